@@ -199,6 +199,7 @@ int kvc_layer_create(const kvc_layer_desc* desc, kvc_layer** out) {
   L->mode = mode;
   L->mk = key_side ? m : desc->n;
   L->mv = value_side ? m : desc->n;
+  L->d_block = nullptr;
   L->d_idx = nullptr;
   L->d_cstatus = nullptr;
   L->d_usum = nullptr;
@@ -208,21 +209,41 @@ int kvc_layer_create(const kvc_layer_desc* desc, kvc_layer** out) {
     const char* ex = std::getenv("KVC_EXPANSION");
     L->use_tc = !ex ? 0 : (std::strcmp(ex, "tcgen05") == 0 ? 1 : (std::strcmp(ex, "pair") == 0 ? 2 : (std::strcmp(ex, "mma") == 0 ? -1 : (std::strcmp(ex, "phases") == 0 ? -2 : (std::strcmp(ex, "split") == 0 ? 3 : (std::strcmp(ex, "resident") == 0 ? 4 : 0))))));
   }
-  if (cudaGetDevice(&L->device) != cudaSuccess ||
-      cudaDeviceGetAttribute(&L->num_sms, cudaDevAttrMultiProcessorCount, L->device) != cudaSuccess ||
-      cudaMalloc(&L->d_idx, idx.size() * sizeof(int32_t)) != cudaSuccess ||
-      cudaMemcpy(L->d_idx, idx.data(), idx.size() * sizeof(int32_t), cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMalloc(&L->d_cstatus, sizeof(int)) != cudaSuccess ||
-      cudaMemset(L->d_cstatus, 0, sizeof(int)) != cudaSuccess ||
-      (!pass && value_side && (cudaMalloc(&L->d_usum, idx.size() * sizeof(float)) != cudaSuccess ||
-                 compute_usum(L, L->d_usum) != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess))) {
-    if (L->d_idx) cudaFree(L->d_idx);
-    if (L->d_cstatus) cudaFree(L->d_cstatus);
-    if (L->d_usum) cudaFree(L->d_usum);
+  // one allocation: index set, status word, row sums of U, and copies of theta and U with rows the TMA engine can address
+  // where n is not a multiple of 64 (bf16)
+  L->np = (int)align_up((size_t)desc->n, 64);
+  L->theta_rows = key_side && !pass ? desc->theta : nullptr;
+  L->U_rows = value_side && !pass ? desc->U : nullptr;
+  const bool pad = desc->dtype == KVC_BF16 && !pass && L->np != desc->n;
+  if (!pad) L->np = desc->n;
+  const size_t rows = (size_t)desc->H_kv * m, padded = rows * L->np * sizeof(__nv_bfloat16);
+  size_t bytes = 0;
+  auto take = [&](size_t b) { const size_t o = bytes; bytes = align_up(bytes + b, 256); return o; };
+  const size_t o_idx = take(rows * sizeof(int32_t)), o_status = take(sizeof(int));
+  const size_t o_usum = take(!pass && value_side ? rows * sizeof(float) : 0);
+  const size_t o_theta = take(pad && key_side ? padded : 0), o_U = take(pad && value_side ? padded : 0);
+  cudaError_t e = cudaGetDevice(&L->device);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&L->num_sms, cudaDevAttrMultiProcessorCount, L->device);
+  if (e == cudaSuccess) e = cudaMalloc(&L->d_block, bytes);
+  if (e == cudaSuccess) {
+    char* base = static_cast<char*>(L->d_block);
+    L->d_idx = reinterpret_cast<int32_t*>(base + o_idx);
+    L->d_cstatus = reinterpret_cast<int*>(base + o_status);
+    e = cudaMemcpy(L->d_idx, idx.data(), idx.size() * sizeof(int32_t), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemset(L->d_cstatus, 0, sizeof(int));
+    if (e == cudaSuccess && !pass && value_side) {
+      L->d_usum = reinterpret_cast<float*>(base + o_usum);
+      e = compute_usum(L, L->d_usum);
+    }
+    if (e == cudaSuccess && pad && key_side) { L->theta_rows = base + o_theta; e = pad_params(desc->theta, base + o_theta, (long long)rows, desc->n, L->np, nullptr); }
+    if (e == cudaSuccess && pad && value_side) { L->U_rows = base + o_U; e = pad_params(desc->U, base + o_U, (long long)rows, desc->n, L->np, nullptr); }
+    if (e == cudaSuccess && !pass) e = cudaDeviceSynchronize();
+  }
+  if (e != cudaSuccess) {
+    if (L->d_block) cudaFree(L->d_block);
     map_cache_destroy(L->maps);
     delete L;
-    cudaGetLastError();
-    return KVC_ERR_CUDA;
+    return cuda_status(e);
   }
   *out = L;
   return KVC_OK;
@@ -230,9 +251,7 @@ int kvc_layer_create(const kvc_layer_desc* desc, kvc_layer** out) {
 
 int kvc_layer_destroy(kvc_layer* L) {
   if (!L) return KVC_OK;
-  if (L->d_idx) cudaFree(L->d_idx);
-  if (L->d_cstatus) cudaFree(L->d_cstatus);
-  if (L->d_usum) cudaFree(L->d_usum);
+  if (L->d_block) cudaFree(L->d_block);
   map_cache_destroy(L->maps);
   delete L;
   return KVC_OK;
@@ -278,14 +297,17 @@ int kvc_compress(const kvc_layer* L, const void* K_vis, const void* V_vis, int B
   void* Kc = capsules;
   void* Vc = static_cast<char*>(capsules) + kbytes;
   const_cast<kvc_layer*>(L)->capsules_fresh = 1;
-  cudaError_t e = cudaMemsetAsync(L->d_cstatus, 0, sizeof(int), st);   // status word of this compress call
-  if (e != cudaSuccess) return cuda_status(e);
   // a side kept verbatim (rho = 0, or the one-sided modes) is a plain copy of its n rows per block
-  if (L->passthrough || L->mode == KVC_MODE_V_ONLY) e = cudaMemcpyAsync(Kc, K_vis, kbytes, cudaMemcpyDeviceToDevice, st);
-  else e = launch_compress_keys(L, K_vis, B, R, Kc, st);
-  if (e != cudaSuccess) return cuda_status(e);
-  if (L->passthrough || L->mode == KVC_MODE_K_ONLY) e = cudaMemcpyAsync(Vc, V_vis, vbytes, cudaMemcpyDeviceToDevice, st);
-  else e = launch_compress_values(L, V_vis, B, R, Vc, st);
+  const bool k_copy = L->passthrough || L->mode == KVC_MODE_V_ONLY, v_copy = L->passthrough || L->mode == KVC_MODE_K_ONLY;
+  bool used = false;
+  cudaError_t e = cudaSuccess;
+  if (!k_copy || !v_copy)       // bf16: both compressed sides in one kernel, which clears the status word of this call
+    e = launch_compress_tc(L, K_vis, V_vis, B, R, (long long)R * L->desc.n, k_copy ? 0 : 1, v_copy ? 0 : 1, Kc, Vc, nullptr, st, &used);
+  if (e == cudaSuccess && !used) e = cudaMemsetAsync(L->d_cstatus, 0, sizeof(int), st);
+  if (e == cudaSuccess && k_copy) e = cudaMemcpyAsync(Kc, K_vis, kbytes, cudaMemcpyDeviceToDevice, st);
+  if (e == cudaSuccess && !k_copy && !used) e = launch_compress_keys(L, K_vis, B, R, Kc, st);
+  if (e == cudaSuccess && v_copy) e = cudaMemcpyAsync(Vc, V_vis, vbytes, cudaMemcpyDeviceToDevice, st);
+  if (e == cudaSuccess && !v_copy && !used) e = launch_compress_values(L, V_vis, B, R, Vc, st);
   return cuda_status(e);
 }
 
@@ -427,8 +449,6 @@ int kvc_compress_ragged(const kvc_layer* L, const void* K_vis, const void* V_vis
     return KVC_ERR_ARG;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const_cast<kvc_layer*>(L)->capsules_fresh = 1;
-  cudaError_t e = cudaMemsetAsync(L->d_cstatus, 0, sizeof(int), st);
-  if (e != cudaSuccess) return cuda_status(e);
   void* Vc = capsules ? static_cast<char*>(capsules) + key_part_bytes(L, B, R_max) : nullptr;
   return cuda_status(launch_compress_ragged(L, K_vis, V_vis, B, N_cap, N_v, R_max, capsules, Vc, K_tail, V_tail, T_cap,
                                             R_b, T_b, st));

@@ -94,6 +94,41 @@ __global__ void __launch_bounds__(256) project_values_kernel(const T* __restrict
   }
 }
 
+// row sums of U (fp32), one warp per row
+template <typename T>
+__global__ void __launch_bounds__(256) usum_kernel(const T* __restrict__ U, float* __restrict__ usum, int rows, int n) {
+  const int row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (row >= rows) return;
+  float s = 0.f;
+  for (int i = lane; i < n; i += 32) s += to_f32(U[(size_t)row * n + i]);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (lane == 0) usum[row] = s;
+}
+
+cudaError_t compute_usum(const kvc_layer* L, float* usum) {
+  const int rows = L->desc.H_kv * L->m;
+  if (L->desc.dtype == KVC_BF16)
+    usum_kernel<__nv_bfloat16><<<ceil_div(rows, 8), 256>>>(static_cast<const __nv_bfloat16*>(L->desc.U), usum, rows, L->desc.n);
+  else
+    usum_kernel<float><<<ceil_div(rows, 8), 256>>>(static_cast<const float*>(L->desc.U), usum, rows, L->desc.n);
+  return cudaGetLastError();
+}
+
+// dst [rows][np] = src [rows][n], zeros behind n (bf16)
+__global__ void __launch_bounds__(256) pad_params_kernel(const __nv_bfloat16* __restrict__ src, __nv_bfloat16* __restrict__ dst,
+                                                         long long rows, int n, int np) {
+  const long long row = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (row >= rows) return;
+  for (int i = threadIdx.x & 31; i < np; i += 32) dst[row * np + i] = i < n ? src[row * n + i] : __float2bfloat16_rn(0.f);
+}
+
+cudaError_t pad_params(const void* src, void* dst, long long rows, int n, int np, cudaStream_t st) {
+  pad_params_kernel<<<(unsigned)((rows + 7) / 8), 256, 0, st>>>(static_cast<const __nv_bfloat16*>(src), static_cast<__nv_bfloat16*>(dst),
+                                                              rows, n, np);
+  return cudaGetLastError();
+}
+
 template <typename T>
 static cudaError_t launch_keys_t(const kvc_layer* L, const void* K_vis, int B, int R, void* Kc, cudaStream_t st) {
   constexpr int RPI = 32 / (D / Elems16<T>::N);
@@ -109,15 +144,7 @@ static cudaError_t launch_keys_t(const kvc_layer* L, const void* K_vis, int B, i
 template <typename T>
 static cudaError_t launch_values_t(const kvc_layer* L, const void* V_vis, int B, int R, void* Vc, cudaStream_t st) {
   const int H_kv = L->desc.H_kv, n = L->desc.n, m = L->m;
-  cudaError_t e;
   ProfScope prof(KVC_KERNEL_PROJECT_VALUES, st);
-  {
-    bool used = false;
-    e = launch_project_values_tc(L, V_vis, B, R, Vc, st, &used);       // bf16: tcgen05, accumulator in tensor memory
-    if (used || e != cudaSuccess) return e;
-    e = launch_project_values_mma(L, V_vis, B, R, Vc, st, &used);      // bf16: mma.sync (kept as the comparison kernel)
-    if (used || e != cudaSuccess) return e;
-  }
   dim3 grid((unsigned)(B * H_kv * R), (unsigned)ceil_div(m, 32));
   project_values_kernel<T><<<grid, 256, 0, st>>>(static_cast<const T*>(V_vis), static_cast<T*>(Vc),
                                                  static_cast<const T*>(L->desc.U),
@@ -208,9 +235,22 @@ static cudaError_t launch_ragged_t(const kvc_layer* L, const void* K_vis, const 
   return e;
 }
 
+// bf16 takes the one-kernel path of kvc_compress_tc.cu (which clears and sets the status word itself); fp32 storage, pointers that
+// are not 16-byte aligned and batches of more sequences than its table holds the kernels above
 cudaError_t launch_compress_ragged(const kvc_layer* L, const void* K_vis, const void* V_vis, int B, int N_cap,
                                    const int* N_v, int R_max, void* Kc, void* Vc, void* K_tail, void* V_tail, int T_cap,
                                    int* R_b, int* T_b, cudaStream_t st) {
+  {
+    const RaggedCompress rag{N_v, N_cap, T_cap, R_b, T_b, K_tail, V_tail};
+    bool used = false;
+    const cudaError_t e = launch_compress_tc(L, K_vis, V_vis, B, R_max, N_cap, L->passthrough || L->mode == KVC_MODE_V_ONLY ? 2 : 1,
+                                             L->passthrough || L->mode == KVC_MODE_K_ONLY ? 2 : 1, Kc, Vc, &rag, st, &used);
+    if (used || e != cudaSuccess) return e;
+  }
+  {
+    const cudaError_t e = cudaMemsetAsync(L->d_cstatus, 0, sizeof(int), st);
+    if (e != cudaSuccess) return e;
+  }
   return L->desc.dtype == KVC_BF16
              ? launch_ragged_t<__nv_bfloat16>(L, K_vis, V_vis, B, N_cap, N_v, R_max, Kc, Vc, K_tail, V_tail, T_cap, R_b, T_b, st)
              : launch_ragged_t<float>(L, K_vis, V_vis, B, N_cap, N_v, R_max, Kc, Vc, K_tail, V_tail, T_cap, R_b, T_b, st);

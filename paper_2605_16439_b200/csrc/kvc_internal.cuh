@@ -121,6 +121,12 @@ struct kvc_layer {
   int32_t* d_idx;        // device [H_kv][m]
   int* d_cstatus;        // device status word of the compress kernels (cleared by every kvc_compress call)
   float* d_usum;         // device [H_kv][m] row sums of U (value compression:  U (V - 1 mu^T) = U V - (U 1) mu^T)
+  // theta and U as tensor maps can address them (bf16): [H_kv][m][np].  The caller's own arrays where n is a multiple of 64
+  // (np = n), otherwise zero-padded copies made when the handle is created (np = n rounded up to 64); nullptr where a side has none
+  int np;
+  const void* theta_rows;
+  const void* U_rows;
+  void* d_block;         // the one device allocation behind d_idx, d_cstatus, d_usum and the padded copies
   kvc_map_cache* maps;   // host: tensor maps keyed by (B, R, capsule pointer, launch plan); guarded by its own mutex
 };
 
@@ -249,8 +255,22 @@ void launch_wait_selftest(int* status, cudaStream_t st);   // one warp, a wait t
 kvc_map_cache* map_cache_create();
 void map_cache_destroy(kvc_map_cache* c);
 cudaError_t compute_usum(const kvc_layer* L, float* usum);
-cudaError_t launch_project_values_tc(const kvc_layer* L, const void* V_vis, int B, int R, void* Vc, cudaStream_t st, bool* used);
-cudaError_t launch_project_values_mma(const kvc_layer* L, const void* V_vis, int B, int R, void* Vc, cudaStream_t st, bool* used);
+// per-sequence lengths of a compress call (see kvc_compress_ragged)
+struct RaggedCompress {
+  const int* N_v;
+  int N_cap, T_cap;
+  int* R_b;
+  int* T_b;
+  void* K_tail;
+  void* V_tail;
+};
+// theta_rows / U_rows can be read by the TMA engine
+inline bool padded_params_ok(const kvc_layer* L) {
+  return ((reinterpret_cast<uintptr_t>(L->theta_rows) | reinterpret_cast<uintptr_t>(L->U_rows)) & 15) == 0;
+}
+cudaError_t pad_params(const void* src, void* dst, long long rows, int n, int np, cudaStream_t st);
+cudaError_t launch_compress_tc(const kvc_layer* L, const void* K_vis, const void* V_vis, int B, int R, long long pitch, int keys,
+                               int values, void* Kc, void* Vc, const RaggedCompress* rag, cudaStream_t st, bool* used);
 cudaError_t launch_compress_ragged(const kvc_layer* L, const void* K_vis, const void* V_vis, int B, int N_cap,
                                    const int* N_v, int R_max, void* Kc, void* Vc, void* K_tail, void* V_tail, int T_cap,
                                    int* R_b, int* T_b, cudaStream_t st);
