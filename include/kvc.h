@@ -93,9 +93,10 @@ KVC_API int kvc_retained_len(int n, int ratio_permille);
  * The device that is current at this call must be current for every later call with the handle.
  * bf16 decode calls run Alg. 1 either as one kernel (steps 2-3 on mma.sync with the logits in registers, or on tcgen05
  * with the logits in tensor memory) or, for block lengths above 640, as three kernels (streaming scores, tcgen05
- * expansion per 128 rows and range of the n axis, streaming output); the library picks per shape (same results within
- * the bf16 tolerance).  The environment variable KVC_EXPANSION = "tcgen05" | "mma" | "pair" | "split" | "resident", read when the
- * handle is created, forces one of them where it applies ("pair": the tcgen05 one-kernel path run by clusters of two
+ * expansion per 128 rows and range of the n axis, streaming output), or, for other block lengths and per-sequence lengths, as
+ * one kernel of CTA clusters that share the n axis; the library picks per shape (same results within
+ * the bf16 tolerance).  The environment variable KVC_EXPANSION = "tcgen05" | "mma" | "pair" | "split" | "resident" | "cluster", read
+ * when the handle is created, forces one of them where it applies ("pair": the tcgen05 one-kernel path run by clusters of two
  * CTAs per (sequence, KV head)); "phases" forces the generic three-phase kernels that also serve fp32 storage. */
 KVC_API int kvc_layer_create(const kvc_layer_desc* desc, kvc_layer** out);
 KVC_API int kvc_layer_destroy(kvc_layer* layer);

@@ -10,6 +10,7 @@
 #include "kvc_internal.cuh"
 #include "kvc_split.cuh"
 #include "kvc_resident.cuh"
+#include "kvc_cluster.cuh"
 
 namespace kvc {
 
@@ -207,7 +208,7 @@ int kvc_layer_create(const kvc_layer_desc* desc, kvc_layer** out) {
   L->num_sms = 0;
   {
     const char* ex = std::getenv("KVC_EXPANSION");
-    L->use_tc = !ex ? 0 : (std::strcmp(ex, "tcgen05") == 0 ? 1 : (std::strcmp(ex, "pair") == 0 ? 2 : (std::strcmp(ex, "mma") == 0 ? -1 : (std::strcmp(ex, "phases") == 0 ? -2 : (std::strcmp(ex, "split") == 0 ? 3 : (std::strcmp(ex, "resident") == 0 ? 4 : 0))))));
+    L->use_tc = !ex ? 0 : (std::strcmp(ex, "tcgen05") == 0 ? 1 : (std::strcmp(ex, "pair") == 0 ? 2 : (std::strcmp(ex, "mma") == 0 ? -1 : (std::strcmp(ex, "phases") == 0 ? -2 : (std::strcmp(ex, "split") == 0 ? 3 : (std::strcmp(ex, "resident") == 0 ? 4 : (std::strcmp(ex, "cluster") == 0 ? 5 : 0)))))));
   }
   // one allocation: index set, status word, row sums of U, and copies of theta and U with rows the TMA engine can address
   // where n is not a multiple of 64 (bf16)
@@ -284,7 +285,8 @@ size_t kvc_capsule_bytes(const kvc_layer* L, int B, int R) {
 
 size_t kvc_workspace_bytes(const kvc_layer* L, int B, int R, int T_cap) {
   if (!L || B < 0 || R < 0 || T_cap < 0) return 0;
-  return ws_layout(L, B, R, T_cap).total;
+  const size_t phases = ws_layout(L, B, R, T_cap).total, cluster = cluster_ws_bytes(L, B, R, T_cap);
+  return phases > cluster ? phases : cluster;
 }
 
 int kvc_compress(const kvc_layer* L, const void* K_vis, const void* V_vis, int B, int R, void* capsules,
@@ -324,6 +326,24 @@ static bool use_split(const kvc_layer* L, int B, int R) {
   return plan_split(L, B, R).ok != 0;
 }
 
+// Which bf16 shapes take the cluster path: those that the one-kernel and three-kernel paths do not serve (per-sequence lengths, block
+// lengths that are no multiple of 64) and whose expansions are worth its chain of hand-overs.  Measured on B200, us per call, three-phase
+// kernels -> cluster path: where those kernels expand on the CUDA cores (n no multiple of 8) it is ahead at every shape tried
+// (8 sequences x 5 blocks of n = 729, 28/4 heads: 277 -> 51; 1 x 1 block: 75 -> 33; 1 x 4 blocks of n = 81, 8/2 heads: 27 -> 22); where
+// they expand on mma.sync it is from about 1.5e8 flop of expansion per call on (lengths per sequence: 8 x 8 blocks of n = 1024: 154 ->
+// 58, 1 x 4: 43 -> 40; uniform 16 x 8 blocks of n = 400, 8/2 heads, 3.3e8: 45 -> 45; 1 x 2 of n = 144, 32/32 heads, 2e6: 17 -> 21) unless
+// each KV head has one query head, whose few rows leave its 128-row tiles empty (8 x 5 of n = 576, 32/32 heads: 70 -> 88).
+// KVC_EXPANSION=cluster forces it where its plan applies, any other value of the variable keeps it off.
+static bool use_cluster(const kvc_layer* L, int B, int R, bool ragged) {
+  if (R < 1 || L->passthrough || L->mode != KVC_MODE_KV || L->desc.dtype != KVC_BF16) return false;
+  if (L->use_tc == 5) return true;
+  const int n = L->desc.n;
+  if (L->use_tc != 0 || n < 64 || (!ragged && n % 64 == 0)) return false;
+  if (ragged && (n == 64 || n == 128 || n == 192 || n == 256) && plan_resident(L, B, R, 0).ok) return false;     // read the lengths itself
+  if (cluster_prec(L, ragged) == 2) return true;
+  return L->G > 1 && 4.0 * B * L->desc.H_q * R * (double)L->m * n >= 1.5e8;
+}
+
 // One token per decode call, process-wide: never 0 and never one of the byte patterns a caller is likely to have
 // filled a fresh workspace with, so that stale workspace contents cannot pass for arrivals of this call.
 static unsigned int next_token() {
@@ -338,7 +358,7 @@ static unsigned int next_token() {
 
 int decode_common(const kvc_layer* L, const void* q, const void* capsules, int B, int R, const void* K_txt,
                   const void* V_txt, int T, int T_cap, void* out, void* workspace, cudaStream_t st, const int* R_b,
-                  const int* T_b) {
+                  const int* T_b, size_t ws_limit) {
   if (!L || B < 0 || R < 0 || T < 0 || T_cap < T) return KVC_ERR_ARG;
   if (B == 0) return KVC_OK;
   if (R == 0 && T == 0) return KVC_ERR_SHAPE;
@@ -346,7 +366,6 @@ int decode_common(const kvc_layer* L, const void* q, const void* capsules, int B
   if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 255)) return KVC_ERR_WORKSPACE;
 
   DecodeArgs a{};
-  a.ws = ws_layout(L, B, R, T);
   char* ws = static_cast<char*>(workspace);
   a.q = q;
   a.Kc = capsules;
@@ -357,8 +376,30 @@ int decode_common(const kvc_layer* L, const void* q, const void* capsules, int B
   a.B = B; a.H_kv = L->desc.H_kv; a.G = L->G; a.R = R; a.m = L->mk; a.ms = (L->mk + 15) / 16 * 16; a.n = L->desc.n;
   a.mv = L->mv; a.msv = (L->mv + 15) / 16 * 16;
   a.id_theta = L->mode == KVC_MODE_V_ONLY; a.id_U = L->mode == KVC_MODE_K_ONLY;
-  a.T = T; a.T_cap = T_cap > 0 ? T_cap : 1; a.Ts = a.ws.Ts;
+  a.T = T; a.T_cap = T_cap > 0 ? T_cap : 1;
   a.passthrough = L->passthrough;
+  a.token = next_token();
+  a.cnt = reinterpret_cast<int*>(ws);                       // counters and the status word lead the workspace on every path
+  a.status = a.cnt + (size_t)B * L->desc.H_kv;
+  a.R_b = R_b; a.T_b = T_b;
+  a.early_capsules = L->capsules_fresh ? 0 : 1;
+  const_cast<kvc_layer*>(L)->capsules_fresh = 0;
+  const bool ragged = R_b != nullptr || T_b != nullptr;
+  const uintptr_t align = reinterpret_cast<uintptr_t>(q) | reinterpret_cast<uintptr_t>(capsules) |
+                          reinterpret_cast<uintptr_t>(out) | (T > 0 ? reinterpret_cast<uintptr_t>(K_txt) |
+                          reinterpret_cast<uintptr_t>(V_txt) : 0) | reinterpret_cast<uintptr_t>(L->desc.mu);
+
+  if ((align & 15) == 0 && use_cluster(L, B, R, ragged)) {
+    const ClusterPlan cp = plan_cluster(L, B, R, T, ragged);
+    if (cp.ok && (ws_limit == 0 || cluster_ws(L, cp, B, R).bytes <= ws_limit)) {
+      bool encoded = false;
+      const cudaError_t ce = launch_cluster(L, a, cp, ws, st, &encoded);
+      if (encoded) return cuda_status(ce);
+    }
+  }
+
+  a.ws = ws_layout(L, B, R, T);
+  a.Ts = a.ws.Ts;
   a.S = reinterpret_cast<float*>(ws + a.ws.off_S);
   a.Sb = reinterpret_cast<__nv_bfloat16*>(ws + a.ws.off_S);
   a.s_txt = reinterpret_cast<float*>(ws + a.ws.off_stxt);
@@ -368,17 +409,11 @@ int decode_common(const kvc_layer* L, const void* q, const void* capsules, int B
   a.statc = reinterpret_cast<float4*>(ws + a.ws.off_statc);
   a.ypart = reinterpret_cast<float*>(ws + a.ws.off_ypart);
   a.ystat = reinterpret_cast<float2*>(ws + a.ws.off_ystat);
-  a.cnt = reinterpret_cast<int*>(ws + a.ws.off_cnt);
   a.fcnt = reinterpret_cast<unsigned long long*>(ws + a.ws.off_fcnt);
-  a.token = next_token();
-  a.status = a.cnt + (size_t)B * L->desc.H_kv;
   a.fpart_y = reinterpret_cast<float*>(ws + a.ws.off_fpy);
   a.fpart_ml = reinterpret_cast<float2*>(ws + a.ws.off_fpml);
   a.split_base = ws + a.ws.off_split;
   a.resident_base = ws + a.ws.off_resident;
-  a.R_b = R_b; a.T_b = T_b;
-  a.early_capsules = L->capsules_fresh ? 0 : 1;
-  const_cast<kvc_layer*>(L)->capsules_fresh = 0;
 
   // bf16 storage with TMA-compatible shapes and pointers: the whole of Algorithm 1 in one kernel
   {
@@ -387,11 +422,7 @@ int decode_common(const kvc_layer* L, const void* q, const void* capsules, int B
     const bool plain = R == 0 || L->passthrough;
     // one-sided modes are served by the three-phase kernels below; so are per-sequence lengths, except on the shapes the
     // resident-parameter kernel takes (it reads the lengths itself)
-    const bool ragged = R_b != nullptr || T_b != nullptr;
     const bool one_sided = (R > 0 && L->mode != KVC_MODE_KV) || ragged;
-    const uintptr_t align = reinterpret_cast<uintptr_t>(q) | reinterpret_cast<uintptr_t>(capsules) |
-                            reinterpret_cast<uintptr_t>(out) | (T > 0 ? reinterpret_cast<uintptr_t>(K_txt) |
-                            reinterpret_cast<uintptr_t>(V_txt) : 0) | reinterpret_cast<uintptr_t>(L->desc.mu);
     // Short blocks whose theta and U fit shared memory (n <= 256, m <= 128, G <= 8) take the resident-parameter kernel: on
     // the n = 256, G = 7, m = 103 shape it ran ahead of the other one-kernel variants at every batch measured (1, 4, 16:
     // 19.2 / 19.5 / 42.4 us against 22.4 / 23.5 / 83.7 us).  KVC_EXPANSION=resident forces it, any other value keeps it off.

@@ -203,7 +203,8 @@ __device__ __forceinline__ void check_seq_lengths(const DecodeArgs& a, int tid, 
 // scratch of ws_layout(L, B, R, T).total bytes
 int decode_common(const kvc_layer* L, const void* q, const void* capsules, int B, int R, const void* K_txt,
                   const void* V_txt, int T, int T_cap, void* out, void* workspace, cudaStream_t st,
-                  const int* R_b = nullptr, const int* T_b = nullptr);
+                  const int* R_b = nullptr, const int* T_b = nullptr, size_t ws_limit = 0);   // ws_limit: bytes of the scratch, 0: as many
+                                                                                              // as kvc_workspace_bytes says
 
 // Raises a kernel's dynamic shared-memory limit to at least `bytes` on the current device.  The attribute is per device
 // (and per kernel), so the record of what has been set is keyed by (kernel, device ordinal); safe from several host threads.

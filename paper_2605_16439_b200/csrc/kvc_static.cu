@@ -54,7 +54,7 @@ int kvc_decode_attend_static(const kvc_layer* L, const void* q, const void* caps
   const int s = scratch_for_current_device(&scratch);
   if (s != KVC_OK) return s;
   return kvc::decode_common(L, q, capsules, B, R, K_txt, V_txt, T, T_cap, out, scratch,
-                            static_cast<cudaStream_t>(stream));
+                            static_cast<cudaStream_t>(stream), nullptr, nullptr, (size_t)KVC_STATIC_SCRATCH_BYTES);
 }
 
 }  // extern "C"

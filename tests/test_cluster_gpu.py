@@ -1,0 +1,105 @@
+"""The cluster decode path (clusters of CTAs that share the n axis of a KV head's blocks) at the sizes where its tiling can go
+wrong, against the fp64 oracle: block lengths around the 64-column groups and the cluster sizes they give, retained lengths around
+the 64-row tiles and beyond 512 (two passes over the weights), units of many sequences and of a few blocks, more units than one wave,
+text lengths around a chunk and beyond sixteen of them, per-sequence lengths with nothing in some sequences.
+
+Bound: the regression bound of the parity tests; shapes whose operands are kept as two bf16 terms (16 bits) stay within it by a
+wide margin, their error is the rounding of the output.
+"""
+import random
+
+import pytest
+import torch
+
+from oracle import kvcapsule_oracle as orc
+from paper_2605_16439_b200 import binding as kvc
+from paper_2605_16439_b200 import build as kvc_build
+from paper_2605_16439_b200 import workloads as wl
+
+import kvc_testlib as tl
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda"
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    kvc_build.build()
+
+
+def _launches(fn):
+    kvc.kvc_profile_start(64)
+    try:
+        out = fn()
+        torch.cuda.synchronize()
+    finally:
+        kvc.kvc_profile_stop()
+    counts = {k: v[1] for k, v in kvc.kvc_profile_read().items()}
+    kvc.kvc_profile_start(0)
+    kvc.kvc_profile_stop()
+    return counts, out
+
+
+@pytest.mark.parametrize("recipe", ["peaked", "structured"])
+@pytest.mark.parametrize("B,H_q,H_kv,grid,R,T,ratio", [
+    (1, 1, 1, 8, 1, 0, 600),         # n = 64: one CTA per cluster, one tile, no text
+    (2, 7, 1, 9, 3, 1, 600),         # n = 81: two groups, the second with 17 columns
+    (1, 8, 2, 16, 2, 127, 500),      # n = 256, m = 128: exactly two tiles
+    (3, 12, 2, 17, 2, 128, 775),     # n = 289, m = 66: two rows in the second tile
+    (2, 28, 4, 27, 3, 129, 600),     # n = 729
+    (1, 4, 2, 31, 2, 40, 300),       # n = 961, m = 673: two passes over the weights
+    (37, 2, 2, 10, 1, 20, 600),      # many sequences per unit
+    (40, 16, 8, 13, 3, 3, 600),      # more units than one wave
+    (1, 2, 1, 12, 1, 2200, 600),     # text beyond sixteen chunks
+    (2, 16, 1, 11, 9, 30, 800),      # G = 16
+])
+def test_uniform(B, H_q, H_kv, grid, R, T, ratio, recipe, monkeypatch):
+    monkeypatch.setenv("KVC_EXPANSION", "cluster")
+    shape = wl.Shape("cluster", 1, B, H_q, H_kv, 128, grid, R, T, 1, "bf16", ratio)
+    p = tl.make_problem(shape, 700 + grid + B, T=T, T_cap=T + 3, recipe=recipe)
+    counts, (_, _, _, out) = _launches(lambda: tl.gpu_run(shape, p))
+    assert counts["fused"] == 1 and counts["scores"] == 0
+    tl.assert_close(tl.np64(out), tl.oracle_run(shape, p, "fused")[2], "bf16")
+
+
+@pytest.mark.parametrize("B,H_q,H_kv,grid,R,T,ratio", [
+    (9, 14, 2, 24, 3, 150, 600), (35, 8, 2, 9, 2, 40, 600), (4, 7, 1, 32, 3, 300, 200), (3, 6, 2, 15, 4, 64, 500),
+])
+def test_per_sequence_lengths(B, H_q, H_kv, grid, R, T, ratio, monkeypatch):
+    monkeypatch.setenv("KVC_EXPANSION", "cluster")
+    rng = random.Random(grid)
+    R_b = [rng.randint(0, R) for _ in range(B)]
+    T_b = [rng.choice([0, 1, T, rng.randint(0, T)]) for _ in range(B)]
+    R_b[1], T_b[1] = 0, 0                              # nothing at all: a zero output row
+    R_b[-1] = R
+    shape = wl.Shape("cluster-ragged", 1, B, H_q, H_kv, 128, grid, R, T, 1, "bf16", ratio)
+    p = tl.make_problem(shape, 800 + grid, T=T, T_cap=T, recipe="peaked")
+    layer = tl.gpu_layer(shape, p)
+    caps = kvc.alloc_capsules(layer, B, R)
+    kvc.kvc_compress(layer, p["K_vis"].to(DEV), p["V_vis"].to(DEV), B, R, caps)
+    K_g, V_g = kvc.capsule_views(layer, caps, B, R)
+    K_txt, V_txt = p["K_txt"].to(DEV), p["V_txt"].to(DEV)
+    for b in range(B):                                 # whatever lies past a sequence's lengths must not be used
+        K_g[b, :, R_b[b]:] = float("nan"); V_g[b, :, R_b[b]:] = float("nan")
+        K_txt[b, :, T_b[b]:] = float("nan"); V_txt[b, :, T_b[b]:] = float("nan")
+    kvc.kvc_layer_capsules_written(layer)
+    ws = kvc.alloc_workspace(layer, B, R, T)
+    ws.fill_(0xFF)
+    out = torch.full((B, H_q, 128), float("nan"), dtype=torch.bfloat16, device=DEV)
+    i32 = lambda x: torch.tensor(list(x), dtype=torch.int32, device=DEV)
+    run = lambda: kvc.kvc_decode_attend_ragged(layer, p["q"].to(DEV), caps, B, R, i32(R_b), K_txt, V_txt, T, i32(T_b), T, out, ws)
+    counts, _ = _launches(run)
+    assert counts["fused"] == 1 and counts["scores"] == 0
+    run()                                              # a second call on the same workspace
+    torch.cuda.synchronize()
+    assert kvc.kvc_read_device_status(layer, B, R, T, ws) == 0
+    K_o, V_o = orc.compress(tl.np64(p["K_vis"]), tl.np64(p["V_vis"]), p["idx"].numpy(), tl.np64(p["U"]), tl.np64(p["mu"]), shape.n, False)
+    want = orc.decode_attend_ragged(tl.np64(p["q"]), K_o, V_o, tl.np64(p["theta"]), tl.np64(p["U"]), tl.np64(p["mu"]),
+                                    tl.np64(p["K_txt"]), tl.np64(p["V_txt"]), R_b, T_b, "kv")
+    tl.assert_close(tl.np64(out), want, "bf16")
+    assert (tl.np64(out)[1] == 0).all()
+    # a length out of range is clamped and reported
+    R_b[0] = R + 1
+    run()
+    torch.cuda.synchronize()
+    assert kvc.kvc_read_device_status(layer, B, R, T, ws) == -8
