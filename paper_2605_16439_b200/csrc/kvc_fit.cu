@@ -4,12 +4,16 @@
 //     (= the top m left singular vectors of the pooled centred columns);
 //   the key reconstructor for a fixed retained index set as the minimiser of the reconstruction term of Alg. 2:
 //     theta = (K_r K_r^T)^+ K_r K^T with K_r the retained rows, the pseudo-inverse taken through the eigen-decomposition.
-// Both rest on one hand-written solver: the cyclic Jacobi method for symmetric matrices with the round-robin ordering,
-// in which the n/2 rotations of a round act on disjoint index pairs, so a round is one data-parallel update
-// A <- J^T A J, Q <- Q J in which every 2 x 2 block of A is transformed in place by the rotations of its row pair and
-// its column pair.
+// Both rest on a hand-written Jacobi solver for symmetric positive semidefinite matrices, in two forms:
+//   up to 640 indices  one-sided (Hestenes): the columns of A + tau I are rotated in pairs until they are orthogonal; they then are
+//                      sigma_i u_i with u_i the eigenvectors and sigma_i - tau the eigenvalues.  One launch, a cluster of CTAs per
+//                      matrix (see jacobi_cluster_kernel)
+//   beyond             two-sided cyclic with the round-robin ordering: the n/2 rotations of a round act on disjoint index pairs, so a
+//                      round is one data-parallel update A <- J^T A J, Q <- Q J in which every 2 x 2 block of A is transformed in
+//                      place by the rotations of its row pair and its column pair (two launches per round)
 #include <vector>
 
+#include "kvc_async.cuh"
 #include "kvc_internal.cuh"
 
 namespace kvc {
@@ -17,6 +21,7 @@ namespace kvc {
 constexpr int FIT_TILE = 64;            // covariance tile per CTA
 constexpr int FIT_KC = 32;              // channels per staged chunk
 constexpr int FIT_MAX_SWEEPS = 40;
+constexpr float FIT_COS_TOL2 = 1e-20f;  // one-sided: stop after a sweep whose largest squared cosine between two columns was below this
 constexpr double FIT_OFF_TOL2 = 1e-22;  // stop when (off-diagonal norm / diagonal norm)^2 falls below this
 
 static inline int even_up(int x) { return (x + 1) & ~1; }
@@ -33,6 +38,7 @@ struct FitLayout {
   size_t off_idx;         // [ne] ints
   size_t off_norm;        // [2]: off-diagonal and diagonal sums of squares
   size_t off_sum;         // [D]
+  size_t off_flag;        // 64 floats: largest squared cosine of every sweep; an int at [60]: sweeps taken (one-sided solver)
   size_t per_head;
 };
 
@@ -49,6 +55,7 @@ static FitLayout fit_layout(int n) {
   f.off_idx = off; off += f.ne;
   f.off_norm = off; off += 2;
   f.off_sum = off; off += D;
+  f.off_flag = off; off += 32;
   f.per_head = (off + 31) / 32 * 32;
   return f;
 }
@@ -352,10 +359,228 @@ __global__ void __launch_bounds__(256) fit_emit_theta_kernel(const double* __res
   if (j0 + ty < m && c0 + tx < n) store_elem(theta + ((size_t)h * m + j0 + ty) * n + c0 + tx, (float)acc);
 }
 
+// ---- one-sided Jacobi, one launch ----------------------------------------------------------------------------------------
+// Bound: latency of a rotation (three dot products over a column reduced across a warp, two double-precision divisions and a root,
+// then the update), n - 1 of them one after the other per sweep whatever the machine's width, about 14 sweeps.  So everything else is
+// taken out of that chain: a cluster of C CTAs owns a matrix, its columns form 2 C blocks of bs, in each of the 2 C - 1 rounds of a
+// sweep a CTA holds two blocks in shared memory (a warp per pair, the first block's column kept in registers) and rotates all pairs
+// between them (in the first round also those inside), and between rounds the columns go through L2 behind one cluster barrier; no
+// launch, no host round trip.  The two-sided form took two launches per round: 24 + 8 ms for n = 256, m = 103, 4 heads
+// (B200, 8600 launches of 4 us); this one 3 ms.
+// The tangent of a rotation is taken in single precision: it only steers the convergence (off-diagonal cosines fall by 1e-7 at worst per
+// sweep once they are small); cosine and sine are made from it in double precision, so that the rotation is orthogonal.
+// tau = 1e-5 of the largest diagonal entry keeps the columns of a rank-deficient matrix away from zero, so that its null space gets
+// orthonormal vectors too.
+template <int EPL>
+__global__ void __launch_bounds__(640, 1) jacobi_cluster_kernel(double* __restrict__ ws, size_t head_stride, size_t off_A, size_t off_Q,
+                                                                size_t off_flag, int size, int C, int bs) {
+  constexpr int LD = 32 * EPL;
+  extern __shared__ __align__(16) double cols[];                 // [2 bs][LD]
+  __shared__ double s_red[32];
+  __shared__ float s_max[32];
+  const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31, nw = bs;
+  const int h = blockIdx.x / C, c = blockIdx.x - h * C, NB = 2 * C;
+  double* A = ws + (size_t)h * head_stride + off_A;
+  double* Q = ws + (size_t)h * head_stride + off_Q;
+  float* flag = reinterpret_cast<float*>(ws + (size_t)h * head_stride + off_flag);
+  double tau = 0.0;
+  for (int i = tid; i < size; i += nw * 32) tau = fmax(tau, A[(size_t)i * size + i]);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) tau = fmax(tau, __shfl_xor_sync(0xffffffffu, tau, o));
+  if (lane == 0) s_red[w] = tau;
+  __syncthreads();
+  tau = 0.0;
+  for (int x = 0; x < nw; ++x) tau = fmax(tau, s_red[x]);
+  tau = tau > 0.0 ? 1e-5 * tau : 1.0;
+  cluster_sync_all();                                            // every CTA has read the diagonal
+
+  float mx = 0.f;
+  // rotates columns a, b towards orthogonality
+  auto rotate = [&](double (&a)[EPL], double (&b)[EPL]) {
+    double al = 0.0, be = 0.0, ga = 0.0;
+#pragma unroll
+    for (int e = 0; e < EPL; ++e) { al = fma(a[e], a[e], al); be = fma(b[e], b[e], be); ga = fma(a[e], b[e], ga); }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      al += __shfl_xor_sync(0xffffffffu, al, o);
+      be += __shfl_xor_sync(0xffffffffu, be, o);
+      ga += __shfl_xor_sync(0xffffffffu, ga, o);
+    }
+    const float cos2 = (float)(ga * ga / (al * be));             // NaN for a zero column (an index beyond the matrix): no rotation
+    if (!(cos2 > 1e-30f)) return;
+    mx = fmaxf(mx, cos2);
+    const float z = (float)((be - al) / (2.0 * ga));
+    const double t = (double)((z >= 0.f ? 1.f : -1.f) / (fabsf(z) + sqrtf(fmaf(z, z, 1.f))));
+    const double cs = rsqrt(fma(t, t, 1.0)), sn = cs * t;
+#pragma unroll
+    for (int e = 0; e < EPL; ++e) {
+      const double x = a[e], y = b[e];
+      a[e] = cs * x - sn * y;
+      b[e] = sn * x + cs * y;
+    }
+  };
+  auto get = [&](double (&x)[EPL], int slot) {
+#pragma unroll
+    for (int e = 0; e < EPL; ++e) x[e] = cols[(size_t)slot * LD + e * 32 + lane];
+  };
+  auto put = [&](const double (&x)[EPL], int slot) {
+#pragma unroll
+    for (int e = 0; e < EPL; ++e) cols[(size_t)slot * LD + e * 32 + lane] = x[e];
+  };
+  auto fetch = [&](double (&x)[EPL], int col, bool shift) {
+#pragma unroll
+    for (int e = 0; e < EPL; ++e) {
+      const int i = e * 32 + lane;
+      x[e] = col < size && i < size ? __ldcg(A + (size_t)col * size + i) : 0.0;
+      if (shift && i == col && col < size) x[e] += tau;
+    }
+  };
+  auto save = [&](const double (&x)[EPL], int col) {
+#pragma unroll
+    for (int e = 0; e < EPL; ++e) {
+      const int i = e * 32 + lane;
+      if (col < size && i < size) __stcg(A + (size_t)col * size + i, x[e]);
+    }
+  };
+
+  int sweep = 0;
+  for (; sweep < FIT_MAX_SWEEPS;) {
+    mx = 0.f;
+    for (int br = 0; br < NB - 1; ++br) {
+      // round robin over the blocks: block 0 stays, the others move one place per round; place c meets place NB - 1 - c
+      auto at = [&](int pos) { return pos == 0 ? 0 : (pos - 1 - br + 2 * (NB - 1)) % (NB - 1) + 1; };
+      const int p = at(c) * bs + w, q = at(NB - 1 - c) * bs + w;
+      double a[EPL], b[EPL];
+      const bool shift = sweep == 0 && br == 0;
+      fetch(a, p, shift);
+      fetch(b, q, shift);
+      put(b, bs + w);
+      if (br == 0) {
+        put(a, w);
+        __syncthreads();
+        const int n2 = 2 * bs;
+        for (int r = 0; r < n2 - 1; ++r) {
+          auto place = [&](int pos) { return pos == 0 ? 0 : (pos - 1 - r + n2 - 1) % (n2 - 1) + 1; };
+          const int i = place(w), j = place(n2 - 1 - w);
+          get(a, i);
+          get(b, j);
+          rotate(a, b);
+          put(a, i);
+          put(b, j);
+          __syncthreads();
+        }
+        get(a, w);
+      } else {
+        __syncthreads();
+        int slot = bs + w;
+        for (int r = 0; r < bs; ++r) {
+          if (r > 0) get(b, slot);
+          rotate(a, b);
+          put(b, slot);
+          slot = slot + 1 < 2 * bs ? slot + 1 : bs;
+          __syncthreads();
+        }
+      }
+      save(a, p);
+      get(b, bs + w);
+      save(b, q);
+      if (br == NB - 2) {
+        if (lane == 0) s_max[w] = mx;
+        __syncthreads();
+        if (tid == 0) {
+          float m = 0.f;
+          for (int x = 0; x < nw; ++x) m = fmaxf(m, s_max[x]);
+          atomicMax(reinterpret_cast<int*>(flag) + sweep, __float_as_int(m));
+        }
+      }
+      cluster_sync_all();                                        // the columns (and the sweep's maximum) are in L2 for their next owners
+    }
+    const float worst = __ldcg(flag + sweep);
+    ++sweep;
+    if (worst < FIT_COS_TOL2) break;
+  }
+
+  // eigenvalues and eigenvectors: Q[i][col] = column / its length, A[col][col] = length - tau
+  double len[2];
+#pragma unroll
+  for (int x = 0; x < 2; ++x) {
+    const int col = (2 * c + x) * bs + w;
+    double a[EPL], al = 0.0;
+    fetch(a, col, false);
+#pragma unroll
+    for (int e = 0; e < EPL; ++e) al = fma(a[e], a[e], al);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) al += __shfl_xor_sync(0xffffffffu, al, o);
+    len[x] = sqrt(al);
+    const double inv = al > 0.0 ? 1.0 / len[x] : 0.0;
+#pragma unroll
+    for (int e = 0; e < EPL; ++e) {
+      const int i = e * 32 + lane;
+      if (col < size && i < size) Q[(size_t)i * size + col] = a[e] * inv;
+    }
+  }
+  cluster_sync_all();                                            // every column has been read
+#pragma unroll
+  for (int x = 0; x < 2; ++x) {
+    const int col = (2 * c + x) * bs + w;
+    if (lane == 0 && col < size) A[(size_t)col * size + col] = len[x] - tau;
+  }
+  if (c == 0 && tid == 0) reinterpret_cast<int*>(flag)[60] = sweep;
+}
+
+// CTAs of a cluster: blocks of about eight columns, as many CTAs as the device places together (sixteen with the non-portable size)
+template <int EPL>
+static cudaError_t launch_jacobi_cluster(double* ws, size_t head_stride, size_t off_A, size_t off_Q, size_t off_flag, int H, int size,
+                                         cudaStream_t st, bool* used) {
+  const void* fn = reinterpret_cast<const void*>(jacobi_cluster_kernel<EPL>);
+  *used = false;
+  int C = ceil_div(size, 16);
+  C = C > 16 ? 16 : C;
+  const int bs = ceil_div(size, 2 * C);
+  if (bs > 20) return cudaSuccess;
+  const size_t smem = sizeof(double) * 2 * (size_t)bs * 32 * EPL;
+  cudaError_t e = ensure_dynamic_smem(fn, smem);
+  if (e != cudaSuccess) return e;
+  if (C > 8) e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(C * H));
+  cfg.blockDim = dim3((unsigned)(bs * 32));
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)C; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int fit = 0;
+  if (C > 8 && (cudaOccupancyMaxActiveClusters(&fit, fn, &cfg) != cudaSuccess || fit < 1)) { cudaGetLastError(); return cudaSuccess; }
+  *used = true;
+  return cudaLaunchKernelEx(&cfg, jacobi_cluster_kernel<EPL>, ws, head_stride, off_A, off_Q, off_flag, size, C, bs);
+}
+
 // ---- host side -------------------------------------------------------------------------------------------------
 // eigen-decomposition of the size x size matrices at off_A (overwritten by their diagonal form), eigenvectors to off_Q
-static cudaError_t jacobi_eigen(double* ws, size_t head_stride, size_t off_A, size_t off_Q, size_t off_rot, size_t off_norm,
-                                int H, int size, cudaStream_t st, int* sweeps_out) {
+// sweeps: one entry per head, complete when the stream has been synchronised
+static cudaError_t jacobi_eigen(double* ws, const FitLayout& f, size_t off_A, size_t off_Q, int H, int size, cudaStream_t st,
+                                std::vector<int>& sweeps) {
+  const size_t head_stride = f.per_head, off_rot = f.off_rot, off_norm = f.off_norm;
+  sweeps.assign(H, 0);
+  {
+    bool used = false;
+    cudaError_t e = cudaSuccess;
+#define KVC_JACOBI(EPL) launch_jacobi_cluster<EPL>(ws, head_stride, off_A, off_Q, f.off_flag, H, size, st, &used)
+    if (size <= 64) e = KVC_JACOBI(2);
+    else if (size <= 128) e = KVC_JACOBI(4);
+    else if (size <= 256) e = KVC_JACOBI(8);
+    else if (size <= 384) e = KVC_JACOBI(12);
+    else if (size <= 640) e = KVC_JACOBI(20);
+#undef KVC_JACOBI
+    if (e != cudaSuccess) return e;
+    if (used)
+      return cudaMemcpy2DAsync(sweeps.data(), sizeof(int), reinterpret_cast<const int*>(ws + f.off_flag) + 60, head_stride * sizeof(double),
+                               sizeof(int), (size_t)H, cudaMemcpyDeviceToHost, st);
+  }
   fit_identity_kernel<<<dim3(64, H), 256, 0, st>>>(ws, head_stride, off_Q, size);
   cudaError_t e = cudaGetLastError();
   std::vector<double> norms((size_t)2 * H);
@@ -378,7 +603,17 @@ static cudaError_t jacobi_eigen(double* ws, size_t head_stride, size_t off_A, si
     }
     e = cudaGetLastError();
   }
-  if (sweeps_out) *sweeps_out = sweep;
+  sweeps.assign(H, sweep);
+  return e;
+}
+
+// completes a fit: the stream is idle, the sweeps are known
+static cudaError_t finish(cudaStream_t st, const std::vector<int>& sweeps, int* sweeps_out) {
+  const cudaError_t e = cudaStreamSynchronize(st);
+  if (e == cudaSuccess && sweeps_out) {
+    *sweeps_out = 0;
+    for (int s : sweeps) *sweeps_out = s > *sweeps_out ? s : *sweeps_out;
+  }
   return e;
 }
 
@@ -399,14 +634,15 @@ static cudaError_t fit_pca_t(const void* V_vis, int B, int R, int H, int n, int 
   const FitLayout f = fit_layout(n);
   cudaError_t e = moments<T>(static_cast<const T*>(V_vis), B, R, H, n, f, ws, f.off_M[0], true, st);
   if (e != cudaSuccess) return e;
-  e = jacobi_eigen(ws, f.per_head, f.off_M[0], f.off_M[1], f.off_rot, f.off_norm, H, f.ne, st, sweeps);
+  std::vector<int> taken;
+  e = jacobi_eigen(ws, f, f.off_M[0], f.off_M[1], H, f.ne, st, taken);
   if (e != cudaSuccess) return e;
   fit_rank_kernel<<<dim3(ceil_div(f.ne, 128), H), 128, 0, st>>>(ws, f.per_head, f.off_M[0], f.off_lam, f.off_order, f.ne, n);
   fit_emit_basis_kernel<T><<<dim3(eig_out ? n : m, H), 128, 0, st>>>(ws, f.per_head, f.off_M[1], f.off_lam, f.off_order, f.ne, n, m,
                                                                      static_cast<T*>(U_out), eig_out);
   fit_emit_mean_kernel<T><<<H, D, 0, st>>>(ws, f.per_head, f.off_sum, (double)B * R * n, static_cast<T*>(mu_out));
   e = cudaGetLastError();
-  return e != cudaSuccess ? e : cudaStreamSynchronize(st);
+  return e != cudaSuccess ? e : finish(st, taken, sweeps);
 }
 
 template <typename T>
@@ -420,7 +656,8 @@ static cudaError_t fit_theta_t(const void* K_vis, int B, int R, int H, int n, in
                         cudaMemcpyHostToDevice, st);
   if (e != cudaSuccess) return e;
   fit_select_kernel<<<dim3(64, H), 256, 0, st>>>(ws, f.per_head, f.off_M[0], f.off_M[1], f.off_idx, f.ne, me, m);
-  e = jacobi_eigen(ws, f.per_head, f.off_M[1], f.off_M[2], f.off_rot, f.off_norm, H, me, st, sweeps);
+  std::vector<int> taken;
+  e = jacobi_eigen(ws, f, f.off_M[1], f.off_M[2], H, me, st, taken);
   if (e != cudaSuccess) return e;
   fit_pinv_kernel<<<H, 256, 0, st>>>(ws, f.per_head, f.off_M[1], f.off_inv, me, m, rcond);
   fit_project_kernel<<<dim3(ceil_div(n, 16), ceil_div(me, 16), H), 256, 0, st>>>(ws, f.per_head, f.off_M[0], f.off_M[2], f.off_M[3],
@@ -428,7 +665,7 @@ static cudaError_t fit_theta_t(const void* K_vis, int B, int R, int H, int n, in
   fit_emit_theta_kernel<T><<<dim3(ceil_div(n, 16), ceil_div(m, 16), H), 256, 0, st>>>(ws, f.per_head, f.off_M[2], f.off_M[3], f.ne, me, m,
                                                                                     n, static_cast<T*>(theta_out));
   e = cudaGetLastError();
-  return e != cudaSuccess ? e : cudaStreamSynchronize(st);
+  return e != cudaSuccess ? e : finish(st, taken, sweeps);
 }
 
 }  // namespace kvc
