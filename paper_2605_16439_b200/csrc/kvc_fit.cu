@@ -20,6 +20,7 @@ namespace kvc {
 
 constexpr int FIT_TILE = 64;            // covariance tile per CTA
 constexpr int FIT_KC = 32;              // channels per staged chunk
+constexpr int FIT_SPLITS = 4;            // parts of the samples, one per matrix of the workspace
 constexpr int FIT_MAX_SWEEPS = 40;
 constexpr float FIT_COS_TOL2 = 1e-20f;  // one-sided: stop after a sweep whose largest squared cosine between two columns was below this
 constexpr double FIT_OFF_TOL2 = 1e-22;  // stop when (off-diagonal norm / diagonal norm)^2 falls below this
@@ -75,16 +76,25 @@ __global__ void __launch_bounds__(256) fit_sum_kernel(const T* __restrict__ X, i
   atomicAdd(sum + (size_t)h * head_stride + c, acc);
 }
 
-// C[h][i][j] = sum over blocks s and channels c of (X_s[i][c] - mu_c)(X_s[j][c] - mu_c), mu = sum / count (0 if !center)
+// Partial sums of the symmetric second-moment matrix: C_split[h][i][j] = sum over the split's blocks s and channels c of
+// (X_s[i][c] - mu_c)(X_s[j][c] - mu_c), mu = sum / count (0 if !center).  Bound: fp64 multiply-adds (and as many shared-memory
+// wavefronts).  Only tiles on and above the diagonal are computed, and the samples are split four ways into the four matrices of the
+// workspace, so that a few heads fill the machine: n = 256, 32 samples, 4 heads 163 us (596 us for the full square in one piece, with
+// each thread's columns side by side, which is a four-way bank conflict).
 template <typename T>
 __global__ void __launch_bounds__(256) fit_moment_kernel(const T* __restrict__ X, int B, int R, int H_kv, int n, int ne,
-                                                         double* __restrict__ ws, size_t head_stride, size_t off_C,
+                                                         double* __restrict__ ws, size_t head_stride, size_t off_C, size_t mat,
                                                          size_t off_sum, int center) {
-  __shared__ double As[FIT_KC][FIT_TILE + 1], Bs[FIT_KC][FIT_TILE + 1];
+  __shared__ double As[FIT_KC][FIT_TILE], Bs[FIT_KC][FIT_TILE];
   __shared__ double mu[D];
-  const int h = blockIdx.z, i0 = blockIdx.y * FIT_TILE, j0 = blockIdx.x * FIT_TILE;
+  const int h = blockIdx.z, split = blockIdx.y;
+  int ti = 0, tj = blockIdx.x;                              // tile (ti, tj), tj >= ti
+  for (int row = (n + FIT_TILE - 1) / FIT_TILE; tj >= row; --row) { tj -= row; ++ti; }
+  tj += ti;
+  const int i0 = ti * FIT_TILE, j0 = tj * FIT_TILE;
   const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
-  double* C = ws + (size_t)h * head_stride + off_C;
+  double* C = ws + (size_t)h * head_stride + off_C + (size_t)split * mat;
+  const bool aligned = (reinterpret_cast<uintptr_t>(X) & 15) == 0;
   if (tid < D) mu[tid] = center ? ws[(size_t)h * head_stride + off_sum + tid] / ((double)B * R * n) : 0.0;
   __syncthreads();
   double acc[4][4];
@@ -92,23 +102,40 @@ __global__ void __launch_bounds__(256) fit_moment_kernel(const T* __restrict__ X
   for (int a = 0; a < 4; ++a)
 #pragma unroll
     for (int b = 0; b < 4; ++b) acc[a][b] = 0.0;
-  const int lrow = tid >> 2, lc = (tid & 3) * 8;          // staging: 64 rows x 4 groups of 8 channels
-  for (int s = 0; s < B * R; ++s) {
+  const int lrow = tid & 63, lc = (tid >> 6) * 8;          // staging: 64 rows x 4 groups of 8 channels, a warp along the rows
+  const int s0 = (int)((long long)B * R * split / FIT_SPLITS), s1 = (int)((long long)B * R * (split + 1) / FIT_SPLITS);
+  for (int s = s0; s < s1; ++s) {
     const int b = s / R, r = s - b * R;
     const T* blk = X + (((size_t)b * H_kv + h) * R + r) * (size_t)n * D;
     for (int c0 = 0; c0 < D; c0 += FIT_KC) {
 #pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        const int c = c0 + lc + e;
-        As[lc + e][lrow] = i0 + lrow < n ? (double)to_f32(blk[(size_t)(i0 + lrow) * D + c]) - mu[c] : 0.0;
-        Bs[lc + e][lrow] = j0 + lrow < n ? (double)to_f32(blk[(size_t)(j0 + lrow) * D + c]) - mu[c] : 0.0;
+      for (int side = 0; side < 2; ++side) {
+        const int row = (side ? j0 : i0) + lrow;
+        float f[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) f[e] = 0.f;
+        if (row < n && !aligned) {
+#pragma unroll
+          for (int e = 0; e < 8; ++e) f[e] = to_f32(blk[(size_t)row * D + c0 + lc + e]);
+        } else if (row < n) {
+          constexpr int EPV = Elems16<T>::N;
+#pragma unroll
+          for (int v = 0; v < 8; v += EPV) {
+            float x[EPV];
+            load16(blk + (size_t)row * D + c0 + lc + v, x);
+#pragma unroll
+            for (int e = 0; e < EPV; ++e) f[v + e] = x[e];
+          }
+        }
+#pragma unroll
+        for (int e = 0; e < 8; ++e) (side ? Bs : As)[lc + e][lrow] = row < n ? (double)f[e] - mu[c0 + lc + e] : 0.0;
       }
       __syncthreads();
 #pragma unroll 8
       for (int k = 0; k < FIT_KC; ++k) {
         double av[4], bv[4];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) { av[e] = As[k][ty * 4 + e]; bv[e] = Bs[k][tx * 4 + e]; }
+        for (int e = 0; e < 4; ++e) { av[e] = As[k][ty + 16 * e]; bv[e] = Bs[k][tx + 16 * e]; }
 #pragma unroll
         for (int a = 0; a < 4; ++a)
 #pragma unroll
@@ -121,9 +148,23 @@ __global__ void __launch_bounds__(256) fit_moment_kernel(const T* __restrict__ X
   for (int a = 0; a < 4; ++a)
 #pragma unroll
     for (int bb = 0; bb < 4; ++bb) {
-      const int i = i0 + ty * 4 + a, j = j0 + tx * 4 + bb;
+      const int i = i0 + ty + 16 * a, j = j0 + tx + 16 * bb;
       if (i < n && j < n) C[(size_t)i * ne + j] = acc[a][bb];
     }
+}
+
+// the splits summed into the first matrix, both triangles
+__global__ void __launch_bounds__(256) fit_moment_sum_kernel(double* __restrict__ ws, size_t head_stride, size_t off_C, size_t mat, int n, int ne) {
+  double* C = ws + (size_t)blockIdx.y * head_stride + off_C;
+  for (int x = blockIdx.x * 256 + threadIdx.x; x < n * n; x += gridDim.x * 256) {
+    const int i = x / n, j = x - i * n;
+    if (j / FIT_TILE < i / FIT_TILE) continue;               // a tile below the diagonal: written by its mirror image
+    double v = 0.0;
+#pragma unroll
+    for (int k = 0; k < FIT_SPLITS; ++k) v += C[(size_t)k * mat + (size_t)i * ne + j];
+    C[(size_t)i * ne + j] = v;
+    if (j / FIT_TILE > i / FIT_TILE) C[(size_t)j * ne + i] = v;
+  }
 }
 
 // ---- cyclic Jacobi with the round-robin ordering --------------------------------------------------------------
@@ -360,15 +401,17 @@ __global__ void __launch_bounds__(256) fit_emit_theta_kernel(const double* __res
 }
 
 // ---- one-sided Jacobi, one launch ----------------------------------------------------------------------------------------
-// Bound: latency of a rotation (three dot products over a column reduced across a warp, two double-precision divisions and a root,
-// then the update), n - 1 of them one after the other per sweep whatever the machine's width, about 14 sweeps.  So everything else is
-// taken out of that chain: a cluster of C CTAs owns a matrix, its columns form 2 C blocks of bs, in each of the 2 C - 1 rounds of a
-// sweep a CTA holds two blocks in shared memory (a warp per pair, the first block's column kept in registers) and rotates all pairs
-// between them (in the first round also those inside), and between rounds the columns go through L2 behind one cluster barrier; no
-// launch, no host round trip.  The two-sided form took two launches per round: 24 + 8 ms for n = 256, m = 103, 4 heads
-// (B200, 8600 launches of 4 us); this one 3 ms.
-// The tangent of a rotation is taken in single precision: it only steers the convergence (off-diagonal cosines fall by 1e-7 at worst per
-// sweep once they are small); cosine and sine are made from it in double precision, so that the rotation is orthogonal.
+// Bound: latency of a rotation (a dot product over a column reduced across a warp, the angle, the update: about 850 cycles), n - 1 of
+// them one after the other per sweep whatever the machine's width, 11 to 14 sweeps.  So everything else is taken out of that chain: a
+// cluster of C CTAs owns a matrix, its columns form 2 C blocks of bs, in each of the 2 C - 1 rounds of a sweep a CTA holds two blocks
+// in shared memory (a warp per pair, the first block's column kept in registers) and rotates all pairs between them (in the first
+// round also those inside), and between rounds the columns go through L2 behind one cluster barrier (about 3 us); no launch, no host
+// round trip.  n = 256, 4 heads on B200: 3.2 ms (n = 103: 0.85 ms); the two-sided form took two launches of 4 us per round, 24 and 8 ms.
+// Half as many CTAs with twice the warps: 3.8 ms (the rotations of 16 warps are bound by shared memory).
+// The angle is taken in single precision: it only steers the convergence (off-diagonal cosines fall by 1e-7 at worst per sweep once
+// they are small); cosine and sine are made from its tangent in double precision, so that the rotation is orthogonal.  The squared
+// lengths that the angle needs are carried along and taken anew in every round; with them as two more dot products and the angle in
+// double precision a rotation took 1.05 us instead of 0.89 (both with their share of the rounds).
 // tau = 1e-5 of the largest diagonal entry keeps the columns of a rank-deficient matrix away from zero, so that its null space gets
 // orthonormal vectors too.
 template <int EPL>
@@ -376,7 +419,7 @@ __global__ void __launch_bounds__(640, 1) jacobi_cluster_kernel(double* __restri
                                                                 size_t off_flag, int size, int C, int bs) {
   constexpr int LD = 32 * EPL;
   extern __shared__ __align__(16) double cols[];                 // [2 bs][LD]
-  __shared__ double s_red[32];
+  __shared__ double s_red[32], s_norm[40];                       // s_norm: squared lengths of the block columns
   __shared__ float s_max[32];
   const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31, nw = bs;
   const int h = blockIdx.x / C, c = blockIdx.x - h * C, NB = 2 * C;
@@ -391,27 +434,41 @@ __global__ void __launch_bounds__(640, 1) jacobi_cluster_kernel(double* __restri
   __syncthreads();
   tau = 0.0;
   for (int x = 0; x < nw; ++x) tau = fmax(tau, s_red[x]);
-  tau = tau > 0.0 ? 1e-5 * tau : 1.0;
+  // the matrix is taken relative to its largest diagonal entry, so that the lengths are numbers of order one
+  const double big = tau > 0.0 ? tau : 1.0, inv_big = 1.0 / big;
+  tau = tau > 0.0 ? 1e-5 : 1.0;
   cluster_sync_all();                                            // every CTA has read the diagonal
 
   float mx = 0.f;
-  // rotates columns a, b towards orthogonality
-  auto rotate = [&](double (&a)[EPL], double (&b)[EPL]) {
-    double al = 0.0, be = 0.0, ga = 0.0;
+  auto length2 = [&](const double (&x)[EPL]) {
+    double l = 0.0;
 #pragma unroll
-    for (int e = 0; e < EPL; ++e) { al = fma(a[e], a[e], al); be = fma(b[e], b[e], be); ga = fma(a[e], b[e], ga); }
+    for (int e = 0; e < EPL; ++e) l = fma(x[e], x[e], l);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      al += __shfl_xor_sync(0xffffffffu, al, o);
-      be += __shfl_xor_sync(0xffffffffu, be, o);
-      ga += __shfl_xor_sync(0xffffffffu, ga, o);
-    }
-    const float cos2 = (float)(ga * ga / (al * be));             // NaN for a zero column (an index beyond the matrix): no rotation
+    for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+    return l;
+  };
+  // rotates columns a, b towards orthogonality; na, nb: their squared lengths, carried along
+  auto rotate = [&](double (&a)[EPL], double (&b)[EPL], double& na, double& nb) {
+    double g0 = 0.0, g1 = 0.0;
+#pragma unroll
+    for (int e = 0; e < EPL; e += 2) { g0 = fma(a[e], b[e], g0); g1 = fma(a[e + 1], b[e + 1], g1); }
+    double ga = g0 + g1;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) ga += __shfl_xor_sync(0xffffffffu, ga, o);
+    const float gf = (float)ga, cosine = gf * rsqrtf((float)na) * rsqrtf((float)nb);      // NaN for a zero column (an index beyond the matrix)
+    const float cos2 = cosine * cosine;
     if (!(cos2 > 1e-30f)) return;
     mx = fmaxf(mx, cos2);
-    const float z = (float)((be - al) / (2.0 * ga));
-    const double t = (double)((z >= 0.f ? 1.f : -1.f) / (fabsf(z) + sqrtf(fmaf(z, z, 1.f))));
-    const double cs = rsqrt(fma(t, t, 1.0)), sn = cs * t;
+    const float z = (float)(nb - na) / (2.f * gf);
+    const float tf = (z >= 0.f ? 1.f : -1.f) / (fabsf(z) + sqrtf(fmaf(z, z, 1.f)));
+    const double t = (double)tf, d = fma(t, t, 1.0);
+    double cs = (double)rsqrtf(fmaf(tf, tf, 1.f));                // two Newton steps: 1e-7 -> 1e-14 -> rounding
+    cs = cs * fma(-0.5 * d, cs * cs, 1.5);
+    cs = cs * fma(-0.5 * d, cs * cs, 1.5);
+    const double sn = cs * t;
+    na = fma(-t, ga, na);
+    nb = fma(t, ga, nb);
 #pragma unroll
     for (int e = 0; e < EPL; ++e) {
       const double x = a[e], y = b[e];
@@ -432,6 +489,7 @@ __global__ void __launch_bounds__(640, 1) jacobi_cluster_kernel(double* __restri
     for (int e = 0; e < EPL; ++e) {
       const int i = e * 32 + lane;
       x[e] = col < size && i < size ? __ldcg(A + (size_t)col * size + i) : 0.0;
+      if (shift) x[e] *= inv_big;
       if (shift && i == col && col < size) x[e] += tau;
     }
   };
@@ -454,9 +512,12 @@ __global__ void __launch_bounds__(640, 1) jacobi_cluster_kernel(double* __restri
       const bool shift = sweep == 0 && br == 0;
       fetch(a, p, shift);
       fetch(b, q, shift);
+      double na = length2(a), nb = length2(b);
       put(b, bs + w);
+      if (lane == 0) s_norm[bs + w] = nb;
       if (br == 0) {
         put(a, w);
+        if (lane == 0) s_norm[w] = na;
         __syncthreads();
         const int n2 = 2 * bs;
         for (int r = 0; r < n2 - 1; ++r) {
@@ -464,9 +525,13 @@ __global__ void __launch_bounds__(640, 1) jacobi_cluster_kernel(double* __restri
           const int i = place(w), j = place(n2 - 1 - w);
           get(a, i);
           get(b, j);
-          rotate(a, b);
+          na = s_norm[i];
+          nb = s_norm[j];
+          rotate(a, b, na, nb);
           put(a, i);
           put(b, j);
+          __syncwarp();
+          if (lane == 0) { s_norm[i] = na; s_norm[j] = nb; }
           __syncthreads();
         }
         get(a, w);
@@ -474,9 +539,11 @@ __global__ void __launch_bounds__(640, 1) jacobi_cluster_kernel(double* __restri
         __syncthreads();
         int slot = bs + w;
         for (int r = 0; r < bs; ++r) {
-          if (r > 0) get(b, slot);
-          rotate(a, b);
+          if (r > 0) { get(b, slot); nb = s_norm[slot]; }
+          rotate(a, b, na, nb);
           put(b, slot);
+          __syncwarp();
+          if (lane == 0) s_norm[slot] = nb;
           slot = slot + 1 < 2 * bs ? slot + 1 : bs;
           __syncthreads();
         }
@@ -505,12 +572,9 @@ __global__ void __launch_bounds__(640, 1) jacobi_cluster_kernel(double* __restri
 #pragma unroll
   for (int x = 0; x < 2; ++x) {
     const int col = (2 * c + x) * bs + w;
-    double a[EPL], al = 0.0;
+    double a[EPL];
     fetch(a, col, false);
-#pragma unroll
-    for (int e = 0; e < EPL; ++e) al = fma(a[e], a[e], al);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) al += __shfl_xor_sync(0xffffffffu, al, o);
+    const double al = length2(a);
     len[x] = sqrt(al);
     const double inv = al > 0.0 ? 1.0 / len[x] : 0.0;
 #pragma unroll
@@ -523,7 +587,7 @@ __global__ void __launch_bounds__(640, 1) jacobi_cluster_kernel(double* __restri
 #pragma unroll
   for (int x = 0; x < 2; ++x) {
     const int col = (2 * c + x) * bs + w;
-    if (lane == 0 && col < size) A[(size_t)col * size + col] = len[x] - tau;
+    if (lane == 0 && col < size) A[(size_t)col * size + col] = (len[x] - tau) * (tau < 1.0 ? big : 0.0);
   }
   if (c == 0 && tid == 0) reinterpret_cast<int*>(flag)[60] = sweep;
 }
@@ -624,7 +688,9 @@ static cudaError_t moments(const T* X, int B, int R, int H, int n, const FitLayo
   if (e != cudaSuccess) return e;
   if (center) fit_sum_kernel<T><<<dim3(H, 64), 256, 0, st>>>(X, B, H, (long long)R * n, ws + f.off_sum, f.per_head);
   const int tiles = ceil_div(n, FIT_TILE);
-  fit_moment_kernel<T><<<dim3(tiles, tiles, H), 256, 0, st>>>(X, B, R, H, n, f.ne, ws, f.per_head, off_C, f.off_sum, center ? 1 : 0);
+  fit_moment_kernel<T><<<dim3(tiles * (tiles + 1) / 2, FIT_SPLITS, H), 256, 0, st>>>(X, B, R, H, n, f.ne, ws, f.per_head, off_C, f.mat, f.off_sum,
+                                                                                   center ? 1 : 0);
+  fit_moment_sum_kernel<<<dim3(ceil_div(n * n, 1024), H), 256, 0, st>>>(ws, f.per_head, off_C, f.mat, n, f.ne);
   return cudaGetLastError();
 }
 
