@@ -11,6 +11,7 @@
 #include "kvc_split.cuh"
 #include "kvc_resident.cuh"
 #include "kvc_cluster.cuh"
+#include "kvc_plain.cuh"
 
 namespace kvc {
 
@@ -286,7 +287,9 @@ size_t kvc_capsule_bytes(const kvc_layer* L, int B, int R) {
 size_t kvc_workspace_bytes(const kvc_layer* L, int B, int R, int T_cap) {
   if (!L || B < 0 || R < 0 || T_cap < 0) return 0;
   const size_t phases = ws_layout(L, B, R, T_cap).total, cluster = cluster_ws_bytes(L, B, R, T_cap);
-  return phases > cluster ? phases : cluster;
+  const size_t most = phases > cluster ? phases : cluster;
+  const size_t plain = (R == 0 || L->passthrough) && L->desc.dtype == KVC_BF16 && B > 0 ? plain_ws(L, B).bytes : 0;
+  return most > plain ? most : plain;
 }
 
 int kvc_compress(const kvc_layer* L, const void* K_vis, const void* V_vis, int B, int R, void* capsules,
@@ -395,6 +398,16 @@ int decode_common(const kvc_layer* L, const void* q, const void* capsules, int B
       bool encoded = false;
       const cudaError_t ce = launch_cluster(L, a, cp, ws, st, &encoded);
       if (encoded) return cuda_status(ce);
+    }
+  }
+
+  // rows stored verbatim only (uncompressed K/V, text alone, the stores of ratio 0)
+  if ((align & 15) == 0 && (R == 0 || L->passthrough) && !ragged && L->use_tc != -2) {
+    const PlainPlan pp = plan_plain(L, B, R * L->desc.n, T);
+    if (pp.ok && (ws_limit == 0 || plain_ws(L, B).bytes <= ws_limit)) {
+      bool encoded = false;
+      const cudaError_t pe = launch_plain(L, a, pp, ws, st, &encoded);
+      if (encoded) return cuda_status(pe);
     }
   }
 
