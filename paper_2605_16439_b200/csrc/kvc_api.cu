@@ -85,16 +85,11 @@ WsLayout ws_layout(const kvc_layer* L, int B, int R, int T_cap) {
   w.off_ypart = take(sizeof(float) * (size_t)B * H_kv * G * w.nsplit * D);
   w.off_ystat = take(sizeof(float2) * (size_t)B * H_kv * G * w.nsplit);
   {
-    // partial outputs of the one-kernel path: per (sequence, KV head) one per unit along the block axis, or, without
-    // vision blocks, one per slice of the text rows (at most 16, whatever T is)
+    // partial outputs of the one-kernel path: per (sequence, KV head) one per unit along the block axis
     size_t np = 0;
     if (B > 0 && R > 0) {
       const FusedPlan fp = plan_fused(L, B, R);
       if (fp.ok && L->mode == KVC_MODE_KV && fp.nrg > 1) np = (size_t)B * H_kv * fp.nrg * G;
-    }
-    if ((R == 0 || L->passthrough) && B > 0 && R * n + T_cap > 0 && plan_fused_text(L, B, R * n + T_cap).ok) {
-      const size_t np_plain = (size_t)B * H_kv * 16 * G;
-      np = np > np_plain ? np : np_plain;
     }
     w.off_fpy = take(sizeof(float) * np * D);
     w.off_fpml = take(sizeof(float2) * np);
@@ -430,9 +425,7 @@ int decode_common(const kvc_layer* L, const void* q, const void* capsules, int B
 
   // bf16 storage with TMA-compatible shapes and pointers: the whole of Algorithm 1 in one kernel
   {
-    // R == 0 (text rows only, the uncompressed comparator): the same kernel with text stages only
-    // rho = 0 stores K and V verbatim: vision rows and text rows are attended as plain rows by the text-only mode
-    const bool plain = R == 0 || L->passthrough;
+    const bool plain = R == 0 || L->passthrough;            // rows stored verbatim only: served above
     // one-sided modes are served by the three-phase kernels below; so are per-sequence lengths, except on the shapes the
     // resident-parameter kernel takes (it reads the lengths itself)
     const bool one_sided = (R > 0 && L->mode != KVC_MODE_KV) || ragged;
@@ -453,8 +446,8 @@ int decode_common(const kvc_layer* L, const void* q, const void* capsules, int B
       const cudaError_t se = launch_split(L, a, sp, st, &encoded);
       if (encoded) return cuda_status(se);
     }
-    FusedPlan fp = plain ? plan_fused_text(L, B, R * L->desc.n + T) : plan_fused(L, B, R);
-    if (one_sided) fp.ok = 0;
+    FusedPlan fp{};
+    if (!plain && !one_sided) fp = plan_fused(L, B, R);
     if (fp.ok && (align & 15) == 0) {
       bool encoded = false;
       const cudaError_t fe = launch_fused(L, a, fp, st, &encoded);

@@ -73,8 +73,8 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
       const int bg = rem / a.nrg, rg = rem - bg * a.nrg;
       const int b0 = bg * a.NB, r0 = rg * a.RB;
       const RowRanges tr = row_ranges(a, rg);
-      const int nts = tr.na + tr.nb;
-      if (first && a.R > 0) {
+      const int nts = tr.nb;
+      if (first) {
         // while the stream's previous kernel drains: the K_tilde rows of the first ring of stages are asked into L2 (a
         // prefetch consumes no data, so it need not wait for that kernel; the loads below do)
         for (int c = 0; c < a.NJ && c < a.stages; ++c) {
@@ -89,16 +89,13 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
           unsigned char* dst = sm + slot * a.stage_bytes;
           uint64_t* bar = &bars.full[slot];
           if (part == 1) {
-            const bool lead = c < tr.na;
-            const int y = lead ? tr.a0 + c * a.TCH : tr.b0 + (c - tr.na) * a.TCH;
-            const CUtensorMap* mk = lead ? &tmK : &tmKt;
-            const CUtensorMap* mv = lead ? &tmV : &tmVt;
+            const int y = tr.b0 + c * a.TCH;
             mbar_expect_tx(bar, 4 * a.txt_half_bytes);
             if (first) { grid_dep_wait(); first = false; }
-            tma_load_4d(dst, mk, 0, y, h, b0, bar);
-            tma_load_4d(dst + a.txt_half_bytes, mk, 64, y, h, b0, bar);
-            tma_load_4d(dst + 2 * a.txt_half_bytes, mv, 0, y, h, b0, bar);
-            tma_load_4d(dst + 3 * a.txt_half_bytes, mv, 64, y, h, b0, bar);
+            tma_load_4d(dst, &tmKt, 0, y, h, b0, bar);
+            tma_load_4d(dst + a.txt_half_bytes, &tmKt, 64, y, h, b0, bar);
+            tma_load_4d(dst + 2 * a.txt_half_bytes, &tmVt, 0, y, h, b0, bar);
+            tma_load_4d(dst + 3 * a.txt_half_bytes, &tmVt, 64, y, h, b0, bar);
           } else {
             const CUtensorMap* tp = part == 0 ? &tmTh : &tmU;
             const CUtensorMap* tk = part == 0 ? &tmK : &tmV;
@@ -199,7 +196,7 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
       const int nbv = min(a.NB, a.B - b0);
       const int rbv = min(RB, a.R - r0);
       const RowRanges tr = row_ranges(a, rg);
-      const int nts = tr.na + tr.nb;
+      const int nts = tr.nb;
       (void)h;
 
       // expansion rows held by this lane: rho = mt*16 + gid + 8*hr  <->  (sequence, block, head)
@@ -459,7 +456,7 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
       const int nbv = min(a.NB, a.B - b0);
       const int rbv = min(RB, a.R - r0);
       const RowRanges tr = row_ranges(a, rg);
-      const int nts = tr.na + tr.nb;
+      const int nts = tr.nb;
 
       // ---- queries of the unit's sequences: [NB][16 heads][128], heads >= G and absent sequences are zero rows
       for (int idx = vtid; idx < a.NB * 256; idx += VTH) {
@@ -535,8 +532,8 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
         wait_on(&bars.full[slot], phase);
         const uint32_t kt_u = sm_u + slot * a.stage_bytes, vt_u = kt_u + 2 * a.txt_half_bytes;
         for (int tile = wig; tile * 16 < a.TCH; tile += WPG) {
-          const int ts1 = ts < tr.na ? tr.a1 : tr.b1;               // end of the row range this stage belongs to
-          const int t_first = (ts < tr.na ? tr.a0 + ts * a.TCH : tr.b0 + (ts - tr.na) * a.TCH) + tile * 16;
+          const int ts1 = tr.b1;
+          const int t_first = tr.b0 + ts * a.TCH + tile * 16;
           if (t_first >= ts1) break;
           const int row0 = bl * a.TCH + tile * 16;
           const uint32_t rowB = (uint32_t)((row0 + lrowB) * 128);
@@ -717,7 +714,7 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
           const int g = g0 + gg;
           float y = 0.f;
           for (int w = tb * WPG; w < (tb + 1) * WPG; ++w) y += yred[(w * YHG + gg) * D + col];
-          if (a.R > 0) y = fmaf(vsum[tb * 16 + g], __bfloat162float(a.mu[h * D + col]), y);
+          y = fmaf(vsum[tb * 16 + g], __bfloat162float(a.mu[h * D + col]), y);
           if (a.nrg == 1)
             a.out[((size_t)(b0 + tb) * a.H_kv * G + (size_t)h * G + g) * D + col] = __float2bfloat16_rn(y / hsum[tb * 16 + g]);
           else
@@ -970,56 +967,6 @@ FusedPlan plan_fused(const kvc_layer* L, int B, int R) {
   return p;
 }
 
-// Text-only attention (no vision blocks: the uncompressed comparator and R == 0 calls) through the same kernel:
-// only text stages, the rows of a (sequence, KV head) cut into `nrg` slices whose partials are merged.
-FusedPlan plan_fused_text(const kvc_layer* L, int B, int T) {   // T = all plain rows (leading segment + text)
-  FusedPlan p{};
-  const int G = L->G, H_kv = L->desc.H_kv;
-  if (L->desc.dtype != KVC_BF16 || B < 1 || T < 1 || G > 16) return p;
-  const int sms = L->num_sms > 0 ? L->num_sms : 148;
-  p.EW = 4; p.VW = 8; p.ktw = 0; p.MT = 1;
-  p.NB = 1; p.RB = 1; p.nbg = B;
-  // slices: enough units for every SM, cut so that the persistent CTAs are evenly loaded, slices of >= 256 rows
-  const long long bh = (long long)B * H_kv;
-  int best_ns = 1;
-  double best_eff = 0;
-  for (int ns = 1; ns <= 16; ++ns) {
-    if (ns > 1 && T / ns < 256) break;
-    const long long units = bh * ns;
-    const long long grid = units < sms ? units : sms;
-    const double eff = (double)units / (double)(((units + grid - 1) / grid) * sms);
-    if (eff > best_eff + 0.02) { best_eff = eff; best_ns = ns; }
-  }
-  p.nrg = best_ns;
-  p.units = (int)(bh * p.nrg);
-  p.ncg = 1; p.JC = 1; p.NJ = 0;
-  p.TCH = 128;
-  p.par_bytes = 0; p.k_half_bytes = 0;
-  p.txt_half_bytes = (uint32_t)p.TCH * 128u;
-  p.stage_bytes = 4 * p.txt_half_bytes;
-  p.msplit = 1; p.mshift = 3;
-  p.sld = 24;
-  uint32_t off = 0;
-  auto take = [&](uint32_t bytes) { uint32_t o = off; off = (off + bytes + 127u) & ~127u; return o; };
-  p.off_q = take((uint32_t)p.NB * 16 * QLD * 2);
-  const int rt = ROWS * p.MT;
-  p.off_S = take((uint32_t)(2 * rt * p.sld + 2 * (rt + 16) * SLD) * 2);
-  p.off_W = p.off_S + (uint32_t)2 * rt * p.sld * 2;
-  p.off_wred = take((uint32_t)2 * p.EW * rt * 16 * 4);
-  p.off_rstat = take((uint32_t)2 * p.EW * rt * 4);
-  p.off_tstat = take((uint32_t)2 * p.VW * 16 * 4);
-  p.off_hstat = take((uint32_t)(5 * p.NB * 16 + rt) * 4);
-  p.yhg = G > 4 ? 8 : (G > 2 ? 4 : 2);
-  p.off_yred = take((uint32_t)p.VW * p.yhg * D * 4);
-  p.misc_bytes = off;
-  const uint32_t avail = SMEM_LIMIT - 1024u - 2048u - p.misc_bytes;
-  p.stages = (int)(avail / p.stage_bytes) > 3 ? 3 : (int)(avail / p.stage_bytes);
-  if (p.stages < 2) return p;
-  p.smem_bytes = (size_t)p.stages * p.stage_bytes + p.misc_bytes + 1024u;
-  p.grid = p.units < sms ? p.units : sms;
-  p.ok = 1;
-  return p;
-}
 
 template <int EW, int VW, int KTW, int NH, int MT>
 static cudaError_t launch_inst(const CUtensorMap* tm, const FusedArgs& fa, const FusedPlan& p, cudaStream_t st) {
@@ -1042,9 +989,8 @@ cudaError_t launch_fused(const kvc_layer* L, const DecodeArgs& a, const FusedPla
   const int H_kv = a.H_kv, m = a.m, n = a.n, R = a.R, B = a.B;
   CUtensorMap tm[6];
   *encoded = false;
-  const bool compressed = R > 0 && !a.passthrough;
   bool cached = false;
-  if (compressed && L->maps) {
+  if (L->maps) {
     std::lock_guard<std::mutex> lock(L->maps->mu);
     for (const auto& x : L->maps->e)
       if (x.valid && x.B == B && x.R == R && x.tc == p.tc && x.JC == p.JC && x.RB == p.RB && x.NB == p.NB && x.Kc == a.Kc) {
@@ -1053,7 +999,7 @@ cudaError_t launch_fused(const kvc_layer* L, const DecodeArgs& a, const FusedPla
         break;
       }
   }
-  if (compressed && !cached) {
+  if (!cached) {
     const uint64_t dims[5] = {(uint64_t)D, (uint64_t)m, (uint64_t)R, (uint64_t)H_kv, (uint64_t)B};
     const uint64_t str[4] = {256ull, (uint64_t)m * 256, (uint64_t)R * m * 256, (uint64_t)H_kv * R * m * 256};
     const uint32_t box[5] = {64u, (uint32_t)(16 * p.JC), (uint32_t)p.RB, 1u, (uint32_t)p.NB};
@@ -1070,18 +1016,7 @@ cudaError_t launch_fused(const kvc_layer* L, const DecodeArgs& a, const FusedPla
     tm[2] = tm[0];
     tm[3] = tm[1];
   }
-  const int S0 = (R > 0 && a.passthrough) ? R * n : 0;   // rho = 0: the store holds K and V verbatim, attended as plain rows
-  if (S0 > 0) {
-    const uint64_t dims[4] = {(uint64_t)D, (uint64_t)S0, (uint64_t)H_kv, (uint64_t)B};
-    const uint64_t str[3] = {256ull, (uint64_t)S0 * 256, (uint64_t)H_kv * S0 * 256};
-    const uint32_t box[4] = {64u, (uint32_t)p.TCH, 1u, (uint32_t)p.NB};
-    if (!encode_tensor_map_bf16(&tm[0], a.Kc, 4, dims, str, box)) return cudaSuccess;
-    if (!encode_tensor_map_bf16(&tm[1], a.Vc, 4, dims, str, box)) return cudaSuccess;
-    if (a.T == 0) { tm[2] = tm[0]; tm[3] = tm[1]; }
-    tm[4] = tm[0]; tm[5] = tm[1];
-  } else if (R == 0) {
-    tm[0] = tm[2]; tm[1] = tm[3]; tm[4] = tm[2]; tm[5] = tm[3];          // never used: no vision stages
-  } else if (!cached) {
+  if (!cached) {
     // theta, U [H_kv][m][n] viewed as (64 columns, m rows, n/64 column groups, H_kv): a box lands as [group][row][64]
     const uint64_t dims[4] = {64ull, (uint64_t)m, (uint64_t)p.ncg, (uint64_t)H_kv};
     const uint64_t str[3] = {(uint64_t)n * 2, 128ull, (uint64_t)m * n * 2};
@@ -1104,13 +1039,11 @@ cudaError_t launch_fused(const kvc_layer* L, const DecodeArgs& a, const FusedPla
   fa.q = static_cast<const __nv_bfloat16*>(a.q);
   fa.mu = static_cast<const __nv_bfloat16*>(a.mu);
   fa.out = static_cast<__nv_bfloat16*>(a.out);
-  const bool plain = R == 0 || a.passthrough;            // text-only mode
-  fa.B = B; fa.H_kv = H_kv; fa.G = a.G; fa.R = plain ? 0 : R; fa.m = plain ? 1 : m; fa.n = plain ? 64 : n; fa.T = a.T;
-  fa.S0 = S0;
+  fa.B = B; fa.H_kv = H_kv; fa.G = a.G; fa.R = R; fa.m = m; fa.n = n; fa.T = a.T;
   fa.NB = p.NB; fa.RB = p.RB; fa.nbg = p.nbg; fa.nrg = p.nrg; fa.units = p.units; fa.JC = p.JC; fa.NJ = p.NJ;
   fa.TCH = p.TCH; fa.ncg = p.ncg; fa.stages = p.stages;
   fa.ktw = p.ktw; fa.msplit = p.msplit; fa.mshift = p.mshift; fa.sld = p.sld; fa.yhg = p.yhg;
-  fa.Tper = (ceil_div(S0 + a.T > 0 ? S0 + a.T : 1, p.nrg) + 15) & ~15;
+  fa.Tper = (ceil_div(a.T > 0 ? a.T : 1, p.nrg) + 15) & ~15;
   fa.par_bytes = p.par_bytes; fa.k_half_bytes = p.k_half_bytes; fa.txt_half_bytes = p.txt_half_bytes;
   fa.stage_bytes = p.stage_bytes;
   const uint32_t ring = (uint32_t)p.stages * p.stage_bytes;

@@ -18,7 +18,6 @@ struct FusedArgs {
   const __nv_bfloat16* mu;
   __nv_bfloat16* out;
   int B, H_kv, G, R, m, n, T;
-  int S0;             // text-only mode: rows of a leading K/V segment (verbatim vision rows of a rho = 0 store), else 0
   int NB, RB, nbg, nrg, units, JC, NJ, TCH, Tper, ncg, stages;
   int ktw;            // 16-column groups of L per expansion warp
   int msplit, mshift; // the 8 row tiles of a value block go to msplit = 8 >> mshift tasks
@@ -49,15 +48,11 @@ constexpr int BAR_S_FREE = 6;    // + b: score tile read     (expansion warps ar
 constexpr int BAR_W_READY = 8;   // + b: weight tile written (expansion warps arrive, value warps wait)
 constexpr int BAR_W_FREE = 10;   // + b: weight tile read    (value warps arrive, expansion warps wait)
 
-// The plain K/V rows a unit attends over: its slice [g0, g1) of the concatenation [leading segment | text rows], as a
-// range of the leading segment (a0, a1; tensor maps tmK / tmV) and a range of the text rows (b0, b1; tmKt / tmVt)
-struct RowRanges { int a0, a1, b0, b1, na, nb; };
+// The text rows a unit attends over: its slice [b0, b1), in nb stages
+struct RowRanges { int b0, b1, nb; };
 __device__ __forceinline__ RowRanges row_ranges(const FusedArgs& a, int rg) {
   RowRanges r;
-  const int g0 = rg * a.Tper, g1 = min(a.S0 + a.T, g0 + a.Tper);
-  r.a0 = min(g0, a.S0); r.a1 = min(g1, a.S0);
-  r.b0 = max(g0, a.S0) - a.S0; r.b1 = max(g1, a.S0) - a.S0;
-  r.na = r.a1 > r.a0 ? (r.a1 - r.a0 + a.TCH - 1) / a.TCH : 0;
+  r.b0 = min(rg * a.Tper, a.T); r.b1 = min(a.T, r.b0 + a.Tper);
   r.nb = r.b1 > r.b0 ? (r.b1 - r.b0 + a.TCH - 1) / a.TCH : 0;
   return r;
 }

@@ -148,7 +148,7 @@ fused_decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_con
       const int rk = PAIR ? (rg & 1) : 0;
       const int b0 = bg * a.NB, r0 = PAIR ? (rg >> 1) * a.RB : rg * a.RB;
       const RowRanges tr = row_ranges(a, rg);
-      const int nts = tr.na + tr.nb;
+      const int nts = tr.nb;
       const int cg0 = PAIR ? rk * ncgl : 0;          // first column group of this CTA
       const int c2first = (PAIR && rk) ? NJ0 : 0, c2count = PAIR ? (rk ? a.NJ - NJ0 : NJ0) : a.NJ;
       // stage sequence of a unit: NJ stages of pass A (theta rows + K_tilde rows); then the column groups of U and
@@ -231,7 +231,7 @@ fused_decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_con
       const int rem = u % per_h;
       const int rg = rem % a.nrg;
       const RowRanges tr = row_ranges(a, rg);
-      const int nts = tr.na + tr.nb;
+      const int nts = tr.nb;
       // ---------------- pass A ----------------
       if (ucount > 0) wait_on(&bars.l_free, (ucount - 1) & 1u);    // the previous unit's logits have been read back
       for (int c = 0; c < a.NJ; ++c) {
@@ -614,7 +614,7 @@ fused_decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_con
     const int nbv = min(a.NB, a.B - b0);
     const int rbv = min(RB, a.R - r0);
     const RowRanges tr = row_ranges(a, rg);
-    const int nts = tr.na + tr.nb;
+    const int nts = tr.nb;
     const int c2first = (PAIR && rk) ? NJ0 : 0, c2count = PAIR ? (rk ? a.NJ - NJ0 : NJ0) : a.NJ;
     (void)r0;
 
@@ -705,8 +705,8 @@ fused_decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_con
       wait_on(&bars.full[slot], phase);
       const uint32_t kt_u = sm_u + slot * a.stage_bytes, vt_u = kt_u + 2 * a.txt_half_bytes;
       for (int tile = wig; tile * 16 < a.TCH; tile += WPG) {
-        const int ts1 = ts < tr.na ? tr.a1 : tr.b1;               // end of the row range this stage belongs to
-        const int t_first = (ts < tr.na ? tr.a0 + ts * a.TCH : tr.b0 + (ts - tr.na) * a.TCH) + tile * 16;
+        const int ts1 = tr.b1;
+        const int t_first = tr.b0 + ts * a.TCH + tile * 16;
         if (t_first >= ts1) break;
         const int row0 = bl * a.TCH + tile * 16;
         const uint32_t rowB = (uint32_t)((row0 + lrowB) * 128);
@@ -894,7 +894,7 @@ fused_decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_con
         const int g = g0 + gg;
         float y = 0.f;
         for (int w = tb * WPG; w < (tb + 1) * WPG; ++w) y += yred[(w * YHG + gg) * D + col];
-        if (a.R > 0) y = fmaf(vsum[tb * 16 + g], __bfloat162float(a.mu[h * D + col]), y);
+        y = fmaf(vsum[tb * 16 + g], __bfloat162float(a.mu[h * D + col]), y);
         if (a.nrg == 1)
           a.out[((size_t)(b0 + tb) * a.H_kv * G + (size_t)h * G + g) * D + col] = __float2bfloat16_rn(y / hsum[tb * 16 + g]);
         else if (pmerge) {

@@ -137,7 +137,6 @@ int cuda_status(cudaError_t e);   // KVC_OK or KVC_ERR_CUDA, remembering the err
 FusedPlan plan_fused(const kvc_layer* L, int B, int R);
 FusedPlan plan_fused_tc(const kvc_layer* L, int B, int R);     // tensor-memory variant; ok == 0 if the shape does not fit it
 FusedPlan plan_fused_pair(const kvc_layer* L, int B, int R);   // its pair mode (clusters of two CTAs)
-FusedPlan plan_fused_text(const kvc_layer* L, int B, int T);   // R == 0: text rows only
 
 struct DecodeArgs {
   const void* q;

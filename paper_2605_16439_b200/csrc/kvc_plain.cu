@@ -249,7 +249,7 @@ plain_decode_kernel(const __grid_constant__ CUtensorMap tmKa, const __grid_const
       __syncthreads();
     }
     const int first = run_owner((long long)p * spp, a.total, gridDim.x), parts = run_owner((long long)(p + 1) * spp - 1, a.total, gridDim.x) - first + 1;
-    const size_t slot = (size_t)p * PN_MAX_PARTS + (blockIdx.x - first);
+    const size_t slot = (size_t)p * a.slots + (blockIdx.x - first);
     for (int idx = tid; idx < G * (D / 4); idx += PN_THREADS) {
       const int head = idx >> 5, c = (idx & 31) * 4;
       float4 y = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -287,7 +287,7 @@ plain_decode_kernel(const __grid_constant__ CUtensorMap tmKa, const __grid_const
     if (s_last) {
       // lane <-> partial for the statistics, the values eight partials at a time
       for (int head = warp; head < G; head += PN_WARPS) {
-        const size_t base = (size_t)p * PN_MAX_PARTS;
+        const size_t base = (size_t)p * a.slots;
         float2 st[2];
 #pragma unroll
         for (int x = 0; x < 2; ++x) st[x] = lane + 32 * x < parts ? __ldcg(&a.pml[(base + lane + 32 * x) * G + head]) : make_float2(-INFINITY, 0.f);
@@ -322,6 +322,12 @@ plain_decode_kernel(const __grid_constant__ CUtensorMap tmKa, const __grid_const
 }
 
 // ------------------------------------------------------------------------------------------ host side
+// partial slots of a pair: CTAs that can share it (pair-aligned runs of at most sms / pairs CTAs, or crossing runs on all SMs)
+static int part_slots(const kvc_layer* L, int B) {
+  const long long n = (L->num_sms > 0 ? L->num_sms : 148) / ((long long)B * L->desc.H_kv) + 2;
+  return (int)(n < PN_MAX_PARTS ? n : PN_MAX_PARTS);
+}
+
 PlainPlan plan_plain(const kvc_layer* L, int B, int S0, int T) {
   PlainPlan p{};
   const int G = L->G, H = L->desc.H_kv;
@@ -357,12 +363,12 @@ PlainPlan plan_plain(const kvc_layer* L, int B, int S0, int T) {
 
 PlainWs plain_ws(const kvc_layer* L, int B) {
   PlainWs w{};
-  const size_t bh = (size_t)B * L->desc.H_kv;
+  const size_t bh = (size_t)B * L->desc.H_kv, slots = (size_t)part_slots(L, B);
   size_t off = align_up(sizeof(int) * (bh + 1), 256);                  // behind the status word of the layout all paths share
   auto take = [&](size_t bytes) { const size_t o = off; off = align_up(off + bytes, 256); return o; };
   w.off_cnt = take(sizeof(unsigned long long) * bh);
-  w.off_pml = take(sizeof(float2) * bh * PN_MAX_PARTS * L->G);
-  w.off_py = take(sizeof(float) * bh * PN_MAX_PARTS * L->G * D);
+  w.off_pml = take(sizeof(float2) * bh * slots * L->G);
+  w.off_py = take(sizeof(float) * bh * slots * L->G * D);
   w.bytes = off;
   return w;
 }
@@ -400,7 +406,7 @@ cudaError_t launch_plain(const kvc_layer* L, const DecodeArgs& d, const PlainPla
   a.pml = reinterpret_cast<float2*>(ws + w.off_pml);
   a.cnt = reinterpret_cast<unsigned long long*>(ws + w.off_cnt);
   a.token = d.token; a.status = d.status;
-  a.G = d.G; a.S0 = S0; a.T = d.T; a.steps_a = p.steps_a; a.spp = p.spp; a.total = p.total; a.off_red = p.off_red;
+  a.G = d.G; a.S0 = S0; a.T = d.T; a.steps_a = p.steps_a; a.spp = p.spp; a.slots = part_slots(L, B); a.total = p.total; a.off_red = p.off_red;
   ProfScope prof(KVC_KERNEL_FUSED, st);
   return d.G > 8 ? launch_plain_inst<2, 3>(tm, a, p, st) : launch_plain_inst<1, 4>(tm, a, p, st);
 }

@@ -31,12 +31,12 @@ cudaError_t launch_plain(const kvc_layer* L, const DecodeArgs& a, const PlainPla
 struct PlainArgs {
   const __nv_bfloat16* q;
   __nv_bfloat16* out;
-  float* py;               // [B*H_kv][PN_MAX_PARTS][G][D]
-  float2* pml;             // [B*H_kv][PN_MAX_PARTS][G]  (maximum in log2 units, sum)
+  float* py;               // [B*H_kv][slots][G][D]
+  float2* pml;             // [B*H_kv][slots][G]  (maximum in log2 units, sum)
   unsigned long long* cnt; // [B*H_kv] arrival words
   unsigned int token;
   int* status;
-  int G, S0, T, steps_a, spp;
+  int G, S0, T, steps_a, spp, slots;
   long long total;
   uint32_t off_red;
 };
