@@ -14,71 +14,107 @@
 
 namespace kvc {
 
+// Bound: latency of the parameter loads from L2 at the few rows this path is used for, fp32 multiply-adds beyond.  A CTA has 16 rows and
+// walks its range of the n axis in chunks of 64 positions:
+//   L      thread <-> (position, quarter of the retained rows), eight loads of theta in flight, 16 rows accumulated in registers
+//          against scores broadcast from shared memory ([j][16 rows]); the quarters meet in shared memory
+//   W      thread <-> a row of U (and every 256th after it), 16-byte loads of its 64 entries, the probabilities broadcast
+// One head of 4 rows, n = 576, m = 231 in fp32: 39 -> 18 us between events (one load of theta in flight per thread and 64 rows of U at a time
+// through shared memory before).
 template <typename T>
 __global__ void __launch_bounds__(256) expand_kernel(DecodeArgs a) {
+  constexpr int R16 = EXP_ROWS;
+  static_assert(EXP_ROWS == 16 && EXP_IC == 64, "thread mapping");
   extern __shared__ __align__(16) float smem[];
   const int ms = a.ms, m = a.m, n = a.n, msv = a.msv, mv = a.mv;
-  float* Ssm = smem;                          // [EXP_ROWS][ms]
-  float* Wacc = Ssm + EXP_ROWS * ms;          // [EXP_ROWS][msv]
-  float* Lsm = Wacc + EXP_ROWS * msv;         // [EXP_ROWS][EXP_IC]
-  float* Usm = Lsm + EXP_ROWS * EXP_IC;       // [64][EXP_IC + 1]
-  float* rowmax = Usm + 64 * (EXP_IC + 1);    // [EXP_ROWS]
-  float* rowsum = rowmax + EXP_ROWS;
-  float* rowscale = rowsum + EXP_ROWS;
+  float* Ssm = smem;                          // [ms][16]
+  float* Wacc = Ssm + R16 * ms;               // [msv][16]
+  float* red = Wacc + R16 * msv;              // [4][64][16 + 1] partial logits of the quarters
+  float* Psm = red + 4 * EXP_IC * (R16 + 1);  // [64][16]
+  float* rowmax = Psm + EXP_IC * R16;         // [16]
+  float* rowsum = rowmax + R16;
+  float* rowscale = rowsum + R16;
 
   const int split = blockIdx.x, rt = blockIdx.y, h = blockIdx.z;
   const int nrows_h = a.B * a.G * a.R;
-  const int row0 = rt * EXP_ROWS;
+  const int row0 = rt * R16;
   const int i_begin = split * a.ws.IR, i_end = min(n, i_begin + a.ws.IR);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const T* theta = static_cast<const T*>(a.theta) + (size_t)h * m * n;
   const T* U = static_cast<const T*>(a.U) + (size_t)h * mv * n;
   const float* S = a.S + (size_t)h * nrows_h * ms;
+  const int ii = tid & 63, qd = tid >> 6;     // position in the chunk, quarter of the retained rows
+  // 16-byte loads of U: rows start on 16-byte boundaries
+  constexpr int EPV = Elems16<T>::N;
+  const bool vec = n % EPV == 0 && (reinterpret_cast<uintptr_t>(U) & 15) == 0;
 
-  for (int x = tid; x < EXP_ROWS * ms; x += 256) {
+  grid_dep_wait();
+  grid_dep_launch();
+  for (int x = tid; x < R16 * ms; x += 256) {
     const int r = x / ms, j = x - r * ms;
-    Ssm[x] = (row0 + r < nrows_h && j < m) ? S[(size_t)(row0 + r) * ms + j] : 0.f;
+    Ssm[j * R16 + r] = (row0 + r < nrows_h && j < m) ? S[(size_t)(row0 + r) * ms + j] : 0.f;
   }
-  for (int x = tid; x < EXP_ROWS * msv; x += 256) Wacc[x] = 0.f;
-  if (tid < EXP_ROWS) { rowmax[tid] = -INFINITY; rowsum[tid] = 0.f; }
+  for (int x = tid; x < R16 * msv; x += 256) Wacc[x] = 0.f;
+  if (tid < R16) { rowmax[tid] = -INFINITY; rowsum[tid] = 0.f; }
   __syncthreads();
 
-  const int ii = tid & 63, rg = tid >> 6;      // column in chunk, group of 4 rows
-  for (int i0 = i_begin; i0 < i_end; i0 += EXP_IC) {
-    // ---- L chunk: [EXP_ROWS x EXP_IC] = S [EXP_ROWS x m] . theta[:, i0:i0+IC]
-    {
-      float acc[4] = {0.f, 0.f, 0.f, 0.f};
-      const bool ok = i0 + ii < i_end;
-      if (ok && a.id_theta) {
+  auto fma16 = [](float (&acc)[R16], const float* v, float x) {      // acc += v[0..15] x, v in shared memory
 #pragma unroll
-        for (int k = 0; k < 4; ++k) acc[k] = Ssm[(rg * 4 + k) * ms + i0 + ii];
+    for (int k = 0; k < R16; k += 4) {
+      const float4 s = *reinterpret_cast<const float4*>(v + k);
+      acc[k] = fmaf(s.x, x, acc[k]); acc[k + 1] = fmaf(s.y, x, acc[k + 1]);
+      acc[k + 2] = fmaf(s.z, x, acc[k + 2]); acc[k + 3] = fmaf(s.w, x, acc[k + 3]);
+    }
+  };
+  for (int i0 = i_begin; i0 < i_end; i0 += EXP_IC) {
+    // ---- L chunk [16 rows x 64] = S theta[:, i0 : i0 + 64]
+    const bool ok = i0 + ii < i_end;
+    {
+      float acc[R16];
+#pragma unroll
+      for (int k = 0; k < R16; ++k) acc[k] = 0.f;
+      if (ok && a.id_theta) {
+        if (qd == 0) fma16(acc, Ssm + (size_t)(i0 + ii) * R16, 1.f);
       } else if (ok) {
         const T* tp = theta + i0 + ii;
-        for (int j = 0; j < m; ++j) {
-          const float t = to_f32(tp[(size_t)j * n]);
+        int j = qd;
+        for (; j + 28 < m; j += 32) {
+          float t[8];
 #pragma unroll
-          for (int k = 0; k < 4; ++k) acc[k] = fmaf(Ssm[(rg * 4 + k) * ms + j], t, acc[k]);
+          for (int e = 0; e < 8; ++e) t[e] = to_f32(tp[(size_t)(j + 4 * e) * n]);
+#pragma unroll
+          for (int e = 0; e < 8; ++e) fma16(acc, Ssm + (size_t)(j + 4 * e) * R16, t[e]);
         }
+        for (; j < m; j += 4) fma16(acc, Ssm + (size_t)j * R16, to_f32(tp[(size_t)j * n]));
       }
 #pragma unroll
-      for (int k = 0; k < 4; ++k) Lsm[(rg * 4 + k) * EXP_IC + ii] = ok ? acc[k] : -INFINITY;
+      for (int k = 0; k < R16; ++k) red[(qd * EXP_IC + ii) * (R16 + 1) + k] = acc[k];
     }
     __syncthreads();
-    // ---- running max, P = exp(L - max), running sum: warp w owns rows 2w and 2w+1
+    // ---- running max, P = exp(L - max), running sum: warp w owns rows 2w and 2w + 1
 #pragma unroll
     for (int rr = 0; rr < 2; ++rr) {
       const int r = warp * 2 + rr;
-      const float l0 = Lsm[r * EXP_IC + lane], l1 = Lsm[r * EXP_IC + lane + 32];
-      float cm = fmaxf(l0, l1);
+      float l[2];
+#pragma unroll
+      for (int x = 0; x < 2; ++x) {
+        const int c = lane + 32 * x;
+        float v = 0.f;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) v += red[(q * EXP_IC + c) * (R16 + 1) + r];
+        l[x] = i0 + c < i_end ? v : -INFINITY;
+      }
+      float cm = fmaxf(l[0], l[1]);
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) cm = fmaxf(cm, __shfl_xor_sync(0xffffffffu, cm, o));
       const float m_old = rowmax[r], m_new = fmaxf(m_old, cm);
-      const float p0 = __expf(l0 - m_new), p1 = __expf(l1 - m_new);
+      const float p0 = __expf(l[0] - m_new), p1 = __expf(l[1] - m_new);
       float ps = p0 + p1;
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) ps += __shfl_xor_sync(0xffffffffu, ps, o);
-      Lsm[r * EXP_IC + lane] = p0;
-      Lsm[r * EXP_IC + lane + 32] = p1;
+      Psm[lane * R16 + r] = p0;
+      Psm[(lane + 32) * R16 + r] = p1;
+      __syncwarp();
       if (lane == 0) {
         const float sc = (m_old == -INFINITY) ? 0.f : __expf(m_old - m_new);
         rowscale[r] = sc;
@@ -89,50 +125,46 @@ __global__ void __launch_bounds__(256) expand_kernel(DecodeArgs a) {
     __syncthreads();
     if (a.id_U) {
       // W = P: the columns of this CTA's range written so far follow the running maximum, the chunk's columns are P
-      for (int x = tid; x < EXP_ROWS * (i0 - i_begin); x += 256) {
-        const int r = x / (i0 - i_begin), j = i_begin + (x - r * (i0 - i_begin));
-        Wacc[r * msv + j] *= rowscale[r];
-      }
-#pragma unroll
-      for (int k = 0; k < 4; ++k)
-        if (i0 + ii < i_end) Wacc[(rg * 4 + k) * msv + i0 + ii] = Lsm[(rg * 4 + k) * EXP_IC + ii];
+      for (int x = tid; x < R16 * (i0 - i_begin); x += 256) Wacc[i_begin * R16 + x] *= rowscale[x & (R16 - 1)];
+      for (int x = tid; x < R16 * min(EXP_IC, i_end - i0); x += 256) Wacc[i0 * R16 + x] = Psm[x];
       __syncthreads();
       continue;
     }
-    // ---- W[:, j] = W[:, j] * scale + P . U[j, i0:i0+IC]^T, 64 rows of U at a time
-    for (int j0 = 0; j0 < mv; j0 += 64) {
-      for (int x = tid; x < 64 * EXP_IC; x += 256) {
-        const int jj = x >> 6, i2 = x & 63;
-        const bool ok = (j0 + jj < mv) && (i0 + i2 < i_end);
-        Usm[jj * (EXP_IC + 1) + i2] = ok ? to_f32(U[(size_t)(j0 + jj) * n + i0 + i2]) : 0.f;
+    // ---- W[:, j] = W[:, j] * scale + P . U[j, i0 : i0 + 64]^T
+    for (int j = tid; j < mv; j += 256) {
+      float acc[R16];
+#pragma unroll
+      for (int k = 0; k < R16; k += 4) {
+        const float4 w = *reinterpret_cast<const float4*>(Wacc + (size_t)j * R16 + k), sc = *reinterpret_cast<const float4*>(rowscale + k);
+        acc[k] = w.x * sc.x; acc[k + 1] = w.y * sc.y; acc[k + 2] = w.z * sc.z; acc[k + 3] = w.w * sc.w;
       }
-      __syncthreads();
-      {
-        const int jj = ii;
-        float acc[4] = {0.f, 0.f, 0.f, 0.f};
-        for (int i2 = 0; i2 < EXP_IC; ++i2) {
-          const float u = Usm[jj * (EXP_IC + 1) + i2];
+      const T* up = U + (size_t)j * n + i0;
+      const int cnt = min(EXP_IC, i_end - i0);
+      int i = 0;
+      if (vec) {
+        for (; i + 4 * EPV <= cnt; i += 4 * EPV) {
+          float u[4][EPV];
 #pragma unroll
-          for (int k = 0; k < 4; ++k) acc[k] = fmaf(Lsm[(rg * 4 + k) * EXP_IC + i2], u, acc[k]);
-        }
-        if (j0 + jj < mv) {
+          for (int v = 0; v < 4; ++v) load16(up + i + v * EPV, u[v]);
 #pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            const int r = rg * 4 + k;
-            Wacc[r * msv + j0 + jj] = Wacc[r * msv + j0 + jj] * rowscale[r] + acc[k];
-          }
+          for (int v = 0; v < 4; ++v)
+#pragma unroll
+            for (int e = 0; e < EPV; ++e) fma16(acc, Psm + (i + v * EPV + e) * R16, u[v][e]);
         }
       }
-      __syncthreads();
+      for (; i < cnt; ++i) fma16(acc, Psm + i * R16, to_f32(up[i]));
+#pragma unroll
+      for (int k = 0; k < R16; k += 4) *reinterpret_cast<float4*>(Wacc + (size_t)j * R16 + k) = make_float4(acc[k], acc[k + 1], acc[k + 2], acc[k + 3]);
     }
+    __syncthreads();
   }
 
   float* Wout = a.W + ((size_t)split * a.H_kv + h) * nrows_h * msv;
-  for (int x = tid; x < EXP_ROWS * msv; x += 256) {
-    const int r = x / msv;
-    if (row0 + r < nrows_h) Wout[(size_t)(row0 + r) * msv + (x - r * msv)] = Wacc[x];
+  for (int x = tid; x < R16 * msv; x += 256) {
+    const int r = x / msv, j = x - r * msv;
+    if (row0 + r < nrows_h) Wout[(size_t)(row0 + r) * msv + j] = Wacc[j * R16 + r];
   }
-  if (tid < EXP_ROWS && row0 + tid < nrows_h)
+  if (tid < R16 && row0 + tid < nrows_h)
     a.wstat[((size_t)split * a.H_kv + h) * nrows_h + row0 + tid] = make_float2(rowmax[tid], rowsum[tid]);
 }
 
@@ -198,7 +230,7 @@ __global__ void __launch_bounds__(256) combine_kernel(DecodeArgs a) {
 }
 
 static size_t expand_smem_bytes(int ms, int msv) {
-  return sizeof(float) * ((size_t)EXP_ROWS * (ms + msv) + EXP_ROWS * EXP_IC + 64 * (EXP_IC + 1) + 3 * EXP_ROWS);
+  return sizeof(float) * ((size_t)EXP_ROWS * (ms + msv) + 4 * EXP_IC * (EXP_ROWS + 1) + EXP_IC * EXP_ROWS + 3 * EXP_ROWS);
 }
 
 template <typename T>
@@ -207,8 +239,7 @@ static cudaError_t launch_expand_t(const DecodeArgs& a, cudaStream_t st) {
   cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(expand_kernel<T>), smem);
   if (e != cudaSuccess) return e;
   dim3 grid(a.ws.NS, ceil_div(a.B * a.G * a.R, EXP_ROWS), a.H_kv);
-  expand_kernel<T><<<grid, 256, smem, st>>>(a);
-  return cudaGetLastError();
+  return launch_dependent(expand_kernel<T>, grid, dim3(256), smem, st, a);
 }
 
 cudaError_t launch_expand(const DecodeArgs& a, int dtype, cudaStream_t st) {
