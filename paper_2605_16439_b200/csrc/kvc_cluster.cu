@@ -2,7 +2,7 @@
 //
 // Bound: latency of the hand-overs (scores -> logits -> probabilities -> weights -> values, each a round trip through L2 or shared
 // memory per unit); the bytes take a tenth to a third of the time.  Measured on B200: 8 sequences x 5 blocks of n = 729, 28/4 heads,
-// 300 text rows: 50 us per call (277 us with the three-phase kernels, whose expansion of such block lengths ran on the CUDA cores);
+// 300 text rows: 37.5 us per call (277 us with the three-phase kernels, whose expansion of such block lengths ran on the CUDA cores);
 // time line: scores until 7 us, logits 14, probabilities 16, weights 18, joined 28, values 36, merged 40.
 // Why one kernel of clusters: a unit's CTAs hand S and the partial weights to each other through L2 behind an mbarrier instead of a
 // kernel boundary, and while the tensor cores expand, the consumers ask the unit's value rows (and the next unit's key rows) into
@@ -30,7 +30,7 @@ struct ClusterBars {
   uint64_t vfull[CL_V_SLOTS], vempty[CL_V_SLOTS];
   uint64_t xfull[CL_X_SLOTS], xempty[CL_X_SLOTS];
   uint64_t l_done, p_ready, w_done, w_free;
-  uint64_t s_ready, w_ready;                                  // cluster-wide: every consumer warp of every CTA
+  uint64_t s_ready, w_ready;                                  // cluster-wide: an arrival of every CTA
   uint64_t text[CL_WARPS][CL_TEXT_SLOTS];
 };
 
@@ -78,6 +78,12 @@ __device__ __forceinline__ uint32_t split_lo(float x0, float x1, uint32_t hi) { 
 }
 
 
+// Slot x of the value ring's weight slices: the first a.nwp behind the groups' reductions in the region of P, which the slices, asked for
+// after w_ready, find free; the others behind the value tiles
+__device__ __forceinline__ uint32_t cl_w_slot(const ClusterArgs& a, int x) {
+  return x < a.nwp ? CL_W_TAIL + (uint32_t)x * a.w_bytes : CL_P_BYTES + a.w_off + (uint32_t)(x - a.nwp) * a.w_bytes;
+}
+
 // What the merge of a (sequence, KV head) has to know about the call's units
 struct ClusterView { const int *pre, *tx; UnitSplit us; int nblk; };
 
@@ -98,30 +104,43 @@ __device__ __forceinline__ int cl_expected(const ClusterArgs& a, const ClusterVi
   return e;
 }
 
-// The last partial of a (sequence, KV head) merges: warps wi of nw take heads wi, wi + nw, ...  A lane finds one partial and its
-// statistics; the values are loaded eight partials at a time
-__device__ __forceinline__ void cl_merge(const ClusterArgs& a, const ClusterView& v, int b, int h, int wi, int nw) {
-  const int G = a.G, lane = fresh(threadIdx.x) & 31, bh = b * a.H_kv + h;
-  const int f0 = cl_first(a, v.pre, b), f1 = cl_first(a, v.pre, b + 1);
-  const int base = h * (v.us.nu * CL_GROUPS * a.NS + a.B) + b;
-  const int total = cl_expected(a, v, b);
-  for (int g = wi; g < G; g += nw) {
+// The last partial of a (sequence, KV head) merges: the G heads of every sequence of list[0 .. n), warps wi of nw taking (sequence, head)
+// pairs wi, wi + nw, ...  A lane finds one partial and its statistics; the values are loaded sixteen partials at a time (L2's latency
+// bounds it: with 8 in flight and a warp group per sequence the merge of 8 sequences of 5 blocks, 28/4 heads, took 8 us, now 3-6).
+__device__ __forceinline__ void cl_merge(const ClusterArgs& a, const ClusterView& v, const int* list, int n, int h, int wi, int nw) {
+  const int G = a.G, lane = fresh(threadIdx.x) & 31;
+#pragma unroll 1
+  for (int e = wi; e < n * G; e += nw) {
+    const int i = e / G, g = e - i * G, b = list[i];
+    const int f0 = cl_first(a, v.pre, b), f1 = cl_first(a, v.pre, b + 1), u0 = f0 / v.us.rb, u1 = (f1 - 1) / v.us.rb;
     float M = -INFINITY, den = 0.f;
     float4 num = make_float4(0.f, 0.f, 0.f, 0.f);
+    int total, p0 = 0;
 #pragma unroll 1
-    for (int p0 = 0; p0 < total; p0 += 32) {
+    do {
       int k = p0 + lane, slot = -1;
-      if (k < total) {
-        if (f0 < f1)
-          for (int u = f0 / v.us.rb; u <= (f1 - 1) / v.us.rb && slot < 0; ++u) {
-            int pa;
-            const int np = cl_pieces(a, v, u, f0, f1, pa);
-            if (k < np) slot = base + u * CL_GROUPS * a.NS + pa + k; else k -= np;
-          }
-        if (slot < 0) slot = a.tslot0 + bh * a.nct + k;
-      }
+      total = 0;
+      if (f0 < f1)
+        for (int u = u0; u <= u1; ++u) {
+          int pa;
+          const int np = cl_pieces(a, v, u, f0, f1, pa);
+          if ((unsigned)k < (unsigned)np) slot = h * (v.us.nu * CL_GROUPS * a.NS + a.B) + b + u * CL_GROUPS * a.NS + pa + k;
+          k -= np; total += np;
+        }
+      const int nt = (cl_text(a, v.tx, b) + a.tc - 1) / a.tc;
+      if ((unsigned)k < (unsigned)nt) slot = a.tslot0 + (b * a.H_kv + h) * a.nct + k;
+      total += nt;
       const float2 st = slot >= 0 ? __ldcg(&a.pml[(size_t)slot * G + g]) : make_float2(-INFINITY, 0.f);
       const int cnt = min(32, total - p0);
+      float4 y[16];
+      auto load = [&](int p) {
+#pragma unroll
+        for (int x = 0; x < 16; ++x) {
+          const int sl = __shfl_sync(0xffffffffu, slot, p + x);
+          y[x] = sl >= 0 ? __ldcg(reinterpret_cast<const float4*>(a.py + ((size_t)sl * G + g) * D + lane * 4)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+      };
+      load(0);
       float mx = st.x;
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
@@ -135,24 +154,21 @@ __device__ __forceinline__ void cl_merge(const ClusterArgs& a, const ClusterView
       den = fmaf(den, sc, d);
       num.x *= sc; num.y *= sc; num.z *= sc; num.w *= sc;
 #pragma unroll 1
-      for (int p = 0; p < cnt; p += 8) {
-        float4 y[8];
+      for (int p = 0;;) {
 #pragma unroll
-        for (int x = 0; x < 8; ++x) {
-          const int sl = __shfl_sync(0xffffffffu, slot, (p + x) & 31);
-          if (p + x < cnt) y[x] = __ldcg(reinterpret_cast<const float4*>(a.py + ((size_t)sl * G + g) * D + lane * 4));
+        for (int x = 0; x < 16; ++x) {
+          const float w = __shfl_sync(0xffffffffu, f, p + x);
+          num.x = fmaf(w, y[x].x, num.x); num.y = fmaf(w, y[x].y, num.y); num.z = fmaf(w, y[x].z, num.z); num.w = fmaf(w, y[x].w, num.w);
         }
-#pragma unroll
-        for (int x = 0; x < 8; ++x) {
-          const float w = __shfl_sync(0xffffffffu, f, (p + x) & 31);
-          if (p + x < cnt) { num.x = fmaf(w, y[x].x, num.x); num.y = fmaf(w, y[x].y, num.y); num.z = fmaf(w, y[x].z, num.z); num.w = fmaf(w, y[x].w, num.w); }
-        }
+        if ((p += 16) >= cnt) break;
+        load(p);
       }
-    }
+      p0 += 32;
+    } while (p0 < total);
     const float inv = den > 0.f ? 1.f / den : 0.f;
     uint2 o;
     o.x = pack2_bf16(num.x * inv, num.y * inv); o.y = pack2_bf16(num.z * inv, num.w * inv);
-    *reinterpret_cast<uint2*>(a.out + ((size_t)bh * G + g) * D + lane * 4) = o;
+    *reinterpret_cast<uint2*>(a.out + ((size_t)(b * a.H_kv + h) * G + g) * D + lane * 4) = o;
   }
 }
 
@@ -358,7 +374,7 @@ __device__ __forceinline__ bool cl_text_part(const CUtensorMap& tmKt, const CUte
     int last = 0;
     if (lane == 0) last = arrive_is_last(&a.cnt[bh], a.token, cl_expected(a, v, b)) ? 1 : 0;
     last = __shfl_sync(0xffffffffu, last, 0);
-    if (last) { __threadfence(); cl_merge(a, v, b, h, 0, 1); }
+    if (last) { __threadfence(); cl_merge(a, v, &b, 1, h, 0, 1); }
   }
   return dead;
 }
@@ -393,7 +409,7 @@ cluster_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
     for (int s = 0; s < CL_V_SLOTS; ++s) { mbar_init(&bars.vfull[s], 1); mbar_init(&bars.vempty[s], 4); }
     for (int s = 0; s < CL_X_SLOTS; ++s) { mbar_init(&bars.xfull[s], 1); mbar_init(&bars.xempty[s], 1); }
     mbar_init(&bars.l_done, 1); mbar_init(&bars.p_ready, CL_WARPS); mbar_init(&bars.w_done, 1); mbar_init(&bars.w_free, CL_WARPS);
-    mbar_init(&bars.s_ready, (uint32_t)(NS * CL_WARPS)); mbar_init(&bars.w_ready, (uint32_t)(NS * CL_WARPS));
+    mbar_init(&bars.s_ready, (uint32_t)NS); mbar_init(&bars.w_ready, (uint32_t)NS);
     for (int w = 0; w < CL_WARPS; ++w)
       for (int s = 0; s < CL_TEXT_SLOTS; ++s) mbar_init(&bars.text[w][s], 1);
     fence_mbar_init();
@@ -539,7 +555,7 @@ cluster_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
           if (vn[g] > 0) bw[g].start(a, pre, u.blk0 + vbl[g]);
         }
         auto w_slice = [&](int x, int jt, int bl) {
-          tma_load_4d(ring + a.w_off + (uint32_t)x * a.w_bytes, &tmWld, jt * CL_TILE, bl * G, 0, cid, &bars.vfull[x]);
+          tma_load_4d(sm + cl_w_slot(a, x), &tmWld, jt * CL_TILE, bl * G, 0, cid, &bars.vfull[x]);
         };
         const int first = most < spg ? most : spg;
         int xd = 0, xg = 0;                                                   // xg: slot of a group's next tile
@@ -672,6 +688,15 @@ cluster_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
 
     const ClusterView view{pre, tx, us, nblk};
     uint32_t round = 0, wpass = 0;
+    // Hand-over to the cluster's CTAs: everything the consumers have written so far, by one arrival per CTA.  The CTA's barrier and one
+    // thread's fence order it (a fence and NS arrivals by every warp took 4 us instead of 2); the readers' proxy fence follows their wait.
+    auto tell_cluster = [&](uint64_t* bar) {
+      named_barrier_sync(1, CL_CONS);
+      if (fresh(tid) < NS) {
+        asm volatile("fence.acq_rel.cluster;\n" ::: "memory");
+        mbar_arrive_remote(map_to_cta(smem_addr(bar), (uint32_t)fresh(tid)));
+      }
+    };
     uint32_t kb = 0, vb = 0;                                    // bit s: parity of the fills of slot s taken so far
     // line gt of a 64-row tile of a capsule store into L2 (gt: thread of the group)
     auto prefetch_tile = [&](const __nv_bfloat16* store, int blk, int jt, int gt) {
@@ -684,7 +709,9 @@ cluster_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
       int b_first, b_last, rr_;
       cl_locate(a, pre, u.blk0, b_first, rr_);
       cl_locate(a, pre, u.blk0 + u.nb - 1, b_last, rr_);
+      int* ndue = reinterpret_cast<int*>(sm + a.tab_off + CL_GROUPS * 512 + (uint32_t)NS * CL_ROWS * 8u + CL_GROUPS * 64);
       named_barrier_sync(1, CL_CONS);                           // the region of P is free (last unit's reductions)
+      if (fresh(tid) == 0) *ndue = 0;
       for (int x = tid; x < (b_last - b_first + 1) * G * 16; x += CL_CONS) {
         const int row = x >> 4, c = x & 15, bb = row / G;
         *reinterpret_cast<uint4*>(sm + (uint32_t)row * CL_QPITCH + c * 16) =
@@ -758,12 +785,7 @@ cluster_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
           jt += P;
           while (jt >= a.vt) { jt -= a.vt; ++bl; if (bl < u.nb) bw.next(a, pre); }
         }
-        fence_proxy_async_all();                                // the scores are read by the TMA engine
-        __syncwarp();
-        if (lane == 0) {
-          asm volatile("fence.acq_rel.cluster;\n" ::: "memory");
-          for (int c = 0; c < NS; ++c) mbar_arrive_remote(map_to_cta(smem_addr(&bars.s_ready), (uint32_t)c));
-        }
+        tell_cluster(&bars.s_ready);
       }
       // the value tiles this group will take into L2 while the expansions run (HBM has nothing else to do)
       {
@@ -924,12 +946,7 @@ cluster_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
         __syncwarp();
         if (wp + 1 < a.npass && lane == 0) mbar_arrive(&bars.w_free);
       }
-      fence_proxy_async_all();
-      __syncwarp();
-      if (lane == 0) {
-        asm volatile("fence.acq_rel.cluster;\n" ::: "memory");
-        for (int c = 0; c < NS; ++c) mbar_arrive_remote(map_to_cta(smem_addr(&bars.w_ready), (uint32_t)c));
-      }
+      tell_cluster(&bars.w_ready);
       // ---------------- step 4: the group's run of value tiles ----------------
       if (!dead && !mbar_wait_cluster_bounded(&bars.w_ready, round & 1u)) dead = true;
       __syncwarp();
@@ -955,7 +972,8 @@ cluster_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
         reset();
         int bl = v0 / a.vt, jt = v0 - bl * a.vt;
         int cur_b = -1, s = grp, nflush = 0;
-        int* flushed = reinterpret_cast<int*>(sm + CL_GROUPS * 16384) + grp * CL_ROWS;      // sequences whose partial of this run is written
+        int mine = 0;                                           // thread x of the group arrives for the run's x-th sequence
+        int* due = reinterpret_cast<int*>(sm + CL_DUE);         // sequences this CTA has to merge
         BlockWalk bw;
         if (v0 < v1) bw.start(a, pre, u.blk0 + bl);
         for (int t = v0; t < v1; ++t) {
@@ -1005,7 +1023,7 @@ cluster_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
           vb ^= 1u << s;
           __syncwarp();
           if (jt * CL_TILE + rg * 16 < a.m) {
-            const unsigned char* wp = ring + a.w_off + s * a.w_bytes;           // [NS][G][64]
+            const unsigned char* wp = sm + cl_w_slot(a, s);           // [NS][G][64]
             uint32_t bw[NH][2], bx[NH][2];
 #pragma unroll
             for (int nh = 0; nh < NH; ++nh) {
@@ -1096,23 +1114,20 @@ cluster_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
               }
               named_barrier_sync(2 + grp, 128);
             }
-            if (gt == 0) flushed[nflush] = b_;
-            ++nflush;
+            if (gt == nflush++) mine = b_;
             reset();
           }
         }
         // the run's partials arrive together: one fence, an atomic per sequence, then the merges that became due
+        const int expected = gt < nflush ? cl_expected(a, view, mine) : 0;
         named_barrier_sync(2 + grp, 128);
         if (gt < nflush) {
-          const int b = flushed[gt];
           __threadfence();                   // the partials of every thread (ordered before by the barrier) before the arrival
-          if (!arrive_is_last(&a.cnt[b * a.H_kv + u.h], a.token, cl_expected(a, view, b))) flushed[gt] = -1;
+          if (arrive_is_last(&a.cnt[mine * a.H_kv + u.h], a.token, expected)) due[atomicAdd(ndue, 1)] = mine;
           __threadfence();
         }
-        named_barrier_sync(2 + grp, 128);
-#pragma unroll 1
-        for (int x = 0; x < nflush; ++x)
-          if (flushed[x] >= 0) cl_merge(a, view, flushed[x], u.h, rg, 4);
+        named_barrier_sync(1, CL_CONS);                         // (a CTA sees a sequence become due once at most)
+        cl_merge(a, view, due, *ndue, u.h, warp, CL_WARPS);
       }
     }
 
@@ -1174,6 +1189,14 @@ int cluster_prec(const kvc_layer* L, bool ragged) {
   return mma ? 1 : 2;
 }
 
+static uint32_t cl_tab_bytes(int ns) { return CL_GROUPS * 512u + (uint32_t)ns * 1024u + 256u; }
+// slots of the value ring (a multiple of the groups) in ring_max bytes and the tail of the region of P
+static int cl_v_slots(uint32_t ring_max, uint32_t w_bytes) {
+  const int tail = (int)((CL_P_BYTES - CL_W_TAIL) / w_bytes);
+  int nv = CL_V_SLOTS;
+  while (nv > 0 && (uint32_t)nv * CL_TILE_BYTES + (uint32_t)(nv > tail ? nv - tail : 0) * w_bytes > ring_max) nv -= CL_GROUPS;
+  return nv;
+}
 static int text_chunk(int T) { return T <= 16 * CL_TEXT_CHUNK ? CL_TEXT_CHUNK : (int)align_up((size_t)ceil_div(T, 16), 16); }
 
 ClusterPlan plan_cluster(const kvc_layer* L, int B, int R, int T, bool ragged) {
@@ -1188,14 +1211,20 @@ ClusterPlan plan_cluster(const kvc_layer* L, int B, int R, int T, bool ragged) {
   p.rbmax = CL_ROWS / G;
   const int nb = B * R;
   // CTAs per cluster: at most 256 columns each (128 where P has two terms); more where the smallest number of units still leaves
-  // SMs to the text (the chain of a unit gets shorter)
+  // SMs to the text (the chain of a unit gets shorter), as long as every group has two slots for value tiles, whose slices of the
+  // weights grow with the ranges (n = 729, 8 sequences, 28/4 heads: 6 CTAs 43.5 us, 8 CTAs with one slot per group 50.3)
   const int gmax = p.prec == 2 ? 2 : 4;
   const int ns_min = ceil_div(p.ncg, gmax);
   if (ns_min > CL_MAX_NS) return p;
   const int nu_min = ceil_div(nb, p.rbmax);
   p.NS = ns_min;
+  const int eb = p.prec >= 1 ? 4 : 2;
+  auto v_slots = [&](int ns) {
+    return cl_v_slots((uint32_t)CL_DYN_LIMIT - 1024u - CL_P_BYTES - cl_tab_bytes(ns) - (ragged ? (uint32_t)(2 * B + 1) * 4u : 0u),
+                      ((uint32_t)(ns * G * 64 * eb) + 127u) & ~127u);
+  };
   for (int ns = p.ncg < CL_MAX_NS ? p.ncg : CL_MAX_NS; ns > ns_min; --ns)
-    if ((long long)H * nu_min * 100 <= (long long)max_clusters(L->device, sms, ns) * 87) { p.NS = ns; break; }
+    if ((long long)H * nu_min * 100 <= (long long)max_clusters(L->device, sms, ns) * 87 && v_slots(ns) >= 2 * CL_GROUPS) { p.NS = ns; break; }
   p.ncl = max_clusters(L->device, sms, p.NS);
   const double kv = 2.0 * nb * m * D * 2 * H + 4.0 * H * m * n, tx = 2.0 * B * H * (double)T * D * 2;
   p.cap = (int)(p.ncl * (kv / (kv + tx)) / H);
@@ -1216,7 +1245,7 @@ ClusterPlan plan_cluster(const kvc_layer* L, int B, int R, int T, bool ragged) {
   p.brow = (int)align_up((size_t)ceil_div(p.prow, p.nbox), 16);
   if (p.npass == 1) p.prow = p.nbox * p.brow;
   p.vt = ceil_div(m, CL_TILE);
-  const int planes = p.prec == 2 ? 2 : 1, eb = p.prec >= 1 ? 4 : 2;
+  const int planes = p.prec == 2 ? 2 : 1;
   {
     const int rows = us.rb * G < CL_ROWS ? us.rb * G : CL_ROWS;
     p.srows = ragged ? CL_ROWS : (int)align_up((size_t)rows, 8);
@@ -1231,21 +1260,21 @@ ClusterPlan plan_cluster(const kvc_layer* L, int B, int R, int T, bool ragged) {
   p.x_bytes = (p.x_bytes + 1023u) & ~1023u;
   p.w_tx = (uint32_t)(p.NS * G * 64 * eb);
   p.w_bytes = (p.w_tx + 127u) & ~127u;
-  const uint32_t tab = CL_GROUPS * 512u + (uint32_t)p.NS * 1024u + 256u;
+  const uint32_t tab = cl_tab_bytes(p.NS);
   const uint32_t pre = ragged ? (uint32_t)(2 * B + 1) * 4u : 0u;
   const uint32_t ring_max = (uint32_t)CL_DYN_LIMIT - 1024u - CL_P_BYTES - tab - pre;
   p.nK = CL_K_SLOTS;
   if ((uint32_t)p.nK * CL_TILE_BYTES > ring_max) p.nK -= CL_GROUPS;
-  p.nV = CL_V_SLOTS;
-  while (p.nV > 0 && (uint32_t)p.nV * (CL_TILE_BYTES + p.w_bytes) > ring_max) p.nV -= CL_GROUPS;
+  p.nV = cl_v_slots(ring_max, p.w_bytes);
   if (p.nV == 0) return p;
+  p.nwp = (int)((CL_P_BYTES - CL_W_TAIL) / p.w_bytes) < p.nV ? (int)((CL_P_BYTES - CL_W_TAIL) / p.w_bytes) : p.nV;
   p.nX = (int)(ring_max / p.x_bytes);
   if (p.nX > CL_X_SLOTS) p.nX = CL_X_SLOTS;
   if (p.nX < 2) return p;
   p.w_off = (uint32_t)p.nV * CL_TILE_BYTES;
   uint32_t ring = (uint32_t)p.nK * CL_TILE_BYTES;
   if ((uint32_t)p.nX * p.x_bytes > ring) ring = (uint32_t)p.nX * p.x_bytes;
-  if (p.w_off + (uint32_t)p.nV * p.w_bytes > ring) ring = p.w_off + (uint32_t)p.nV * p.w_bytes;
+  if (p.w_off + (uint32_t)(p.nV - p.nwp) * p.w_bytes > ring) ring = p.w_off + (uint32_t)(p.nV - p.nwp) * p.w_bytes;
   if (ring + CL_P_BYTES < (uint32_t)CL_WARPS * CL_TEXT_SLOTS * 4096u) ring = (uint32_t)CL_WARPS * CL_TEXT_SLOTS * 4096u - CL_P_BYTES;
   ring = (ring + 127u) & ~127u;
   p.tab_off = CL_P_BYTES + ring;
@@ -1260,6 +1289,11 @@ ClusterPlan plan_cluster(const kvc_layer* L, int B, int R, int T, bool ragged) {
   if (p.ucl < p.ncl && p.text_items > 0) {
     const double share = (kv + tx) * (p.ncl - p.ucl) / p.ncl / tx;
     p.text_ded = share >= 1.0 ? p.text_items : (long long)(share * p.text_items);
+    // ... and at least what they can do while the units' chain runs (a unit: 18 us and 0.3 us per tile of a CTA; a warp's item: 9 us
+    // with its arrival): an item behind the units ends 8-14 us after them, by the latency of one warp's pieces and merge
+    const double unit_us = ceil_div(H * us.nu, p.ucl) * (18.0 + 0.3 * 2.0 * us.rb * p.vt / p.NS);
+    const long long spare = (long long)(unit_us / 9.0) * (p.ncl - p.ucl) * p.NS * CL_WARPS;
+    if (p.text_ded < spare) p.text_ded = spare < p.text_items ? spare : p.text_items;
     // no more clusters than the text has use for
     const long long need = (p.text_ded + (long long)p.NS * CL_WARPS - 1) / ((long long)p.NS * CL_WARPS);
     if (need < p.ncl - p.ucl) p.ncl = p.ucl + (int)need;
@@ -1388,7 +1422,7 @@ cudaError_t launch_cluster(const kvc_layer* L, const DecodeArgs& d, const Cluste
   a.B = B; a.H_kv = H; a.G = G; a.R = R; a.m = m; a.n = n; a.T = d.T;
   a.NS = p.NS; a.ncl = p.ncl; a.ucl = p.ucl; a.cap = p.cap; a.rbmax = p.rbmax; a.ncg = p.ncg; a.ms = p.ms; a.nk1 = p.nk1;
   a.npass = p.npass; a.prow = p.prow; a.nbox = p.nbox; a.brow = p.brow; a.vt = p.vt; a.srows = p.srows; a.nK = p.nK; a.nX = p.nX; a.nV = p.nV;
-  a.x_bytes = p.x_bytes; a.s_bytes = p.s_bytes; a.w_off = p.w_off; a.w_bytes = p.w_bytes; a.w_tx = p.w_tx;
+  a.x_bytes = p.x_bytes; a.s_bytes = p.s_bytes; a.w_off = p.w_off; a.w_bytes = p.w_bytes; a.w_tx = p.w_tx; a.nwp = p.nwp;
   a.tab_off = p.tab_off; a.pre_off = p.pre_off;
   a.tc = p.tc; a.nct = p.nct; a.text_items = (int)p.text_items; a.text_ded = (int)p.text_ded;
   ProfScope prof(KVC_KERNEL_FUSED, st);

@@ -24,6 +24,7 @@ constexpr int CL_ROWS = 128;                       // expansion rows of a unit
 constexpr int CL_TILE = 64;                        // key / value rows per tile
 constexpr uint32_t CL_HALF = CL_TILE * 128;        // one 64-channel half of a tile
 constexpr uint32_t CL_TILE_BYTES = 2 * CL_HALF;
+constexpr uint32_t CL_DUE = CL_GROUPS * 16384, CL_W_TAIL = CL_DUE + 512;      // in the region of P while values are summed: behind the groups' reductions
 constexpr uint32_t CL_P_BYTES = 65536;             // probabilities; queries, weight staging and the warps' parked accumulators in turn
 constexpr int CL_K_SLOTS = 3 * CL_GROUPS, CL_V_SLOTS = 3 * CL_GROUPS, CL_X_SLOTS = 6;      // upper bounds of the rings' slots
 constexpr int CL_MAX_NS = 8;
@@ -47,6 +48,7 @@ struct ClusterPlan {
   int vt;                // 64-row tiles per block
   int srows;             // rows of S loaded per chunk
   int nK, nX, nV;        // slots of the key ring, the expansion ring and the value ring
+  int nwp;                                             // weight slices of the value ring kept in the region of P
   uint32_t x_bytes, s_bytes, w_off, w_bytes, w_tx;     // slot sizes (w_tx: bytes of a slice); the value ring's weights lie behind its tiles
   uint32_t tab_off, pre_off;
   size_t smem;
@@ -97,6 +99,7 @@ struct ClusterArgs {
   int early;
   int B, H_kv, G, R, m, n, T;
   int NS, ncl, ucl, cap, rbmax, ncg, ms, nk1, npass, prow, nbox, brow, vt, srows, nK, nX, nV;
+  int nwp;
   uint32_t x_bytes, s_bytes, w_off, w_bytes, w_tx, tab_off, pre_off;
   int tc, nct;
   int text_items, text_ded;
