@@ -1,4 +1,5 @@
 // Host side of the C ABI: validation, layer handles, workspace layout, kernel sequencing.
+#include <algorithm>
 #include <atomic>
 #include <map>
 #include <mutex>
@@ -88,8 +89,10 @@ WsLayout ws_layout(const kvc_layer* L, int B, int R, int T_cap) {
     // partial outputs of the one-kernel path: per (sequence, KV head) one per unit along the block axis
     size_t np = 0;
     if (B > 0 && R > 0) {
-      const FusedPlan fp = plan_fused(L, B, R);
-      if (fp.ok && L->mode == KVC_MODE_KV && fp.nrg > 1) np = (size_t)B * H_kv * fp.nrg * G;
+      for (int ragged = 0; ragged < 2; ++ragged) {
+        const FusedPlan fp = plan_fused(L, B, R, ragged != 0);
+        if (fp.ok && L->mode == KVC_MODE_KV && fp.nrg > 1) np = std::max(np, (size_t)B * H_kv * fp.nrg * G);
+      }
     }
     w.off_fpy = take(sizeof(float) * np * D);
     w.off_fpml = take(sizeof(float2) * np);
@@ -324,22 +327,74 @@ static bool use_split(const kvc_layer* L, int B, int R) {
   return plan_split(L, B, R).ok != 0;
 }
 
-// Which bf16 shapes take the cluster path: those that the one-kernel and three-kernel paths do not serve (per-sequence lengths, block
-// lengths that are no multiple of 64) and whose expansions are worth its chain of hand-overs.  Measured on B200, us per call, three-phase
-// kernels -> cluster path: where those kernels expand on the CUDA cores (n no multiple of 8) it is ahead at every shape tried
-// (8 sequences x 5 blocks of n = 729, 28/4 heads: 277 -> 51; 1 x 1 block: 75 -> 33; 1 x 4 blocks of n = 81, 8/2 heads: 27 -> 22); where
-// they expand on mma.sync it is from about 1.5e8 flop of expansion per call on (lengths per sequence: 8 x 8 blocks of n = 1024: 154 ->
-// 58, 1 x 4: 43 -> 40; uniform 16 x 8 blocks of n = 400, 8/2 heads, 3.3e8: 45 -> 45; 1 x 2 of n = 144, 32/32 heads, 2e6: 17 -> 21) unless
-// each KV head has one query head, whose few rows leave its 128-row tiles empty (8 x 5 of n = 576, 32/32 heads: 70 -> 88).
+// Which calls with per-sequence lengths and n a multiple of 64 take the one-kernel path (1), which the cluster path (2), which the
+// three-phase kernels (0).  The one-kernel path's time goes with the rounds of its units over the SMs (a unit: 9 us and 0.09 us per retained
+// row, or its bytes, parameters included, at 45 GB/s, up to 90 where few units of long blocks share the L2); the three-phase kernels'
+// with the bytes and the block length; the cluster path's is a chain of some 28 us, long for text, but it spreads few blocks over more SMs.
+// Measured on B200, us per call, one-kernel / cluster / three-phase:
+// One query head per KV head: 8 x 5 blocks of n = 576, 512 text rows 47.7 / 76.7 / 70.1; 8 x 4 of 1024 78 / 99 / 116; 1 x 5 of 576 30.0 /
+// 31.2 / 30.8; 32 x 5 of 576 160 / 205 / 183; 64 x 1 of 576 208 / 153 / 123; 24 x 1 of 1024 136 / 104 / 118; 4 x 16 of 1024 153 / 101 / 153.
+// Groups of query heads, units within one round: 16 x 2 of 1024, 32/8 heads, 80 MB of rows 47 / 59 / 79, 16 x 2 of 576 32 / 41 / 48, 6 x 8 of
+// 320, m = 128, 26 / 30 / 35, but 2 x 2 of 576, 10 MB, 29 / 25 / 29, 4 x 4 of 1024, 28/4 heads, 50 / 37 / 72; more rounds: 16 x 5 of 576,
+// 28/4 heads 66 / 39 / 102.
+static int ragged_path(const kvc_layer* L, int B, int R, int T) {
+  if (L->mode != KVC_MODE_KV || L->passthrough || R < 1 || (L->use_tc != 0 && L->use_tc != -1)) return 0;
+  const FusedPlan f = plan_fused(L, B, R, true);
+  if (L->use_tc == -1) return f.ok;
+  const int sms = L->num_sms > 0 ? L->num_sms : 148, n = L->desc.n, m = L->m, H = L->desc.H_kv;
+  const double rows = 512.0 * B * R * H * m, text = 512.0 * B * H * (double)T, par = 4.0 * m * n;
+  if (L->G > 1) return f.ok && f.units <= sms && (m <= 144 || rows >= 2.5e7) ? 1 : 2;
+  const double floor_us = (rows + text + H * par) / 6.5e6, phases = 8.0 + 0.042 * n + 1.3 * floor_us;
+  const ClusterPlan c = plan_cluster(L, B, R, T, true);
+  const double cluster = c.ok && c.units <= c.ucl ? 28.0 + (n > 576 ? 0.06 * (n - 576) : 0.0) + (1.15 * (rows + H * par) + 2.5 * text) / 6.5e6 : 1e30;
+  double fused = 1e30;
+  if (f.ok) {
+    const int last = (f.units + sms - 1) / sms, ctas = f.units < sms ? f.units : sms;
+    const double rate = n <= 640 || 148 * 45 > 90 * ctas ? (n <= 640 ? 45e3 : 90e3) : 45e3 * 148 / ctas;
+    const double rounds = last > 1 ? 0.5 * ((double)f.units / sms + last) : 1.0;
+    fused = std::max(last * (9.0 + 0.09 * m), rounds * ((rows + text) / f.units + par) / rate);
+  }
+  if (fused < 0.95 * std::min(phases, cluster)) return 1;
+  return cluster < 0.9 * phases ? 2 : 0;
+}
+
+// Which bf16 shapes take the cluster path.  Measured on B200, us per call, cluster / other paths.
+// Block lengths that are no multiple of 64, and per-sequence lengths outside the path above: the other way is the three-phase kernels.
+// It is ahead at every shape tried where those expand on the CUDA cores (n no multiple of 8: 8 x 5 blocks of n = 729, 28/4 heads: 37 /
+// 277) and, with more than one query head per KV head, where they expand on mma.sync (4 x 1 of 400: 22 / 29; 16 x 4 of 196, 32/8 heads:
+// 31 / 65; 1 x 1 of 784, 8/2 heads: 23 / 25; 8 x 2 of 144: 18.8 / 18.6; with lengths per sequence from 1e7 flop of expansion on: 8 x 5 of
+// 144, 6/2 heads, 8e6: 21.7 / 20.8; 2 x 5 of 144, 28/4 heads, 9e6: 22 / 27); with one, its 128-row tiles stay empty (8 x 4 of 400, 32/32
+// heads: 60 / 50).
+// Whole multiples of 64 up to 640, groups of query heads: the other way is the one-kernel path, whose time goes with the rounds of its
+// units and the retained rows (9 us + 0.09 us a row).  The cluster path is ahead (a) on the smallest calls, one unit per KV head, from m
+// = 224 on (1 x 1 of n = 576, 28/4 heads: 21.7 / 25.5; n = 640: 22 / 26.5; m = 205: 21.4 / 20.7), (b) where the rounds of the other are many
+// and its own units are one wave or fill the last (16 x 5 of 576: 43 / 59; 8 x 16 of 640: 50 / 63; 16 x 20 of 576, 16/2 heads: 53 / 92; 64
+// x 8 of 576: 168 / 202; but 32 x 8 of 576, 32/8 heads, 290 MB: 154 / 121).
 // KVC_EXPANSION=cluster forces it where its plan applies, any other value of the variable keeps it off.
-static bool use_cluster(const kvc_layer* L, int B, int R, bool ragged) {
+static bool use_cluster(const kvc_layer* L, int B, int R, int T, bool ragged) {
   if (R < 1 || L->passthrough || L->mode != KVC_MODE_KV || L->desc.dtype != KVC_BF16) return false;
   if (L->use_tc == 5) return true;
-  const int n = L->desc.n;
-  if (L->use_tc != 0 || n < 64 || (!ragged && n % 64 == 0)) return false;
-  if (ragged && (n == 64 || n == 128 || n == 192 || n == 256) && plan_resident(L, B, R, 0).ok) return false;     // read the lengths itself
-  if (cluster_prec(L, ragged) == 2) return true;
-  return L->G > 1 && 4.0 * B * L->desc.H_q * R * (double)L->m * n >= 1.5e8;
+  const int n = L->desc.n, G = L->G;
+  if (L->use_tc != 0 || n < 64) return false;
+  if (ragged || n % 64 != 0) {
+    if (ragged && (n == 64 || n == 128 || n == 192 || n == 256) && plan_resident(L, B, R, 0).ok) return false;     // read the lengths itself
+    if (ragged && n % 64 == 0 && n <= 1024 && cluster_terms(L) == 1) {
+      const int path = ragged_path(L, B, R, T);
+      if (path != 2 || G == 1) return path == 2;
+    }
+    return cluster_terms(L) == 2 || (G > 1 && (!ragged || 4.0 * B * L->desc.H_q * R * (double)L->m * n >= 1e7));
+  }
+  if (n <= 256 || n > 640 || G == 1) return false;
+  const int sms = L->num_sms > 0 ? L->num_sms : 148;
+  const double rows = 512.0 * B * R * L->desc.H_kv * L->m, bytes = rows + 512.0 * B * L->desc.H_kv * (double)T;
+  if (B * R * (long long)G <= 64) return bytes < 8e6 && L->m >= 224;
+  const FusedPlan f = plan_fused(L, B, R);
+  if (f.ok && f.units <= sms) return false;
+  const ClusterPlan c = plan_cluster(L, B, R, T, false);
+  if (!f.ok || !c.ok) return c.ok != 0;
+  const int rounds = (c.units + c.ucl - 1) / c.ucl;
+  if (10ll * c.units < 7ll * rounds * c.ucl) return false;
+  return 1.1 * (25.0 * rounds + 4.0 + 2.4e-6 * bytes / 6.5) < (f.units + sms - 1) / sms * (9.0 + 0.09 * L->m);
 }
 
 // One token per decode call, process-wide: never 0 and never one of the byte patterns a caller is likely to have
@@ -387,7 +442,7 @@ int decode_common(const kvc_layer* L, const void* q, const void* capsules, int B
                           reinterpret_cast<uintptr_t>(out) | (T > 0 ? reinterpret_cast<uintptr_t>(K_txt) |
                           reinterpret_cast<uintptr_t>(V_txt) : 0) | reinterpret_cast<uintptr_t>(L->desc.mu);
 
-  if ((align & 15) == 0 && use_cluster(L, B, R, ragged)) {
+  if ((align & 15) == 0 && use_cluster(L, B, R, T, ragged)) {
     const ClusterPlan cp = plan_cluster(L, B, R, T, ragged);
     if (cp.ok && (ws_limit == 0 || cluster_ws(L, cp, B, R).bytes <= ws_limit)) {
       bool encoded = false;
@@ -426,9 +481,8 @@ int decode_common(const kvc_layer* L, const void* q, const void* capsules, int B
   // bf16 storage with TMA-compatible shapes and pointers: the whole of Algorithm 1 in one kernel
   {
     const bool plain = R == 0 || L->passthrough;            // rows stored verbatim only: served above
-    // one-sided modes are served by the three-phase kernels below; so are per-sequence lengths, except on the shapes the
-    // resident-parameter kernel takes (it reads the lengths itself)
-    const bool one_sided = (R > 0 && L->mode != KVC_MODE_KV) || ragged;
+    // one-sided modes are served by the three-phase kernels below
+    const bool one_sided = R > 0 && L->mode != KVC_MODE_KV;
     // Short blocks whose theta and U fit shared memory (n <= 256, m <= 128, G <= 8) take the resident-parameter kernel: on
     // the n = 256, G = 7, m = 103 shape it ran ahead of the other one-kernel variants at every batch measured (1, 4, 16:
     // 19.2 / 19.5 / 42.4 us against 22.4 / 23.5 / 83.7 us).  KVC_EXPANSION=resident forces it, any other value keeps it off.
@@ -440,14 +494,14 @@ int decode_common(const kvc_layer* L, const void* q, const void* capsules, int B
         if (encoded) return cuda_status(re);
       }
     }
-    if (!plain && !one_sided && (align & 15) == 0 && T <= 64 * SP_OUT_ROWS * SP_TEXT_CHUNK && use_split(L, B, R)) {
+    if (!plain && !one_sided && !ragged && (align & 15) == 0 && T <= 64 * SP_OUT_ROWS * SP_TEXT_CHUNK && use_split(L, B, R)) {
       const SplitPlan sp = plan_split(L, B, R);
       bool encoded = false;
       const cudaError_t se = launch_split(L, a, sp, st, &encoded);
       if (encoded) return cuda_status(se);
     }
     FusedPlan fp{};
-    if (!plain && !one_sided) fp = plan_fused(L, B, R);
+    if (!plain && !one_sided && (!ragged || ragged_path(L, B, R, T) == 1)) fp = plan_fused(L, B, R, ragged);
     if (fp.ok && (align & 15) == 0) {
       bool encoded = false;
       const cudaError_t fe = launch_fused(L, a, fp, st, &encoded);

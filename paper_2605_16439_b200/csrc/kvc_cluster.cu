@@ -3,7 +3,7 @@
 // Bound: latency of the hand-overs (scores -> logits -> probabilities -> weights -> values, each a round trip through L2 or shared
 // memory per unit); the bytes take a tenth to a third of the time.  Measured on B200: 8 sequences x 5 blocks of n = 729, 28/4 heads,
 // 300 text rows: 37.5 us per call (277 us with the three-phase kernels, whose expansion of such block lengths ran on the CUDA cores);
-// time line: scores until 7 us, logits 14, probabilities 16, weights 18, joined 28, values 36, merged 40.
+// time line: scores until 5 us, logits 11, probabilities 13, weights 16, joined 20, values 25, merged 27-34.
 // Why one kernel of clusters: a unit's CTAs hand S and the partial weights to each other through L2 behind an mbarrier instead of a
 // kernel boundary, and while the tensor cores expand, the consumers ask the unit's value rows (and the next unit's key rows) into
 // L2, so that HBM does not idle.
@@ -72,10 +72,6 @@ __device__ __forceinline__ int cl_text(const ClusterArgs& a, const int* tx, int 
 // The value tiles of a unit are dealt in contiguous runs to its P = CL_GROUPS NS pieces (piece p: CTA p mod NS, group p / NS)
 __device__ __forceinline__ int run_start(int p, int nt, int P) { return nt >= P ? p * nt / P : (p < nt ? p : nt); }
 __device__ __forceinline__ int run_of(int t, int nt, int P) { return nt >= P ? ((t + 1) * P - 1) / nt : t; }
-
-__device__ __forceinline__ uint32_t split_lo(float x0, float x1, uint32_t hi) {     // the remainders of a packed pair, packed
-  return pack2_bf16(x0 - __uint_as_float(hi << 16), x1 - __uint_as_float(hi & 0xffff0000u));
-}
 
 
 // Slot x of the value ring's weight slices: the first a.nwp behind the groups' reductions in the region of P, which the slices, asked for
@@ -174,7 +170,7 @@ __device__ __forceinline__ void cl_merge(const ClusterArgs& a, const ClusterView
 
 // Text rows: items of up to tc rows of a (sequence, KV head), a warp each, through the warp's own ring of 16-row pieces (4 KB, keys
 // and values in turn), flash-style; the item's partial goes straight from the registers to the workspace.  True if a wait gave up.
-template <int NH, bool SPLIT_P>
+template <int NH>
 __device__ __forceinline__ bool cl_text_part(const CUtensorMap& tmKt, const CUtensorMap& tmVt, const ClusterArgs& a, const ClusterView& v,
                                              unsigned char* sm, ClusterBars& bars) {
   const Lanes ln = lanes_of(threadIdx.x);
@@ -329,7 +325,8 @@ __device__ __forceinline__ bool cl_text_part(const CUtensorMap& tmKt, const CUte
 #pragma unroll
         for (int nh = 0; nh < NH; ++nh) {
           pb[nh][0] = pack2_bf16(cc[0][2 * nh], cc[0][2 * nh + 1]); pb[nh][1] = pack2_bf16(cc[1][2 * nh], cc[1][2 * nh + 1]);
-          if (SPLIT_P) { px[nh][0] = split_lo(cc[0][2 * nh], cc[0][2 * nh + 1], pb[nh][0]); px[nh][1] = split_lo(cc[1][2 * nh], cc[1][2 * nh + 1], pb[nh][1]); }
+          px[nh][0] = split_lo(cc[0][2 * nh], cc[0][2 * nh + 1], pb[nh][0]);
+          px[nh][1] = split_lo(cc[1][2 * nh], cc[1][2 * nh + 1], pb[nh][1]);
         }
         const uint32_t v_u = tring_u + s * 4096u + (uint32_t)lrowB * 128u;
 #pragma unroll
@@ -339,7 +336,7 @@ __device__ __forceinline__ bool cl_text_part(const CUtensorMap& tmKt, const CUte
 #pragma unroll
           for (int nh = 0; nh < NH; ++nh) {
             mma_bf16_16816(yacc[mt][nh], av, pb[nh][0], pb[nh][1]);
-            if (SPLIT_P) mma_bf16_16816(yacc[mt][nh], av, px[nh][0], px[nh][1]);
+            mma_bf16_16816(yacc[mt][nh], av, px[nh][0], px[nh][1]);
           }
         }
       }
@@ -379,7 +376,7 @@ __device__ __forceinline__ bool cl_text_part(const CUtensorMap& tmKt, const CUte
   return dead;
 }
 
-template <int NH, int PREC>
+template <int NH, int PL>
 __global__ void __launch_bounds__(CL_THREADS, 1)
 cluster_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
                       const __grid_constant__ CUtensorMap tmKt, const __grid_constant__ CUtensorMap tmVt,
@@ -387,8 +384,6 @@ cluster_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
                       const __grid_constant__ CUtensorMap tmTh1, const __grid_constant__ CUtensorMap tmU,
                       const __grid_constant__ CUtensorMap tmWld,
                       const __grid_constant__ ClusterArgs a) {
-  constexpr int PL = PREC == 2 ? 2 : 1;                       // bf16 terms of S and P
-  constexpr bool WF32 = PREC >= 1;                            // partial weights kept in fp32
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* sm = smem_raw + ((1024u - (smem_addr(smem_raw) & 1023u)) & 1023u);
   __shared__ __align__(8) ClusterBars bars;
@@ -908,7 +903,7 @@ cluster_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
           // A step is 128 bytes of every row, alternating over the column warps.  In the last pass the region of P is free: the rows
           // are turned through it so that a store instruction covers four rows of 128 bytes (a lane storing its own row in 16-byte
           // pieces writes half sectors: 5 us instead of 2 at 128 x 410)
-          constexpr int EB = WF32 ? 4 : 2, CWD = 128 / EB;
+          constexpr int EB = 4, CWD = 128 / EB;
           const bool last = wp == a.npass - 1;
           unsigned char* stage = sm + (uint32_t)warp * 4096u;
           unsigned char* wrow = static_cast<unsigned char*>(a.W) + (((size_t)cid * NS + rank) * CL_ROWS + rg * 32) * a.ms * EB;
@@ -921,9 +916,7 @@ cluster_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
               tmem_ld_wait_x32(v);
 #pragma unroll
               for (int q = 0; q < 32 * EB / 16; ++q) {
-                const uint4 x = WF32 ? make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3])
-                                     : make_uint4(pack2_bf16(__uint_as_float(v[(8 * q) & 31]), __uint_as_float(v[(8 * q + 1) & 31])), pack2_bf16(__uint_as_float(v[(8 * q + 2) & 31]), __uint_as_float(v[(8 * q + 3) & 31])),
-                                                  pack2_bf16(__uint_as_float(v[(8 * q + 4) & 31]), __uint_as_float(v[(8 * q + 5) & 31])), pack2_bf16(__uint_as_float(v[(8 * q + 6) & 31]), __uint_as_float(v[(8 * q + 7) & 31])));
+                const uint4 x = make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
                 const int piece = cc * EB / 16 + q, j = j0 + c0 + piece * (16 / EB);
                 if (last) *reinterpret_cast<uint4*>(stage + swz(lane, piece)) = x;
                 else if (row < rows && j < jend) *reinterpret_cast<uint4*>(wrow + ((size_t)lane * a.ms + j) * EB) = x;
@@ -1030,25 +1023,20 @@ cluster_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
               const int g = gid + 8 * nh;
               float w0 = 0.f, w1 = 0.f, w2 = 0.f, w3 = 0.f;
               if (g < G) {
-                const unsigned char* wr = wp + (size_t)g * (WF32 ? 256 : 128) + (rg * 16 + 2 * t4) * (WF32 ? 4 : 2);
+                const unsigned char* wr = wp + (size_t)g * 256 + (rg * 16 + 2 * t4) * 4;
 #pragma unroll
                 for (int sx = 0; sx < CL_MAX_NS; ++sx)
                   if (sx < NS) {
                     const float ff = f[nh][sx];
-                    if (WF32) {
-                      const float2 lo = *reinterpret_cast<const float2*>(wr), hi = *reinterpret_cast<const float2*>(wr + 32);
-                      w0 = fmaf(ff, lo.x, w0); w1 = fmaf(ff, lo.y, w1); w2 = fmaf(ff, hi.x, w2); w3 = fmaf(ff, hi.y, w3);
-                    } else {
-                      const uint32_t lo = *reinterpret_cast<const uint32_t*>(wr), hi = *reinterpret_cast<const uint32_t*>(wr + 16);
-                      w0 = fmaf(ff, __uint_as_float(lo << 16), w0); w1 = fmaf(ff, __uint_as_float(lo & 0xffff0000u), w1);
-                      w2 = fmaf(ff, __uint_as_float(hi << 16), w2); w3 = fmaf(ff, __uint_as_float(hi & 0xffff0000u), w3);
-                    }
-                    wr += (size_t)G * (WF32 ? 256 : 128);
+                    const float2 lo = *reinterpret_cast<const float2*>(wr), hi = *reinterpret_cast<const float2*>(wr + 32);
+                    w0 = fmaf(ff, lo.x, w0); w1 = fmaf(ff, lo.y, w1); w2 = fmaf(ff, hi.x, w2); w3 = fmaf(ff, hi.y, w3);
+                    wr += (size_t)G * 256;
                   }
               }
               bw[nh][0] = pack2_bf16(w0, w1);
               bw[nh][1] = pack2_bf16(w2, w3);
-              if (WF32) { bx[nh][0] = split_lo(w0, w1, bw[nh][0]); bx[nh][1] = split_lo(w2, w3, bw[nh][1]); }
+              bx[nh][0] = split_lo(w0, w1, bw[nh][0]);
+              bx[nh][1] = split_lo(w2, w3, bw[nh][1]);
             }
             const uint32_t v_u = ring_u + s * CL_TILE_BYTES;
             const uint32_t rowB = (uint32_t)((rg * 16 + lrowB) * 128);
@@ -1059,7 +1047,7 @@ cluster_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
 #pragma unroll
               for (int nh = 0; nh < NH; ++nh) {
                 mma_bf16_16816(yacc[mt][nh], av, bw[nh][0], bw[nh][1]);
-                if (WF32) mma_bf16_16816(yacc[mt][nh], av, bx[nh][0], bx[nh][1]);
+                mma_bf16_16816(yacc[mt][nh], av, bx[nh][0], bx[nh][1]);
               }
             }
           }
@@ -1132,7 +1120,7 @@ cluster_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
     }
 
     if (units > 0) { fence_proxy_async(); named_barrier_sync(1, CL_CONS); }      // the text's pieces take the memory the units' tiles were in
-    if (cl_text_part<NH, WF32>(tmKt, tmVt, a, view, sm, bars)) dead = true;
+    if (cl_text_part<NH>(tmKt, tmVt, a, view, sm, bars)) dead = true;
     if (dead && lane == 0) atomicExch(a.status, (int)KVC_ERR_TIMEOUT);
   }
   tc_fence_before();
@@ -1142,12 +1130,8 @@ cluster_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
 }
 
 // ------------------------------------------------------------------------------------------ host side
-template <int NH, int PREC>
-static const void* cluster_kernel_ptr() { return reinterpret_cast<const void*>(cluster_decode_kernel<NH, PREC>); }
-static const void* cluster_kernel_of(int G, int prec) {
-  if (G > 8) return prec == 0 ? cluster_kernel_ptr<2, 0>() : (prec == 1 ? cluster_kernel_ptr<2, 1>() : cluster_kernel_ptr<2, 2>());
-  return prec == 0 ? cluster_kernel_ptr<1, 0>() : (prec == 1 ? cluster_kernel_ptr<1, 1>() : cluster_kernel_ptr<1, 2>());
-}
+template <int NH, int PL>
+static const void* cluster_kernel_ptr() { return reinterpret_cast<const void*>(cluster_decode_kernel<NH, PL>); }
 
 constexpr size_t CL_DYN_LIMIT = 231424;       // 227 KB less the barriers
 
@@ -1160,7 +1144,7 @@ static int max_clusters(int device, int sms, int ns) {
   std::lock_guard<std::mutex> lock(mu);
   int& k = known[device][ns];
   if (k > 0) return k;
-  const void* fn = cluster_kernel_of(1, 0);
+  const void* fn = cluster_kernel_ptr<1, 1>();
   int n = 0;
   if (ensure_dynamic_smem(fn, CL_DYN_LIMIT) == cudaSuccess) {
     cudaLaunchConfig_t cfg = {};
@@ -1178,12 +1162,9 @@ static int max_clusters(int device, int sms, int ns) {
   return k;
 }
 
-// How the scores, probabilities and partial weights are carried.  Calls that the one-kernel and three-kernel bf16 paths serve keep
-// their bf16 operands.  The others (per-sequence lengths, block lengths that are no multiple of 64) used to run on the three-phase
-// kernels, with fp32 weights, or, where n is no multiple of 8 or a score row was too long for those kernels' tensor-core
-// expansion, with fp32 scores and probabilities as well: they keep that precision (two bf16 terms per operand, 16 bits).
-int cluster_prec(const kvc_layer* L, bool ragged) {
-  if (L->desc.n % 64 == 0 && !ragged) return 0;
+// How the scores and probabilities are carried: as one bf16 term, or, where n is no multiple of 8 or a score row is too long for the
+// tensor-core expansion of the three-phase kernels (which kept them in fp32 there), as two (16 bits).  The partial weights are fp32.
+int cluster_terms(const kvc_layer* L) {
   const int ms = (L->mk + 15) / 16 * 16, cg = ceil_div(ms, 256);
   const bool mma = L->desc.n % 8 == 0 && expand_mma_smem_bytes(ms, (int)align_up((size_t)ceil_div(ms, cg), 16)) <= 227u * 1024u;
   return mma ? 1 : 2;
@@ -1206,22 +1187,21 @@ ClusterPlan plan_cluster(const kvc_layer* L, int B, int R, int T, bool ragged) {
   if (!padded_params_ok(L) || (ragged && B > CL_MAX_RAGGED_B)) return p;
   if ((long long)B * R >= (1 << 28) || (long long)B * H * R >= (1ll << 31)) return p;
   const int sms = L->num_sms > 0 ? L->num_sms : 148;
-  p.prec = cluster_prec(L, ragged);
+  p.terms = cluster_terms(L);
   p.ncg = ceil_div(n, 64);
   p.rbmax = CL_ROWS / G;
   const int nb = B * R;
   // CTAs per cluster: at most 256 columns each (128 where P has two terms); more where the smallest number of units still leaves
   // SMs to the text (the chain of a unit gets shorter), as long as every group has two slots for value tiles, whose slices of the
   // weights grow with the ranges (n = 729, 8 sequences, 28/4 heads: 6 CTAs 43.5 us, 8 CTAs with one slot per group 50.3)
-  const int gmax = p.prec == 2 ? 2 : 4;
+  const int gmax = p.terms == 2 ? 2 : 4;
   const int ns_min = ceil_div(p.ncg, gmax);
   if (ns_min > CL_MAX_NS) return p;
   const int nu_min = ceil_div(nb, p.rbmax);
   p.NS = ns_min;
-  const int eb = p.prec >= 1 ? 4 : 2;
   auto v_slots = [&](int ns) {
     return cl_v_slots((uint32_t)CL_DYN_LIMIT - 1024u - CL_P_BYTES - cl_tab_bytes(ns) - (ragged ? (uint32_t)(2 * B + 1) * 4u : 0u),
-                      ((uint32_t)(ns * G * 64 * eb) + 127u) & ~127u);
+                      ((uint32_t)(ns * G * 256) + 127u) & ~127u);
   };
   for (int ns = p.ncg < CL_MAX_NS ? p.ncg : CL_MAX_NS; ns > ns_min; --ns)
     if ((long long)H * nu_min * 100 <= (long long)max_clusters(L->device, sms, ns) * 87 && v_slots(ns) >= 2 * CL_GROUPS) { p.NS = ns; break; }
@@ -1235,7 +1215,10 @@ ClusterPlan plan_cluster(const kvc_layer* L, int B, int R, int T, bool ragged) {
     if (p.nu_max < 1) p.nu_max = 1;
   }
   const UnitSplit us = split_units(nb, p.rbmax, p.cap);
-  p.ucl = (long long)H * us.nu < p.ncl ? H * us.nu : p.ncl;
+  // fewer blocks than the plan's may split into more units (5 blocks into 5, but 8 into 4 of 2): with lengths per sequence, clusters for
+  // all that the cap allows (else the odd ones take a second round: 38 us instead of 21 at 4 x 2 blocks of n = 400, 8/2 heads)
+  const int nu_most = ragged && p.cap < nb && p.cap > us.nu ? p.cap : us.nu;
+  p.ucl = (long long)H * nu_most < p.ncl ? H * nu_most : p.ncl;
   p.ms = (m + 7) & ~7;
   p.nk1 = ceil_div(m, 64);
   const int mpad = (m + 15) & ~15;
@@ -1245,7 +1228,7 @@ ClusterPlan plan_cluster(const kvc_layer* L, int B, int R, int T, bool ragged) {
   p.brow = (int)align_up((size_t)ceil_div(p.prow, p.nbox), 16);
   if (p.npass == 1) p.prow = p.nbox * p.brow;
   p.vt = ceil_div(m, CL_TILE);
-  const int planes = p.prec == 2 ? 2 : 1;
+  const int planes = p.terms;
   {
     const int rows = us.rb * G < CL_ROWS ? us.rb * G : CL_ROWS;
     p.srows = ragged ? CL_ROWS : (int)align_up((size_t)rows, 8);
@@ -1258,7 +1241,7 @@ ClusterPlan plan_cluster(const kvc_layer* L, int B, int R, int T, bool ragged) {
   if (p.x_bytes < reach) p.x_bytes = reach;
   if (p.x_bytes < ub) p.x_bytes = ub;
   p.x_bytes = (p.x_bytes + 1023u) & ~1023u;
-  p.w_tx = (uint32_t)(p.NS * G * 64 * eb);
+  p.w_tx = (uint32_t)(p.NS * G * 256);
   p.w_bytes = (p.w_tx + 127u) & ~127u;
   const uint32_t tab = cl_tab_bytes(p.NS);
   const uint32_t pre = ragged ? (uint32_t)(2 * B + 1) * 4u : 0u;
@@ -1300,6 +1283,7 @@ ClusterPlan plan_cluster(const kvc_layer* L, int B, int R, int T, bool ragged) {
   } else {
     p.ncl = p.ucl;
   }
+  p.units = H * us.nu;
   p.ok = 1;
   return p;
 }
@@ -1311,8 +1295,8 @@ ClusterWs cluster_ws(const kvc_layer* L, const ClusterPlan& p, int B, int R) {
   size_t off = align_up(sizeof(int) * ((size_t)B * H + 1), 256);       // behind the status word of the layout all paths share
   auto take = [&](size_t bytes) { const size_t o = off; off = align_up(off + bytes, 256); return o; };
   const size_t ncl = (size_t)max_clusters(L->device, sms, p.NS), slots = (size_t)H * ((size_t)p.nu_max * CL_GROUPS * p.NS + B);
-  w.off_S = take(sizeof(__nv_bfloat16) * ncl * (p.prec == 2 ? 2 : 1) * CL_ROWS * p.ms);
-  w.off_W = take((p.prec >= 1 ? 4 : 2) * ncl * p.NS * CL_ROWS * p.ms);
+  w.off_S = take(sizeof(__nv_bfloat16) * ncl * p.terms * CL_ROWS * p.ms);
+  w.off_W = take(sizeof(float) * ncl * p.NS * CL_ROWS * p.ms);
   w.off_cnt = take(sizeof(unsigned long long) * (size_t)B * H);
   w.unit_slots = slots;
   const size_t all = slots + (size_t)B * H * p.nct;
@@ -1335,9 +1319,9 @@ size_t cluster_ws_bytes(const kvc_layer* L, int B, int R, int T_cap) {
   return most;
 }
 
-template <int NH, int PREC>
+template <int NH, int PL>
 static cudaError_t launch_cluster_inst(const CUtensorMap* tm, const ClusterArgs& a, const ClusterPlan& p, cudaStream_t st) {
-  cudaError_t e = ensure_dynamic_smem(cluster_kernel_ptr<NH, PREC>(), CL_DYN_LIMIT);
+  cudaError_t e = ensure_dynamic_smem(cluster_kernel_ptr<NH, PL>(), CL_DYN_LIMIT);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(p.ncl * p.NS));
@@ -1351,7 +1335,7 @@ static cudaError_t launch_cluster_inst(const CUtensorMap* tm, const ClusterArgs&
   attr[1].val.clusterDim.x = (unsigned)p.NS; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = p.NS > 1 ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, cluster_decode_kernel<NH, PREC>, tm[0], tm[1], tm[2], tm[3], tm[4], tm[5], tm[6], tm[7], tm[8], a);
+  return cudaLaunchKernelEx(&cfg, cluster_decode_kernel<NH, PL>, tm[0], tm[1], tm[2], tm[3], tm[4], tm[5], tm[6], tm[7], tm[8], a);
 }
 
 cudaError_t launch_cluster(const kvc_layer* L, const DecodeArgs& d, const ClusterPlan& p, char* ws, cudaStream_t st, bool* encoded) {
@@ -1359,7 +1343,7 @@ cudaError_t launch_cluster(const kvc_layer* L, const DecodeArgs& d, const Cluste
   const int B = d.B, H = d.H_kv, R = d.R, G = d.G, m = L->m, n = L->desc.n;
   const ClusterWs w = cluster_ws(L, p, B, R);
   const int ncl = max_clusters(L->device, L->num_sms > 0 ? L->num_sms : 148, p.NS);
-  const int planes = p.prec == 2 ? 2 : 1, eb = p.prec >= 1 ? 4 : 2;
+  const int planes = p.terms;
   CUtensorMap tm[9];
   {
     // capsule rows as (64 channels, m rows of a block, channel half, blocks): a box lands as [half][64 rows][64]
@@ -1399,10 +1383,9 @@ cudaError_t launch_cluster(const kvc_layer* L, const DecodeArgs& d, const Cluste
   }
   {
     const uint64_t dims[4] = {(uint64_t)p.ms, (uint64_t)CL_ROWS, (uint64_t)p.NS, (uint64_t)ncl};
-    const uint64_t str[3] = {(uint64_t)p.ms * eb, (uint64_t)CL_ROWS * p.ms * eb, (uint64_t)p.NS * CL_ROWS * p.ms * eb};
+    const uint64_t str[3] = {(uint64_t)p.ms * 4, (uint64_t)CL_ROWS * p.ms * 4, (uint64_t)p.NS * CL_ROWS * p.ms * 4};
     const uint32_t box_ld[4] = {64u, (uint32_t)G, (uint32_t)p.NS, 1u};
-    const bool ok = p.prec >= 1 ? encode_tensor_map_f32(&tm[8], ws + w.off_W, 4, dims, str, box_ld, false)
-                                : encode_tensor_map_bf16(&tm[8], ws + w.off_W, 4, dims, str, box_ld, false);
+    const bool ok = encode_tensor_map_f32(&tm[8], ws + w.off_W, 4, dims, str, box_ld, false);
     if (!ok) return cudaSuccess;
   }
   *encoded = true;
@@ -1427,8 +1410,8 @@ cudaError_t launch_cluster(const kvc_layer* L, const DecodeArgs& d, const Cluste
   a.tc = p.tc; a.nct = p.nct; a.text_items = (int)p.text_items; a.text_ded = (int)p.text_ded;
   ProfScope prof(KVC_KERNEL_FUSED, st);
   if (G > 8)
-    return p.prec == 0 ? launch_cluster_inst<2, 0>(tm, a, p, st) : (p.prec == 1 ? launch_cluster_inst<2, 1>(tm, a, p, st) : launch_cluster_inst<2, 2>(tm, a, p, st));
-  return p.prec == 0 ? launch_cluster_inst<1, 0>(tm, a, p, st) : (p.prec == 1 ? launch_cluster_inst<1, 1>(tm, a, p, st) : launch_cluster_inst<1, 2>(tm, a, p, st));
+    return p.terms == 1 ? launch_cluster_inst<2, 1>(tm, a, p, st) : launch_cluster_inst<2, 2>(tm, a, p, st);
+  return p.terms == 1 ? launch_cluster_inst<1, 1>(tm, a, p, st) : launch_cluster_inst<1, 2>(tm, a, p, st);
 }
 
 }  // namespace kvc

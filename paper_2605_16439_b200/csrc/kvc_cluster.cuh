@@ -34,7 +34,8 @@ constexpr int CL_TEXT_CHUNK = 128;                 // text rows per item (more f
 
 struct ClusterPlan {
   int ok;
-  int prec;              // 0: S, P and Wp in bf16.  1: Wp in fp32, its product as two bf16 terms.  2: S and P as two bf16 terms too
+  int units;             // work units of the call
+  int terms;             // bf16 terms of S and P
   int NS;                // CTAs per cluster
   int ncl;               // clusters of the grid
   int ucl;               // the first ucl of them take units
@@ -74,7 +75,7 @@ __host__ __device__ __forceinline__ UnitSplit split_units(int nb, int rbmax, int
   return s;
 }
 
-int cluster_prec(const kvc_layer* L, bool ragged);     // operand precision of a call's kind (0, 1, 2)
+int cluster_terms(const kvc_layer* L);                 // bf16 terms of the scores and probabilities (1, 2)
 ClusterPlan plan_cluster(const kvc_layer* L, int B, int R, int T, bool ragged);
 ClusterWs cluster_ws(const kvc_layer* L, const ClusterPlan& p, int B, int R);
 size_t cluster_ws_bytes(const kvc_layer* L, int B, int R, int T_cap);     // for uniform and ragged calls alike; 0 if the path never applies

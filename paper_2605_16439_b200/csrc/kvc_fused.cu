@@ -29,7 +29,14 @@ namespace kvc {
 
 // EW expansion warps, VW value warps, one producer warp.  Every expansion warp owns up to KTW 16-column groups of
 // the logits; NH = 8-head tiles of the group (1: G <= 8, 2: G <= 16); MT = 16-row tiles of expansion rows per unit
-template <int EW, int VW, int KTW, int NH, int MT>
+//
+// RG: the calls with per-sequence lengths.  Blocks and text rows past a sequence's lengths are neither loaded nor computed on, so the
+// capsule rows come in one copy per block; sequences are dealt to the units in the order of their work (the lengths are on the
+// device: every CTA sorts them itself), long ones with short ones.  The weights enter the product with the values as two bf16 terms:
+// these calls had fp32 weights before this kernel took them.
+// Bound as the uniform calls are (8 x 5 blocks of n = 576, 32/32 heads, half to all of 512 text rows: 235 MB in 47.7 us, 4.9 TB/s; the
+// three-phase kernels took 70).
+template <int EW, int VW, int KTW, int NH, int MT, bool RG>
 __global__ void __launch_bounds__((EW + VW + 1) * 32, 1)
 fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
                     const __grid_constant__ CUtensorMap tmKt, const __grid_constant__ CUtensorMap tmVt,
@@ -52,12 +59,79 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
   // score and weight tiles start as zeros: their padding rows and columns are read by the MMAs
   {
     uint32_t* z = reinterpret_cast<uint32_t*>(sm + a.off_S);
-    const int words = (2 * RT * a.sld + 2 * (RT + 16) * SLD) / 2;
+    const int words = (2 * RT * a.sld + (RG ? 4 : 2) * (RT + 16) * SLD) / 2;
     for (int i = tid; i < words; i += FTHREADS) z[i] = 0u;
+  }
+  FusedSeq* tab = reinterpret_cast<FusedSeq*>(sm + a.off_seq);               // RG: [nbg][NB]
+  if (RG) {
+    if (warp == CW && lane == 0 && blockIdx.x < a.units) {
+      // parameters do not depend on the previous kernel: the first stages' into L2 while it drains
+      const int h = blockIdx.x % a.H_kv;
+      for (int c = 0; c < a.NJ && c < a.stages; ++c) tma_prefetch_l2_4d(&tmTh, 0, c * 16 * a.JC, 0, h);
+    }
+    grid_dep_wait();
+    if (blockIdx.x == 0 && tid == 0) *a.status = 0;
+    const int slots = a.nbg * a.NB;
+    // the sorting keys behind the table: (blocks, text rows) of every sequence
+    int2* len = reinterpret_cast<int2*>(tab + slots);
+    for (int b = tid; b < slots; b += FTHREADS) tab[b].b = -1, tab[b].rb = 0, tab[b].tb = 0;
+    for (int b = tid; b < a.B; b += FTHREADS) {
+      const int r = a.R_b ? a.R_b[b] : a.R, t = a.T_b ? a.T_b[b] : a.T;
+      len[b] = make_int2(min(max(r, 0), a.R), min(max(t, 0), a.T));
+    }
+    __syncthreads();
+    for (int b = tid; b < a.B; b += FTHREADS) {
+      const int2 l = len[b];
+      const unsigned work = (unsigned)l.x * a.m + l.y;
+      int rank = 0;
+      for (int o = 0; o < a.B; ++o) {
+        const int2 x = len[o];
+        const unsigned w = (unsigned)x.x * a.m + x.y;
+        rank += w > work || (w == work && o < b) ? 1 : 0;
+      }
+      const int tb = rank / a.nbg, pos = rank - tb * a.nbg, bg = tb & 1 ? a.nbg - 1 - pos : pos;
+      tab[bg * a.NB + tb].b = b; tab[bg * a.NB + tb].rb = l.x; tab[bg * a.NB + tb].tb = l.y;
+      if (blockIdx.x == 0) {
+        const bool bad = (a.R_b && a.R_b[b] != l.x) || (a.T_b && a.T_b[b] != l.y);
+        if (bad) atomicExch(a.status, (int)KVC_ERR_BOUNDS);
+      }
+    }
   }
   __syncthreads();
 
   const int per_h = a.nbg * a.nrg;
+  // unit u -> KV head, group of sequences, group of blocks
+  auto unit_of = [&](int u, int& h, int& bg, int& rg) {
+    if (RG) {                                   // long sequences first
+      const int k = u / a.H_kv;
+      h = u - k * a.H_kv;
+      bg = k / a.nrg; rg = k - bg * a.nrg;
+    } else {
+      h = u / per_h;
+      const int rem = u - h * per_h;
+      bg = rem / a.nrg; rg = rem - bg * a.nrg;
+    }
+  };
+  // sequence tb of group bg (-1: none), and how many of the RB blocks from r0 on it has
+  auto seq_of = [&](int bg, int tb) { return RG ? tab[bg * a.NB + tb].b : (bg * a.NB + tb < a.B ? bg * a.NB + tb : -1); };
+  auto blocks_of = [&](int bg, int tb, int r0) {
+    if (RG) return min(max(tab[bg * a.NB + tb].rb - r0, 0), a.RB);
+    return bg * a.NB + tb < a.B ? min(a.RB, a.R - r0) : 0;
+  };
+  // stages of a pass over the m axis
+  auto stages_of = [&](int bg, int r0) {
+    if (!RG) return a.NJ;
+    int n = 0;
+    for (int x = 0; x < a.NB; ++x) n += blocks_of(bg, x, r0);
+    return n > 0 ? a.NJ : 0;
+  };
+  // text rows of the longest sequence of the group
+  auto text_of = [&](int bg) {
+    if (!RG) return a.T;
+    int t = 0;
+    for (int x = 0; x < a.NB; ++x) t = max(t, tab[bg * a.NB + x].tb);
+    return t;
+  };
 
   if (warp == CW) {
     // ================= producer: one thread feeds the ring =================
@@ -69,11 +143,52 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     bool first = true;
     uint32_t slot = 0, phase = 1;              // parity to wait for on the empty barrier: 1 passes on a fresh barrier
     for (int u = blockIdx.x; u < a.units; u += gridDim.x) {
-      const int h = u / per_h, rem = u - h * per_h;
-      const int bg = rem / a.nrg, rg = rem - bg * a.nrg;
+      int h, bg, rg;
+      unit_of(u, h, bg, rg);
       const int b0 = bg * a.NB, r0 = rg * a.RB;
-      const RowRanges tr = row_ranges(a, rg);
+      const RowRanges tr = row_ranges(a, rg, text_of(bg));
       const int nts = tr.nb;
+      if (RG) {
+        first = false;
+        int nblk = 0;
+        for (int tb = 0; tb < a.NB; ++tb) nblk += blocks_of(bg, tb, r0);
+        const uint32_t blk = (uint32_t)a.JC * 4096u;
+        for (int part = 0; part < 3; ++part) {
+          const int count = part == 1 ? nts : stages_of(bg, r0);
+          for (int c = 0; c < count; ++c) {
+            if (!mbar_wait_bounded(&bars.empty[slot], phase)) { atomicExch(a.status, (int)KVC_ERR_TIMEOUT); return; }
+            unsigned char* dst = sm + slot * a.stage_bytes;
+            uint64_t* bar = &bars.full[slot];
+            if (part == 1) {
+              const int y = tr.b0 + c * a.TCH;
+              uint32_t halves = 0;
+              for (int tb = 0; tb < a.NB; ++tb) halves += min(tr.b1, tab[b0 + tb].tb) > y ? 4u : 0u;
+              const uint32_t seq = (uint32_t)a.TCH * 128u;
+              mbar_expect_tx(bar, halves * seq);
+              for (int tb = 0; tb < a.NB; ++tb) {
+                if (min(tr.b1, tab[b0 + tb].tb) <= y) continue;
+                const int b = tab[b0 + tb].b;
+                unsigned char* d = dst + tb * seq;
+                tma_load_4d(d, &tmKt, 0, y, h, b, bar);
+                tma_load_4d(d + a.txt_half_bytes, &tmKt, 64, y, h, b, bar);
+                tma_load_4d(d + 2 * a.txt_half_bytes, &tmVt, 0, y, h, b, bar);
+                tma_load_4d(d + 3 * a.txt_half_bytes, &tmVt, 64, y, h, b, bar);
+              }
+            } else {
+              const int j0 = c * 16 * a.JC;
+              mbar_expect_tx(bar, a.par_bytes + (uint32_t)nblk * blk);
+              tma_load_4d(dst, part == 0 ? &tmTh : &tmU, 0, j0, 0, h, bar);
+              for (int tb = 0; tb < a.NB; ++tb) {
+                const int nb = blocks_of(bg, tb, r0), k0 = (tab[b0 + tb].b * a.H_kv + h) * a.R + r0;
+                unsigned char* d = dst + a.par_bytes + (uint32_t)(tb * a.RB) * blk;
+                for (int rl = 0; rl < nb; ++rl) tma_load_4d(d + (uint32_t)rl * blk, part == 0 ? &tmK : &tmV, 0, j0, 0, k0 + rl, bar);
+              }
+            }
+            if (++slot == (uint32_t)a.stages) { slot = 0; phase ^= 1u; }
+          }
+        }
+        continue;
+      }
       if (first) {
         // while the stream's previous kernel drains: the K_tilde rows of the first ring of stages are asked into L2 (a
         // prefetch consumes no data, so it need not wait for that kernel; the loads below do)
@@ -117,6 +232,7 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
   const int gid = lane >> 2, t4 = lane & 3;
   const int G = a.G, RB = a.RB, JC = a.JC;
   const int rows16 = 16 * JC;                      // rows of one block inside a stage
+  const int blk16 = RG ? 2 * rows16 : rows16;      // from one block's rows to the next one's, in 128-byte rows
   const int sld = a.sld;
   const uint32_t sm_u = smem_addr(sm);
   const uint32_t q_u = sm_u + a.off_q, S_u = sm_u + a.off_S, W_u = sm_u + a.off_W;
@@ -143,18 +259,20 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
   const int lmid = (lane >> 3) & 1;
   const int WPG = VW / a.NB;                       // value warps per sequence of the unit
 
-  if (warp >= EW && blockIdx.x < a.units) {
+  if (!RG && warp >= EW && blockIdx.x < a.units) {
     // the queries of the first unit: into L2 (and the TLB) before the wait, read after it
-    const int u = blockIdx.x, h = u / per_h, rem = u - h * per_h, b0 = (rem / a.nrg) * a.NB;
+    int h, bg, rg;
+    unit_of(blockIdx.x, h, bg, rg);
+    const int b0 = bg * a.NB;
     const int vt = tid - EW * 32;
     if (vt < a.NB * 32) {
       const int tb = vt >> 5, g = (vt >> 1) & 15, half = vt & 1;     // 128-byte halves of a 256-byte query row
       if (b0 + tb < a.B && g < a.G) prefetch_l2(a.q + ((size_t)(b0 + tb) * a.H_kv * a.G + (size_t)h * a.G + g) * D + half * 64);
     }
   }
-  grid_dep_wait();
+  if (!RG) grid_dep_wait();
   grid_dep_launch();
-  if (blockIdx.x == 0 && tid == 0) *a.status = 0;
+  if (!RG && blockIdx.x == 0 && tid == 0) *a.status = 0;
 
   uint32_t slot = 0, phase = 0;
   uint32_t si = 0, wi = 0;                         // score tiles and weight tiles handed over so far (buffer = count & 1)
@@ -190,14 +308,10 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     }
 
     for (int u = blockIdx.x; u < a.units; u += gridDim.x) {
-      const int h = u / per_h, rem = u - h * per_h;
-      const int bg = rem / a.nrg, rg = rem - bg * a.nrg;
-      const int b0 = bg * a.NB, r0 = rg * a.RB;
-      const int nbv = min(a.NB, a.B - b0);
-      const int rbv = min(RB, a.R - r0);
-      const RowRanges tr = row_ranges(a, rg);
-      const int nts = tr.nb;
-      (void)h;
+      int h, bg, rg;
+      unit_of(u, h, bg, rg);
+      const int r0 = rg * a.RB;
+      const int nts = row_ranges(a, rg, text_of(bg)).nb, NJ = stages_of(bg, r0);
 
       // expansion rows held by this lane: rho = mt*16 + gid + 8*hr  <->  (sequence, block, head)
       bool rvalid[MT][2];
@@ -209,7 +323,7 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
           const int rho = mt * 16 + gid + 8 * hr;
           const int bi = rho / G, g = rho - bi * G;
           const int rbl = bi / RB, rrl = bi - rbl * RB;
-          rvalid[mt][hr] = rho < a.NB * RB * G && rbl < nbv && rrl < rbv;
+          rvalid[mt][hr] = rho < a.NB * RB * G && rrl < blocks_of(bg, rbl, r0);
           rhead[mt][hr] = rvalid[mt][hr] ? rbl * 16 + g : 0;
         }
 
@@ -222,7 +336,7 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
           for (int e = 0; e < 4; ++e) accL[mt][nt][e] = 0.f;
 
       // ---------------- pass A: L[:, my column groups] += S theta ----------------
-      for (int c = 0; c < a.NJ; ++c) {
+      for (int c = 0; c < NJ; ++c) {
         wait_on(&bars.full[slot], phase);
         const uint32_t par_u = sm_u + slot * a.stage_bytes;
         const int nsub = min(JC, (a.m - c * rows16 + 15) >> 4);          // 16-row sub-chunks with rows below m
@@ -300,8 +414,9 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
         for (int x = lane; x < a.NB * 16; x += 32) {
           const int tb = x >> 4, g = x & 15;
           float mx = 0.f;
-          if (g < G && tb < nbv) {
+          if (g < G && seq_of(bg, tb) >= 0) {
             mx = -INFINITY;
+            const int rbv = blocks_of(bg, tb, r0);
             for (int rl = 0; rl < rbv; ++rl) mx = fmaxf(mx, rmax[(tb * RB + rl) * G + g]);
           }
           hvmax[x] = mx;
@@ -354,10 +469,10 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
         for (int x = lane; x < a.NB * 16; x += 32) {
           const int tb = x >> 4, g = x & 15;
           float mx = 0.f, f = 0.f;
-          if (g < G && tb < nbv) {
+          if (g < G && seq_of(bg, tb) >= 0) {
             mx = hvmax[x];
             for (int w = tb * WPG; w < (tb + 1) * WPG; ++w) mx = fmaxf(mx, tmax[w * 16 + g]);
-            f = fast_exp2(hvmax[x] - mx);
+            f = RG && mx == -INFINITY ? 0.f : fast_exp2(hvmax[x] - mx);      // RG: a unit may hold nothing of a sequence
           }
           hmax[x] = mx;
           hfv[x] = f;
@@ -374,7 +489,8 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
         for (int x = lane; x < a.NB * 16; x += 32) {
           const int tb = x >> 4, g = x & 15;
           float vs = 0.f, tsm = 0.f;
-          if (g < G && tb < nbv) {
+          if (g < G && seq_of(bg, tb) >= 0) {
+            const int rbv = blocks_of(bg, tb, r0);
             for (int rl = 0; rl < rbv; ++rl) vs += rsum[(tb * RB + rl) * G + g];
             vs *= hfv[x];
             for (int w = tb * WPG; w < (tb + 1) * WPG; ++w) tsm += tsum[w * 16 + g];
@@ -386,7 +502,7 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
       named_barrier_sync(1, FCONS);                                   // B4: head sums
 
       // ---------------- pass C: W = P U^T, reduced over the expansion warps ----------------
-      for (int c = 0; c < a.NJ; ++c) {
+      for (int c = 0; c < NJ; ++c) {
         wait_on(&bars.full[slot], phase);
         const uint32_t par_u = sm_u + slot * a.stage_bytes;
         const int nsub = min(JC, (a.m - c * rows16 + 15) >> 4);
@@ -432,7 +548,10 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
             float w = 0.f;
 #pragma unroll
             for (int x = 0; x < EW; ++x) w += wp[x * RT * 16];
-            W_sm[wbuf * ((RT + 16) * SLD) + (idx >> 4) * SLD + (idx & 15)] = __float2bfloat16_rn(w * rowf[idx >> 4]);
+            w *= rowf[idx >> 4];
+            const __nv_bfloat16 hi = __float2bfloat16_rn(w);
+            W_sm[wbuf * ((RT + 16) * SLD) + (idx >> 4) * SLD + (idx & 15)] = hi;
+            if (RG) W_sm[(2 + wbuf) * ((RT + 16) * SLD) + (idx >> 4) * SLD + (idx & 15)] = __float2bfloat16_rn(w - __bfloat162float(hi));
           }
           named_barrier_arrive(BAR_W_READY + (int)wbuf, FCONS);
           ++wi;
@@ -450,20 +569,21 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     const int msplit = a.msplit, mshift = a.mshift;           // a task covers the row tiles mt with (mt >> mshift) == its group
 
     for (int u = blockIdx.x; u < a.units; u += gridDim.x) {
-      const int h = u / per_h, rem = u - h * per_h;
-      const int bg = rem / a.nrg, rg = rem - bg * a.nrg;
-      const int b0 = bg * a.NB, r0 = rg * a.RB;
-      const int nbv = min(a.NB, a.B - b0);
-      const int rbv = min(RB, a.R - r0);
-      const RowRanges tr = row_ranges(a, rg);
-      const int nts = tr.nb;
+      int h, bg, rg;
+      unit_of(u, h, bg, rg);
+      const int r0 = rg * a.RB;
+      const RowRanges tr = row_ranges(a, rg, text_of(bg));
+      const int nts = tr.nb, NJ = stages_of(bg, r0);
+      const int rbv = blocks_of(bg, bl, r0);                     // blocks and text rows of this warp's sequence
+      const int ts1 = RG ? min(tr.b1, tab[bg * a.NB + bl].tb) : tr.b1;
 
       // ---- queries of the unit's sequences: [NB][16 heads][128], heads >= G and absent sequences are zero rows
       for (int idx = vtid; idx < a.NB * 256; idx += VTH) {
         const int tb = idx >> 8, g = (idx >> 4) & 15, piece = idx & 15;
         uint4 v = make_uint4(0u, 0u, 0u, 0u);
-        if (tb < nbv && g < G)
-          v = *reinterpret_cast<const uint4*>(a.q + ((size_t)(b0 + tb) * a.H_kv * G + (size_t)h * G + g) * D + piece * 8);
+        const int b = seq_of(bg, tb);
+        if (b >= 0 && g < G)
+          v = *reinterpret_cast<const uint4*>(a.q + ((size_t)b * a.H_kv * G + (size_t)h * G + g) * D + piece * 8);
         *reinterpret_cast<uint4*>(q_sm + (tb * 16 + g) * QLD + piece * 8) = v;
       }
       named_barrier_sync(3, VTH);
@@ -479,7 +599,7 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
         }
 
       // ---------------- pass A: S[rows of block][16] = sigma q K^T for my (block, sub-chunk) tasks ----------------
-      for (int c = 0; c < a.NJ; ++c) {
+      for (int c = 0; c < NJ; ++c) {
         wait_on(&bars.full[slot], phase);
         const uint32_t k_u = sm_u + slot * a.stage_bytes + a.par_bytes;
         const int nsub = min(JC, (a.m - c * rows16 + 15) >> 4);
@@ -488,8 +608,9 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
         __nv_bfloat16* Sb = S_sm + sbuf * (RT * sld);
         for (int task = wig; task < RB * nsub; task += WPG) {
           const int rl = nsub == 1 ? task : task / nsub, s = task - rl * nsub;
+          if (RG && rl >= rbv) continue;
           const int bi = bl * RB + rl;
-          const uint32_t rowoff = k_u + (uint32_t)((bi * rows16 + s * 16 + lrow) * 128);
+          const uint32_t rowoff = k_u + (uint32_t)((bi * blk16 + s * 16 + lrow) * 128);
           uint32_t af[8][4];
 #pragma unroll
           for (int ks = 0; ks < 8; ++ks)
@@ -532,7 +653,6 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
         wait_on(&bars.full[slot], phase);
         const uint32_t kt_u = sm_u + slot * a.stage_bytes, vt_u = kt_u + 2 * a.txt_half_bytes;
         for (int tile = wig; tile * 16 < a.TCH; tile += WPG) {
-          const int ts1 = tr.b1;
           const int t_first = tr.b0 + ts * a.TCH + tile * 16;
           if (t_first >= ts1) break;
           const int row0 = bl * a.TCH + tile * 16;
@@ -608,10 +728,26 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
               }
             }
           }
+          if (RG && t_first + 16 > ts1) {
+            // rows past the sequence's length may hold anything: out of the product, and of the way of the next copy into this stage
+            for (int x = lane; x < (t_first + 16 - ts1) * 16; x += 32) {
+              const int rr = row0 + (ts1 - t_first) + (x >> 4), c = x & 15;
+              *reinterpret_cast<uint4*>(sm + slot * a.stage_bytes + (2 + (c >> 3)) * a.txt_half_bytes + (uint32_t)(rr * 128 + (c & 7) * 16)) = make_uint4(0u, 0u, 0u, 0u);
+            }
+            fence_proxy_async();
+            __syncwarp();
+          }
           // y^T[128][heads] += V_txt^T[128][16 rows] P^T[16 rows][heads]
           uint32_t pb[2][2];
           pb[0][0] = pack2_bf16(cc[0][0], cc[0][1]); pb[0][1] = pack2_bf16(cc[1][0], cc[1][1]);
           pb[1][0] = pack2_bf16(cc[0][2], cc[0][3]); pb[1][1] = pack2_bf16(cc[1][2], cc[1][3]);
+          uint32_t px[2][2];                           // RG: the second terms of the probabilities
+          if (RG) {
+#pragma unroll
+            for (int nh = 0; nh < NH; ++nh)
+#pragma unroll
+              for (int x = 0; x < 2; ++x) px[nh][x] = split_lo(cc[x][2 * nh], cc[x][2 * nh + 1], pb[nh][x]);
+          }
           uint32_t av[8][4];
 #pragma unroll
           for (int mt = 0; mt < 8; ++mt)
@@ -619,7 +755,10 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
 #pragma unroll
           for (int mt = 0; mt < 8; ++mt)
 #pragma unroll
-            for (int nh = 0; nh < NH; ++nh) mma_bf16_16816(yacc[mt][nh], av[mt], pb[nh][0], pb[nh][1]);
+            for (int nh = 0; nh < NH; ++nh) {
+              mma_bf16_16816(yacc[mt][nh], av[mt], pb[nh][0], pb[nh][1]);
+              if (RG) mma_bf16_16816(yacc[mt][nh], av[mt], px[nh][0], px[nh][1]);
+            }
         }
         release();
       }
@@ -655,7 +794,7 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
       named_barrier_sync(1, FCONS);                                   // B4: head sums
 
       // ---------------- pass C: y^T[128][heads] += V^T[128][16 rows of block] W^T[16][heads of block] ----------------
-      for (int c = 0; c < a.NJ; ++c) {
+      for (int c = 0; c < NJ; ++c) {
         wait_on(&bars.full[slot], phase);
         const uint32_t v_u = sm_u + slot * a.stage_bytes + a.par_bytes;
         const int nsub = min(JC, (a.m - c * rows16 + 15) >> 4);
@@ -664,11 +803,12 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
           named_barrier_sync(BAR_W_READY + (int)wbuf, FCONS);
           for (int task = wig; task < RB * msplit; task += WPG) {          // my (block, row-tile group) tasks
             const int rl = task >> (3 - mshift), mg = task & (msplit - 1);
-            if (rl >= rbv || bl >= nbv) continue;
+            if (rl >= rbv) continue;
             const int bi = bl * RB + rl;
-            uint32_t bw[4];
+            uint32_t bw[4], bx[4];
             ldsm_x4(bw, W_u + (uint32_t)((wbuf * ((RT + 16) * SLD) + (bi * G + lrowB) * SLD + lmid * 8) * 2));
-            const uint32_t rowoff = v_u + (uint32_t)((bi * rows16 + s * 16 + lrowB) * 128);
+            if (RG) ldsm_x4(bx, W_u + (uint32_t)(((2 + wbuf) * ((RT + 16) * SLD) + (bi * G + lrowB) * SLD + lmid * 8) * 2));
+            const uint32_t rowoff = v_u + (uint32_t)((bi * blk16 + s * 16 + lrowB) * 128);
             uint32_t av[8][4];
 #pragma unroll
             for (int mt = 0; mt < 8; ++mt)
@@ -678,7 +818,10 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
             for (int mt = 0; mt < 8; ++mt)
               if ((mt >> mshift) == mg) {
 #pragma unroll
-                for (int nh = 0; nh < NH; ++nh) mma_bf16_16816(yacc[mt][nh], av[mt], bw[2 * nh], bw[2 * nh + 1]);
+                for (int nh = 0; nh < NH; ++nh) {
+                  mma_bf16_16816(yacc[mt][nh], av[mt], bw[2 * nh], bw[2 * nh + 1]);
+                  if (RG) mma_bf16_16816(yacc[mt][nh], av[mt], bx[2 * nh], bx[2 * nh + 1]);
+                }
               }
           }
           named_barrier_arrive(BAR_W_FREE + (int)wbuf, FCONS);
@@ -688,7 +831,7 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
       }
 
       // ---------------- unit end: reduce over the value warps, mu term, normalise or leave a partial ----------------
-      const int bh = b0 * a.H_kv + h;                    // used when the block axis is split (NB == 1)
+      const int bh = max(seq_of(bg, 0), 0) * a.H_kv + h; // used when the block axis is split (NB == 1)
       const size_t pbase = ((size_t)bh * a.nrg + rg) * G;
       const int YHG = a.yhg;
       for (int g0 = 0; g0 < G; g0 += YHG) {
@@ -709,14 +852,16 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
           }
         named_barrier_sync(3, VTH);
         const int hg = min(YHG, G - g0);
-        for (int idx = vtid; idx < nbv * hg * D; idx += VTH) {
+        for (int idx = vtid; idx < a.NB * hg * D; idx += VTH) {
           const int col = idx & (D - 1), gg = (idx >> 7) % hg, tb = idx / (D * hg);
-          const int g = g0 + gg;
+          const int g = g0 + gg, b = seq_of(bg, tb);
+          if (b < 0) continue;
           float y = 0.f;
           for (int w = tb * WPG; w < (tb + 1) * WPG; ++w) y += yred[(w * YHG + gg) * D + col];
           y = fmaf(vsum[tb * 16 + g], __bfloat162float(a.mu[h * D + col]), y);
           if (a.nrg == 1)
-            a.out[((size_t)(b0 + tb) * a.H_kv * G + (size_t)h * G + g) * D + col] = __float2bfloat16_rn(y / hsum[tb * 16 + g]);
+            a.out[((size_t)b * a.H_kv * G + (size_t)h * G + g) * D + col] =
+                __float2bfloat16_rn(RG && hsum[tb * 16 + g] == 0.f ? 0.f : y / hsum[tb * 16 + g]);       // RG: nothing to attend to
           else
             a.part_y[(pbase + g) * D + col] = y;
         }
@@ -749,8 +894,8 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
               float M = -INFINITY, den = 0.f;
               for (int p = 0; p < a.nrg; ++p) M = fmaxf(M, mlm[p * G + vtid]);
               for (int p = 0; p < a.nrg; ++p) den = fmaf(fast_exp2(mlm[p * G + vtid] - M), mlm[npg + p * G + vtid], den);
-              const float inv = 1.f / den;
-              for (int p = 0; p < a.nrg; ++p) mlm[2 * npg + p * G + vtid] = fast_exp2(mlm[p * G + vtid] - M) * inv;
+              const float inv = RG && M == -INFINITY ? 0.f : 1.f / den;
+              for (int p = 0; p < a.nrg; ++p) mlm[2 * npg + p * G + vtid] = RG && M == -INFINITY ? 0.f : fast_exp2(mlm[p * G + vtid] - M) * inv;
             }
             named_barrier_sync(3, VTH);
             // four output columns per thread, up to eight partials' loads in flight: the merge is a chain of L2 round trips
@@ -780,7 +925,7 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
               for (; p < a.nrg; ++p) acc(__ldcg(reinterpret_cast<const float4*>(yp + (size_t)p * G * D)), wp[p * G]);
               uint2 o;
               o.x = pack2_bf16(num.x, num.y); o.y = pack2_bf16(num.z, num.w);
-              *reinterpret_cast<uint2*>(a.out + ((size_t)b0 * a.H_kv * G + (size_t)h * G + g) * D + col) = o;
+              *reinterpret_cast<uint2*>(a.out + ((size_t)bh * G + g) * D + col) = o;
             }
           } else {
             for (int idx = vtid; idx < G * D; idx += VTH) {
@@ -788,13 +933,13 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
               float M = -INFINITY;
               for (int p = 0; p < a.nrg; ++p) M = fmaxf(M, __ldcg(&a.part_ml[p0 + (size_t)p * G + g]).x);
               float num = 0.f, den = 0.f;
-              for (int p = 0; p < a.nrg; ++p) {
+              for (int p = 0; p < a.nrg && !(RG && M == -INFINITY); ++p) {
                 const float2 ml = __ldcg(&a.part_ml[p0 + (size_t)p * G + g]);
                 const float w = fast_exp2(ml.x - M);
                 den = fmaf(w, ml.y, den);
                 num = fmaf(w, __ldcg(&a.part_y[(p0 + (size_t)p * G + g) * D + col]), num);
               }
-              a.out[((size_t)b0 * a.H_kv * G + (size_t)h * G + g) * D + col] = __float2bfloat16_rn(num / den);
+              a.out[((size_t)bh * G + g) * D + col] = __float2bfloat16_rn(RG && M == -INFINITY ? 0.f : num / den);
             }
           }
         }
@@ -811,7 +956,7 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
 // the text length: a decode loop re-encodes them for the same few stores again and again, so a handle keeps the last few.
 struct kvc_map_cache {
   struct Entry {
-    bool valid;
+    bool valid, rg;
     int B, R, tc, JC, RB, NB;
     const void* Kc;
     CUtensorMap tm[4];          // K_tilde, V_tilde, theta, U
@@ -879,9 +1024,9 @@ static void warp_split(int n, int* ew, int* vw, int* ktw_max) {
   else { *ew = 11; *vw = 4; *ktw_max = 6; }                  // n <= 1024: the expansion dominates
 }
 
-FusedPlan plan_fused(const kvc_layer* L, int B, int R) {
+FusedPlan plan_fused(const kvc_layer* L, int B, int R, bool ragged) {
   if (L->use_tc == -2) return FusedPlan{};      // the three-phase kernels were asked for
-  if (L->use_tc >= 0 && L->use_tc != 3) {
+  if (!ragged && L->use_tc >= 0 && L->use_tc != 3) {
     // The tensor-memory variant pays per tcgen05.mma, not per expansion row: it wins for long blocks once two row
     // tiles per unit still give most SMs a unit (measured on the n = 1024, G = 7 shape: ahead from batch 16 on,
     // behind at batches 1-4 where units of half the size halve the latency).
@@ -899,6 +1044,7 @@ FusedPlan plan_fused(const kvc_layer* L, int B, int R) {
   const int G = L->G, n = L->desc.n, m = L->m, H_kv = L->desc.H_kv;
   if (L->desc.dtype != KVC_BF16 || L->passthrough || R < 1 || B < 1 || n % 64 != 0 || n > 1024 || G > 16) return p;
   if (reinterpret_cast<uintptr_t>(L->desc.theta) & 15 || reinterpret_cast<uintptr_t>(L->desc.U) & 15) return p;
+  if (ragged && (B > FUSED_MAX_RAGGED_B || (long long)B * H_kv * R >= (1ll << 31))) return p;
   const int sms = L->num_sms > 0 ? L->num_sms : 148;
   int ktw_max = 0;
   warp_split(n, &p.EW, &p.VW, &ktw_max);
@@ -930,6 +1076,7 @@ FusedPlan plan_fused(const kvc_layer* L, int B, int R) {
   p.par_bytes = (uint32_t)p.ncg * p.JC * 2048u;
   p.k_half_bytes = (uint32_t)p.NB * p.RB * p.JC * 2048u;
   p.stage_bytes = p.par_bytes + 2 * p.k_half_bytes;
+  if (ragged) p.k_half_bytes = (uint32_t)p.JC * 2048u;          // of one block
   int tch = (int)(p.stage_bytes / (p.NB * 512u)) & ~15;
   p.TCH = tch > 256 ? 256 : tch;
   if (p.TCH < 16) return p;
@@ -948,7 +1095,7 @@ FusedPlan plan_fused(const kvc_layer* L, int B, int R) {
   auto take = [&](uint32_t bytes) { uint32_t o = off; off = (off + bytes + 127u) & ~127u; return o; };
   p.off_q = take((uint32_t)p.NB * 16 * QLD * 2);
   const int rt = ROWS * p.MT;
-  p.off_S = take((uint32_t)(2 * rt * p.sld + 2 * (rt + 16) * SLD) * 2);
+  p.off_S = take((uint32_t)(2 * rt * p.sld + (ragged ? 4 : 2) * (rt + 16) * SLD) * 2);
   p.off_W = p.off_S + (uint32_t)2 * rt * p.sld * 2;
   p.off_wred = take((uint32_t)2 * p.EW * rt * 16 * 4);
   p.off_rstat = take((uint32_t)2 * p.EW * rt * 4);
@@ -956,6 +1103,7 @@ FusedPlan plan_fused(const kvc_layer* L, int B, int R) {
   p.off_hstat = take((uint32_t)(5 * p.NB * 16 + rt) * 4);
   p.yhg = G > 4 ? 8 : (G > 2 ? 4 : 2);
   p.off_yred = take((uint32_t)p.VW * p.yhg * D * 4);
+  p.off_seq = take(ragged ? (uint32_t)(p.nbg * p.NB * sizeof(FusedSeq) + B * 8) : 0u);
   p.misc_bytes = off;
   const uint32_t avail = SMEM_LIMIT - 1024u - 2048u - p.misc_bytes;   // alignment slack; static shared memory and its padding
   int stages = (int)(avail / p.stage_bytes);
@@ -968,32 +1116,33 @@ FusedPlan plan_fused(const kvc_layer* L, int B, int R) {
 }
 
 
-template <int EW, int VW, int KTW, int NH, int MT>
+template <int EW, int VW, int KTW, int NH, int MT, bool RG>
 static cudaError_t launch_inst(const CUtensorMap* tm, const FusedArgs& fa, const FusedPlan& p, cudaStream_t st) {
   {
-    cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(fused_decode_kernel<EW, VW, KTW, NH, MT>), p.smem_bytes);
+    cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(fused_decode_kernel<EW, VW, KTW, NH, MT, RG>), p.smem_bytes);
     if (e != cudaSuccess) return e;
   }
-  return launch_dependent(fused_decode_kernel<EW, VW, KTW, NH, MT>, dim3(p.grid), dim3((EW + VW + 1) * 32), p.smem_bytes, st, tm[0],
+  return launch_dependent(fused_decode_kernel<EW, VW, KTW, NH, MT, RG>, dim3(p.grid), dim3((EW + VW + 1) * 32), p.smem_bytes, st, tm[0],
                           tm[1], tm[2], tm[3], tm[4], tm[5], fa);
 }
 
-template <int NH>
+template <int NH, bool RG>
 static cudaError_t launch_nh(const CUtensorMap* tm, const FusedArgs& fa, const FusedPlan& p, cudaStream_t st) {
-  if (p.EW == 4) return p.MT == 2 ? launch_inst<4, 8, 4, NH, 2>(tm, fa, p, st) : launch_inst<4, 8, 4, NH, 1>(tm, fa, p, st);
-  if (p.EW == 5) return launch_inst<5, 10, 8, NH, 1>(tm, fa, p, st);
-  return launch_inst<11, 4, 6, NH, 1>(tm, fa, p, st);
+  if (p.EW == 4) return p.MT == 2 ? launch_inst<4, 8, 4, NH, 2, RG>(tm, fa, p, st) : launch_inst<4, 8, 4, NH, 1, RG>(tm, fa, p, st);
+  if (p.EW == 5) return launch_inst<5, 10, 8, NH, 1, RG>(tm, fa, p, st);
+  return launch_inst<11, 4, 6, NH, 1, RG>(tm, fa, p, st);
 }
 
 cudaError_t launch_fused(const kvc_layer* L, const DecodeArgs& a, const FusedPlan& p, cudaStream_t st, bool* encoded) {
   const int H_kv = a.H_kv, m = a.m, n = a.n, R = a.R, B = a.B;
+  const bool rg = a.R_b != nullptr || a.T_b != nullptr;
   CUtensorMap tm[6];
   *encoded = false;
   bool cached = false;
   if (L->maps) {
     std::lock_guard<std::mutex> lock(L->maps->mu);
     for (const auto& x : L->maps->e)
-      if (x.valid && x.B == B && x.R == R && x.tc == p.tc && x.JC == p.JC && x.RB == p.RB && x.NB == p.NB && x.Kc == a.Kc) {
+      if (x.valid && x.rg == rg && x.B == B && x.R == R && x.tc == p.tc && x.JC == p.JC && x.RB == p.RB && x.NB == p.NB && x.Kc == a.Kc) {
         tm[0] = x.tm[0]; tm[1] = x.tm[1]; tm[4] = x.tm[2]; tm[5] = x.tm[3];
         cached = true;
         break;
@@ -1003,13 +1152,17 @@ cudaError_t launch_fused(const kvc_layer* L, const DecodeArgs& a, const FusedPla
     const uint64_t dims[5] = {(uint64_t)D, (uint64_t)m, (uint64_t)R, (uint64_t)H_kv, (uint64_t)B};
     const uint64_t str[4] = {256ull, (uint64_t)m * 256, (uint64_t)R * m * 256, (uint64_t)H_kv * R * m * 256};
     const uint32_t box[5] = {64u, (uint32_t)(16 * p.JC), (uint32_t)p.RB, 1u, (uint32_t)p.NB};
-    if (!encode_tensor_map_bf16(&tm[0], a.Kc, 5, dims, str, box)) return cudaSuccess;
-    if (!encode_tensor_map_bf16(&tm[1], a.Vc, 5, dims, str, box)) return cudaSuccess;
+    // per-sequence lengths: a block per copy, viewed as (64 columns, m rows, 2 halves of a row, blocks)
+    const uint64_t dims_rg[4] = {64ull, (uint64_t)m, 2ull, (uint64_t)B * H_kv * R};
+    const uint64_t str_rg[3] = {256ull, 128ull, (uint64_t)m * 256};
+    const uint32_t box_rg[4] = {64u, (uint32_t)(16 * p.JC), 2u, 1u};
+    if (!encode_tensor_map_bf16(&tm[0], a.Kc, rg ? 4 : 5, rg ? dims_rg : dims, rg ? str_rg : str, rg ? box_rg : box)) return cudaSuccess;
+    if (!encode_tensor_map_bf16(&tm[1], a.Vc, rg ? 4 : 5, rg ? dims_rg : dims, rg ? str_rg : str, rg ? box_rg : box)) return cudaSuccess;
   }
   if (a.T > 0) {
     const uint64_t dims[4] = {(uint64_t)D, (uint64_t)a.T, (uint64_t)H_kv, (uint64_t)B};
     const uint64_t str[3] = {256ull, (uint64_t)a.T_cap * 256, (uint64_t)H_kv * a.T_cap * 256};
-    const uint32_t box[4] = {64u, (uint32_t)p.TCH, 1u, (uint32_t)p.NB};
+    const uint32_t box[4] = {64u, (uint32_t)p.TCH, 1u, rg ? 1u : (uint32_t)p.NB};
     if (!encode_tensor_map_bf16(&tm[2], a.K_txt, 4, dims, str, box)) return cudaSuccess;
     if (!encode_tensor_map_bf16(&tm[3], a.V_txt, 4, dims, str, box)) return cudaSuccess;
   } else {
@@ -1028,7 +1181,7 @@ cudaError_t launch_fused(const kvc_layer* L, const DecodeArgs& a, const FusedPla
       std::lock_guard<std::mutex> lock(L->maps->mu);
       auto& x = L->maps->e[L->maps->next];
       L->maps->next = (L->maps->next + 1) % 8;
-      x.B = B; x.R = R; x.tc = p.tc; x.JC = p.JC; x.RB = p.RB; x.NB = p.NB; x.Kc = a.Kc;
+      x.rg = rg; x.B = B; x.R = R; x.tc = p.tc; x.JC = p.JC; x.RB = p.RB; x.NB = p.NB; x.Kc = a.Kc;
       x.tm[0] = tm[0]; x.tm[1] = tm[1]; x.tm[2] = tm[4]; x.tm[3] = tm[5];
       x.valid = true;
     }
@@ -1057,11 +1210,13 @@ cudaError_t launch_fused(const kvc_layer* L, const DecodeArgs& a, const FusedPla
   fa.cnt = a.fcnt;
   fa.token = a.token;
   fa.status = a.status;
+  fa.R_b = a.R_b; fa.T_b = a.T_b; fa.off_seq = ring + p.off_seq;
   fa.early = a.early_capsules;
 
   ProfScope prof(p.tc == 2 ? KVC_KERNEL_FUSED_PAIR : (p.tc ? KVC_KERNEL_FUSED_TC : KVC_KERNEL_FUSED), st);
   if (p.tc) return launch_fused_tc_kernel(tm, fa, p, st);
-  return a.G > 8 ? launch_nh<2>(tm, fa, p, st) : launch_nh<1>(tm, fa, p, st);
+  if (rg) return a.G > 8 ? launch_nh<2, true>(tm, fa, p, st) : launch_nh<1, true>(tm, fa, p, st);
+  return a.G > 8 ? launch_nh<2, false>(tm, fa, p, st) : launch_nh<1, false>(tm, fa, p, st);
 }
 
 }  // namespace kvc

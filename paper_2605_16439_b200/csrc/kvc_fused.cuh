@@ -34,6 +34,8 @@ struct FusedArgs {
   unsigned long long* cnt;   // [B*H_kv] arrival words in the caller's workspace (see arrive_is_last)
   unsigned int token;        // this call's token, never 0
   int* status;        // device status word
+  const int *R_b, *T_b;      // per-sequence block counts (<= R) and text lengths (<= T), device arrays; nullptr: R and T for all
+  uint32_t off_seq;          // with them: the table of sequences (FusedSeq [nbg][NB], then the lengths as given)
   int early;          // 1: capsule rows may be loaded before the stream's previous kernel has finished (see kvc.h)
 };
 
@@ -48,11 +50,14 @@ constexpr int BAR_S_FREE = 6;    // + b: score tile read     (expansion warps ar
 constexpr int BAR_W_READY = 8;   // + b: weight tile written (expansion warps arrive, value warps wait)
 constexpr int BAR_W_FREE = 10;   // + b: weight tile read    (value warps arrive, expansion warps wait)
 
+struct FusedSeq { int b, rb, tb, pad; };         // a sequence (-1: none), its blocks, its text rows
+constexpr int FUSED_MAX_RAGGED_B = 512;
+
 // The text rows a unit attends over: its slice [b0, b1), in nb stages
 struct RowRanges { int b0, b1, nb; };
-__device__ __forceinline__ RowRanges row_ranges(const FusedArgs& a, int rg) {
+__device__ __forceinline__ RowRanges row_ranges(const FusedArgs& a, int rg, int T) {
   RowRanges r;
-  r.b0 = min(rg * a.Tper, a.T); r.b1 = min(a.T, r.b0 + a.Tper);
+  r.b0 = min(rg * a.Tper, T); r.b1 = min(T, r.b0 + a.Tper);
   r.nb = r.b1 > r.b0 ? (r.b1 - r.b0 + a.TCH - 1) / a.TCH : 0;
   return r;
 }

@@ -147,7 +147,7 @@ fused_decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_con
       // pair mode: the units 2k, 2k+1 of a (sequence, head) are the two CTAs (rank rk) of a cluster on block group k
       const int rk = PAIR ? (rg & 1) : 0;
       const int b0 = bg * a.NB, r0 = PAIR ? (rg >> 1) * a.RB : rg * a.RB;
-      const RowRanges tr = row_ranges(a, rg);
+      const RowRanges tr = row_ranges(a, rg, a.T);
       const int nts = tr.nb;
       const int cg0 = PAIR ? rk * ncgl : 0;          // first column group of this CTA
       const int c2first = (PAIR && rk) ? NJ0 : 0, c2count = PAIR ? (rk ? a.NJ - NJ0 : NJ0) : a.NJ;
@@ -230,7 +230,7 @@ fused_decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_con
     for (int u = blockIdx.x; u < a.units; u += gridDim.x, ++ucount) {
       const int rem = u % per_h;
       const int rg = rem % a.nrg;
-      const RowRanges tr = row_ranges(a, rg);
+      const RowRanges tr = row_ranges(a, rg, a.T);
       const int nts = tr.nb;
       // ---------------- pass A ----------------
       if (ucount > 0) wait_on(&bars.l_free, (ucount - 1) & 1u);    // the previous unit's logits have been read back
@@ -613,7 +613,7 @@ fused_decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_con
     const int b0 = bg * a.NB, r0 = PAIR ? (rg >> 1) * a.RB : rg * a.RB;
     const int nbv = min(a.NB, a.B - b0);
     const int rbv = min(RB, a.R - r0);
-    const RowRanges tr = row_ranges(a, rg);
+    const RowRanges tr = row_ranges(a, rg, a.T);
     const int nts = tr.nb;
     const int c2first = (PAIR && rk) ? NJ0 : 0, c2count = PAIR ? (rk ? a.NJ - NJ0 : NJ0) : a.NJ;
     (void)r0;

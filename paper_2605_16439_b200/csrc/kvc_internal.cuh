@@ -93,7 +93,7 @@ struct FusedPlan {
   int yhg;           // heads per round of the final reduction over the value warps
   int stages, grid;
   uint32_t par_bytes, k_half_bytes, txt_half_bytes, stage_bytes, misc_bytes;
-  uint32_t off_q, off_S, off_W, off_wred, off_rstat, off_tstat, off_hstat, off_yred;   // relative to the end of the ring
+  uint32_t off_q, off_S, off_W, off_wred, off_rstat, off_tstat, off_hstat, off_yred, off_seq;   // relative to the end of the ring
   int tc;            // 1: the expansions run on tcgen05 with the logits in tensor memory (kvc_fused_tc.cu); 2: its pair mode
   uint32_t off_P, off_rtab, off_xstat, off_wrecv;
   int tmem_cols;
@@ -117,7 +117,8 @@ struct kvc_layer {
   int device;
   int num_sms;
   int use_tc;            // expansions of the one-kernel decode path: 0 chosen per shape, 1 tcgen05, 2 tcgen05 in pairs of CTAs,
-                         // -1 mma.sync (environment KVC_EXPANSION=tcgen05 | pair | mma when the handle is created)
+                         // -1 mma.sync; -2 three-phase kernels, 3 three-kernel path, 4 resident parameters, 5 clusters (environment
+                         // KVC_EXPANSION=tcgen05 | pair | mma | phases | split | resident | cluster when the handle is created)
   int32_t* d_idx;        // device [H_kv][m]
   int* d_cstatus;        // device status word of the compress kernels (cleared by every kvc_compress call)
   float* d_usum;         // device [H_kv][m] row sums of U (value compression:  U (V - 1 mu^T) = U V - (U 1) mu^T)
@@ -134,7 +135,7 @@ namespace kvc {
 
 WsLayout ws_layout(const kvc_layer* L, int B, int R, int T_cap);
 int cuda_status(cudaError_t e);   // KVC_OK or KVC_ERR_CUDA, remembering the error for kvc_last_cuda_error
-FusedPlan plan_fused(const kvc_layer* L, int B, int R);
+FusedPlan plan_fused(const kvc_layer* L, int B, int R, bool ragged = false);
 FusedPlan plan_fused_tc(const kvc_layer* L, int B, int R);     // tensor-memory variant; ok == 0 if the shape does not fit it
 FusedPlan plan_fused_pair(const kvc_layer* L, int B, int R);   // its pair mode (clusters of two CTAs)
 
