@@ -297,14 +297,15 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     const int KT = a.n >> 4;
     const int kt0 = warp * a.ktw;
     const int my_kt = max(0, min(a.ktw, KT - kt0));
-    // byte offsets of this warp's fragments inside a parameter tile [column group][row][64]
-    uint32_t th_off[KTW], u_off[KTW];              // theta: [k = row][n = col] read transposed;  U: [n = row][k = col]
+    // byte offsets of this warp's fragments inside a parameter tile [column group][row][64]: those of its first four 16-column groups;
+    // group kt's lies (kt / 4) column groups further (all KTW of both kinds in registers spilled, see below)
+    uint32_t th_off[4], u_off[4];                  // theta: [k = row][n = col] read transposed;  U: [n = row][k = col]
+    const uint32_t grp4 = (uint32_t)rows16 * 128u;
 #pragma unroll
-    for (int kt = 0; kt < KTW; ++kt) {
-      const int ktc = kt < my_kt ? kt0 + kt : 0;
-      const int col_t = ktc * 16 + lhi * 8, col_u = ktc * 16 + lmid * 8;
-      th_off[kt] = (uint32_t)(((col_t >> 6) * rows16 + lrow) * 128 + ((((col_t & 63) >> 3) ^ l7) << 4));
-      u_off[kt] = (uint32_t)(((col_u >> 6) * rows16 + lrowB) * 128 + ((((col_u & 63) >> 3) ^ l7) << 4));
+    for (int x = 0; x < 4; ++x) {
+      const int col_t = (kt0 + x) * 16 + lhi * 8, col_u = (kt0 + x) * 16 + lmid * 8;
+      th_off[x] = (uint32_t)(((col_t >> 6) * rows16 + lrow) * 128 + ((((col_t & 63) >> 3) ^ l7) << 4));
+      u_off[x] = (uint32_t)(((col_u >> 6) * rows16 + lrowB) * 128 + ((((col_u & 63) >> 3) ^ l7) << 4));
     }
 
     for (int u = blockIdx.x; u < a.units; u += gridDim.x) {
@@ -352,7 +353,7 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
             uint32_t bf[4][4];
 #pragma unroll
             for (int x = 0; x < 4; ++x)
-              if (kq + x < KTW && kq + x < my_kt) ldsm_x4_t(bf[x], par_u + th_off[(kq + x < KTW) ? kq + x : 0] + (uint32_t)(s * 2048));
+              if (kq + x < KTW && kq + x < my_kt) ldsm_x4_t(bf[x], par_u + th_off[x] + (uint32_t)(kq >> 2) * grp4 + (uint32_t)(s * 2048));
 #pragma unroll
             for (int x = 0; x < 4; ++x)
               if (kq + x < KTW && kq + x < my_kt) {
@@ -519,7 +520,7 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
             uint32_t bu[4][4];
 #pragma unroll
             for (int x = 0; x < 4; ++x)
-              if (kq + x < KTW && kq + x < my_kt) ldsm_x4(bu[x], par_u + u_off[(kq + x < KTW) ? kq + x : 0] + (uint32_t)(s * 2048));
+              if (kq + x < KTW && kq + x < my_kt) ldsm_x4(bu[x], par_u + u_off[x] + (uint32_t)(kq >> 2) * grp4 + (uint32_t)(s * 2048));
 #pragma unroll
             for (int x = 0; x < 4; ++x)
               if (kq + x < KTW && kq + x < my_kt) {
