@@ -39,7 +39,6 @@ struct Unit { int h, blk0, nb, nt; };
 // A thread's roles, derived anew where a step begins: kept across the loop over units they (and everything the compiler hoists with
 // them) took some 100 registers more than a thread has, and with the L1 given to shared memory a spill is an L2 round trip.
 struct Lanes { int warp, lane, grp, rg, gid, t4, l7, lmid, lrowB; };
-__device__ __forceinline__ int fresh(int x) { asm volatile("" : "+r"(x)); return x; }
 __device__ __forceinline__ Lanes lanes_of(int tid) {
   tid = fresh(tid);
   const int warp = tid >> 5, lane = tid & 31;

@@ -27,6 +27,15 @@
 
 namespace kvc {
 
+// A lane's roles in the fragments, derived anew in every section that uses them: kept across the loop over units they spilled (see par_off)
+struct FusedLanes { int lane, gid, t4, l7, lrow, lhi, lrowB, lmid; };
+__device__ __forceinline__ FusedLanes fused_lanes() {
+  const int lane = fresh(threadIdx.x) & 31;
+  const int l7 = lane & 7, lhi = lane >> 4, lmid = (lane >> 3) & 1;
+  // fragment row and column pair; ldmatrix address patterns: rows 0-15 by lanes 0-15, twice; rows 0-7 | 0-7 | 8-15 | 8-15
+  return {lane, lane >> 2, lane & 3, l7, l7 + lmid * 8, lhi, l7 + lhi * 8, lmid};
+}
+
 // EW expansion warps, VW value warps, one producer warp.  Every expansion warp owns up to KTW 16-column groups of
 // the logits; NH = 8-head tiles of the group (1: G <= 8, 2: G <= 16); MT = 16-row tiles of expansion rows per unit
 //
@@ -46,6 +55,7 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
   constexpr int FCONS = CW * 32;
   constexpr int FTHREADS = FCONS + 32;
   constexpr int RT = ROWS * MT;               // expansion rows of a unit
+  constexpr int VT = NH == 2 ? 4 : 8;         // value fragments in flight per warp (two head tiles' accumulators leave room for four)
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* sm = smem_raw + ((1024u - (smem_addr(smem_raw) & 1023u)) & 1023u);
   __shared__ __align__(8) FusedBars bars;
@@ -229,7 +239,6 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
   }
 
   // ================= consumers: common set-up =================
-  const int gid = lane >> 2, t4 = lane & 3;
   const int G = a.G, RB = a.RB, JC = a.JC;
   const int rows16 = 16 * JC;                      // rows of one block inside a stage
   const int blk16 = RG ? 2 * rows16 : rows16;      // from one block's rows to the next one's, in 128-byte rows
@@ -252,11 +261,6 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
   float* rowf = hfv + a.NB * 16;                                             // [RT] that factor per expansion row
   float* yred = reinterpret_cast<float*>(sm + a.off_yred);                   // [VW][yhg][D]
   const float qscale = 0.08838834764831845f * 1.4426950408889634f;   // sigma = 1/sqrt(128), logits kept in log2 units
-  const int l7 = lane & 7;
-  const int lrow = l7 + ((lane >> 3) & 1) * 8;     // ldmatrix address pattern A: rows 0-15 by lanes 0-15, twice
-  const int lhi = lane >> 4;
-  const int lrowB = l7 + lhi * 8;                  // address pattern B: rows 0-7 | 0-7 | 8-15 | 8-15
-  const int lmid = (lane >> 3) & 1;
   const int WPG = VW / a.NB;                       // value warps per sequence of the unit
 
   if (!RG && warp >= EW && blockIdx.x < a.units) {
@@ -285,7 +289,7 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
   // the stage in `slot` has been consumed by this warp
   auto release = [&]() {
     __syncwarp();
-    if (lane == 0) mbar_arrive(&bars.empty[slot]);
+    if ((fresh(threadIdx.x) & 31) == 0) mbar_arrive(&bars.empty[slot]);
     if (++slot == (uint32_t)a.stages) { slot = 0; phase ^= 1u; }
   };
 
@@ -297,17 +301,6 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     const int KT = a.n >> 4;
     const int kt0 = warp * a.ktw;
     const int my_kt = max(0, min(a.ktw, KT - kt0));
-    // byte offsets of this warp's fragments inside a parameter tile [column group][row][64]: those of its first four 16-column groups;
-    // group kt's lies (kt / 4) column groups further (all KTW of both kinds in registers spilled, see below)
-    uint32_t th_off[4], u_off[4];                  // theta: [k = row][n = col] read transposed;  U: [n = row][k = col]
-    const uint32_t grp4 = (uint32_t)rows16 * 128u;
-#pragma unroll
-    for (int x = 0; x < 4; ++x) {
-      const int col_t = (kt0 + x) * 16 + lhi * 8, col_u = (kt0 + x) * 16 + lmid * 8;
-      th_off[x] = (uint32_t)(((col_t >> 6) * rows16 + lrow) * 128 + ((((col_t & 63) >> 3) ^ l7) << 4));
-      u_off[x] = (uint32_t)(((col_u >> 6) * rows16 + lrowB) * 128 + ((((col_u & 63) >> 3) ^ l7) << 4));
-    }
-
     for (int u = blockIdx.x; u < a.units; u += gridDim.x) {
       int h, bg, rg;
       unit_of(u, h, bg, rg);
@@ -321,6 +314,7 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
       for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
         for (int hr = 0; hr < 2; ++hr) {
+          const int gid = (fresh(threadIdx.x) & 31) >> 2;
           const int rho = mt * 16 + gid + 8 * hr;
           const int bi = rho / G, g = rho - bi * G;
           const int rbl = bi / RB, rrl = bi - rbl * RB;
@@ -336,8 +330,23 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
 #pragma unroll
           for (int e = 0; e < 4; ++e) accL[mt][nt][e] = 0.f;
 
+      // Byte offsets of this warp's fragments inside a parameter tile [column group][row][64] (theta: [k = row][n = col] read transposed;
+      // U: [n = row][k = col]): those of its first four 16-column groups; group kt's lies (kt / 4) column groups further.  Worked out
+      // before each pass: kept for every group of both kinds they spilled, and with the L1 given to shared memory a spilled value is
+      // an L2 round trip per stage (8 x 5 blocks of n = 576, 32/32 heads: 41.0 us, now 38.1).
+      uint32_t par_off[4];
+      const uint32_t grp4 = (uint32_t)rows16 * 128u;
+      {
+        const int ln = fresh(threadIdx.x) & 31;
+#pragma unroll
+        for (int x = 0; x < 4; ++x) {
+          const int col = (kt0 + x) * 16 + (ln >> 4) * 8, row = (ln & 7) + ((ln >> 3) & 1) * 8;
+          par_off[x] = (uint32_t)(((col >> 6) * rows16 + row) * 128 + ((((col & 63) >> 3) ^ (ln & 7)) << 4));
+        }
+      }
       // ---------------- pass A: L[:, my column groups] += S theta ----------------
       for (int c = 0; c < NJ; ++c) {
+        const auto [lane, gid, t4, l7, lrow, lhi, lrowB, lmid] = fused_lanes();
         wait_on(&bars.full[slot], phase);
         const uint32_t par_u = sm_u + slot * a.stage_bytes;
         const int nsub = min(JC, (a.m - c * rows16 + 15) >> 4);          // 16-row sub-chunks with rows below m
@@ -353,7 +362,7 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
             uint32_t bf[4][4];
 #pragma unroll
             for (int x = 0; x < 4; ++x)
-              if (kq + x < KTW && kq + x < my_kt) ldsm_x4_t(bf[x], par_u + th_off[x] + (uint32_t)(kq >> 2) * grp4 + (uint32_t)(s * 2048));
+              if (kq + x < KTW && kq + x < my_kt) ldsm_x4_t(bf[x], par_u + par_off[x] + (uint32_t)(kq >> 2) * grp4 + (uint32_t)(s * 2048));
 #pragma unroll
             for (int x = 0; x < 4; ++x)
               if (kq + x < KTW && kq + x < my_kt) {
@@ -399,6 +408,7 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
             if (nt < 2 * my_kt) mx = fmaxf(mx, fmaxf(accL[mt][nt][2 * hr], accL[mt][nt][2 * hr + 1]));
           mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
           mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+          const int gid = (fresh(threadIdx.x) & 31) >> 2, t4 = fresh(threadIdx.x) & 3;
           if (t4 == 0) rmax[warp * RT + mt * 16 + gid + 8 * hr] = rvalid[mt][hr] ? mx : -INFINITY;
         }
       pass_text(false);
@@ -443,6 +453,7 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
             }
           sum += __shfl_xor_sync(0xffffffffu, sum, 1);
           sum += __shfl_xor_sync(0xffffffffu, sum, 2);
+          const int gid = (fresh(threadIdx.x) & 31) >> 2, t4 = fresh(threadIdx.x) & 3;
           if (t4 == 0) rsum[warp * RT + mt * 16 + gid + 8 * hr] = sum;
         }
 #pragma unroll
@@ -484,7 +495,10 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
       for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
         for (int hr = 0; hr < 2; ++hr)
+        {
+          const int gid = (fresh(threadIdx.x) & 31) >> 2, t4 = fresh(threadIdx.x) & 3;
           if (warp == 0 && t4 == 0) rowf[mt * 16 + gid + 8 * hr] = rvalid[mt][hr] ? hfv[rhead[mt][hr]] : 0.f;
+        }
       named_barrier_sync(1, FCONS);                                   // B3: text sums are in place
       if (warp == 0) {
         for (int x = lane; x < a.NB * 16; x += 32) {
@@ -503,7 +517,16 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
       named_barrier_sync(1, FCONS);                                   // B4: head sums
 
       // ---------------- pass C: W = P U^T, reduced over the expansion warps ----------------
+      {
+        const int ln = fresh(threadIdx.x) & 31;
+#pragma unroll
+        for (int x = 0; x < 4; ++x) {
+          const int col = (kt0 + x) * 16 + ((ln >> 3) & 1) * 8, row = (ln & 7) + (ln >> 4) * 8;
+          par_off[x] = (uint32_t)(((col >> 6) * rows16 + row) * 128 + ((((col & 63) >> 3) ^ (ln & 7)) << 4));
+        }
+      }
       for (int c = 0; c < NJ; ++c) {
+        const auto [lane, gid, t4, l7, lrow, lhi, lrowB, lmid] = fused_lanes();
         wait_on(&bars.full[slot], phase);
         const uint32_t par_u = sm_u + slot * a.stage_bytes;
         const int nsub = min(JC, (a.m - c * rows16 + 15) >> 4);
@@ -520,7 +543,7 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
             uint32_t bu[4][4];
 #pragma unroll
             for (int x = 0; x < 4; ++x)
-              if (kq + x < KTW && kq + x < my_kt) ldsm_x4(bu[x], par_u + u_off[x] + (uint32_t)(kq >> 2) * grp4 + (uint32_t)(s * 2048));
+              if (kq + x < KTW && kq + x < my_kt) ldsm_x4(bu[x], par_u + par_off[x] + (uint32_t)(kq >> 2) * grp4 + (uint32_t)(s * 2048));
 #pragma unroll
             for (int x = 0; x < 4; ++x)
               if (kq + x < KTW && kq + x < my_kt) {
@@ -593,6 +616,7 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
       for (int nh = 0; nh < NH; ++nh)
 #pragma unroll
         for (int k2 = 0; k2 < 4; ++k2) {
+          const int lane = fresh(threadIdx.x) & 31, l7 = lane & 7;
           uint32_t r[4];
           ldsm_x4(r, q_u + (uint32_t)(((bl * 16 + nh * 8 + l7) * QLD + k2 * 32 + (lane >> 3) * 8) * 2));
           qf[nh][2 * k2][0] = r[0]; qf[nh][2 * k2][1] = r[1];
@@ -601,6 +625,7 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
 
       // ---------------- pass A: S[rows of block][16] = sigma q K^T for my (block, sub-chunk) tasks ----------------
       for (int c = 0; c < NJ; ++c) {
+        const auto [lane, gid, t4, l7, lrow, lhi, lrowB, lmid] = fused_lanes();
         wait_on(&bars.full[slot], phase);
         const uint32_t k_u = sm_u + slot * a.stage_bytes + a.par_bytes;
         const int nsub = min(JC, (a.m - c * rows16 + 15) >> 4);
@@ -651,6 +676,7 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
           for (int e = 0; e < 4; ++e) yacc[mt][nh][e] = 0.f;
       float m_run[2] = {-INFINITY, -INFINITY}, l_run[2] = {0.f, 0.f};   // heads gid and gid + 8
       for (int ts = 0; ts < nts; ++ts) {
+        const auto [lane, gid, t4, l7, lrow, lhi, lrowB, lmid] = fused_lanes();
         wait_on(&bars.full[slot], phase);
         const uint32_t kt_u = sm_u + slot * a.stage_bytes, vt_u = kt_u + 2 * a.txt_half_bytes;
         for (int tile = wig; tile * 16 < a.TCH; tile += WPG) {
@@ -749,26 +775,35 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
 #pragma unroll
               for (int x = 0; x < 2; ++x) px[nh][x] = split_lo(cc[x][2 * nh], cc[x][2 * nh + 1], pb[nh][x]);
           }
-          uint32_t av[8][4];
 #pragma unroll
-          for (int mt = 0; mt < 8; ++mt)
-            ldsm_x4_t(av[mt], vt_u + (mt >> 2) * a.txt_half_bytes + rowB + (uint32_t)(((((mt & 3) * 2 + lmid)) ^ l7) << 4));
+          for (int mq = 0; mq < 8; mq += VT) {
+            uint32_t av[VT][4];
 #pragma unroll
-          for (int mt = 0; mt < 8; ++mt)
-#pragma unroll
-            for (int nh = 0; nh < NH; ++nh) {
-              mma_bf16_16816(yacc[mt][nh], av[mt], pb[nh][0], pb[nh][1]);
-              if (RG) mma_bf16_16816(yacc[mt][nh], av[mt], px[nh][0], px[nh][1]);
+            for (int x = 0; x < VT; ++x) {
+              const int mt = mq + x;
+              ldsm_x4_t(av[x], vt_u + (mt >> 2) * a.txt_half_bytes + rowB + (uint32_t)(((((mt & 3) * 2 + lmid)) ^ l7) << 4));
             }
+#pragma unroll
+            for (int x = 0; x < VT; ++x)
+#pragma unroll
+              for (int nh = 0; nh < NH; ++nh) {
+                mma_bf16_16816(yacc[mq + x][nh], av[x], pb[nh][0], pb[nh][1]);
+                if (RG) mma_bf16_16816(yacc[mq + x][nh], av[x], px[nh][0], px[nh][1]);
+              }
+          }
         }
         release();
       }
 
       // ---------------- joint softmax: the text accumulators move to the unit's reference maximum ----------------
-      if (t4 == 0) { tmax[vw * 16 + gid] = m_run[0]; tmax[vw * 16 + gid + 8] = m_run[1]; }
+      {
+        const auto [lane, gid, t4, l7, lrow, lhi, lrowB, lmid] = fused_lanes();
+        if (t4 == 0) { tmax[vw * 16 + gid] = m_run[0]; tmax[vw * 16 + gid + 8] = m_run[1]; }
+      }
       named_barrier_sync(1, FCONS);                                   // B1
       named_barrier_sync(1, FCONS);                                   // B2: head maxima
       {
+        const auto [lane, gid, t4, l7, lrow, lhi, lrowB, lmid] = fused_lanes();
         float scl[2];
 #pragma unroll
         for (int hr = 0; hr < 2; ++hr) {
@@ -796,6 +831,7 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
 
       // ---------------- pass C: y^T[128][heads] += V^T[128][16 rows of block] W^T[16][heads of block] ----------------
       for (int c = 0; c < NJ; ++c) {
+        const auto [lane, gid, t4, l7, lrow, lhi, lrowB, lmid] = fused_lanes();
         wait_on(&bars.full[slot], phase);
         const uint32_t v_u = sm_u + slot * a.stage_bytes + a.par_bytes;
         const int nsub = min(JC, (a.m - c * rows16 + 15) >> 4);
@@ -810,20 +846,27 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
             ldsm_x4(bw, W_u + (uint32_t)((wbuf * ((RT + 16) * SLD) + (bi * G + lrowB) * SLD + lmid * 8) * 2));
             if (RG) ldsm_x4(bx, W_u + (uint32_t)(((2 + wbuf) * ((RT + 16) * SLD) + (bi * G + lrowB) * SLD + lmid * 8) * 2));
             const uint32_t rowoff = v_u + (uint32_t)((bi * blk16 + s * 16 + lrowB) * 128);
-            uint32_t av[8][4];
 #pragma unroll
-            for (int mt = 0; mt < 8; ++mt)
-              if ((mt >> mshift) == mg)
-                ldsm_x4_t(av[mt], rowoff + (mt >> 2) * a.k_half_bytes + (uint32_t)(((((mt & 3) * 2 + lmid)) ^ l7) << 4));
+            for (int mq = 0; mq < 8; mq += VT) {
+              uint32_t av[VT][4];
 #pragma unroll
-            for (int mt = 0; mt < 8; ++mt)
-              if ((mt >> mshift) == mg) {
+              for (int x = 0; x < VT; ++x) {
+                const int mt = mq + x;
+                if ((mt >> mshift) == mg)
+                  ldsm_x4_t(av[x], rowoff + (mt >> 2) * a.k_half_bytes + (uint32_t)(((((mt & 3) * 2 + lmid)) ^ l7) << 4));
+              }
 #pragma unroll
-                for (int nh = 0; nh < NH; ++nh) {
-                  mma_bf16_16816(yacc[mt][nh], av[mt], bw[2 * nh], bw[2 * nh + 1]);
-                  if (RG) mma_bf16_16816(yacc[mt][nh], av[mt], bx[2 * nh], bx[2 * nh + 1]);
+              for (int x = 0; x < VT; ++x) {
+                const int mt = mq + x;
+                if ((mt >> mshift) == mg) {
+#pragma unroll
+                  for (int nh = 0; nh < NH; ++nh) {
+                    mma_bf16_16816(yacc[mt][nh], av[x], bw[2 * nh], bw[2 * nh + 1]);
+                    if (RG) mma_bf16_16816(yacc[mt][nh], av[x], bx[2 * nh], bx[2 * nh + 1]);
+                  }
                 }
               }
+            }
           }
           named_barrier_arrive(BAR_W_FREE + (int)wbuf, FCONS);
           ++wi;
@@ -836,6 +879,7 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
       const size_t pbase = ((size_t)bh * a.nrg + rg) * G;
       const int YHG = a.yhg;
       for (int g0 = 0; g0 < G; g0 += YHG) {
+        const auto [lane, gid, t4, l7, lrow, lhi, lrowB, lmid] = fused_lanes();
         // every warp parks its tile columns of heads g0 .. g0+YHG-1; then the warps of a sequence are summed
 #pragma unroll
         for (int nh = 0; nh < NH; ++nh)
@@ -948,7 +992,7 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
       }
     }
   }
-  if (dead && lane == 0) atomicExch(a.status, (int)KVC_ERR_TIMEOUT);
+  if (dead && (threadIdx.x & 31) == 0) atomicExch(a.status, (int)KVC_ERR_TIMEOUT);
 }
 
 }  // namespace kvc
