@@ -32,7 +32,9 @@ constexpr uint32_t CT_V_BYTES = CT_BK * D * 2;              // 16 KB: 64 rows of
 constexpr int CT_EPI_WARPS = 8;
 constexpr uint32_t CT_OUT_WARP = 32 * 128;                  // epilogue staging of a warp: 32 rows, one 64-channel half
 constexpr uint32_t CT_TMEM_COLS = 512;
-constexpr int CT_COPY_WARPS = 8;
+// Six: sixteen warps have 128 registers a thread; with eight (96 registers) the copy loop's two steps in flight spilled, an L2 round trip
+// each with the L1 given to shared memory (8 x 5 blocks of n = 576, 32 heads, ratio 0.6: 78 us, six 74.5; 32 x 8 of 256: 31 and 27)
+constexpr int CT_COPY_WARPS = 6;
 constexpr int CT_THREADS = (CT_EPI_WARPS + 2 + CT_COPY_WARPS) * 32;
 constexpr uint32_t CT_SMEM_LIMIT = 231424;                  // dynamic part of the 227 KB; the barriers take the rest
 constexpr int CT_MAX_B = 8192;                              // sequences of a ragged batch: their block counts sit in shared memory
