@@ -36,10 +36,10 @@ NOMINAL_HBM_GBS = 8000.0        # nominal HBM3e bandwidth: the roofline fraction
 
 # DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) of the dominant kernel from one ncu capture,
 # keyed by (kernel, workload name): (bytes, digest of the kernel's source files when the counters were taken).  The
-# captures ran at 4 decode steps (text length 130 / 258 / 514; profiles/*.md give the commands); a text row adds exactly
-# 2 * B * H_kv * d * 2 bytes, and the figure here is scaled by that amount to the mid-run text length.  For the three-kernel
-# path the figure is the sum over its three kernels (one layer call).  When the sources no longer match the digest the
-# bench reports traffic = null: the counters belong to another kernel.
+# captures ran one launch of every kernel at the workload's full batch and layer size and its mid-run text length (256 / 512 /
+# 1024 rows), other layers' launches before it.  For the three-kernel path the figure is the sum over its three kernels (one
+# layer call).  When the sources no longer match the digest the bench reports traffic = null: the counters belong to
+# another kernel.
 KERNEL_SOURCES = {
     "fused": ("kvc_fused.cu", "kvc_fused.cuh", "kvc_tma.cuh", "kvc_async.cuh"),
     "fused_tc": ("kvc_fused_tc.cu", "kvc_fused.cuh", "kvc_tcgen05.cuh", "kvc_tma.cuh", "kvc_async.cuh"),
@@ -49,9 +49,9 @@ KERNEL_SOURCES = {
                                                "kvc_tcgen05.cuh", "kvc_tma.cuh", "kvc_async.cuh"),
 }
 NCU_TRAFFIC_BYTES = {
-    ("fused", "config1-llava-next-7b"): (208.4e6, "3788d05ac9fe"),
-    ("split_scores+split_expand+split_output", "config2-qwen2-vl-7b"): (147.7e6, "b9ec0383c83b"),
-    ("resident", "config3-internvl3-8b-video"): (36.0e6, "1e4ede360c43"),
+    ("fused", "config1-llava-next-7b"): (206.2e6, "9e8c36e90b98"),
+    ("split_scores+split_expand+split_output", "config2-qwen2-vl-7b"): (147.1e6, "4fedd6d75f9c"),
+    ("resident", "config3-internvl3-8b-video"): (36.0e6, "57710997d7a9"),
 }
 
 

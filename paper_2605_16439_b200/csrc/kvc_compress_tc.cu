@@ -12,7 +12,7 @@
 //                   (about 3.6 k cycles) runs behind the next unit's products
 //   warp 9          TMA producer: per 64 vision positions one 48 KB stage (U 16 KB, V 2 x 16 KB, 128-byte swizzle), a ring of
 //                   stages that runs on across units
-//   warps 10-17     row copies: the retained key rows, a side stored verbatim, the rows left over by a ragged batch
+//   warps 10-15     row copies: the retained key rows, a side stored verbatim, the rows left over by a ragged batch
 // Measured on B200 (per layer, back to back): 8 x 32 x 5 blocks of n = 576, m = 231: 81 us (5.3 TB/s of 426 MB; 129 us with one
 // launch for the keys and one CTA per (block, row tile)); 8 sequences of up to 8 blocks x 4 heads of n = 1024, m = 410 with their
 // own lengths: 42 us (1108 us on the CUDA cores before).  Tried: both row tiles of a pair in one unit, which fills the tensor memory
