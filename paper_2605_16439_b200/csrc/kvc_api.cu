@@ -332,11 +332,11 @@ static bool use_split(const kvc_layer* L, int B, int R) {
 // row, or its bytes, parameters included, at 45 GB/s, up to 90 where few units of long blocks share the L2); the three-phase kernels'
 // with the bytes and the block length; the cluster path's is a chain of some 28 us, long for text, but it spreads few blocks over more SMs.
 // Measured on B200, us per call, one-kernel / cluster / three-phase:
-// One query head per KV head: 8 x 5 blocks of n = 576, 512 text rows 47.7 / 76.7 / 70.1; 8 x 4 of 1024 78 / 99 / 116; 1 x 5 of 576 30.0 /
-// 31.2 / 30.8; 32 x 5 of 576 160 / 205 / 183; 64 x 1 of 576 208 / 153 / 123; 24 x 1 of 1024 136 / 104 / 118; 4 x 16 of 1024 153 / 101 / 153.
-// Groups of query heads, units within one round: 16 x 2 of 1024, 32/8 heads, 80 MB of rows 47 / 59 / 79, 16 x 2 of 576 32 / 41 / 48, 6 x 8 of
-// 320, m = 128, 26 / 30 / 35, but 2 x 2 of 576, 10 MB, 29 / 25 / 29, 4 x 4 of 1024, 28/4 heads, 50 / 37 / 72; more rounds: 16 x 5 of 576,
-// 28/4 heads 66 / 39 / 102.
+// One query head per KV head: 8 x 5 blocks of n = 576, 512 text rows 43.9 / 75.1 / 70.2; 8 x 4 of 1024 76 / 97 / 116; 1 x 5 of 576 29.1 /
+// 31.1 / 31.3; 32 x 5 of 576 147 / 205 / 183; 64 x 1 of 576 194 / 148 / 123; 24 x 1 of 1024 136 / 104 / 118.
+// Groups of query heads, units within one round: 16 x 2 of 1024, 32/8 heads, 80 MB of rows 47 / 58 / 79, 16 x 2 of 576 31 / 41 / 48, 6 x 8 of
+// 320, m = 128, 25 / 30 / 34, but 2 x 2 of 576, 4 MB, 28 / 25 / 29, 4 x 4 of 1024, 28/4 heads, 49 / 37 / 72; more rounds: 16 x 5 of 576,
+// 28/4 heads 63 / 39 / 102.
 static int ragged_path(const kvc_layer* L, int B, int R, int T) {
   if (L->mode != KVC_MODE_KV || L->passthrough || R < 1 || (L->use_tc != 0 && L->use_tc != -1)) return 0;
   const FusedPlan f = plan_fused(L, B, R, true);
@@ -367,9 +367,9 @@ static int ragged_path(const kvc_layer* L, int B, int R, int T) {
 // heads: 60 / 50).
 // Whole multiples of 64 up to 640, groups of query heads: the other way is the one-kernel path, whose time goes with the rounds of its
 // units and the retained rows (9 us + 0.09 us a row).  The cluster path is ahead (a) on the smallest calls, one unit per KV head, from m
-// = 224 on (1 x 1 of n = 576, 28/4 heads: 21.7 / 25.5; n = 640: 22 / 26.5; m = 205: 21.4 / 20.7), (b) where the rounds of the other are many
-// and its own units are one wave or fill the last (16 x 5 of 576: 43 / 59; 8 x 16 of 640: 50 / 63; 16 x 20 of 576, 16/2 heads: 53 / 92; 64
-// x 8 of 576: 168 / 202; but 32 x 8 of 576, 32/8 heads, 290 MB: 154 / 121).
+// = 224 on (1 x 1 of n = 576, 28/4 heads: 22.0 / 24.8; n = 640: 22 / 26; m = 205: 21.6 / 20.0), (b) where the rounds of the other are many
+// and its own units are one wave or fill the last (16 x 5 of 576: 43 / 57; 8 x 16 of 640: 49 / 62; 16 x 20 of 576, 16/2 heads: 53 / 88; 64
+// x 8 of 576: 169 / 193; but 32 x 8 of 576, 32/8 heads, 290 MB: 151 / 114).
 // KVC_EXPANSION=cluster forces it where its plan applies, any other value of the variable keeps it off.
 static bool use_cluster(const kvc_layer* L, int B, int R, int T, bool ragged) {
   if (R < 1 || L->passthrough || L->mode != KVC_MODE_KV || L->desc.dtype != KVC_BF16) return false;

@@ -43,7 +43,7 @@ __device__ __forceinline__ FusedLanes fused_lanes() {
 // capsule rows come in one copy per block; sequences are dealt to the units in the order of their work (the lengths are on the
 // device: every CTA sorts them itself), long ones with short ones.  The weights enter the product with the values as two bf16 terms:
 // these calls had fp32 weights before this kernel took them.
-// Bound as the uniform calls are (8 x 5 blocks of n = 576, 32/32 heads, half to all of 512 text rows: 235 MB in 47.7 us, 4.9 TB/s; the
+// Bound as the uniform calls are (8 x 5 blocks of n = 576, 32/32 heads, half to all of 512 text rows: 235 MB in 43.9 us, 5.4 TB/s; the
 // three-phase kernels took 70).
 template <int EW, int VW, int KTW, int NH, int MT, bool RG>
 __global__ void __launch_bounds__((EW + VW + 1) * 32, 1)
@@ -333,7 +333,8 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
       // Byte offsets of this warp's fragments inside a parameter tile [column group][row][64] (theta: [k = row][n = col] read transposed;
       // U: [n = row][k = col]): those of its first four 16-column groups; group kt's lies (kt / 4) column groups further.  Worked out
       // before each pass: kept for every group of both kinds they spilled, and with the L1 given to shared memory a spilled value is
-      // an L2 round trip per stage (8 x 5 blocks of n = 576, 32/32 heads: 41.0 us, now 38.1).
+      // an L2 round trip per stage (8 x 5 blocks of n = 576, 32/32 heads: 41.0 us, and
+      // 37.5 without those and the lane roles below).
       uint32_t par_off[4];
       const uint32_t grp4 = (uint32_t)rows16 * 128u;
       {
