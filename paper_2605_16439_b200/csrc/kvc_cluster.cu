@@ -651,8 +651,9 @@ cluster_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
     if (dead && lane == 0) atomicExch(a.status, (int)KVC_ERR_TIMEOUT);
   } else {
     // =========================================== consumers ===========================================
-    // the parameters of the first unit into L2 (fixed at inference, so before the wait), a share by each of the head's clusters
-    if (units > 0) {
+    // the parameters of the first unit into L2 (fixed at inference, so before the wait), a share by each of the head's clusters.  Lengths
+    // on the device may give fewer units than the clusters launched for them: those without one have no head either
+    if (cid < units) {
       const int h = cid / us.nu, lines = a.m * ngrp, step = min(us.nu, a.ucl) * CL_CONS;
       for (int x = (cid - h * us.nu) * CL_CONS + tid; x < lines; x += step) {
         const int row = x / ngrp, c = cg0 + x - row * ngrp;
