@@ -24,6 +24,8 @@ namespace kvc {
 
 constexpr float CL_QSCALE = 0.08838834764831845f * 1.4426950408889634f;      // sigma = 1/sqrt(128), logits in log2 units
 constexpr uint32_t CL_QPITCH = 272;                                          // bytes per staged query row (conflict-free ldmatrix)
+static_assert((CL_ROWS + 15) * CL_QPITCH <= CL_DUE, "a unit's queries (and the rows a fragment reads past them) in the region of P");
+static_assert(CL_ROWS * sizeof(int) <= CL_W_TAIL - CL_DUE && CL_MAX_RAGGED_B < (1 << 16), "the unit's sequences");
 
 struct ClusterBars {
   uint64_t kfull[CL_K_SLOTS], kempty[CL_K_SLOTS];
@@ -701,16 +703,33 @@ cluster_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
       const Unit u = unit_at(w);
       const int rows = u.nb * G;
       // ---------------- queries of the unit's sequences ----------------
-      int b_first, b_last, rr_;
-      cl_locate(a, pre, u.blk0, b_first, rr_);
-      cl_locate(a, pre, u.blk0 + u.nb - 1, b_last, rr_);
+      // A sequence's G rows lie where its first block's expansion rows are: within the unit's 128 rows whatever lies between its sequences
+      // (with per-sequence lengths there may be any number without a block)
       int* ndue = reinterpret_cast<int*>(sm + a.tab_off + CL_GROUPS * 512 + (uint32_t)NS * CL_ROWS * 8u + CL_GROUPS * 64);
+      int* nseq_sm = ndue + 1;
+      int* seq_sm = reinterpret_cast<int*>(sm + CL_DUE);        // (sequence, its first block of the unit) in any order
+      if (fresh(tid) == 0) *nseq_sm = 0;
       named_barrier_sync(1, CL_CONS);                           // the region of P is free (last unit's reductions)
       if (fresh(tid) == 0) *ndue = 0;
-      for (int x = tid; x < (b_last - b_first + 1) * G * 16; x += CL_CONS) {
-        const int row = x >> 4, c = x & 15, bb = row / G;
-        *reinterpret_cast<uint4*>(sm + (uint32_t)row * CL_QPITCH + c * 16) =
-            __ldg(reinterpret_cast<const uint4*>(a.q + (((size_t)(b_first + bb) * a.H_kv + u.h) * G + (row - bb * G)) * D + c * 8));
+      int b_first, nseq, rr_;
+      if (pre) {
+        if (fresh(tid) < u.nb) {
+          int b, r;
+          cl_locate(a, pre, u.blk0 + fresh(tid), b, r);
+          if (r == 0 || fresh(tid) == 0) seq_sm[atomicAdd(nseq_sm, 1)] = b | fresh(tid) << 16;
+        }
+        named_barrier_sync(1, CL_CONS);
+        b_first = 0;
+        nseq = *nseq_sm;
+      } else {
+        cl_locate(a, pre, u.blk0, b_first, rr_);
+        nseq = (u.blk0 + u.nb - 1) / a.R - b_first + 1;
+      }
+      for (int x = tid; x < nseq * G * 16; x += CL_CONS) {
+        const int row = x >> 4, c = x & 15, k = row / G, g = row - k * G;
+        const int b = pre ? seq_sm[k] & 0xffff : b_first + k, blk = pre ? seq_sm[k] >> 16 : max(b * a.R - u.blk0, 0);
+        *reinterpret_cast<uint4*>(sm + (uint32_t)(blk * G + g) * CL_QPITCH + c * 16) =
+            __ldg(reinterpret_cast<const uint4*>(a.q + (((size_t)b * a.H_kv + u.h) * G + g) * D + c * 8));
       }
       named_barrier_sync(1, CL_CONS);
       // ---------------- step 1: scores ----------------
@@ -729,7 +748,7 @@ cluster_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
           const int b = bw.b;
           if (b != cur_b) {
             cur_b = b;
-            const uint32_t qrow = sm_u + (uint32_t)((b - b_first) * G + (lane & 15)) * CL_QPITCH + (uint32_t)(lane >> 4) * 16u;
+            const uint32_t qrow = sm_u + (uint32_t)((bl - min(bw.r, bl)) * G + (lane & 15)) * CL_QPITCH + (uint32_t)(lane >> 4) * 16u;
 #pragma unroll
             for (int ks = 0; ks < 8; ++ks) ldsm_x4(qa[ks], qrow + (uint32_t)ks * 32u);
           }

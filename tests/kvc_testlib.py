@@ -97,5 +97,59 @@ def gpu_run(shape: wl.Shape, p, dev="cuda", mode: str = "kv"):
     return layer, K_t, V_t, out
 
 
+def launches(fn):
+    """({kernel name: launches}, result) of fn run with the library's event brackets on."""
+    kvc.kvc_profile_start(64)
+    try:
+        out = fn()
+        torch.cuda.synchronize()
+    finally:
+        kvc.kvc_profile_stop()
+    counts = {k: v[1] for k, v in kvc.kvc_profile_read().items()}
+    kvc.kvc_profile_start(0)
+    kvc.kvc_profile_stop()
+    return counts, out
+
+
+def check_ragged(shape: wl.Shape, seed: int, R_b, T_b, dev="cuda"):
+    """One layer's decode with per-sequence lengths (shape.R blocks and shape.T0 text rows at most) against the oracle, twice on one
+    workspace; whatever lies past a sequence's lengths is NaN.  Then a length out of range, which is clamped and reported.  Returns
+    ({kernel name: launches} of the first call, output)."""
+    B, R, T = shape.B, shape.R, shape.T0
+    R_b, T_b = list(R_b), list(T_b)
+    p = make_problem(shape, seed, T=T, T_cap=T, recipe="peaked")
+    layer = gpu_layer(shape, p, dev)
+    caps = kvc.alloc_capsules(layer, B, R, dev)
+    kvc.kvc_compress(layer, p["K_vis"].to(dev), p["V_vis"].to(dev), B, R, caps)
+    K_g, V_g = kvc.capsule_views(layer, caps, B, R)
+    K_txt, V_txt = p["K_txt"].to(dev), p["V_txt"].to(dev)
+    for b in range(B):
+        K_g[b, :, R_b[b]:] = float("nan"); V_g[b, :, R_b[b]:] = float("nan")
+        K_txt[b, :, T_b[b]:] = float("nan"); V_txt[b, :, T_b[b]:] = float("nan")
+    kvc.kvc_layer_capsules_written(layer)
+    ws = kvc.alloc_workspace(layer, B, R, T, dev)
+    ws.fill_(0xFF)
+    out = torch.full((B, shape.H_q, 128), float("nan"), dtype=wl.torch_dtype(shape.dtype), device=dev)
+    i32 = lambda x: torch.tensor(list(x), dtype=torch.int32, device=dev)
+    run = lambda: kvc.kvc_decode_attend_ragged(layer, p["q"].to(dev), caps, B, R, i32(R_b), K_txt, V_txt, T, i32(T_b), T, out, ws)
+    counts, _ = launches(run)
+    run()                                              # a second call on the same workspace
+    torch.cuda.synchronize()
+    assert kvc.kvc_read_device_status(layer, B, R, T, ws) == 0
+    K_o, V_o = orc.compress(np64(p["K_vis"]), np64(p["V_vis"]), p["idx"].numpy(), np64(p["U"]), np64(p["mu"]), shape.n, False)
+    want = orc.decode_attend_ragged(np64(p["q"]), K_o, V_o, np64(p["theta"]), np64(p["U"]), np64(p["mu"]), np64(p["K_txt"]),
+                                    np64(p["V_txt"]), R_b, T_b, "kv")
+    got = np64(out)
+    assert_close(got, want, shape.dtype)
+    for b in range(B):
+        if R_b[b] == 0 and T_b[b] == 0:
+            assert (got[b] == 0).all()
+    R_b[0] = R + 1
+    run()
+    torch.cuda.synchronize()
+    assert kvc.kvc_read_device_status(layer, B, R, T, ws) == -8
+    return counts, got
+
+
 def small(shape: wl.Shape, **kw) -> wl.Shape:
     return dataclasses.replace(shape, **kw)

@@ -103,3 +103,19 @@ def test_per_sequence_lengths(B, H_q, H_kv, grid, R, T, ratio, monkeypatch):
     run()
     torch.cuda.synchronize()
     assert kvc.kvc_read_device_status(layer, B, R, T, ws) == -8
+
+
+@pytest.mark.parametrize("B,H_q,H_kv,grid,R,T,ratio,where", [
+    (64, 28, 4, 27, 1, 40, 600, range(0, 64, 9)),       # n = 729: eight of 64 sequences have a block
+    (128, 14, 2, 9, 1, 300, 600, (0, 127)),             # the first and the last of 128, in one unit
+    (60, 16, 1, 11, 2, 20, 600, (3, 59)),               # G = 16
+    (300, 2, 2, 9, 3, 5, 600, (1, 2, 298)),             # G = 1
+])
+def test_long_runs_of_sequences_without_blocks(B, H_q, H_kv, grid, R, T, ratio, where, monkeypatch):
+    """A unit's sequences may lie any number of block-less ones apart: its staged queries stay within its 128 rows."""
+    monkeypatch.setenv("KVC_EXPANSION", "cluster")
+    shape = wl.Shape("cluster-sparse", 1, B, H_q, H_kv, 128, grid, R, T, 1, "bf16", ratio)
+    R_b = [R if b in where else 0 for b in range(B)]
+    T_b = [T - b % 3 if b % 7 else 0 for b in range(B)]
+    counts, _ = tl.check_ragged(shape, 820 + grid, R_b, T_b)
+    assert counts["fused"] == 1 and counts["scores"] == 0
