@@ -21,7 +21,8 @@ namespace kvc {
 //   W      thread <-> a row of U (and every 256th after it), 16-byte loads of its 64 entries, the probabilities broadcast
 // One head of 4 rows, n = 576, m = 231 in fp32: 39 -> 18 us between events (one load of theta in flight per thread and 64 rows of U at a time
 // through shared memory before).
-template <typename T>
+// RP: pitch of a position's 16 partial logits, 17 against bank conflicts, 16 where retained rows take the last of the shared memory
+template <typename T, int RP>
 __global__ void __launch_bounds__(256) expand_kernel(DecodeArgs a) {
   constexpr int R16 = EXP_ROWS;
   static_assert(EXP_ROWS == 16 && EXP_IC == 64, "thread mapping");
@@ -29,8 +30,8 @@ __global__ void __launch_bounds__(256) expand_kernel(DecodeArgs a) {
   const int ms = a.ms, m = a.m, n = a.n, msv = a.msv, mv = a.mv;
   float* Ssm = smem;                          // [ms][16]
   float* Wacc = Ssm + R16 * ms;               // [msv][16]
-  float* red = Wacc + R16 * msv;              // [4][64][16 + 1] partial logits of the quarters
-  float* Psm = red + 4 * EXP_IC * (R16 + 1);  // [64][16]
+  float* red = Wacc + R16 * msv;              // [4][64][RP] partial logits of the quarters
+  float* Psm = red + 4 * EXP_IC * RP;  // [64][16]
   float* rowmax = Psm + EXP_IC * R16;         // [16]
   float* rowsum = rowmax + R16;
   float* rowscale = rowsum + R16;
@@ -88,7 +89,7 @@ __global__ void __launch_bounds__(256) expand_kernel(DecodeArgs a) {
         for (; j < m; j += 4) fma16(acc, Ssm + (size_t)j * R16, to_f32(tp[(size_t)j * n]));
       }
 #pragma unroll
-      for (int k = 0; k < R16; ++k) red[(qd * EXP_IC + ii) * (R16 + 1) + k] = acc[k];
+      for (int k = 0; k < R16; ++k) red[(qd * EXP_IC + ii) * RP + k] = acc[k];
     }
     __syncthreads();
     // ---- running max, P = exp(L - max), running sum: warp w owns rows 2w and 2w + 1
@@ -101,7 +102,7 @@ __global__ void __launch_bounds__(256) expand_kernel(DecodeArgs a) {
         const int c = lane + 32 * x;
         float v = 0.f;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) v += red[(q * EXP_IC + c) * (R16 + 1) + r];
+        for (int q = 0; q < 4; ++q) v += red[(q * EXP_IC + c) * RP + r];
         l[x] = i0 + c < i_end ? v : -INFINITY;
       }
       float cm = fmaxf(l[0], l[1]);
@@ -229,17 +230,23 @@ __global__ void __launch_bounds__(256) combine_kernel(DecodeArgs a) {
   if (lane == 0) a.statc[row] = make_float4(mx, sum, 0.f, 0.f);
 }
 
-static size_t expand_smem_bytes(int ms, int msv) {
-  return sizeof(float) * ((size_t)EXP_ROWS * (ms + msv) + 4 * EXP_IC * (EXP_ROWS + 1) + EXP_IC * EXP_ROWS + 3 * EXP_ROWS);
+static size_t expand_smem_bytes(int ms, int msv, int rp) {
+  return sizeof(float) * ((size_t)EXP_ROWS * (ms + msv) + 4 * EXP_IC * rp + EXP_IC * EXP_ROWS + 3 * EXP_ROWS);
+}
+
+template <typename T, int RP>
+static cudaError_t launch_expand_rp(const DecodeArgs& a, cudaStream_t st) {
+  const size_t smem = expand_smem_bytes(a.ms, a.msv, RP);
+  cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(expand_kernel<T, RP>), smem);
+  if (e != cudaSuccess) return e;
+  dim3 grid(a.ws.NS, ceil_div(a.B * a.G * a.R, EXP_ROWS), a.H_kv);
+  return launch_dependent(expand_kernel<T, RP>, grid, dim3(256), smem, st, a);
 }
 
 template <typename T>
 static cudaError_t launch_expand_t(const DecodeArgs& a, cudaStream_t st) {
-  const size_t smem = expand_smem_bytes(a.ms, a.msv);
-  cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(expand_kernel<T>), smem);
-  if (e != cudaSuccess) return e;
-  dim3 grid(a.ws.NS, ceil_div(a.B * a.G * a.R, EXP_ROWS), a.H_kv);
-  return launch_dependent(expand_kernel<T>, grid, dim3(256), smem, st, a);
+  // 3280 and 3296 score and weight entries a row (rounded up to 16 each) are the most the two pitches leave room for
+  return expand_smem_bytes(a.ms, a.msv, EXP_ROWS + 1) <= 227u * 1024u ? launch_expand_rp<T, EXP_ROWS + 1>(a, st) : launch_expand_rp<T, EXP_ROWS>(a, st);
 }
 
 cudaError_t launch_expand(const DecodeArgs& a, int dtype, cudaStream_t st) {

@@ -28,3 +28,16 @@ def test_fp32_expansion(B, H_q, H_kv, grid, R, T, ratio, mode):
     p = tl.make_problem(shape, 400 + grid, T=T, T_cap=T + 1, recipe="peaked")
     _, _, _, out = tl.gpu_run(shape, p, mode=mode)
     tl.assert_close(tl.np64(out), tl.oracle_run(shape, p, "fused", mode)[2], "f32", mode)
+
+
+@pytest.mark.parametrize("grid,ratio,mode", [(43, 110, "kv"), (48, 580, "k"), (48, 570, "k"), (48, 570, "v")])
+def test_most_retained_rows_that_fit(grid, ratio, mode):
+    """A score and a weight row of 3280 and of 3296 entries together, all that a CTA's shared memory holds."""
+    n = grid * grid
+    m = (n * (1000 - ratio) + 999) // 1000
+    pitch = lambda x: (x + 15) // 16 * 16
+    assert pitch(n if mode == "v" else m) + pitch(n if mode == "k" else m) == (3280 if ratio == 580 else 3296)
+    shape = wl.Shape("fp32-long", 1, 1, 2, 1, 128, grid, 1, 3, 1, "f32", ratio)
+    p = tl.make_problem(shape, 500 + grid, T=3, T_cap=4, recipe="peaked")
+    _, _, _, out = tl.gpu_run(shape, p, mode=mode)
+    tl.assert_close(tl.np64(out), tl.oracle_run(shape, p, "fused", mode)[2], "f32", mode)
