@@ -14,6 +14,7 @@
 // kept apart).
 //
 // Roles: warps 0-11 consumers, warp 12 MMA issue, warp 13 TMA producer.
+#include <algorithm>
 #include <mutex>
 
 #include "kvc_cluster.cuh"
@@ -101,14 +102,23 @@ __device__ __forceinline__ int cl_expected(const ClusterArgs& a, const ClusterVi
   return e;
 }
 
-// The last partial of a (sequence, KV head) merges: the G heads of every sequence of list[0 .. n), warps wi of nw taking (sequence, head)
-// pairs wi, wi + nw, ...  A lane finds one partial and its statistics; the values are loaded sixteen partials at a time (L2's latency
-// bounds it: with 8 in flight and a warp group per sequence the merge of 8 sequences of 5 blocks, 28/4 heads, took 8 us, now 3-6).
-__device__ __forceinline__ void cl_merge(const ClusterArgs& a, const ClusterView& v, const int* list, int n, int h, int wi, int nw) {
+// the same by all lanes of a warp, one of the sequence's units each
+__device__ __forceinline__ int cl_expected_warp(const ClusterArgs& a, const ClusterView& v, int b) {
+  const int f0 = cl_first(a, v.pre, b), f1 = cl_first(a, v.pre, b + 1);
+  int e = 0, pa;
+  if (f0 < f1)
+    for (int u = f0 / v.us.rb + (fresh(threadIdx.x) & 31); u <= (f1 - 1) / v.us.rb; u += 32) e += cl_pieces(a, v, u, f0, f1, pa);
+  return __reduce_add_sync(0xffffffffu, e) + (cl_text(a, v.tx, b) + a.tc - 1) / a.tc;
+}
+
+// The last partial of a (sequence, KV head) merges: the G query heads of every pair b H_kv + h of list[0 .. n), warps wi of nw taking
+// (pair, query head) wi, wi + nw, ...  A lane finds one partial and its statistics; the values are loaded sixteen partials at a time (L2's
+// latency bounds it: with 8 in flight and a warp group per sequence the merge of 8 sequences of 5 blocks, 28/4 heads, took 8 us, now 3-6).
+__device__ __forceinline__ void cl_merge(const ClusterArgs& a, const ClusterView& v, const int* list, int n, int wi, int nw) {
   const int G = a.G, lane = fresh(threadIdx.x) & 31;
 #pragma unroll 1
   for (int e = wi; e < n * G; e += nw) {
-    const int i = e / G, g = e - i * G, b = list[i];
+    const int i = e / G, g = e - i * G, bh = list[i], b = bh / a.H_kv, h = bh - b * a.H_kv;
     const int f0 = cl_first(a, v.pre, b), f1 = cl_first(a, v.pre, b + 1), u0 = f0 / v.us.rb, u1 = (f1 - 1) / v.us.rb;
     float M = -INFINITY, den = 0.f;
     float4 num = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -165,9 +175,13 @@ __device__ __forceinline__ void cl_merge(const ClusterArgs& a, const ClusterView
     const float inv = den > 0.f ? 1.f / den : 0.f;
     uint2 o;
     o.x = pack2_bf16(num.x * inv, num.y * inv); o.y = pack2_bf16(num.z * inv, num.w * inv);
-    *reinterpret_cast<uint2*>(a.out + ((size_t)(b * a.H_kv + h) * G + g) * D + lane * 4) = o;
+    *reinterpret_cast<uint2*>(a.out + ((size_t)bh * G + g) * D + lane * 4) = o;
   }
 }
+
+// The list of the pairs a CTA has to merge after its text items, their number in front of it; the list lies in the units' tables, whose
+// last use is over by then
+__device__ __forceinline__ int* cl_text_due(const ClusterArgs& a, unsigned char* sm) { return reinterpret_cast<int*>(sm + a.tab_off) + 1; }
 
 // Text rows: items of up to tc rows of a (sequence, KV head), a warp each, through the warp's own ring of 16-row pieces (4 KB, keys
 // and values in turn), flash-style; the item's partial goes straight from the registers to the workspace.  True if a wait gave up.
@@ -187,6 +201,7 @@ __device__ __forceinline__ bool cl_text_part(const CUtensorMap& tmKt, const CUte
     it_step = (a.ncl - a.ucl) * a.NS * CL_WARPS; it_end = a.text_ded;
     it = warp * (a.ncl - a.ucl) * a.NS + (int)blockIdx.x - a.ucl * a.NS;
   }
+  if (it - warp * (it_step / CL_WARPS) >= it_end) return false;      // no item for any warp of the CTA
   unsigned char* tring = sm + (uint32_t)warp * (CL_TEXT_SLOTS * 4096u);
   const uint32_t tring_u = smem_addr(tring);
   auto item_rows = [&](int k, int& b, int& h, int& t0) {
@@ -369,11 +384,19 @@ __device__ __forceinline__ bool cl_text_part(const CUtensorMap& tmKt, const CUte
     }
     __threadfence();
     __syncwarp();
-    int last = 0;
-    if (lane == 0) last = arrive_is_last(&a.cnt[bh], a.token, cl_expected(a, v, b)) ? 1 : 0;
-    last = __shfl_sync(0xffffffffu, last, 0);
-    if (last) { __threadfence(); cl_merge(a, v, &b, 1, h, 0, 1); }
+    const int expected = cl_expected_warp(a, v, b);
+    if (lane == 0 && arrive_is_last(&a.cnt[bh], a.token, expected)) {
+      __threadfence();
+      int* due = cl_text_due(a, sm);
+      due[atomicAdd(due - 1, 1)] = bh;
+    }
   }
+  // The pairs whose last partial was one of the text's, by all warps of the CTA: a warp that merged its own alone took a round trip to L2
+  // per query head and sixteen partials, one after the other (2 x 15 blocks of n = 81, 16/1 heads, 338 text rows: 58 us per call,
+  // now 31; 28/4 heads, 2 x 15 of n = 81, 1500 rows: 46 and 26)
+  named_barrier_sync(1, CL_CONS);
+  const int* due = cl_text_due(a, sm);
+  cl_merge(a, v, due, due[-1], fresh(threadIdx.x) >> 5, CL_WARPS);
   return dead;
 }
 
@@ -409,6 +432,7 @@ cluster_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
     for (int w = 0; w < CL_WARPS; ++w)
       for (int s = 0; s < CL_TEXT_SLOTS; ++s) mbar_init(&bars.text[w][s], 1);
     fence_mbar_init();
+    cl_text_due(a, sm)[-1] = 0;
   }
   if (warp == CL_WARPS) tmem_alloc(&s_tmem, 512u);
   // per-sequence lengths are inputs like the queries: read after the stream's previous kernel
@@ -985,7 +1009,7 @@ cluster_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
         int bl = v0 / a.vt, jt = v0 - bl * a.vt;
         int cur_b = -1, s = grp, nflush = 0;
         int mine = 0;                                           // thread x of the group arrives for the run's x-th sequence
-        int* due = reinterpret_cast<int*>(sm + CL_DUE);         // sequences this CTA has to merge
+        int* due = reinterpret_cast<int*>(sm + CL_DUE);         // pairs this CTA has to merge
         BlockWalk bw;
         if (v0 < v1) bw.start(a, pre, u.blk0 + bl);
         for (int t = v0; t < v1; ++t) {
@@ -1130,15 +1154,19 @@ cluster_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
         named_barrier_sync(2 + grp, 128);
         if (gt < nflush) {
           __threadfence();                   // the partials of every thread (ordered before by the barrier) before the arrival
-          if (arrive_is_last(&a.cnt[mine * a.H_kv + u.h], a.token, expected)) due[atomicAdd(ndue, 1)] = mine;
+          if (arrive_is_last(&a.cnt[mine * a.H_kv + u.h], a.token, expected)) due[atomicAdd(ndue, 1)] = mine * a.H_kv + u.h;
           __threadfence();
         }
         named_barrier_sync(1, CL_CONS);                         // (a CTA sees a sequence become due once at most)
-        cl_merge(a, view, due, *ndue, u.h, warp, CL_WARPS);
+        cl_merge(a, view, due, *ndue, warp, CL_WARPS);
       }
     }
 
-    if (units > 0) { fence_proxy_async(); named_barrier_sync(1, CL_CONS); }      // the text's pieces take the memory the units' tiles were in
+    if (units > 0) {                                            // the text's pieces take the memory the units' tiles were in
+      if (fresh(tid) == 0) cl_text_due(a, sm)[-1] = 0;
+      fence_proxy_async();
+      named_barrier_sync(1, CL_CONS);
+    }
     if (cl_text_part<NH>(tmKt, tmVt, a, view, sm, bars)) dead = true;
     if (dead && lane == 0) atomicExch(a.status, (int)KVC_ERR_TIMEOUT);
   }
@@ -1302,6 +1330,10 @@ ClusterPlan plan_cluster(const kvc_layer* L, int B, int R, int T, bool ragged) {
   } else {
     p.ncl = p.ucl;
   }
+  // a CTA's list of the pairs it merges after its text items holds as many as it can have items
+  const long long with = (long long)p.ucl * p.NS, without = (long long)(p.ncl - p.ucl) * p.NS;
+  const long long most = std::max((p.text_items - p.text_ded + with - 1) / with, without > 0 ? (p.text_ded + without - 1) / without : 0ll);
+  if (most > (long long)(CL_GROUPS * 512u + (uint32_t)p.NS * 1024u) / 4 - 1) return p;
   p.units = H * us.nu;
   p.ok = 1;
   return p;

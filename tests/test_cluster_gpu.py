@@ -52,6 +52,8 @@ def _launches(fn):
     (40, 16, 8, 13, 3, 3, 600),      # more units than one wave
     (1, 2, 1, 12, 1, 2200, 600),     # text beyond sixteen chunks
     (2, 16, 1, 11, 9, 30, 800),      # G = 16
+    (2, 16, 1, 9, 15, 1500, 525),    # the text ends last and merges more partials than a warp has lanes
+    (200, 8, 4, 9, 1, 40, 600),      # more text items than warps
 ])
 def test_uniform(B, H_q, H_kv, grid, R, T, ratio, recipe, monkeypatch):
     monkeypatch.setenv("KVC_EXPANSION", "cluster")
