@@ -1225,7 +1225,17 @@ static int cl_v_slots(uint32_t ring_max, uint32_t w_bytes) {
   while (nv > 0 && (uint32_t)nv * CL_TILE_BYTES + (uint32_t)(nv > tail ? nv - tail : 0) * w_bytes > ring_max) nv -= CL_GROUPS;
   return nv;
 }
-static int text_chunk(int T) { return T <= 16 * CL_TEXT_CHUNK ? CL_TEXT_CHUNK : (int)align_up((size_t)ceil_div(T, 16), 16); }
+// Text items per (sequence, KV head): chunks of CL_TEXT_CHUNK rows, longer ones past 64 of them where the device has a warp for every
+// item, past 16 where it has not.  A warp's rows are a chain of some 0.8 us per 16 of them; partials cost the merge.  4 x 2 blocks of n = 400,
+// 8/2 heads, 13095 text rows: 16 items 71 us per call, 64 36.9, 128 37.1; one sequence, 32768 rows: 132, 51, 42; 2 sequences of 30000, 64/8
+// heads: 154, 82, 91; more items than warps (8 sequences of 2500, 32/8 heads): 47, at 20 items 64.
+static int text_items(const kvc_layer* L, int B) {
+  return 64ll * B * L->desc.H_kv <= (long long)(L->num_sms > 0 ? L->num_sms : 148) * CL_WARPS ? 64 : 16;
+}
+static int text_chunk(const kvc_layer* L, int B, int T) {
+  const int most = text_items(L, B);
+  return T <= most * CL_TEXT_CHUNK ? CL_TEXT_CHUNK : (int)align_up((size_t)ceil_div(T, most), 16);
+}
 
 ClusterPlan plan_cluster(const kvc_layer* L, int B, int R, int T, bool ragged) {
   ClusterPlan p{};
@@ -1311,7 +1321,7 @@ ClusterPlan plan_cluster(const kvc_layer* L, int B, int R, int T, bool ragged) {
   p.pre_off = p.tab_off + tab;
   p.smem = 1024u + (size_t)p.pre_off + pre;
   if (p.smem > CL_DYN_LIMIT) return p;
-  p.tc = text_chunk(T);
+  p.tc = text_chunk(L, B, T);
   p.nct = ceil_div(T, p.tc);
   p.text_items = (long long)B * H * p.nct;
   if (p.text_items >= (1ll << 30)) return p;
@@ -1362,8 +1372,8 @@ size_t cluster_ws_bytes(const kvc_layer* L, int B, int R, int T_cap) {
   for (int ragged = 0; ragged < 2; ++ragged) {
     ClusterPlan p = plan_cluster(L, B, R, T_cap, ragged != 0);
     if (!p.ok) continue;
-    // the chunks of a shorter text: never more than 16, nor than whole chunks of the smallest size
-    p.nct = ceil_div(T_cap, CL_TEXT_CHUNK) < 16 ? ceil_div(T_cap, CL_TEXT_CHUNK) : 16;
+    // the chunks of a shorter text: never more than the most of a pair, nor than whole chunks of the smallest size
+    p.nct = std::min(ceil_div(T_cap, CL_TEXT_CHUNK), text_items(L, B));
     const size_t b = cluster_ws(L, p, B, R).bytes;
     most = b > most ? b : most;
   }

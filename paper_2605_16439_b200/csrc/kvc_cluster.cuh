@@ -30,7 +30,7 @@ constexpr int CL_K_SLOTS = 3 * CL_GROUPS, CL_V_SLOTS = 3 * CL_GROUPS, CL_X_SLOTS
 constexpr int CL_MAX_NS = 8;
 constexpr int CL_MAX_RAGGED_B = 512;
 constexpr int CL_TEXT_SLOTS = 4;                   // 16-row pieces in flight per warp of the text part
-constexpr int CL_TEXT_CHUNK = 128;                 // text rows per item (more for very long tails)
+constexpr int CL_TEXT_CHUNK = 128;                 // text rows per item (more where a pair has as many items as it may)
 
 struct ClusterPlan {
   int ok;

@@ -51,6 +51,8 @@ def _launches(fn):
     (37, 2, 2, 10, 1, 20, 600),      # many sequences per unit
     (40, 16, 8, 13, 3, 3, 600),      # more units than one wave
     (1, 2, 1, 12, 1, 2200, 600),     # text beyond sixteen chunks
+    (2, 2, 2, 9, 1, 8200, 600),      # text beyond sixty-four
+    (8, 4, 4, 9, 1, 2100, 600),      # text beyond sixteen chunks of more items than warps
     (2, 16, 1, 11, 9, 30, 800),      # G = 16
     (2, 16, 1, 9, 15, 1500, 525),    # the text ends last and merges more partials than a warp has lanes
     (200, 8, 4, 9, 1, 40, 600),      # more text items than warps
