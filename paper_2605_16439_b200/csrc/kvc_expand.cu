@@ -18,7 +18,9 @@ namespace kvc {
 // walks its range of the n axis in chunks of 64 positions:
 //   L      thread <-> (position, quarter of the retained rows), eight loads of theta in flight, 16 rows accumulated in registers
 //          against scores broadcast from shared memory ([j][16 rows]); the quarters meet in shared memory
-//   W      thread <-> a row of U (and every 256th after it), 16-byte loads of its 64 entries, the probabilities broadcast
+//   W      thread <-> a row of U (and every 256th after it), 16-byte loads of its 64 entries, the probabilities broadcast; rows that do not
+//          start on 16-byte boundaries, or at most 64 of them, 64 at a time through shared memory, thread <-> (row, 4 expansion rows)
+//          (32 sequences of one block of n = 529, m = 212, bf16, 4/4 heads: a call 61 us with a thread per row, now 37)
 // One head of 4 rows, n = 576, m = 231 in fp32: 39 -> 18 us between events (one load of theta in flight per thread and 64 rows of U at a time
 // through shared memory before).
 // RP: pitch of a position's 16 partial logits, 17 against bank conflicts, 16 where retained rows take the last of the shared memory
@@ -45,9 +47,9 @@ __global__ void __launch_bounds__(256) expand_kernel(DecodeArgs a) {
   const T* U = static_cast<const T*>(a.U) + (size_t)h * mv * n;
   const float* S = a.S + (size_t)h * nrows_h * ms;
   const int ii = tid & 63, qd = tid >> 6;     // position in the chunk, quarter of the retained rows
-  // 16-byte loads of U: rows start on 16-byte boundaries
+  // U read from L2 by its rows' threads: rows start on 16-byte boundaries, and there are enough of them to keep the warps busy
   constexpr int EPV = Elems16<T>::N;
-  const bool vec = n % EPV == 0 && (reinterpret_cast<uintptr_t>(U) & 15) == 0;
+  const bool direct = mv > 64 && n % EPV == 0 && (reinterpret_cast<uintptr_t>(U) & 15) == 0;
 
   grid_dep_wait();
   grid_dep_launch();
@@ -132,17 +134,17 @@ __global__ void __launch_bounds__(256) expand_kernel(DecodeArgs a) {
       continue;
     }
     // ---- W[:, j] = W[:, j] * scale + P . U[j, i0 : i0 + 64]^T
-    for (int j = tid; j < mv; j += 256) {
-      float acc[R16];
+    const int cnt = min(EXP_IC, i_end - i0);
+    if (direct) {
+      for (int j = tid; j < mv; j += 256) {
+        float acc[R16];
 #pragma unroll
-      for (int k = 0; k < R16; k += 4) {
-        const float4 w = *reinterpret_cast<const float4*>(Wacc + (size_t)j * R16 + k), sc = *reinterpret_cast<const float4*>(rowscale + k);
-        acc[k] = w.x * sc.x; acc[k + 1] = w.y * sc.y; acc[k + 2] = w.z * sc.z; acc[k + 3] = w.w * sc.w;
-      }
-      const T* up = U + (size_t)j * n + i0;
-      const int cnt = min(EXP_IC, i_end - i0);
-      int i = 0;
-      if (vec) {
+        for (int k = 0; k < R16; k += 4) {
+          const float4 w = *reinterpret_cast<const float4*>(Wacc + (size_t)j * R16 + k), sc = *reinterpret_cast<const float4*>(rowscale + k);
+          acc[k] = w.x * sc.x; acc[k + 1] = w.y * sc.y; acc[k + 2] = w.z * sc.z; acc[k + 3] = w.w * sc.w;
+        }
+        const T* up = U + (size_t)j * n + i0;
+        int i = 0;
         for (; i + 4 * EPV <= cnt; i += 4 * EPV) {
           float u[4][EPV];
 #pragma unroll
@@ -152,12 +154,35 @@ __global__ void __launch_bounds__(256) expand_kernel(DecodeArgs a) {
 #pragma unroll
             for (int e = 0; e < EPV; ++e) fma16(acc, Psm + (i + v * EPV + e) * R16, u[v][e]);
         }
-      }
-      for (; i < cnt; ++i) fma16(acc, Psm + i * R16, to_f32(up[i]));
+        for (; i < cnt; ++i) fma16(acc, Psm + i * R16, to_f32(up[i]));
 #pragma unroll
-      for (int k = 0; k < R16; k += 4) *reinterpret_cast<float4*>(Wacc + (size_t)j * R16 + k) = make_float4(acc[k], acc[k + 1], acc[k + 2], acc[k + 3]);
+        for (int k = 0; k < R16; k += 4) *reinterpret_cast<float4*>(Wacc + (size_t)j * R16 + k) = make_float4(acc[k], acc[k + 1], acc[k + 2], acc[k + 3]);
+      }
+      __syncthreads();
+    } else {
+      // 64 rows of U at a time through shared memory (the partial logits' region), each row turned by its number against bank conflicts
+      for (int j0 = 0; j0 < mv; j0 += 64) {
+#pragma unroll
+        for (int x = 0; x < 16; ++x) {
+          const int jj = qd + 4 * x;
+          red[jj * 64 + ((ii + jj) & 63)] = j0 + jj < mv && ii < cnt ? to_f32(U[(size_t)(j0 + jj) * n + i0 + ii]) : 0.f;
+        }
+        __syncthreads();
+        if (j0 + ii < mv) {
+          float4* wp = reinterpret_cast<float4*>(Wacc + (size_t)(j0 + ii) * R16 + qd * 4);
+          const float4 w = *wp, sc = *reinterpret_cast<const float4*>(rowscale + qd * 4);
+          float4 acc = make_float4(w.x * sc.x, w.y * sc.y, w.z * sc.z, w.w * sc.w);
+#pragma unroll 8
+          for (int i = 0; i < cnt; ++i) {
+            const float u = red[ii * 64 + ((i + ii) & 63)];
+            const float4 p = *reinterpret_cast<const float4*>(Psm + i * R16 + qd * 4);
+            acc.x = fmaf(p.x, u, acc.x); acc.y = fmaf(p.y, u, acc.y); acc.z = fmaf(p.z, u, acc.z); acc.w = fmaf(p.w, u, acc.w);
+          }
+          *wp = acc;
+        }
+        __syncthreads();
+      }
     }
-    __syncthreads();
   }
 
   float* Wout = a.W + ((size_t)split * a.H_kv + h) * nrows_h * msv;
@@ -240,7 +265,11 @@ static cudaError_t launch_expand_rp(const DecodeArgs& a, cudaStream_t st) {
   cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(expand_kernel<T, RP>), smem);
   if (e != cudaSuccess) return e;
   dim3 grid(a.ws.NS, ceil_div(a.B * a.G * a.R, EXP_ROWS), a.H_kv);
-  return launch_dependent(expand_kernel<T, RP>, grid, dim3(256), smem, st, a);
+  // Programmatic overlap with the fp32 score kernel only (one sequence, one layer: 37.6 us per call, 40.7 without); behind the bf16 one, which
+  // does not let it start early, it costs (32 sequences of one block of n = 81, 4/4 heads: 29.6 us per call, 21.7 without)
+  if (sizeof(T) == sizeof(float)) return launch_dependent(expand_kernel<T, RP>, grid, dim3(256), smem, st, a);
+  expand_kernel<T, RP><<<grid, 256, smem, st>>>(a);
+  return cudaGetLastError();
 }
 
 template <typename T>

@@ -19,7 +19,7 @@ def _built():
 @pytest.mark.parametrize("mode", ["kv", "k", "v"])
 @pytest.mark.parametrize("B,H_q,H_kv,grid,R,T,ratio", [
     (1, 1, 1, 3, 1, 2, 900), (1, 5, 1, 8, 3, 0, 500), (4, 4, 1, 9, 1, 7, 600), (1, 17, 1, 11, 1, 3, 730), (2, 6, 2, 16, 2, 20, 200),
-    (1, 3, 1, 27, 2, 5, 550),
+    (1, 3, 1, 27, 2, 5, 550), (2, 4, 2, 16, 1, 3, 750), (2, 4, 2, 16, 1, 3, 746),       # (the last two: m = 64 and 66)
 ])
 def test_fp32_expansion(B, H_q, H_kv, grid, R, T, ratio, mode):
     if H_q // H_kv > 16:
