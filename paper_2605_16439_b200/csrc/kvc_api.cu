@@ -358,10 +358,30 @@ static int ragged_path(const kvc_layer* L, int B, int R, int T) {
   return cluster < 0.9 * phases ? 2 : 0;
 }
 
+// Few query heads per KV head, expansions in fp32 where the three-phase kernels make them: whether those are ahead of the cluster path.  The
+// cluster path's time goes with the rounds of its units (18 us each, and its tiles, sequences and row chunks), the three-phase kernels'
+// with the chunks of 64 positions of 16 expansion rows, the retained rows they walk, and the bytes.  Constants fitted (least squares of the
+// relative error: 8 % and 12 %) to 1620 uniform calls on B200: 1/1 to 32/32 and 8/2, 32/8 heads, 1 x 1 to 64 x 2 blocks of n = 81 to 961, m = 11
+// to 769, 0 to 700 text rows; routed by it the calls take 0.6 % more than each on its better path, and 16 of 2430 more than 10 %
+// over what the three-phase kernels took before there was a cluster path (at worst 20.0 for 16.3).  us per call, cluster / three-phase: 16/16 heads, 64 x 2 of n = 81, m = 11,
+// 60 text rows 78 / 33; 32/32, 7 x 2 of 529, m = 67 53 / 31, m = 424 92 / 107; 4/4, 64 x 2 of 81, 700 rows 85 / 50; 8/2, 16 x 5 of 729, m = 292 45 / 143.
+static bool cuda_core_expansion_wins(const kvc_layer* L, int B, int R, int T, bool ragged) {
+  const ClusterPlan c = plan_cluster(L, B, R, T, ragged);
+  if (!c.ok) return true;
+  const int n = L->desc.n, m = L->m, H = L->desc.H_kv, nb = B * R;
+  const double rows = 512.0 * nb * H * (double)m, text = 512.0 * B * H * (double)T;
+  const double rounds = (c.units + c.ucl - 1) / c.ucl, rb = ceil_div(nb, c.units / H), seqs = std::min(rb, rb / R + (R > 1 && rb > 1 ? 1.0 : 0.0));
+  const double cluster = rounds * (18.0 + (0.6 * rb * c.vt + 0.44 * seqs) / c.NS + 1.4 * c.nk1) - 2.0 + (rows + 4.0 * H * m * n + 1.2 * text) / 6.5e6;
+  const WsLayout w = ws_layout(L, B, R, T);
+  const double walk = w.IR / EXP_IC, chunks = (double)H * ceil_div(nb * L->G, EXP_ROWS) * ceil_div(n, EXP_IC);
+  const double phases = 15.7 + walk * (0.063 * m - 2.5) + chunks * (2.24e-4 * m + 0.0132) + (1.7 * rows + 1.57 * text) / 6.5e6 + 1.35 * (L->G - 1) + c.nk1;
+  return phases < cluster;
+}
+
 // Which bf16 shapes take the cluster path.  Measured on B200, us per call, cluster / other paths.
 // Block lengths that are no multiple of 64, and per-sequence lengths outside the path above: the other way is the three-phase kernels.
-// It is ahead at every shape tried where those expand on the CUDA cores (n no multiple of 8: 8 x 5 blocks of n = 729, 28/4 heads: 37 /
-// 277) and, with more than one query head per KV head, where they expand on mma.sync (4 x 1 of 400: 22 / 29; 16 x 4 of 196, 32/8 heads:
+// Where those expand on the CUDA cores (n no multiple of 8) it is ahead from seven query heads per KV head on (8 x 5 blocks of n = 729,
+// 28/4 heads: 37 / 277); below, by the estimate above (cuda_core_expansion_wins).  And, with more than one query head per KV head, where they expand on mma.sync (4 x 1 of 400: 22 / 29; 16 x 4 of 196, 32/8 heads:
 // 31 / 65; 1 x 1 of 784, 8/2 heads: 23 / 25; 8 x 2 of 144: 18.8 / 18.6; with lengths per sequence from 1e7 flop of expansion on: 8 x 5 of
 // 144, 6/2 heads, 8e6: 21.7 / 20.8; 2 x 5 of 144, 28/4 heads, 9e6: 22 / 27); with one, its 128-row tiles stay empty (8 x 4 of 400, 32/32
 // heads: 60 / 50).
@@ -382,7 +402,8 @@ static bool use_cluster(const kvc_layer* L, int B, int R, int T, bool ragged) {
       const int path = ragged_path(L, B, R, T);
       if (path != 2 || G == 1) return path == 2;
     }
-    return cluster_terms(L) == 2 || (G > 1 && (!ragged || 4.0 * B * L->desc.H_q * R * (double)L->m * n >= 1e7));
+    if (cluster_terms(L) == 2) return G > 4 || !cuda_core_expansion_wins(L, B, R, T, ragged);
+    return G > 1 && (!ragged || 4.0 * B * L->desc.H_q * R * (double)L->m * n >= 1e7);
   }
   if (n <= 256 || n > 640 || G == 1) return false;
   const int sms = L->num_sms > 0 ? L->num_sms : 148;

@@ -123,3 +123,16 @@ def test_long_runs_of_sequences_without_blocks(B, H_q, H_kv, grid, R, T, ratio, 
     T_b = [T - b % 3 if b % 7 else 0 for b in range(B)]
     counts, _ = tl.check_ragged(shape, 820 + grid, R_b, T_b)
     assert counts["fused"] == 1 and counts["scores"] == 0
+
+
+@pytest.mark.parametrize("H_q,H_kv,B,R,grid,T,ratio,cluster", [
+    (16, 16, 64, 2, 9, 60, 875, False), (4, 4, 64, 2, 9, 700, 600, False), (8, 2, 32, 1, 9, 700, 600, False), (16, 16, 7, 2, 31, 60, 875, False),
+    (8, 2, 16, 5, 19, 60, 600, True), (4, 4, 7, 2, 27, 60, 600, True), (28, 4, 1, 1, 9, 60, 875, True),
+])
+def test_odd_block_lengths_take_the_faster_path(H_q, H_kv, B, R, grid, T, ratio, cluster):
+    """Block lengths off the tensor-core expansion of the three-phase kernels: both sides of the rule, by default routing."""
+    shape = wl.Shape("odd-route", 1, B, H_q, H_kv, 128, grid, R, T, 1, "bf16", ratio)
+    p = tl.make_problem(shape, 850 + grid, T=T, T_cap=T, recipe="peaked")
+    counts, (_, _, _, out) = tl.launches(lambda: tl.gpu_run(shape, p))
+    assert counts["scores"] == (0 if cluster else 1)
+    tl.assert_close(tl.np64(out), tl.oracle_run(shape, p, "fused")[2], "bf16")
