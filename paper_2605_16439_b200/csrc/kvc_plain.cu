@@ -348,6 +348,10 @@ PlainPlan plan_plain(const kvc_layer* L, int B, int S0, int T) {
     long long cpb = sms / bh, most = p.spp <= 48 ? 1 : ceil_div(p.spp, 16);
     cpb = cpb < most ? cpb : most;
     grid = bh * (cpb < PN_MAX_PARTS - 2 ? cpb : PN_MAX_PARTS - 2);
+    // one CTA per pair on at most three quarters of the SMs: they cannot draw the bandwidth, and long runs are worth the crossings (80 pairs x
+    // 1250 steps: 148.9 us, crossing 134.2; x 563: 73.2 and 66.0; x 188: 27.4 and 30.7; 104 x 563: 84.5 and 82.3, x 188: 34.1 and 34.6; 120 x
+    // 563: 93.6 and 94.1)
+    if (cpb == 1 && p.spp > 448 && 4 * bh < 3 * sms) grid = sms;
   } else {
     const long long waves = (bh + sms - 1) / sms;
     grid = p.spp > 96 && bh * 5 < waves * sms * 4 ? sms : bh;

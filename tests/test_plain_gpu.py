@@ -26,6 +26,7 @@ def _built():
 @pytest.mark.parametrize("B,H_q,H_kv,S", [
     (1, 1, 1, 1), (1, 7, 1, 15), (2, 4, 2, 17), (1, 8, 1, 191), (1, 7, 1, 769), (1, 16, 1, 3000), (1, 2, 2, 9000), (3, 12, 1, 800),
     (37, 8, 4, 50), (75, 4, 2, 33), (80, 4, 2, 1600), (151, 1, 1, 1700), (40, 28, 4, 300),
+    (80, 1, 1, 7200), (20, 4, 4, 7150),        # one pair per CTA with crossing runs (a pair on up to three CTAs), and just not
 ])
 def test_attend_full(B, H_q, H_kv, S):
     gen = torch.Generator().manual_seed(S + B)
