@@ -426,12 +426,13 @@ cudaError_t launch_compress_tc(const kvc_layer* L, const void* K_vis, const void
   a.B = B; a.H_kv = H_kv; a.R = R; a.n = n; a.m = m; a.pitch = pitch;
   const long long blocks = (long long)B * H_kv * R;
   const int sms = L->num_sms > 0 ? L->num_sms : 148;
-  // Two blocks per unit give the MMA its full width of 256 columns (141 cycles per K step of 16 against 95 for half the width);
-  // where that leaves SMs without a unit, one block per unit.
-  a.bpu = 2;
+  // Two blocks per unit give the MMA its full width of 256 columns (141 cycles per K step of 16 against 95 for half the width); one
+  // where those units are no more than the SMs (2 x 3 blocks of n = 576, m = 288, 8 heads: 9.4 us, in pairs 10.3), since a second wave of
+  // them costs more than the width (3 x 3: 13.5 and 10.9; 2 x 5 of 1024, m = 410, 4 heads: 18.8 and 13.6).
+  a.bpu = 1;
   a.mtiles = ceil_div(m, CT_BM);
   auto unit_count = [&]() { return ((long long)B * R + a.bpu - 1) / a.bpu * H_kv * a.mtiles; };
-  if (unit_count() < sms) a.bpu = 1;
+  if (unit_count() > sms) a.bpu = 2;
   if (unit_count() >= (1ll << 31)) return cudaSuccess;
   *used = true;
   a.status = L->d_cstatus;
