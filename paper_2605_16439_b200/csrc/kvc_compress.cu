@@ -241,10 +241,17 @@ cudaError_t launch_compress_ragged(const kvc_layer* L, const void* K_vis, const 
                                    const int* N_v, int R_max, void* Kc, void* Vc, void* K_tail, void* V_tail, int T_cap,
                                    int* R_b, int* T_b, cudaStream_t st) {
   {
-    const RaggedCompress rag{N_v, N_cap, T_cap, R_b, T_b, K_tail, V_tail};
+    // lengths written over the ones they come from: after the kernel, whose CTAs read those until they end
+    auto same = [&](const int* out) { return out < N_v + B && N_v < out + B; };
+    const bool in_place = same(R_b) || same(T_b);
+    const RaggedCompress rag{N_v, N_cap, T_cap, in_place ? nullptr : R_b, in_place ? nullptr : T_b, K_tail, V_tail};
     bool used = false;
-    const cudaError_t e = launch_compress_tc(L, K_vis, V_vis, B, R_max, N_cap, L->passthrough || L->mode == KVC_MODE_V_ONLY ? 2 : 1,
-                                             L->passthrough || L->mode == KVC_MODE_K_ONLY ? 2 : 1, Kc, Vc, &rag, st, &used);
+    cudaError_t e = launch_compress_tc(L, K_vis, V_vis, B, R_max, N_cap, L->passthrough || L->mode == KVC_MODE_V_ONLY ? 2 : 1,
+                                       L->passthrough || L->mode == KVC_MODE_K_ONLY ? 2 : 1, Kc, Vc, &rag, st, &used);
+    if (used && e == cudaSuccess && in_place) {
+      ragged_lengths_kernel<<<ceil_div(B, 128), 128, 0, st>>>(N_v, B, L->desc.n, N_cap, R_max, T_cap, R_b, T_b, L->d_cstatus);
+      e = cudaGetLastError();
+    }
     if (used || e != cudaSuccess) return e;
   }
   {

@@ -62,7 +62,7 @@ struct CompressTcArgs {
   // per-sequence lengths (nullptr: R blocks each)
   const int* N_v;
   int N_cap, T_cap;
-  int* R_b;
+  int* R_b;                  // written by CTA 0 (nullptr: not at all)
   int* T_b;
   const __nv_bfloat16* Ktail_src;
   const __nv_bfloat16* Vtail_src;
@@ -140,8 +140,7 @@ compress_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant__
       bool ok = true;
       if (b < a.B) ok = ragged_split(a.N_v[b], a, r, t);
       if (b < a.B && blockIdx.x == 0) {
-        a.R_b[b] = r;
-        a.T_b[b] = t;
+        if (a.R_b) { a.R_b[b] = r; a.T_b[b] = t; }
         if (!ok) atomicExch(a.status, (int)KVC_ERR_BOUNDS);
       }
       int x = r;

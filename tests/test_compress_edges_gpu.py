@@ -84,3 +84,30 @@ def test_ragged_compression(grid, mode):
             _assert_capsules(V_g[b, :, :r], V_o[b, :, :r], f"values of sequence {b}")
         assert torch.equal(kt[b, :, :t].cpu(), p["K_vis"][b, :, r * n:r * n + t]) and (kt[b, :, t:] == 7).all()
         assert torch.equal(vt[b, :, :t].cpu(), p["V_vis"][b, :, r * n:r * n + t]) and (vt[b, :, t:] == 7).all()
+
+
+@pytest.mark.parametrize("over", ["R_b", "T_b"])
+def test_lengths_may_be_written_over_the_row_counts(over):
+    """N_v and R_b (or T_b) one array: capsules, rows left over and lengths as with arrays of their own."""
+    n, B, H, R, N_cap = 81, 40, 4, 3, 4 * 81
+    shape = wl.Shape("compress-in-place", 1, B, H, H, 128, 9, 4, 1, 1, "bf16", 600)
+    p = tl.make_problem(shape, 961, recipe="peaked")
+    layer = tl.gpu_layer(shape, p)
+    K, V = p["K_vis"].to(DEV), p["V_vis"].to(DEV)
+    lengths = [(37 * b) % (3 * n + 50) for b in range(B)]
+    i32 = lambda x: torch.tensor(list(x), dtype=torch.int32, device=DEV)
+    got = []
+    for shared in (False, True):
+        caps = kvc.alloc_capsules(layer, B, R)
+        caps.fill_(0)
+        kt, vt = (torch.zeros((B, H, n, 128), dtype=torch.bfloat16, device=DEV) for _ in range(2))
+        N_v, out = i32(lengths), dict(R_b=i32([-1] * B), T_b=i32([-1] * B))
+        if shared:
+            out[over] = N_v
+        kvc.kvc_compress_ragged(layer, K, V, B, N_cap, N_v, R, caps, kt, vt, n, out["R_b"], out["T_b"])
+        torch.cuda.synchronize()
+        assert kvc.kvc_read_compress_status(layer) == 0
+        got.append((caps, kt, vt, out["R_b"], out["T_b"]))
+    assert got[0][3].tolist() == [x // n for x in lengths] and got[0][4].tolist() == [x % n for x in lengths]
+    for a, b in zip(*got):
+        assert torch.equal(a, b)
