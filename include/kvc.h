@@ -12,8 +12,10 @@
  *
  * Conventions
  *   - Every tensor pointer is a DEVICE pointer to caller-owned, contiguous memory unless a
- *     comment says "host".  The library owns only the opaque kvc_layer (a host struct plus a
- *     small device copy of the index set).
+ *     comment says "host".  The library owns only the opaque kvc_layer: a host struct plus device
+ *     copies of the index set and the row sums of U (a few KB) and, for bf16 block lengths off
+ *     64 (theta) or 8 (U) that kernels read by the TMA engine, copies of theta and U with padded rows
+ *     (up to 4 H_kv m (n rounded up to 64) bytes: n = 729 at ratio 0.6 with 4 KV heads 3.6 MB a layer).
  *   - Calls are asynchronous on the given CUDA stream (a cudaStream_t passed as void*; NULL is
  *     the legacy default stream).  They never synchronise and, except kvc_layer_create /
  *     kvc_layer_destroy, never allocate or free device memory.
@@ -88,7 +90,8 @@ KVC_API int kvc_retained_len(int n, int ratio_permille);
 
 /* Validates the descriptor (KVC_ERR_SHAPE / _DTYPE / _NO_PARAMS / _BOUNDS), copies the index set
  * to device memory and returns a handle.  theta, U and mu are borrowed: they must stay valid and
- * unchanged while the handle is in use.  ratio_permille == 0 is the pass-through limit: m = n,
+ * unchanged from this call on while the handle is in use.  The call waits for the device (writes to theta and U
+ * that are on their way on any stream are seen) and reads theta and U.  ratio_permille == 0 is the pass-through limit: m = n,
  * capsules hold K and V verbatim, idx / theta / U / mu are ignored.
  * The device that is current at this call must be current for every later call with the handle.
  * bf16 decode calls run Alg. 1 either as one kernel (steps 2-3 on mma.sync with the logits in registers, or on tcgen05

@@ -209,19 +209,22 @@ int kvc_layer_create(const kvc_layer_desc* desc, kvc_layer** out) {
     const char* ex = std::getenv("KVC_EXPANSION");
     L->use_tc = !ex ? 0 : (std::strcmp(ex, "tcgen05") == 0 ? 1 : (std::strcmp(ex, "pair") == 0 ? 2 : (std::strcmp(ex, "mma") == 0 ? -1 : (std::strcmp(ex, "phases") == 0 ? -2 : (std::strcmp(ex, "split") == 0 ? 3 : (std::strcmp(ex, "resident") == 0 ? 4 : (std::strcmp(ex, "cluster") == 0 ? 5 : 0)))))));
   }
-  // one allocation: index set, status word, row sums of U, and copies of theta and U with rows the TMA engine can address
-  // where n is not a multiple of 64 (bf16)
-  L->np = (int)align_up((size_t)desc->n, 64);
-  L->theta_rows = key_side && !pass ? desc->theta : nullptr;
+  // one allocation: index set, status word, row sums of U, and where a kernel would read them, copies of theta and U with rows the TMA
+  // engine can address (bf16): theta for the cluster path, whose tensor map cuts rows in groups of 64, U where its rows do not start on 16 bytes
+  const int np = (int)align_up((size_t)desc->n, 64);
+  const bool pad_theta = np != desc->n && cluster_may_serve(L);
+  const bool pad_U = desc->dtype == KVC_BF16 && !pass && value_side && np != desc->n &&
+                     (desc->n % 8 != 0 || !tma_rows(desc->U));
+  L->theta_np = pad_theta ? np : desc->n;
+  L->U_np = pad_U ? np : desc->n;
+  L->theta_rows = key_side && !pass && np == desc->n ? desc->theta : nullptr;
   L->U_rows = value_side && !pass ? desc->U : nullptr;
-  const bool pad = desc->dtype == KVC_BF16 && !pass && L->np != desc->n;
-  if (!pad) L->np = desc->n;
-  const size_t rows = (size_t)desc->H_kv * m, padded = rows * L->np * sizeof(__nv_bfloat16);
+  const size_t rows = (size_t)desc->H_kv * m, padded = rows * np * sizeof(__nv_bfloat16);
   size_t bytes = 0;
   auto take = [&](size_t b) { const size_t o = bytes; bytes = align_up(bytes + b, 256); return o; };
   const size_t o_idx = take(rows * sizeof(int32_t)), o_status = take(sizeof(int));
   const size_t o_usum = take(!pass && value_side ? rows * sizeof(float) : 0);
-  const size_t o_theta = take(pad && key_side ? padded : 0), o_U = take(pad && value_side ? padded : 0);
+  const size_t o_theta = take(pad_theta ? padded : 0), o_U = take(pad_U ? padded : 0);
   cudaError_t e = cudaGetDevice(&L->device);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&L->num_sms, cudaDevAttrMultiProcessorCount, L->device);
   if (e == cudaSuccess) e = cudaMalloc(&L->d_block, bytes);
@@ -231,12 +234,14 @@ int kvc_layer_create(const kvc_layer_desc* desc, kvc_layer** out) {
     L->d_cstatus = reinterpret_cast<int*>(base + o_status);
     e = cudaMemcpy(L->d_idx, idx.data(), idx.size() * sizeof(int32_t), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemset(L->d_cstatus, 0, sizeof(int));
+    // theta and U may still be on their way on any stream
+    if (e == cudaSuccess && !pass) e = cudaDeviceSynchronize();
     if (e == cudaSuccess && !pass && value_side) {
       L->d_usum = reinterpret_cast<float*>(base + o_usum);
       e = compute_usum(L, L->d_usum);
     }
-    if (e == cudaSuccess && pad && key_side) { L->theta_rows = base + o_theta; e = pad_params(desc->theta, base + o_theta, (long long)rows, desc->n, L->np, nullptr); }
-    if (e == cudaSuccess && pad && value_side) { L->U_rows = base + o_U; e = pad_params(desc->U, base + o_U, (long long)rows, desc->n, L->np, nullptr); }
+    if (e == cudaSuccess && pad_theta) { L->theta_rows = base + o_theta; e = pad_params(desc->theta, base + o_theta, (long long)rows, desc->n, np, nullptr); }
+    if (e == cudaSuccess && pad_U) { L->U_rows = base + o_U; e = pad_params(desc->U, base + o_U, (long long)rows, desc->n, np, nullptr); }
     if (e == cudaSuccess && !pass) e = cudaDeviceSynchronize();
   }
   if (e != cudaSuccess) {

@@ -683,9 +683,8 @@ cluster_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
       const int h = cid / us.nu, lines = a.m * ngrp, step = min(us.nu, a.ucl) * CL_CONS;
       for (int x = (cid - h * us.nu) * CL_CONS + tid; x < lines; x += step) {
         const int row = x / ngrp, c = cg0 + x - row * ngrp;
-        const size_t at = ((size_t)h * a.m + row) * a.np + (size_t)c * 64;
-        prefetch_l2(a.theta + at);
-        prefetch_l2(a.U + at);
+        prefetch_l2(a.theta + ((size_t)h * a.m + row) * a.theta_np + (size_t)c * 64);
+        prefetch_l2(a.U + ((size_t)h * a.m + row) * a.U_np + (size_t)c * 64);
       }
     }
     if (!ragged) grid_dep_wait();
@@ -949,7 +948,7 @@ cluster_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
           constexpr int EB = 4, CWD = 128 / EB;
           const bool last = wp == a.npass - 1;
           unsigned char* stage = sm + (uint32_t)warp * 4096u;
-          unsigned char* wrow = static_cast<unsigned char*>(a.W) + (((size_t)cid * NS + rank) * CL_ROWS + rg * 32) * a.ms * EB;
+          unsigned char* wrow = reinterpret_cast<unsigned char*>(a.W) + (((size_t)cid * NS + rank) * CL_ROWS + rg * 32) * a.ms * EB;
           const int jend = min(a.ms, j0 + a.prow);
           for (int c0 = hf * CWD; j0 + c0 < jend; c0 += CL_GROUPS * CWD) {
 #pragma unroll
@@ -1217,6 +1216,15 @@ int cluster_terms(const kvc_layer* L) {
   return mma ? 1 : 2;
 }
 
+// CTAs a cluster has at least: at most 256 columns each, 128 where P has two terms
+static int cluster_min(const kvc_layer* L) { return ceil_div(ceil_div(L->desc.n, 64), cluster_terms(L) == 2 ? 2 : 4); }
+
+// (what decode_common's rule for the path and plan_cluster say of the handle alone)
+bool cluster_may_serve(const kvc_layer* L) {
+  if (L->desc.dtype != KVC_BF16 || L->passthrough || L->mode != KVC_MODE_KV || cluster_min(L) > CL_MAX_NS) return false;
+  return L->use_tc == 5 || (L->use_tc == 0 && L->desc.n >= 64 && (L->desc.n % 64 == 0 || cluster_terms(L) == 2 || L->G > 1));
+}
+
 static uint32_t cl_tab_bytes(int ns) { return CL_GROUPS * 512u + (uint32_t)ns * 1024u + 256u; }
 // slots of the value ring (a multiple of the groups) in ring_max bytes and the tail of the region of P
 static int cl_v_slots(uint32_t ring_max, uint32_t w_bytes) {
@@ -1241,7 +1249,7 @@ ClusterPlan plan_cluster(const kvc_layer* L, int B, int R, int T, bool ragged) {
   ClusterPlan p{};
   const int G = L->G, n = L->desc.n, m = L->m, H = L->desc.H_kv;
   if (L->desc.dtype != KVC_BF16 || L->passthrough || L->mode != KVC_MODE_KV || R < 1 || B < 1 || G > 16) return p;
-  if (!padded_params_ok(L) || (ragged && B > CL_MAX_RAGGED_B)) return p;
+  if (!tma_rows(L->theta_rows) || !tma_rows(L->U_rows) || (ragged && B > CL_MAX_RAGGED_B)) return p;
   if ((long long)B * R >= (1 << 28) || (long long)B * H * R >= (1ll << 31)) return p;
   const int sms = L->num_sms > 0 ? L->num_sms : 148;
   p.terms = cluster_terms(L);
@@ -1251,8 +1259,7 @@ ClusterPlan plan_cluster(const kvc_layer* L, int B, int R, int T, bool ragged) {
   // CTAs per cluster: at most 256 columns each (128 where P has two terms); more where the smallest number of units still leaves
   // SMs to the text (the chain of a unit gets shorter), as long as every group has two slots for value tiles, whose slices of the
   // weights grow with the ranges (n = 729, 8 sequences, 28/4 heads: 6 CTAs 43.5 us, 8 CTAs with one slot per group 50.3)
-  const int gmax = p.terms == 2 ? 2 : 4;
-  const int ns_min = ceil_div(p.ncg, gmax);
+  const int ns_min = cluster_min(L);
   if (ns_min > CL_MAX_NS) return p;
   const int nu_min = ceil_div(nb, p.rbmax);
   p.NS = ns_min;
@@ -1432,13 +1439,13 @@ cudaError_t launch_cluster(const kvc_layer* L, const DecodeArgs& d, const Cluste
     // theta as (64 columns, m rows, 64-column groups, H_kv): a box lands as [group][64 rows][64]; boxes of ceil and floor(ncg / NS)
     const int groups = x == 0 ? ceil_div(p.ncg, p.NS) : (p.ncg / p.NS > 0 ? p.ncg / p.NS : 1);
     const uint64_t dims[4] = {64ull, (uint64_t)m, (uint64_t)p.ncg, (uint64_t)H};
-    const uint64_t str[3] = {(uint64_t)L->np * 2, 128ull, (uint64_t)m * L->np * 2};
+    const uint64_t str[3] = {(uint64_t)L->theta_np * 2, 128ull, (uint64_t)m * L->theta_np * 2};
     const uint32_t box[4] = {64u, 64u, (uint32_t)groups, 1u};
     if (!encode_tensor_map_bf16(&tm[5 + x], L->theta_rows, 4, dims, str, box)) return cudaSuccess;
   }
   {
-    const uint64_t dims[3] = {(uint64_t)L->np, (uint64_t)m, (uint64_t)H};
-    const uint64_t str[2] = {(uint64_t)L->np * 2, (uint64_t)m * L->np * 2};
+    const uint64_t dims[3] = {(uint64_t)n, (uint64_t)m, (uint64_t)H};           // columns past n are zero-filled
+    const uint64_t str[2] = {(uint64_t)L->U_np * 2, (uint64_t)m * L->U_np * 2};
     const uint32_t box[3] = {64u, (uint32_t)p.brow, 1u};
     if (!encode_tensor_map_bf16(&tm[7], L->U_rows, 3, dims, str, box)) return cudaSuccess;
   }
@@ -1454,10 +1461,11 @@ cudaError_t launch_cluster(const kvc_layer* L, const DecodeArgs& d, const Cluste
   a.q = static_cast<const __nv_bfloat16*>(d.q);
   a.mu = static_cast<const __nv_bfloat16*>(d.mu);
   a.Kc = static_cast<const __nv_bfloat16*>(d.Kc); a.Vc = static_cast<const __nv_bfloat16*>(d.Vc);
-  a.theta = static_cast<const __nv_bfloat16*>(L->theta_rows); a.U = static_cast<const __nv_bfloat16*>(L->U_rows); a.np = L->np;
+  a.theta = static_cast<const __nv_bfloat16*>(L->theta_rows); a.U = static_cast<const __nv_bfloat16*>(L->U_rows);
+  a.theta_np = L->theta_np; a.U_np = L->U_np;
   a.out = static_cast<__nv_bfloat16*>(d.out);
   a.S = reinterpret_cast<__nv_bfloat16*>(ws + w.off_S);
-  a.W = ws + w.off_W;
+  a.W = reinterpret_cast<float*>(ws + w.off_W);
   a.py = reinterpret_cast<float*>(ws + w.off_py);
   a.pml = reinterpret_cast<float2*>(ws + w.off_pml);
   a.tslot0 = (int)w.unit_slots;

@@ -85,10 +85,10 @@ struct ClusterArgs {
   const __nv_bfloat16* q;
   const __nv_bfloat16* mu;
   const __nv_bfloat16 *Kc, *Vc, *theta, *U;      // for L2 prefetches
-  int np;                // pitch of theta and U rows
+  int theta_np, U_np;    // pitches of their rows
   __nv_bfloat16* out;
   __nv_bfloat16* S;      // [ncl][planes][128][ms]
-  void* W;               // [ncl][NS][128][ms] partial weights, fp32 or bf16
+  float* W;              // [ncl][NS][128][ms] partial weights
   float* py;             // [slots][G][D] partials: one per (piece, sequence) of the units, then (from tslot0) [B*H_kv][nct] of the text
   float2* pml;           // [slots][G] (maximum in log2 units, sum)
   int tslot0;

@@ -397,10 +397,10 @@ cudaError_t launch_compress_tc(const kvc_layer* L, const void* K_vis, const void
   CUtensorMap tmU{}, tmV{};
   const bool project = values == 1 && R > 0;
   if (project) {
-    if ((reinterpret_cast<uintptr_t>(L->desc.mu) & 7) || !L->d_usum || !padded_params_ok(L)) return cudaSuccess;
+    if ((reinterpret_cast<uintptr_t>(L->desc.mu) & 7) || !L->d_usum || !tma_rows(L->U_rows)) return cudaSuccess;
     {
       const uint64_t dims[3] = {(uint64_t)n, (uint64_t)m, (uint64_t)H_kv};
-      const uint64_t str[2] = {(uint64_t)L->np * 2, (uint64_t)m * L->np * 2};
+      const uint64_t str[2] = {(uint64_t)L->U_np * 2, (uint64_t)m * L->U_np * 2};
       const uint32_t box[3] = {64u, (uint32_t)CT_BM, 1u};
       if (!encode_tensor_map_bf16(&tmU, L->U_rows, 3, dims, str, box)) return cudaSuccess;
     }

@@ -122,9 +122,10 @@ struct kvc_layer {
   int32_t* d_idx;        // device [H_kv][m]
   int* d_cstatus;        // device status word of the compress kernels (cleared by every kvc_compress call)
   float* d_usum;         // device [H_kv][m] row sums of U (value compression:  U (V - 1 mu^T) = U V - (U 1) mu^T)
-  // theta and U as tensor maps can address them (bf16): [H_kv][m][np].  The caller's own arrays where n is a multiple of 64
-  // (np = n), otherwise zero-padded copies made when the handle is created (np = n rounded up to 64); nullptr where a side has none
-  int np;
+  // theta [H_kv][m][theta_np] and U [H_kv][m][U_np] as the tensor maps read them (bf16): the caller's own arrays where those can be
+  // addressed, otherwise zero-padded copies made when the handle is created (rows of n rounded up to 64).  nullptr: none (a side kept verbatim;
+  // theta of a block length off 64 that the cluster path never serves)
+  int theta_np, U_np;
   const void* theta_rows;
   const void* U_rows;
   void* d_block;         // the one device allocation behind d_idx, d_cstatus, d_usum and the padded copies
@@ -265,10 +266,8 @@ struct RaggedCompress {
   void* K_tail;
   void* V_tail;
 };
-// theta_rows / U_rows can be read by the TMA engine
-inline bool padded_params_ok(const kvc_layer* L) {
-  return ((reinterpret_cast<uintptr_t>(L->theta_rows) | reinterpret_cast<uintptr_t>(L->U_rows)) & 15) == 0;
-}
+inline bool tma_rows(const void* p) { return p && (reinterpret_cast<uintptr_t>(p) & 15) == 0; }      // theta_rows / U_rows the TMA engine can read
+bool cluster_may_serve(const kvc_layer* L);      // some call on the handle may take the cluster path (kvc_cluster.cu)
 cudaError_t pad_params(const void* src, void* dst, long long rows, int n, int np, cudaStream_t st);
 cudaError_t launch_compress_tc(const kvc_layer* L, const void* K_vis, const void* V_vis, int B, int R, long long pitch, int keys,
                                int values, void* Kc, void* Vc, const RaggedCompress* rag, cudaStream_t st, bool* used);
