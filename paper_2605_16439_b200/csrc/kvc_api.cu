@@ -205,6 +205,7 @@ int kvc_layer_create(const kvc_layer_desc* desc, kvc_layer** out) {
   L->d_usum = nullptr;
   L->maps = map_cache_create();
   L->num_sms = 0;
+  std::memset(L->clusters, 0, sizeof(L->clusters));
   {
     const char* ex = std::getenv("KVC_EXPANSION");
     L->use_tc = !ex ? 0 : (std::strcmp(ex, "tcgen05") == 0 ? 1 : (std::strcmp(ex, "pair") == 0 ? 2 : (std::strcmp(ex, "mma") == 0 ? -1 : (std::strcmp(ex, "phases") == 0 ? -2 : (std::strcmp(ex, "split") == 0 ? 3 : (std::strcmp(ex, "resident") == 0 ? 4 : (std::strcmp(ex, "cluster") == 0 ? 5 : 0)))))));
@@ -227,6 +228,7 @@ int kvc_layer_create(const kvc_layer_desc* desc, kvc_layer** out) {
   const size_t o_theta = take(pad_theta ? padded : 0), o_U = take(pad_U ? padded : 0);
   cudaError_t e = cudaGetDevice(&L->device);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&L->num_sms, cudaDevAttrMultiProcessorCount, L->device);
+  if (e == cudaSuccess && cluster_may_serve(L)) cluster_occupancy(L->device, L->num_sms, L->clusters);
   if (e == cudaSuccess) e = cudaMalloc(&L->d_block, bytes);
   if (e == cudaSuccess) {
     char* base = static_cast<char*>(L->d_block);

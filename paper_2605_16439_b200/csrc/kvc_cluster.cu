@@ -1181,31 +1181,31 @@ static const void* cluster_kernel_ptr() { return reinterpret_cast<const void*>(c
 
 constexpr size_t CL_DYN_LIMIT = 231424;       // 227 KB less the barriers
 
-// clusters of ns CTAs the device holds at once (one CTA per SM), asked once per device and size
-static int max_clusters(int device, int sms, int ns) {
-  if (ns == 1) return sms;
+// Clusters of 1 to CL_MAX_NS CTAs the device holds at once (one CTA per SM), asked once per device.  Where the query fails, clusters of that size
+// are not used by the handle, and the next handle asks again: a layout and the launch that fills it always see the same answer.
+void cluster_occupancy(int device, int sms, int* out) {
   static std::mutex mu;
   static int known[16][CL_MAX_NS + 1];
-  if (device < 0 || device >= 16) return sms / ns;
   std::lock_guard<std::mutex> lock(mu);
-  int& k = known[device][ns];
-  if (k > 0) return k;
   const void* fn = cluster_kernel_ptr<1, 1>();
-  int n = 0;
-  if (ensure_dynamic_smem(fn, CL_DYN_LIMIT) == cudaSuccess) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(sms / ns * ns));
-    cfg.blockDim = dim3(CL_THREADS);
-    cfg.dynamicSmemBytes = CL_DYN_LIMIT;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)ns; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    if (cudaOccupancyMaxActiveClusters(&n, fn, &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
+  out[1] = sms;
+  for (int ns = 2; ns <= CL_MAX_NS; ++ns) {
+    int n = device >= 0 && device < 16 ? known[device][ns] : 0;
+    if (n == 0 && ensure_dynamic_smem(fn, CL_DYN_LIMIT) == cudaSuccess) {
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3((unsigned)(sms / ns * ns));
+      cfg.blockDim = dim3(CL_THREADS);
+      cfg.dynamicSmemBytes = CL_DYN_LIMIT;
+      cudaLaunchAttribute attr[1];
+      attr[0].id = cudaLaunchAttributeClusterDimension;
+      attr[0].val.clusterDim.x = (unsigned)ns; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+      cfg.attrs = attr;
+      cfg.numAttrs = 1;
+      if (cudaOccupancyMaxActiveClusters(&n, fn, &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
+    }
+    if (n > 0 && device >= 0 && device < 16) known[device][ns] = n;
+    out[ns] = n;
   }
-  k = n > 0 ? n : 1;
-  return k;
 }
 
 // How the scores and probabilities are carried: as one bf16 term, or, where n is no multiple of 8 or a score row is too long for the
@@ -1251,7 +1251,6 @@ ClusterPlan plan_cluster(const kvc_layer* L, int B, int R, int T, bool ragged) {
   if (L->desc.dtype != KVC_BF16 || L->passthrough || L->mode != KVC_MODE_KV || R < 1 || B < 1 || G > 16) return p;
   if (!tma_rows(L->theta_rows) || !tma_rows(L->U_rows) || (ragged && B > CL_MAX_RAGGED_B)) return p;
   if ((long long)B * R >= (1 << 28) || (long long)B * H * R >= (1ll << 31)) return p;
-  const int sms = L->num_sms > 0 ? L->num_sms : 148;
   p.terms = cluster_terms(L);
   p.ncg = ceil_div(n, 64);
   p.rbmax = CL_ROWS / G;
@@ -1268,8 +1267,9 @@ ClusterPlan plan_cluster(const kvc_layer* L, int B, int R, int T, bool ragged) {
                       ((uint32_t)(ns * G * 256) + 127u) & ~127u);
   };
   for (int ns = p.ncg < CL_MAX_NS ? p.ncg : CL_MAX_NS; ns > ns_min; --ns)
-    if ((long long)H * nu_min * 100 <= (long long)max_clusters(L->device, sms, ns) * 87 && v_slots(ns) >= 2 * CL_GROUPS) { p.NS = ns; break; }
-  p.ncl = max_clusters(L->device, sms, p.NS);
+    if ((long long)H * nu_min * 100 <= (long long)L->clusters[ns] * 87 && v_slots(ns) >= 2 * CL_GROUPS) { p.NS = ns; break; }
+  p.ncl = L->clusters[p.NS];
+  if (p.ncl < 1) return p;
   const double kv = 2.0 * nb * m * D * 2 * H + 4.0 * H * m * n, tx = 2.0 * B * H * (double)T * D * 2;
   p.cap = (int)(p.ncl * (kv / (kv + tx)) / H);
   if (p.cap < 1) p.cap = 1;
@@ -1359,10 +1359,10 @@ ClusterPlan plan_cluster(const kvc_layer* L, int B, int R, int T, bool ragged) {
 ClusterWs cluster_ws(const kvc_layer* L, const ClusterPlan& p, int B, int R) {
   (void)R;
   ClusterWs w{};
-  const int H = L->desc.H_kv, G = L->G, sms = L->num_sms > 0 ? L->num_sms : 148;
+  const int H = L->desc.H_kv, G = L->G;
   size_t off = align_up(sizeof(int) * ((size_t)B * H + 1), 256);       // behind the status word of the layout all paths share
   auto take = [&](size_t bytes) { const size_t o = off; off = align_up(off + bytes, 256); return o; };
-  const size_t ncl = (size_t)max_clusters(L->device, sms, p.NS), slots = (size_t)H * ((size_t)p.nu_max * CL_GROUPS * p.NS + B);
+  const size_t ncl = (size_t)L->clusters[p.NS], slots = (size_t)H * ((size_t)p.nu_max * CL_GROUPS * p.NS + B);
   w.off_S = take(sizeof(__nv_bfloat16) * ncl * p.terms * CL_ROWS * p.ms);
   w.off_W = take(sizeof(float) * ncl * p.NS * CL_ROWS * p.ms);
   w.off_cnt = take(sizeof(unsigned long long) * (size_t)B * H);
@@ -1410,7 +1410,7 @@ cudaError_t launch_cluster(const kvc_layer* L, const DecodeArgs& d, const Cluste
   *encoded = false;
   const int B = d.B, H = d.H_kv, R = d.R, G = d.G, m = L->m, n = L->desc.n;
   const ClusterWs w = cluster_ws(L, p, B, R);
-  const int ncl = max_clusters(L->device, L->num_sms > 0 ? L->num_sms : 148, p.NS);
+  const int ncl = L->clusters[p.NS];
   const int planes = p.terms;
   CUtensorMap tm[9];
   {

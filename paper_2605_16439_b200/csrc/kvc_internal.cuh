@@ -116,6 +116,7 @@ struct kvc_layer {
   int passthrough;       // ratio_permille == 0
   int device;
   int num_sms;
+  int clusters[9];       // clusters of 1 to 8 CTAs of the cluster decode kernel the device holds at once (0: not to be used)
   int use_tc;            // expansions of the one-kernel decode path: 0 chosen per shape, 1 tcgen05, 2 tcgen05 in pairs of CTAs,
                          // -1 mma.sync; -2 three-phase kernels, 3 three-kernel path, 4 resident parameters, 5 clusters (environment
                          // KVC_EXPANSION=tcgen05 | pair | mma | phases | split | resident | cluster when the handle is created)
@@ -267,6 +268,7 @@ struct RaggedCompress {
   void* V_tail;
 };
 inline bool tma_rows(const void* p) { return p && (reinterpret_cast<uintptr_t>(p) & 15) == 0; }      // theta_rows / U_rows the TMA engine can read
+void cluster_occupancy(int device, int sms, int* out);      // kvc_layer.clusters
 bool cluster_may_serve(const kvc_layer* L);      // some call on the handle may take the cluster path (kvc_cluster.cu)
 cudaError_t pad_params(const void* src, void* dst, long long rows, int n, int np, cudaStream_t st);
 cudaError_t launch_compress_tc(const kvc_layer* L, const void* K_vis, const void* V_vis, int B, int R, long long pitch, int keys,
