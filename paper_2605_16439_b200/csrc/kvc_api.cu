@@ -472,7 +472,7 @@ int decode_common(const kvc_layer* L, const void* q, const void* capsules, int B
 
   if ((align & 15) == 0 && use_cluster(L, B, R, T, ragged)) {
     const ClusterPlan cp = plan_cluster(L, B, R, T, ragged);
-    if (cp.ok && (ws_limit == 0 || cluster_ws(L, cp, B, R).bytes <= ws_limit)) {
+    if (cp.ok && (ws_limit == 0 || cluster_ws(L, cp, B).bytes <= ws_limit)) {
       bool encoded = false;
       const cudaError_t ce = launch_cluster(L, a, cp, ws, st, &encoded);
       if (encoded) return cuda_status(ce);

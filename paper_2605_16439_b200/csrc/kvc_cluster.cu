@@ -761,7 +761,7 @@ cluster_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
         const uint32_t sm_u = (uint32_t)fresh((int)smem_addr(sm)), ring_u = sm_u + CL_P_BYTES;
         uint32_t qa[8][4];
         int cur_b = -1;
-        __nv_bfloat16* S0 = a.S + (size_t)cid * PL * CL_ROWS * a.ms;
+        __nv_bfloat16* S0 = a.S + (size_t)cid * PL * a.srows * a.ms;
         const int t0 = rank + grp * NS;
         int bl = t0 / a.vt, jt = t0 - bl * a.vt;
         BlockWalk bw;
@@ -810,7 +810,7 @@ cluster_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
                     const float v1 = (cc[0][nt][2 * hh + 1] + cc[1][nt][2 * hh + 1]) * CL_QSCALE;
                     const uint32_t hi = pack2_bf16(v0, v1);
                     *reinterpret_cast<uint32_t*>(row + j) = hi;
-                    if (PL == 2) *reinterpret_cast<uint32_t*>(row + (size_t)CL_ROWS * a.ms + j) = split_lo(v0, v1, hi);
+                    if (PL == 2) *reinterpret_cast<uint32_t*>(row + (size_t)a.srows * a.ms + j) = split_lo(v0, v1, hi);
                   }
                 }
               }
@@ -948,7 +948,7 @@ cluster_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
           constexpr int EB = 4, CWD = 128 / EB;
           const bool last = wp == a.npass - 1;
           unsigned char* stage = sm + (uint32_t)warp * 4096u;
-          unsigned char* wrow = reinterpret_cast<unsigned char*>(a.W) + (((size_t)cid * NS + rank) * CL_ROWS + rg * 32) * a.ms * EB;
+          unsigned char* wrow = reinterpret_cast<unsigned char*>(a.W) + (((size_t)cid * NS + rank) * a.srows + rg * 32) * a.ms * EB;
           const int jend = min(a.ms, j0 + a.prow);
           for (int c0 = hf * CWD; j0 + c0 < jend; c0 += CL_GROUPS * CWD) {
 #pragma unroll
@@ -1245,6 +1245,19 @@ static int text_chunk(const kvc_layer* L, int B, int T) {
   return T <= most * CL_TEXT_CHUNK ? CL_TEXT_CHUNK : (int)align_up((size_t)ceil_div(T, most), 16);
 }
 
+// Most units of a KV head and most blocks of a unit.  Uniform calls: their split.  With lengths per sequence fewer blocks than nb may split into
+// more units (5 blocks into 5, but 8 into 4 of 2): clusters for all that the cap allows (else the odd ones take a second round: 38 us instead
+// of 21 at 4 x 2 blocks of n = 400, 8/2 heads), of no more blocks than nb over the cap.
+static UnitSplit most_units(int nb, int rbmax, int cap, bool ragged) {
+  UnitSplit us = split_units(nb, rbmax, cap);
+  if (!ragged || nb <= 0) return us;
+  us.rb = std::min(rbmax, ceil_div(nb, cap < nb ? cap : nb));
+  if (cap < nb && cap > us.nu) us.nu = cap;
+  return us;
+}
+// expansion rows a unit of rb blocks has room for (a multiple of 8: the second term of S starts on a swizzle period)
+static int unit_rows(int rb, int G) { return (int)align_up((size_t)(rb * G < CL_ROWS ? rb * G : CL_ROWS), 8); }
+
 ClusterPlan plan_cluster(const kvc_layer* L, int B, int R, int T, bool ragged) {
   ClusterPlan p{};
   const int G = L->G, n = L->desc.n, m = L->m, H = L->desc.H_kv;
@@ -1279,10 +1292,8 @@ ClusterPlan plan_cluster(const kvc_layer* L, int B, int R, int T, bool ragged) {
     if (p.nu_max < 1) p.nu_max = 1;
   }
   const UnitSplit us = split_units(nb, p.rbmax, p.cap);
-  // fewer blocks than the plan's may split into more units (5 blocks into 5, but 8 into 4 of 2): with lengths per sequence, clusters for
-  // all that the cap allows (else the odd ones take a second round: 38 us instead of 21 at 4 x 2 blocks of n = 400, 8/2 heads)
-  const int nu_most = ragged && p.cap < nb && p.cap > us.nu ? p.cap : us.nu;
-  p.ucl = (long long)H * nu_most < p.ncl ? H * nu_most : p.ncl;
+  const UnitSplit most = most_units(nb, p.rbmax, p.cap, ragged);
+  p.ucl = (long long)H * most.nu < p.ncl ? H * most.nu : p.ncl;
   p.ms = (m + 7) & ~7;
   p.nk1 = ceil_div(m, 64);
   const int mpad = (m + 15) & ~15;
@@ -1293,10 +1304,7 @@ ClusterPlan plan_cluster(const kvc_layer* L, int B, int R, int T, bool ragged) {
   if (p.npass == 1) p.prow = p.nbox * p.brow;
   p.vt = ceil_div(m, CL_TILE);
   const int planes = p.terms;
-  {
-    const int rows = us.rb * G < CL_ROWS ? us.rb * G : CL_ROWS;
-    p.srows = ragged ? CL_ROWS : (int)align_up((size_t)rows, 8);
-  }
+  p.srows = unit_rows(most.rb, G);
   p.s_bytes = (uint32_t)planes * p.srows * 128u;
   const uint32_t th = (uint32_t)ceil_div(p.ncg, p.NS) * 8192u, ub = (uint32_t)p.brow * 128u;
   p.x_bytes = p.s_bytes + th;
@@ -1349,31 +1357,32 @@ ClusterPlan plan_cluster(const kvc_layer* L, int B, int R, int T, bool ragged) {
   }
   // a CTA's list of the pairs it merges after its text items holds as many as it can have items
   const long long with = (long long)p.ucl * p.NS, without = (long long)(p.ncl - p.ucl) * p.NS;
-  const long long most = std::max((p.text_items - p.text_ded + with - 1) / with, without > 0 ? (p.text_ded + without - 1) / without : 0ll);
-  if (most > (long long)(CL_GROUPS * 512u + (uint32_t)p.NS * 1024u) / 4 - 1) return p;
+  const long long items = std::max((p.text_items - p.text_ded + with - 1) / with, without > 0 ? (p.text_ded + without - 1) / without : 0ll);
+  if (items > (long long)(CL_GROUPS * 512u + (uint32_t)p.NS * 1024u) / 4 - 1) return p;
   p.units = H * us.nu;
   p.ok = 1;
   return p;
 }
 
-ClusterWs cluster_ws(const kvc_layer* L, const ClusterPlan& p, int B, int R) {
-  (void)R;
+// rows: of S and of the partial weights, of all clusters that take units
+static ClusterWs cluster_layout(const kvc_layer* L, const ClusterPlan& p, int B, int rows) {
   ClusterWs w{};
   const int H = L->desc.H_kv, G = L->G;
   size_t off = align_up(sizeof(int) * ((size_t)B * H + 1), 256);       // behind the status word of the layout all paths share
   auto take = [&](size_t bytes) { const size_t o = off; off = align_up(off + bytes, 256); return o; };
-  const size_t ncl = (size_t)L->clusters[p.NS], slots = (size_t)H * ((size_t)p.nu_max * CL_GROUPS * p.NS + B);
-  w.off_S = take(sizeof(__nv_bfloat16) * ncl * p.terms * CL_ROWS * p.ms);
-  w.off_W = take(sizeof(float) * ncl * p.NS * CL_ROWS * p.ms);
+  w.off_S = take(sizeof(__nv_bfloat16) * (size_t)rows * p.terms * p.ms);
+  w.off_W = take(sizeof(float) * (size_t)rows * p.NS * p.ms);
   w.off_cnt = take(sizeof(unsigned long long) * (size_t)B * H);
-  w.unit_slots = slots;
-  const size_t all = slots + (size_t)B * H * p.nct;
+  w.unit_slots = (size_t)H * ((size_t)p.nu_max * CL_GROUPS * p.NS + B);
+  const size_t all = w.unit_slots + (size_t)B * H * p.nct;
   w.off_py = take(sizeof(float) * all * G * D);
   w.off_pml = take(sizeof(float2) * all * G);
   w.bytes = off;
   return w;
 }
+ClusterWs cluster_ws(const kvc_layer* L, const ClusterPlan& p, int B) { return cluster_layout(L, p, B, p.ucl * p.srows); }
 
+// enough for every T <= T_cap: shorter text leaves more clusters to the units (never more than without any), which then have fewer rows each
 size_t cluster_ws_bytes(const kvc_layer* L, int B, int R, int T_cap) {
   size_t most = 0;
   for (int ragged = 0; ragged < 2; ++ragged) {
@@ -1381,8 +1390,13 @@ size_t cluster_ws_bytes(const kvc_layer* L, int B, int R, int T_cap) {
     if (!p.ok) continue;
     // the chunks of a shorter text: never more than the most of a pair, nor than whole chunks of the smallest size
     p.nct = std::min(ceil_div(T_cap, CL_TEXT_CHUNK), text_items(L, B));
-    const size_t b = cluster_ws(L, p, B, R).bytes;
-    most = b > most ? b : most;
+    const int top = plan_cluster(L, B, R, 0, ragged != 0).cap;
+    int rows = 0;
+    for (int cap = 1; cap <= top; ++cap) {
+      const UnitSplit us = most_units(B * R, p.rbmax, cap, ragged != 0);
+      rows = std::max(rows, std::min(L->desc.H_kv * us.nu, L->clusters[p.NS]) * unit_rows(us.rb, L->G));
+    }
+    most = std::max(most, cluster_layout(L, p, B, rows).bytes);
   }
   return most;
 }
@@ -1409,8 +1423,7 @@ static cudaError_t launch_cluster_inst(const CUtensorMap* tm, const ClusterArgs&
 cudaError_t launch_cluster(const kvc_layer* L, const DecodeArgs& d, const ClusterPlan& p, char* ws, cudaStream_t st, bool* encoded) {
   *encoded = false;
   const int B = d.B, H = d.H_kv, R = d.R, G = d.G, m = L->m, n = L->desc.n;
-  const ClusterWs w = cluster_ws(L, p, B, R);
-  const int ncl = L->clusters[p.NS];
+  const ClusterWs w = cluster_ws(L, p, B);
   const int planes = p.terms;
   CUtensorMap tm[9];
   {
@@ -1430,8 +1443,8 @@ cudaError_t launch_cluster(const kvc_layer* L, const DecodeArgs& d, const Cluste
     tm[3] = tm[0];
   }
   {
-    const uint64_t dims[4] = {(uint64_t)m, (uint64_t)CL_ROWS, (uint64_t)planes, (uint64_t)ncl};
-    const uint64_t str[3] = {(uint64_t)p.ms * 2, (uint64_t)CL_ROWS * p.ms * 2, (uint64_t)planes * CL_ROWS * p.ms * 2};
+    const uint64_t dims[4] = {(uint64_t)m, (uint64_t)p.srows, (uint64_t)planes, (uint64_t)p.ucl};
+    const uint64_t str[3] = {(uint64_t)p.ms * 2, (uint64_t)p.srows * p.ms * 2, (uint64_t)planes * p.srows * p.ms * 2};
     const uint32_t box[4] = {64u, (uint32_t)p.srows, (uint32_t)planes, 1u};
     if (!encode_tensor_map_bf16(&tm[4], ws + w.off_S, 4, dims, str, box)) return cudaSuccess;
   }
@@ -1450,8 +1463,8 @@ cudaError_t launch_cluster(const kvc_layer* L, const DecodeArgs& d, const Cluste
     if (!encode_tensor_map_bf16(&tm[7], L->U_rows, 3, dims, str, box)) return cudaSuccess;
   }
   {
-    const uint64_t dims[4] = {(uint64_t)p.ms, (uint64_t)CL_ROWS, (uint64_t)p.NS, (uint64_t)ncl};
-    const uint64_t str[3] = {(uint64_t)p.ms * 4, (uint64_t)CL_ROWS * p.ms * 4, (uint64_t)p.NS * CL_ROWS * p.ms * 4};
+    const uint64_t dims[4] = {(uint64_t)p.ms, (uint64_t)p.srows, (uint64_t)p.NS, (uint64_t)p.ucl};
+    const uint64_t str[3] = {(uint64_t)p.ms * 4, (uint64_t)p.srows * p.ms * 4, (uint64_t)p.NS * p.srows * p.ms * 4};
     const uint32_t box_ld[4] = {64u, (uint32_t)G, (uint32_t)p.NS, 1u};
     const bool ok = encode_tensor_map_f32(&tm[8], ws + w.off_W, 4, dims, str, box_ld, false);
     if (!ok) return cudaSuccess;

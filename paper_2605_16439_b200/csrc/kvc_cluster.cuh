@@ -47,7 +47,7 @@ struct ClusterPlan {
   int nk1;               // 64-row chunks of the m axis
   int npass, prow, nbox, brow;   // passes over the weights (<= 512 columns each), boxes of brow rows of U
   int vt;                // 64-row tiles per block
-  int srows;             // rows of S loaded per chunk
+  int srows;             // expansion rows of a unit: rows of S and W in the workspace, and of S loaded per chunk
   int nK, nX, nV;        // slots of the key ring, the expansion ring and the value ring
   int nwp;                                             // weight slices of the value ring kept in the region of P
   uint32_t x_bytes, s_bytes, w_off, w_bytes, w_tx;     // slot sizes (w_tx: bytes of a slice); the value ring's weights lie behind its tiles
@@ -77,7 +77,7 @@ __host__ __device__ __forceinline__ UnitSplit split_units(int nb, int rbmax, int
 
 int cluster_terms(const kvc_layer* L);                 // bf16 terms of the scores and probabilities (1, 2)
 ClusterPlan plan_cluster(const kvc_layer* L, int B, int R, int T, bool ragged);
-ClusterWs cluster_ws(const kvc_layer* L, const ClusterPlan& p, int B, int R);
+ClusterWs cluster_ws(const kvc_layer* L, const ClusterPlan& p, int B);
 size_t cluster_ws_bytes(const kvc_layer* L, int B, int R, int T_cap);     // for uniform and ragged calls alike; 0 if the path never applies
 cudaError_t launch_cluster(const kvc_layer* L, const DecodeArgs& a, const ClusterPlan& p, char* ws, cudaStream_t st, bool* encoded);
 
@@ -87,8 +87,8 @@ struct ClusterArgs {
   const __nv_bfloat16 *Kc, *Vc, *theta, *U;      // for L2 prefetches
   int theta_np, U_np;    // pitches of their rows
   __nv_bfloat16* out;
-  __nv_bfloat16* S;      // [ncl][planes][128][ms]
-  float* W;              // [ncl][NS][128][ms] partial weights
+  __nv_bfloat16* S;      // [ucl][planes][srows][ms]
+  float* W;              // [ucl][NS][srows][ms] partial weights
   float* py;             // [slots][G][D] partials: one per (piece, sequence) of the units, then (from tslot0) [B*H_kv][nct] of the text
   float2* pml;           // [slots][G] (maximum in log2 units, sum)
   int tslot0;

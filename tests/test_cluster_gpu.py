@@ -136,3 +136,44 @@ def test_odd_block_lengths_take_the_faster_path(H_q, H_kv, B, R, grid, T, ratio,
     counts, (_, _, _, out) = tl.launches(lambda: tl.gpu_run(shape, p))
     assert counts["scores"] == (0 if cluster else 1)
     tl.assert_close(tl.np64(out), tl.oracle_run(shape, p, "fused")[2], "bf16")
+
+
+@pytest.mark.parametrize("B,H_q,H_kv,grid,R,ratio", [(8, 28, 4, 27, 5, 600), (3, 16, 1, 11, 9, 800), (5, 8, 2, 20, 3, 300), (40, 14, 2, 9, 1, 600)])
+def test_workspace_holds_every_shorter_text(B, H_q, H_kv, grid, R, ratio, monkeypatch):
+    """A workspace of kvc_workspace_bytes(.., T_cap) serves every T <= T_cap, whatever the split of the clusters between units and text:
+    nothing behind it is written."""
+    monkeypatch.setenv("KVC_EXPANSION", "cluster")
+    T_cap = 3000
+    shape = wl.Shape("cluster-ws", 1, B, H_q, H_kv, 128, grid, R, T_cap, 1, "bf16", ratio)
+    p = tl.make_problem(shape, 870 + grid, T=T_cap, T_cap=T_cap)
+    layer = tl.gpu_layer(shape, p)
+    caps = kvc.alloc_capsules(layer, B, R)
+    kvc.kvc_compress(layer, p["K_vis"].to(DEV), p["V_vis"].to(DEV), B, R, caps)
+    need = kvc.kvc_workspace_bytes(layer, B, R, T_cap)
+    ws = torch.full((need + (8 << 20),), 0xA5, dtype=torch.uint8, device=DEV)
+    q, K_txt, V_txt = p["q"].to(DEV), p["K_txt"].to(DEV), p["V_txt"].to(DEV)
+    out = torch.empty((B, H_q, 128), dtype=torch.bfloat16, device=DEV)
+    full = torch.full((B,), R, dtype=torch.int32, device=DEV)
+    for T in (0, 1, 100, 700, 2048, 2049, T_cap):
+        counts, _ = tl.launches(lambda: kvc.kvc_decode_attend(layer, q, caps, B, R, K_txt, V_txt, T, T_cap, out, ws))
+        assert counts["fused"] == 1
+        kvc.kvc_decode_attend_ragged(layer, q, caps, B, R, full, K_txt, V_txt, T, None, T_cap, out, ws)
+        torch.cuda.synchronize()
+        assert kvc.kvc_read_device_status(layer, B, R, T, ws) == 0
+        assert bool((ws[need:] == 0xA5).all()), T
+
+
+def test_static_entry_point_takes_the_cluster_path():
+    """8 x 5 blocks of n = 729: the workspace of the call itself fits the fixed scratch."""
+    shape = wl.Shape("cluster-static", 1, 8, 28, 4, 128, 27, 5, 300, 1, "bf16", 600)
+    p = tl.make_problem(shape, 890, T=300, T_cap=300, recipe="peaked")
+    layer = tl.gpu_layer(shape, p)
+    caps = kvc.alloc_capsules(layer, 8, 5)
+    kvc.kvc_compress(layer, p["K_vis"].to(DEV), p["V_vis"].to(DEV), 8, 5, caps)
+    out = torch.full((8, 28, 128), float("nan"), dtype=torch.bfloat16, device=DEV)
+    run = lambda: kvc.kvc_decode_attend_static(layer, p["q"].to(DEV), caps, 8, 5, p["K_txt"].to(DEV), p["V_txt"].to(DEV), 300, 300, out)
+    run()
+    counts, _ = tl.launches(run)
+    assert counts["fused"] == 1 and counts["scores"] == 0
+    assert kvc.kvc_workspace_bytes(layer, 8, 5, 300) <= kvc.kvc_static_scratch_bytes()
+    tl.assert_close(tl.np64(out), tl.oracle_run(shape, p, "fused")[2], "bf16")
