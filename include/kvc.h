@@ -214,9 +214,10 @@ KVC_API int kvc_attend_full(const kvc_layer* layer, const void* q, const void* K
  * that cannot allocate where they decode: an engine whose memory pool is fully committed to KV
  * blocks, code running under an allocator it does not own, or a loop in which an allocation's
  * implicit device synchronisation is unacceptable.
- *   - Limit: the shape must need at most KVC_STATIC_SCRATCH_BYTES of scratch (what
- *     kvc_workspace_bytes(layer, B, R, T) reports); larger shapes return KVC_ERR_WORKSPACE
- *     ("workspace ...: static scratch too small") and nothing is launched.
+ *   - Limit: a shape whose kvc_workspace_bytes(layer, B, R, T) is at most KVC_STATIC_SCRATCH_BYTES is
+ *     always taken.  That figure also covers calls with per-sequence lengths and the fastest path; a
+ *     larger shape may be taken where only those need more (a slower path then serves it).  Otherwise
+ *     KVC_ERR_WORKSPACE ("workspace ...: static scratch too small"), and nothing is launched.
  *   - The array costs KVC_STATIC_SCRATCH_BYTES of device memory on every GPU that loads the
  *     library, for the life of the process.
  *   - The first call on each device looks up the array's device address (with that device

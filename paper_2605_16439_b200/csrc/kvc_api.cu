@@ -18,7 +18,7 @@ namespace kvc {
 
 static size_t elem_bytes(int dtype) { return dtype == KVC_BF16 ? 2 : 4; }
 
-WsLayout ws_layout(const kvc_layer* L, int B, int R, int T_cap) {
+WsLayout ws_layout(const kvc_layer* L, int B, int R, int T_cap, int forms) {
   WsLayout w{};
   const int H_kv = L->desc.H_kv, G = L->G, n = L->desc.n;
   const int ms = (L->mk + 15) / 16 * 16, msv = (L->mv + 15) / 16 * 16;
@@ -90,6 +90,7 @@ WsLayout ws_layout(const kvc_layer* L, int B, int R, int T_cap) {
     size_t np = 0;
     if (B > 0 && R > 0) {
       for (int ragged = 0; ragged < 2; ++ragged) {
+        if (!(forms & (ragged ? WS_RAGGED : WS_UNIFORM))) continue;
         const FusedPlan fp = plan_fused(L, B, R, ragged != 0);
         if (fp.ok && L->mode == KVC_MODE_KV && fp.nrg > 1) np = std::max(np, (size_t)B * H_kv * fp.nrg * G);
       }
@@ -291,7 +292,7 @@ size_t kvc_capsule_bytes(const kvc_layer* L, int B, int R) {
 
 size_t kvc_workspace_bytes(const kvc_layer* L, int B, int R, int T_cap) {
   if (!L || B < 0 || R < 0 || T_cap < 0) return 0;
-  const size_t phases = ws_layout(L, B, R, T_cap).total, cluster = cluster_ws_bytes(L, B, R, T_cap);
+  const size_t phases = ws_layout(L, B, R, T_cap, WS_UNIFORM | WS_RAGGED).total, cluster = cluster_ws_bytes(L, B, R, T_cap);
   const size_t most = phases > cluster ? phases : cluster;
   const size_t plain = (R == 0 || L->passthrough) && L->desc.dtype == KVC_BF16 && B > 0 ? plain_ws(L, B).bytes : 0;
   return most > plain ? most : plain;
@@ -489,7 +490,7 @@ int decode_common(const kvc_layer* L, const void* q, const void* capsules, int B
     }
   }
 
-  a.ws = ws_layout(L, B, R, T);
+  a.ws = ws_layout(L, B, R, T, ragged ? WS_RAGGED : WS_UNIFORM);
   a.Ts = a.ws.Ts;
   a.S = reinterpret_cast<float*>(ws + a.ws.off_S);
   a.Sb = reinterpret_cast<__nv_bfloat16*>(ws + a.ws.off_S);

@@ -135,7 +135,9 @@ struct kvc_layer {
 
 namespace kvc {
 
-WsLayout ws_layout(const kvc_layer* L, int B, int R, int T_cap);
+// regions of the paths behind decode_common's first two (the fused one differs for calls with per-sequence lengths)
+enum { WS_UNIFORM = 1, WS_RAGGED = 2 };
+WsLayout ws_layout(const kvc_layer* L, int B, int R, int T_cap, int forms = WS_UNIFORM);
 int cuda_status(cudaError_t e);   // KVC_OK or KVC_ERR_CUDA, remembering the error for kvc_last_cuda_error
 FusedPlan plan_fused(const kvc_layer* L, int B, int R, bool ragged = false);
 FusedPlan plan_fused_tc(const kvc_layer* L, int B, int R);     // tensor-memory variant; ok == 0 if the shape does not fit it
