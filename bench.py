@@ -559,12 +559,12 @@ def measure(shape, config_index, dev, rank, world, local, steps, warmup, profile
     # per-kernel durations: the same steps again with every launch bracketed by two CUDA events on the launching
     # stream (the brackets sit between the kernels, so the programmatic overlap of consecutive kernels is off in this
     # pass and the pass is a little slower than the timed region above)
-    prof, ms_bracketed = {}, None
+    prof, parts, ms_bracketed = {}, {}, None
     if profile:
         kvc.kvc_profile_start(steps * (5 * calls + 2 * shape.layers))
         ms_bracketed = timed(job.step, steps, dev) / steps
         kvc.kvc_profile_stop()
-        prof = kvc.kvc_profile_read()
+        prof, parts = kvc.kvc_profile_read(), kvc.kvc_profile_parts()
         kvc.kvc_profile_start(0)
         kvc.kvc_profile_stop()
         job.launches = int(sum(v[1] for v in prof.values())) // max(steps, 1) * steps
@@ -585,6 +585,9 @@ def measure(shape, config_index, dev, rank, world, local, steps, warmup, profile
             if n:
                 kernels[k] = {"launches": n, "total_ms": round(t, 3), "avg_us": round(t / n * 1e3, 3),
                               "share": round(t / tot, 4)}
+        for k, (t, n) in parts.items():         # kernels that a name above covers among others
+            if n:
+                kernels[k] = {"launches": n, "total_ms": round(t, 3), "avg_us": round(t / n * 1e3, 3), "counted_above": True}
         dom = max(decode_kernels, key=lambda k: prof.get(k, (0.0, 0))[0])
         t_dom, n_dom = prof[dom]
         if dom in ("fused", "fused_tc", "fused_pair", "resident"):

@@ -300,7 +300,11 @@ typedef enum {
   KVC_KERNEL_SPLIT_EXPAND = 11,   /* its steps 2-3 on tcgen05, per 128 expansion rows and range of the n axis; the text rows on idle SMs */
   KVC_KERNEL_SPLIT_OUTPUT = 12,   /* its step 4 and the normalisation, one pass over V_tilde, merged with the text partials */
   KVC_KERNEL_RESIDENT = 13,       /* one-kernel bf16 path for short blocks whose theta and U stay in shared memory */
-  KVC_KERNEL_COUNT = 14
+  KVC_KERNEL_COUNT = 14,          /* the ids up to here share the launches out; the next ones name some of them once more: */
+  KVC_KERNEL_CLUSTER = 14,        /* of FUSED: the kernel of CTA clusters that share the n axis */
+  KVC_KERNEL_PLAIN = 15,          /* of FUSED: attention over rows stored verbatim */
+  KVC_KERNEL_COMPRESS = 16,       /* of PROJECT_VALUES (GATHER_KEYS where no side is projected): the one-kernel bf16 compression */
+  KVC_KERNEL_ID_END = 17
 } kvc_kernel_id;
 KVC_API int kvc_profile_start(int max_launches);
 KVC_API int kvc_profile_stop(void);

@@ -304,6 +304,7 @@ def capsule_views(layer: Layer, capsules, B: int, R: int):
 
 
 KVC_KERNEL_COUNT = 14
+KVC_KERNEL_ID_END = 17
 
 
 def kvc_profile_start(max_launches: int) -> None:
@@ -314,11 +315,20 @@ def kvc_profile_stop() -> None:
     _check(_lib().kvc_profile_stop(), "kvc_profile_stop")
 
 
-def kvc_profile_read() -> dict:
-    """{kernel name: (total_ms, launches)} of the bracketed launches; synchronise the stream first."""
+def _profile(ids) -> dict:
     out = {}
-    for k in range(KVC_KERNEL_COUNT):
+    for k in ids:
         ms, n = C.c_double(), C.c_longlong()
         _check(_lib().kvc_profile_read(k, C.byref(ms), C.byref(n)), "kvc_profile_read")
         out[_lib().kvc_kernel_name(k).decode()] = (ms.value, n.value)
     return out
+
+
+def kvc_profile_read() -> dict:
+    """{kernel name: (total_ms, launches)} of the bracketed launches; synchronise the stream first."""
+    return _profile(range(KVC_KERNEL_COUNT))
+
+
+def kvc_profile_parts() -> dict:
+    """The same for the kernels that kvc_profile_read counts among others (cluster and plain under fused, compress under project_values)."""
+    return _profile(range(KVC_KERNEL_COUNT, KVC_KERNEL_ID_END))

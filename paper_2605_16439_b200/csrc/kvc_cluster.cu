@@ -1490,7 +1490,7 @@ cudaError_t launch_cluster(const kvc_layer* L, const DecodeArgs& d, const Cluste
   a.x_bytes = p.x_bytes; a.s_bytes = p.s_bytes; a.w_off = p.w_off; a.w_bytes = p.w_bytes; a.w_tx = p.w_tx; a.nwp = p.nwp;
   a.tab_off = p.tab_off; a.pre_off = p.pre_off;
   a.tc = p.tc; a.nct = p.nct; a.text_items = (int)p.text_items; a.text_ded = (int)p.text_ded;
-  ProfScope prof(KVC_KERNEL_FUSED, st);
+  ProfScope prof(KVC_KERNEL_FUSED, st, KVC_KERNEL_CLUSTER);
   if (G > 8)
     return p.terms == 1 ? launch_cluster_inst<2, 1>(tm, a, p, st) : launch_cluster_inst<2, 2>(tm, a, p, st);
   return p.terms == 1 ? launch_cluster_inst<1, 1>(tm, a, p, st) : launch_cluster_inst<1, 2>(tm, a, p, st);

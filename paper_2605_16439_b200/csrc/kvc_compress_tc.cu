@@ -447,7 +447,7 @@ cudaError_t launch_compress_tc(const kvc_layer* L, const void* K_vis, const void
   const size_t smem = (size_t)a.stages * a.stage_bytes + fixed;
   cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(compress_kernel), smem);
   if (e != cudaSuccess) return e;
-  ProfScope prof(project ? KVC_KERNEL_PROJECT_VALUES : KVC_KERNEL_GATHER_KEYS, st);
+  ProfScope prof(project ? KVC_KERNEL_PROJECT_VALUES : KVC_KERNEL_GATHER_KEYS, st, KVC_KERNEL_COMPRESS);
   long long grid = project ? unit_count() : 1;
   for (int s = 0; s < 2; ++s) {
     const long long c = (blocks * ceil_div(a.copy[s].rows, 16) + CT_COPY_WARPS - 1) / CT_COPY_WARPS;

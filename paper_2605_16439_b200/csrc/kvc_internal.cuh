@@ -215,11 +215,11 @@ int decode_common(const kvc_layer* L, const void* q, const void* capsules, int B
 cudaError_t ensure_dynamic_smem(const void* kernel, size_t bytes);
 
 // optional event brackets around a launch (kvc_profile_*)
-bool prof_begin(int kernel_id, cudaStream_t st);
+bool prof_begin(int kernel_id, int part, cudaStream_t st);
 void prof_end(cudaStream_t st);
 struct ProfScope {
   cudaStream_t st; bool on;
-  ProfScope(int kernel_id, cudaStream_t s) : st(s), on(prof_begin(kernel_id, s)) {}
+  ProfScope(int kernel_id, cudaStream_t s, int part = -1) : st(s), on(prof_begin(kernel_id, part, s)) {}
   ~ProfScope() { if (on) prof_end(st); }
 };
 

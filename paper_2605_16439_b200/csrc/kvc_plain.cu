@@ -411,7 +411,7 @@ cudaError_t launch_plain(const kvc_layer* L, const DecodeArgs& d, const PlainPla
   a.cnt = reinterpret_cast<unsigned long long*>(ws + w.off_cnt);
   a.token = d.token; a.status = d.status;
   a.G = d.G; a.S0 = S0; a.T = d.T; a.steps_a = p.steps_a; a.spp = p.spp; a.slots = part_slots(L, B); a.total = p.total; a.off_red = p.off_red;
-  ProfScope prof(KVC_KERNEL_FUSED, st);
+  ProfScope prof(KVC_KERNEL_FUSED, st, KVC_KERNEL_PLAIN);
   return d.G > 8 ? launch_plain_inst<2, 3>(tm, a, p, st) : launch_plain_inst<1, 4>(tm, a, p, st);
 }
 

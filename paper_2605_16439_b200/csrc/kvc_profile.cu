@@ -11,13 +11,15 @@ struct Profile {
   size_t cap = 0;                         // bracketed launches that fit the event pool
   std::vector<cudaEvent_t> ev;            // 2 events per bracketed launch
   std::vector<int> kid;                   // kernel id per bracketed launch
+  std::vector<int> part;                  // its id beyond KVC_KERNEL_COUNT, -1: none
 };
 static Profile g_prof;
 
-bool prof_begin(int kernel_id, cudaStream_t st) {
+bool prof_begin(int kernel_id, int part, cudaStream_t st) {
   Profile& p = g_prof;
   if (!p.on || p.kid.size() >= p.cap) return false;
   p.kid.push_back(kernel_id);
+  p.part.push_back(part);
   cudaEventRecord(p.ev[2 * (p.kid.size() - 1)], st);
   return true;
 }
@@ -38,11 +40,13 @@ int kvc_profile_start(int max_launches) {
   for (cudaEvent_t e : p.ev) cudaEventDestroy(e);
   p.ev.clear();
   p.kid.clear();
+  p.part.clear();
   p.ev.resize((size_t)2 * max_launches);
   for (auto& e : p.ev)
     if (cudaEventCreate(&e) != cudaSuccess) return KVC_ERR_CUDA;
   p.cap = (size_t)max_launches;
   p.kid.reserve(p.cap);
+  p.part.reserve(p.cap);
   p.on = true;
   return KVC_OK;
 }
@@ -54,11 +58,11 @@ int kvc_profile_stop(void) {
 
 int kvc_profile_read(int kernel_id, double* total_ms, long long* launches) {
   Profile& p = g_prof;
-  if (!total_ms || !launches || kernel_id < 0 || kernel_id >= KVC_KERNEL_COUNT) return KVC_ERR_ARG;
+  if (!total_ms || !launches || kernel_id < 0 || kernel_id >= KVC_KERNEL_ID_END) return KVC_ERR_ARG;
   double t = 0;
   long long n = 0;
   for (size_t i = 0; i < p.kid.size(); ++i) {
-    if (p.kid[i] != kernel_id) continue;
+    if (p.kid[i] != kernel_id && p.part[i] != kernel_id) continue;
     float ms = 0.f;
     if (cudaEventElapsedTime(&ms, p.ev[2 * i], p.ev[2 * i + 1]) != cudaSuccess) return KVC_ERR_CUDA;
     t += ms;
@@ -85,6 +89,9 @@ const char* kvc_kernel_name(int kernel_id) {
     case KVC_KERNEL_SPLIT_EXPAND: return "split_expand";
     case KVC_KERNEL_SPLIT_OUTPUT: return "split_output";
     case KVC_KERNEL_RESIDENT: return "resident";
+    case KVC_KERNEL_CLUSTER: return "cluster";
+    case KVC_KERNEL_PLAIN: return "plain";
+    case KVC_KERNEL_COMPRESS: return "compress";
     default: return "?";
   }
 }

@@ -98,14 +98,14 @@ def gpu_run(shape: wl.Shape, p, dev="cuda", mode: str = "kv"):
 
 
 def launches(fn):
-    """({kernel name: launches}, result) of fn run with the library's event brackets on."""
+    """({kernel name: launches}, result) of fn run with the library's event brackets on; cluster, plain and compress beside what they count under."""
     kvc.kvc_profile_start(64)
     try:
         out = fn()
         torch.cuda.synchronize()
     finally:
         kvc.kvc_profile_stop()
-    counts = {k: v[1] for k, v in kvc.kvc_profile_read().items()}
+    counts = {k: v[1] for k, v in {**kvc.kvc_profile_read(), **kvc.kvc_profile_parts()}.items()}
     kvc.kvc_profile_start(0)
     kvc.kvc_profile_stop()
     return counts, out

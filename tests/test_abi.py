@@ -45,6 +45,14 @@ def test_retained_len_matches_oracle_bit_exactly(lib):
     assert lib.kvc_retained_len(16, -1) == -1
 
 
+def test_every_kernel_id_has_a_name_of_its_own(lib):
+    header = open(os.path.join(ROOT, "include", "kvc.h")).read()
+    assert int(re.search(r"KVC_KERNEL_COUNT = (\d+)", header)[1]) == kvc.KVC_KERNEL_COUNT
+    assert int(re.search(r"KVC_KERNEL_ID_END = (\d+)", header)[1]) == kvc.KVC_KERNEL_ID_END
+    names = [lib.kvc_kernel_name(k).decode() for k in range(kvc.KVC_KERNEL_ID_END)]
+    assert len(set(names)) == kvc.KVC_KERNEL_ID_END and {"cluster", "plain", "compress"} <= set(names)
+
+
 def test_strerror_covers_all_codes(lib):
     seen = {lib.kvc_strerror(s).decode() for s in range(0, -9, -1)}
     assert len(seen) == 9 and "unknown status" not in seen

@@ -45,8 +45,8 @@ def test_uniform_compression(B, H, grid, R, ratio):
     p = tl.make_problem(shape, 900 + grid + R, recipe="peaked")
     layer = tl.gpu_layer(shape, p)
     caps = kvc.alloc_capsules(layer, B, R)
-    kvc.kvc_compress(layer, p["K_vis"].to(DEV), p["V_vis"].to(DEV), B, R, caps)
-    torch.cuda.synchronize()
+    counts, _ = tl.launches(lambda: kvc.kvc_compress(layer, p["K_vis"].to(DEV), p["V_vis"].to(DEV), B, R, caps))
+    assert counts["compress"] == 1
     assert kvc.kvc_read_compress_status(layer) == 0
     K_t, V_t = orc.compress(tl.np64(p["K_vis"]), tl.np64(p["V_vis"]), p["idx"].numpy(), tl.np64(p["U"]), tl.np64(p["mu"]), shape.n, False)
     K_g, V_g = (tl.np64(x) for x in kvc.capsule_views(layer, caps, B, R))

@@ -40,8 +40,8 @@ def test_attend_full(B, H_q, H_kv, S):
     out = torch.full((B, H_q, 128), float("nan"), dtype=torch.bfloat16, device=DEV)
     Kd, Vd, qd = K.to(DEV), V.to(DEV), q.to(DEV)
     for _ in range(2):                                 # the second call meets the first one's arrival words
-        kvc.kvc_attend_full(layer, qd, Kd, Vd, B, S, S_cap, out, ws)
-    torch.cuda.synchronize()
+        counts, _ = tl.launches(lambda: kvc.kvc_attend_full(layer, qd, Kd, Vd, B, S, S_cap, out, ws))
+        assert counts["plain"] == 1
     assert kvc.kvc_read_device_status(layer, B, 0, S, ws) == 0
     k64, v64 = (np.repeat(tl.np64(x)[:, :, :S], H_q // H_kv, axis=1) for x in (K, V))
     logits = np.einsum("bhd,bhsd->bhs", tl.np64(q), k64) / np.sqrt(128.0)
@@ -54,5 +54,6 @@ def test_attend_full(B, H_q, H_kv, S):
 def test_ratio_zero_store_with_text(B, H_q, H_kv, grid, R, T):
     shape = wl.Shape("rho0", 1, B, H_q, H_kv, 128, grid, R, T, 1, "bf16", ratio_permille=0)
     p = tl.make_problem(shape, 640 + grid, T=T, T_cap=T + 4)
-    _, _, _, out = tl.gpu_run(shape, p)
+    counts, (_, _, _, out) = tl.launches(lambda: tl.gpu_run(shape, p))
+    assert counts["plain"] == 1
     tl.assert_close(tl.np64(out), tl.oracle_run(shape, p, "fused")[2], "bf16")
