@@ -18,8 +18,9 @@ namespace kvc {
 // walks its range of the n axis in chunks of 64 positions:
 //   L      thread <-> (position, quarter of the retained rows), eight loads of theta in flight, 16 rows accumulated in registers
 //          against scores broadcast from shared memory ([j][16 rows]); the quarters meet in shared memory
-//   W      thread <-> a row of U (and every 256th after it), 16-byte loads of its 64 entries, the probabilities broadcast; rows that do not
-//          start on 16-byte boundaries, or at most 64 of them, 64 at a time through shared memory, thread <-> (row, 4 expansion rows)
+//   W      thread <-> a row of U (and every 256th after it), 16-byte loads of its 64 entries, the probabilities broadcast; in bf16,
+//          rows that do not start on 16-byte boundaries, or at most 64 of them, 64 at a time through shared memory, thread <-> (row, 4
+//          expansion rows)
 //          (32 sequences of one block of n = 529, m = 212, bf16, 4/4 heads: a call 61 us with a thread per row, now 37)
 // One head of 4 rows, n = 576, m = 231 in fp32: 39 -> 18 us between events (one load of theta in flight per thread and 64 rows of U at a time
 // through shared memory before).
@@ -47,9 +48,11 @@ __global__ void __launch_bounds__(256) expand_kernel(DecodeArgs a) {
   const T* U = static_cast<const T*>(a.U) + (size_t)h * mv * n;
   const float* S = a.S + (size_t)h * nrows_h * ms;
   const int ii = tid & 63, qd = tid >> 6;     // position in the chunk, quarter of the retained rows
-  // U read from L2 by its rows' threads: rows start on 16-byte boundaries, and there are enough of them to keep the warps busy
+  // 16-byte loads of U: rows start on 16-byte boundaries.  U read from L2 by its rows' threads: in bf16 only so and where there are enough of
+  // them to keep the warps busy; in fp32 always (staged it was 24 % faster to 11 % slower over 60 calls of other block lengths)
   constexpr int EPV = Elems16<T>::N;
-  const bool direct = mv > 64 && n % EPV == 0 && (reinterpret_cast<uintptr_t>(U) & 15) == 0;
+  const bool vec = n % EPV == 0 && (reinterpret_cast<uintptr_t>(U) & 15) == 0;
+  const bool direct = sizeof(T) == sizeof(float) || (vec && mv > 64);
 
   grid_dep_wait();
   grid_dep_launch();
@@ -145,7 +148,7 @@ __global__ void __launch_bounds__(256) expand_kernel(DecodeArgs a) {
         }
         const T* up = U + (size_t)j * n + i0;
         int i = 0;
-        for (; i + 4 * EPV <= cnt; i += 4 * EPV) {
+        for (; vec && i + 4 * EPV <= cnt; i += 4 * EPV) {
           float u[4][EPV];
 #pragma unroll
           for (int v = 0; v < 4; ++v) load16(up + i + v * EPV, u[v]);
