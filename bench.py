@@ -49,7 +49,7 @@ KERNEL_SOURCES = {
                                                "kvc_tcgen05.cuh", "kvc_tma.cuh", "kvc_async.cuh"),
 }
 NCU_TRAFFIC_BYTES = {
-    ("fused", "config1-llava-next-7b"): (206.2e6, "52a0ec99407f"),
+    ("fused", "config1-llava-next-7b"): (206.2e6, "d7375d60c1e9"),
     ("split_scores+split_expand+split_output", "config2-qwen2-vl-7b"): (147.1e6, "4fedd6d75f9c"),
     ("resident", "config3-internvl3-8b-video"): (36.0e6, "57710997d7a9"),
 }

@@ -94,11 +94,13 @@ KVC_API int kvc_retained_len(int n, int ratio_permille);
  * that are on their way on any stream are seen) and reads theta and U.  ratio_permille == 0 is the pass-through limit: m = n,
  * capsules hold K and V verbatim, idx / theta / U / mu are ignored.
  * The device that is current at this call must be current for every later call with the handle.
- * bf16 decode calls run Alg. 1 either as one kernel (steps 2-3 on mma.sync with the logits in registers, or on tcgen05
- * with the logits in tensor memory) or, for block lengths above 640, as three kernels (streaming scores, tcgen05
- * expansion per 128 rows and range of the n axis, streaming output), or, for other block lengths and per-sequence lengths, as
- * one kernel of CTA clusters that share the n axis; the library picks per shape (same results within
- * the bf16 tolerance).  The environment variable KVC_EXPANSION = "tcgen05" | "mma" | "pair" | "split" | "resident" | "cluster", read
+ * bf16 decode calls run Alg. 1 as one kernel (theta and U resident in shared memory for short blocks; steps 2-3 on mma.sync with
+ * the logits in registers up to n = 640, with per-sequence lengths up to 1024; or on tcgen05 with the logits in tensor memory), for
+ * uniform calls of longer blocks as three kernels (streaming scores, tcgen05 expansion per 128 rows and range of the n axis, streaming
+ * output), or as one kernel of CTA clusters that share the n axis: block lengths off 64, the smallest and the many-round
+ * calls with groups of query heads, and per-sequence lengths where it is ahead.  What none of them takes, and block lengths off 64 with few
+ * query heads per KV head where they are ahead, goes to the generic three-phase kernels.  The library picks per shape
+ * (same results within the bf16 tolerance).  The environment variable KVC_EXPANSION = "tcgen05" | "mma" | "pair" | "split" | "resident" | "cluster", read
  * when the handle is created, forces one of them where it applies ("pair": the tcgen05 one-kernel path run by clusters of two
  * CTAs per (sequence, KV head)); "phases" forces the generic three-phase kernels that also serve fp32 storage. */
 KVC_API int kvc_layer_create(const kvc_layer_desc* desc, kvc_layer** out);
@@ -178,15 +180,15 @@ KVC_API int kvc_decode_attend_ragged(const kvc_layer* layer, const void* q, cons
                              int T_cap, void* out, void* workspace, void* stream);
 
 /* Parameter fits from activations (App. C, Algorithm 2), on the device in fp64.  Calibration-time calls: each one
- * SYNCHRONISES the stream several times (the eigen-solver checks convergence on the host) and returns with its outputs
- * complete.  X_vis: [B][H_kv][R*n][d] device, storage type `dtype`; every n-row block of every sequence is one sample.
+ * SYNCHRONISES the stream (once at its end up to n = 640, where the eigen-solver is one launch; beyond several times, since
+ * convergence is then checked on the host) and returns with its outputs complete.  X_vis: [B][H_kv][R*n][d] device, storage type `dtype`; every n-row block of every sequence is one sample.
  * workspace: kvc_fit_workspace_bytes(H_kv, n) bytes, 256-byte aligned, device.  sweeps_out (may be NULL): sweeps the
  * eigen-solver took.  Errors: KVC_ERR_ARG / _SHAPE (m outside [1, n]) / _DTYPE / _WORKSPACE / _BOUNDS (index set) / _CUDA.
  *
  * kvc_fit_value_pca: FitValuePCA (Sec. 3.1 "Sequence-Level Low-Rank Compression for Values"): mu_out [H_kv][d] = the
  * mean of the value rows over samples and positions; U_out [H_kv][m][n] = the top-m principal directions along the
- * token axis of the centred values (eigenvectors of the n x n token covariance by a hand-written cyclic Jacobi solver;
- * rows orthonormal, each with its entry of largest magnitude positive), both written in `dtype`.  eig_out (may be
+ * token axis of the centred values (eigenvectors of the n x n token covariance by a hand-written Jacobi solver,
+ * one-sided up to n = 640, two-sided cyclic beyond; rows orthonormal, each with its entry of largest magnitude positive), both written in `dtype`.  eig_out (may be
  * NULL): DEVICE double [H_kv][n], the covariance eigenvalues in descending order (squared singular values of the
  * pooled centred columns; the energy the projection loses is the sum of entries m..n-1).
  *

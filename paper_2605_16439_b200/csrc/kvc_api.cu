@@ -335,6 +335,8 @@ static bool use_split(const kvc_layer* L, int B, int R) {
   return plan_split(L, B, R).ok != 0;
 }
 
+constexpr double HBM_US = 6.5e6;      // bytes a microsecond at the measured copy bandwidth, in the estimates below
+
 // Which calls with per-sequence lengths and n a multiple of 64 take the one-kernel path (1), which the cluster path (2), which the
 // three-phase kernels (0).  The one-kernel path's time goes with the rounds of its units over the SMs (a unit: 9 us and 0.09 us per retained
 // row, or its bytes, parameters included, at 45 GB/s, up to 90 where few units of long blocks share the L2); the three-phase kernels'
@@ -352,13 +354,13 @@ static int ragged_path(const kvc_layer* L, int B, int R, int T) {
   const int sms = L->num_sms > 0 ? L->num_sms : 148, n = L->desc.n, m = L->m, H = L->desc.H_kv;
   const double rows = 512.0 * B * R * H * m, text = 512.0 * B * H * (double)T, par = 4.0 * m * n;
   if (L->G > 1) return f.ok && f.units <= sms && (m <= 144 || rows >= 2.5e7) ? 1 : 2;
-  const double floor_us = (rows + text + H * par) / 6.5e6, phases = 8.0 + 0.042 * n + 1.3 * floor_us;
+  const double floor_us = (rows + text + H * par) / HBM_US, phases = 8.0 + 0.042 * n + 1.3 * floor_us;
   const ClusterPlan c = plan_cluster(L, B, R, T, true);
-  const double cluster = c.ok && c.units <= c.ucl ? 28.0 + (n > 576 ? 0.06 * (n - 576) : 0.0) + (1.15 * (rows + H * par) + 2.5 * text) / 6.5e6 : 1e30;
+  const double cluster = c.ok && c.units <= c.ucl ? 28.0 + (n > 576 ? 0.06 * (n - 576) : 0.0) + (1.15 * (rows + H * par) + 2.5 * text) / HBM_US : 1e30;
   double fused = 1e30;
   if (f.ok) {
     const int last = (f.units + sms - 1) / sms, ctas = f.units < sms ? f.units : sms;
-    const double rate = n <= 640 || 148 * 45 > 90 * ctas ? (n <= 640 ? 45e3 : 90e3) : 45e3 * 148 / ctas;
+    const double rate = n <= 640 || sms * 45 > 90 * ctas ? (n <= 640 ? 45e3 : 90e3) : 45e3 * sms / ctas;
     const double rounds = last > 1 ? 0.5 * ((double)f.units / sms + last) : 1.0;
     fused = std::max(last * (9.0 + 0.09 * m), rounds * ((rows + text) / f.units + par) / rate);
   }
@@ -371,26 +373,26 @@ static int ragged_path(const kvc_layer* L, int B, int R, int T) {
 // with the chunks of 64 positions of 16 expansion rows, the retained rows they walk, and the bytes.  Constants fitted (least squares of the
 // relative error: 8 % and 12 %) to 1620 uniform calls on B200: 1/1 to 32/32 and 8/2, 32/8 heads, 1 x 1 to 64 x 2 blocks of n = 81 to 961, m = 11
 // to 769, 0 to 700 text rows; routed by it the calls take 0.6 % more than each on its better path, and 16 of 2430 more than 10 %
-// over what the three-phase kernels took before there was a cluster path (at worst 20.0 for 16.3).  us per call, cluster / three-phase: 16/16 heads, 64 x 2 of n = 81, m = 11,
-// 60 text rows 78 / 33; 32/32, 7 x 2 of 529, m = 67 53 / 31, m = 424 92 / 107; 4/4, 64 x 2 of 81, 700 rows 85 / 50; 8/2, 16 x 5 of 729, m = 292 45 / 143.
+// over what the three-phase kernels took before there was a cluster path (at worst 20.0 for 16.3).
+// us per call, cluster / three-phase: 16/16 heads, 64 x 2 of n = 81, m = 11, 60 text rows 78 / 33; 32/32, 7 x 2 of 529, m = 67 53 / 31, m = 424 92 / 107; 4/4, 64 x 2 of 81, 700 rows 85 / 50; 8/2, 16 x 5 of 729, m = 292 45 / 143.
 static bool cuda_core_expansion_wins(const kvc_layer* L, int B, int R, int T, bool ragged) {
   const ClusterPlan c = plan_cluster(L, B, R, T, ragged);
   if (!c.ok) return true;
   const int n = L->desc.n, m = L->m, H = L->desc.H_kv, nb = B * R;
   const double rows = 512.0 * nb * H * (double)m, text = 512.0 * B * H * (double)T;
   const double rounds = (c.units + c.ucl - 1) / c.ucl, rb = ceil_div(nb, c.units / H), seqs = std::min(rb, rb / R + (R > 1 && rb > 1 ? 1.0 : 0.0));
-  const double cluster = rounds * (18.0 + (0.6 * rb * c.vt + 0.44 * seqs) / c.NS + 1.4 * c.nk1) - 2.0 + (rows + 4.0 * H * m * n + 1.2 * text) / 6.5e6;
+  const double cluster = rounds * (18.0 + (0.6 * rb * c.vt + 0.44 * seqs) / c.NS + 1.4 * c.nk1) - 2.0 + (rows + 4.0 * H * m * n + 1.2 * text) / HBM_US;
   const WsLayout w = ws_layout(L, B, R, T);
   const double walk = w.IR / EXP_IC, chunks = (double)H * ceil_div(nb * L->G, EXP_ROWS) * ceil_div(n, EXP_IC);
-  const double phases = 15.7 + walk * (0.063 * m - 2.5) + chunks * (2.24e-4 * m + 0.0132) + (1.7 * rows + 1.57 * text) / 6.5e6 + 1.35 * (L->G - 1) + c.nk1;
+  const double phases = 15.7 + walk * (0.063 * m - 2.5) + chunks * (2.24e-4 * m + 0.0132) + (1.7 * rows + 1.57 * text) / HBM_US + 1.35 * (L->G - 1) + c.nk1;
   return phases < cluster;
 }
 
 // Which bf16 shapes take the cluster path.  Measured on B200, us per call, cluster / other paths.
 // Block lengths that are no multiple of 64, and per-sequence lengths outside the path above: the other way is the three-phase kernels.
 // Where those expand on the CUDA cores (n no multiple of 8) it is ahead from seven query heads per KV head on (8 x 5 blocks of n = 729,
-// 28/4 heads: 37 / 277); below, by the estimate above (cuda_core_expansion_wins).  And, with more than one query head per KV head, where they expand on mma.sync (4 x 1 of 400: 22 / 29; 16 x 4 of 196, 32/8 heads:
-// 31 / 65; 1 x 1 of 784, 8/2 heads: 23 / 25; 8 x 2 of 144: 18.8 / 18.6; with lengths per sequence from 1e7 flop of expansion on: 8 x 5 of
+// 28/4 heads: 37 / 277); below, by the estimate above (cuda_core_expansion_wins).  And it is ahead, with more than one query head per KV
+// head, where they expand on mma.sync (4 x 1 of 400: 22 / 29; 16 x 4 of 196, 32/8 heads: 31 / 65; 1 x 1 of 784, 8/2 heads: 23 / 25; 8 x 2 of 144: 18.8 / 18.6; with lengths per sequence from 1e7 flop of expansion on: 8 x 5 of
 // 144, 6/2 heads, 8e6: 21.7 / 20.8; 2 x 5 of 144, 28/4 heads, 9e6: 22 / 27); with one, its 128-row tiles stay empty (8 x 4 of 400, 32/32
 // heads: 60 / 50).
 // Whole multiples of 64 up to 640, groups of query heads: the other way is the one-kernel path, whose time goes with the rounds of its
@@ -423,7 +425,7 @@ static bool use_cluster(const kvc_layer* L, int B, int R, int T, bool ragged) {
   if (!f.ok || !c.ok) return c.ok != 0;
   const int rounds = (c.units + c.ucl - 1) / c.ucl;
   if (10ll * c.units < 7ll * rounds * c.ucl) return false;
-  return 1.1 * (25.0 * rounds + 4.0 + 2.4e-6 * bytes / 6.5) < (f.units + sms - 1) / sms * (9.0 + 0.09 * L->m);
+  return 1.1 * (25.0 * rounds + 4.0 + 2.4 * bytes / HBM_US) < (f.units + sms - 1) / sms * (9.0 + 0.09 * L->m);
 }
 
 // One token per decode call, process-wide: never 0 and never one of the byte patterns a caller is likely to have

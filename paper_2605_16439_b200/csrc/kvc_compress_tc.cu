@@ -13,7 +13,7 @@
 //   warp 9          TMA producer: per 64 vision positions one 48 KB stage (U 16 KB, V 2 x 16 KB, 128-byte swizzle), a ring of
 //                   stages that runs on across units
 //   warps 10-15     row copies: the retained key rows, a side stored verbatim, the rows left over by a ragged batch
-// Measured on B200 (per layer, back to back): 8 x 32 x 5 blocks of n = 576, m = 231: 81 us (5.3 TB/s of 426 MB; 129 us with one
+// Measured on B200 (per layer, back to back): 8 x 32 x 5 blocks of n = 576, m = 231: 84 us (5.1 TB/s of 426 MB; 129 us with one
 // launch for the keys and one CTA per (block, row tile)); 8 sequences of up to 8 blocks x 4 heads of n = 1024, m = 410 with their
 // own lengths: 42 us (1108 us on the CUDA cores before).  Tried: both row tiles of a pair in one unit, which fills the tensor memory
 // and leaves the epilogue exposed (N = 256: 103 us at the first shape; N = 128: 94 us).
@@ -33,7 +33,7 @@ constexpr int CT_EPI_WARPS = 8;
 constexpr uint32_t CT_OUT_WARP = 32 * 128;                  // epilogue staging of a warp: 32 rows, one 64-channel half
 constexpr uint32_t CT_TMEM_COLS = 512;
 // Six: sixteen warps have 128 registers a thread; with eight (96 registers) the copy loop's two steps in flight spilled, an L2 round trip
-// each with the L1 given to shared memory (8 x 5 blocks of n = 576, 32 heads, ratio 0.6: 78 us, six 74.5; 32 x 8 of 256: 31 and 27)
+// each with the L1 given to shared memory (one layer's buffers again and again: 8 x 5 blocks of n = 576, 32 heads, ratio 0.6: 78 us, six 74.5; 32 x 8 of 256: 31 and 27)
 constexpr int CT_COPY_WARPS = 6;
 constexpr int CT_THREADS = (CT_EPI_WARPS + 2 + CT_COPY_WARPS) * 32;
 constexpr uint32_t CT_SMEM_LIMIT = 231424;                  // dynamic part of the 227 KB; the barriers take the rest

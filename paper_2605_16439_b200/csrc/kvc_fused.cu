@@ -42,9 +42,10 @@ __device__ __forceinline__ FusedLanes fused_lanes() {
 // RG: the calls with per-sequence lengths.  Blocks and text rows past a sequence's lengths are neither loaded nor computed on, so the
 // capsule rows come in one copy per block; sequences are dealt to the units in the order of their work (the lengths are on the
 // device: every CTA sorts them itself), long ones with short ones.  The weights enter the product with the values as two bf16 terms:
-// these calls had fp32 weights before this kernel took them.
-// Bound as the uniform calls are (8 x 5 blocks of n = 576, 32/32 heads, half to all of 512 text rows: 235 MB in 43.9 us, 5.4 TB/s; the
-// three-phase kernels took 70).
+// these calls had fp32 weights before this kernel took them.  The scores are rounded to bf16 in log2 units, as on the uniform calls (those of
+// the three-phase kernels before that scaling): as many bits, other rounding points.
+// Bound as the uniform calls are (8 x 5 blocks of n = 576, 32/32 heads, half to all of 512 text rows: 235 MB in 46.3 us, 5.1 TB/s; the
+// three-phase kernels took 72).
 template <int EW, int VW, int KTW, int NH, int MT, bool RG>
 __global__ void __launch_bounds__((EW + VW + 1) * 32, 1)
 fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,

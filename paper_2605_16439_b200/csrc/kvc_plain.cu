@@ -5,7 +5,7 @@
 // CTA's part of a pair ends, and the copies of the next part are already in flight then.  Twelve warps with four pieces (192 KB a SM) cover
 // the round trip to HBM: 64 CTAs already draw 5.6 TB/s.
 // Measured on B200 (us per call, before: the text-only mode of the one-kernel path, equal slices per pair through CTA-wide stages):
-// 16 x 8704 rows, 28/4 heads 72 -> 51.5 (285 MB, 5.5 TB/s); 8 x 8448 38 -> 29; 32 x 2304 75 -> 29; 8 x 3000, 32/32 heads 89 -> 63;
+// 16 x 8704 rows, 28/4 heads 72 -> 52 (285 MB, 5.5 TB/s); 8 x 8448 38 -> 29; 32 x 2304 75 -> 29; 8 x 3000, 32/32 heads 89 -> 63;
 // 64 x 33000 642 -> 640; 1 x 2304 12.1 -> 10.3; 1 x 33000 27.5 -> 20.
 #include "kvc_fused.cuh"
 #include "kvc_plain.cuh"
