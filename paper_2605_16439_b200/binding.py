@@ -304,7 +304,7 @@ def capsule_views(layer: Layer, capsules, B: int, R: int):
 
 
 KVC_KERNEL_COUNT = 14
-KVC_KERNEL_ID_END = 17
+KVC_KERNEL_ID_END = 18
 
 
 def kvc_profile_start(max_launches: int) -> None:

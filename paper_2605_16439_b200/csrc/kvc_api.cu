@@ -13,6 +13,7 @@
 #include "kvc_resident.cuh"
 #include "kvc_cluster.cuh"
 #include "kvc_plain.cuh"
+#include "kvc_spread.cuh"
 
 namespace kvc {
 
@@ -209,12 +210,12 @@ int kvc_layer_create(const kvc_layer_desc* desc, kvc_layer** out) {
   std::memset(L->clusters, 0, sizeof(L->clusters));
   {
     const char* ex = std::getenv("KVC_EXPANSION");
-    L->use_tc = !ex ? 0 : (std::strcmp(ex, "tcgen05") == 0 ? 1 : (std::strcmp(ex, "pair") == 0 ? 2 : (std::strcmp(ex, "mma") == 0 ? -1 : (std::strcmp(ex, "phases") == 0 ? -2 : (std::strcmp(ex, "split") == 0 ? 3 : (std::strcmp(ex, "resident") == 0 ? 4 : (std::strcmp(ex, "cluster") == 0 ? 5 : 0)))))));
+    L->use_tc = !ex ? 0 : (std::strcmp(ex, "tcgen05") == 0 ? 1 : (std::strcmp(ex, "pair") == 0 ? 2 : (std::strcmp(ex, "mma") == 0 ? -1 : (std::strcmp(ex, "phases") == 0 ? -2 : (std::strcmp(ex, "split") == 0 ? 3 : (std::strcmp(ex, "resident") == 0 ? 4 : (std::strcmp(ex, "cluster") == 0 ? 5 : (std::strcmp(ex, "spread") == 0 ? 6 : 0))))))));
   }
   // one allocation: index set, status word, row sums of U, and where a kernel would read them, copies of theta and U with rows the TMA
   // engine can address (bf16): theta for the cluster path, whose tensor map cuts rows in groups of 64, U where its rows do not start on 16 bytes
   const int np = (int)align_up((size_t)desc->n, 64);
-  const bool pad_theta = np != desc->n && cluster_may_serve(L);
+  const bool pad_theta = np != desc->n && (cluster_may_serve(L) || (spread_may_serve(L) && desc->n % 8 != 0));
   const bool pad_U = desc->dtype == KVC_BF16 && !pass && value_side && np != desc->n &&
                      (desc->n % 8 != 0 || !tma_rows(desc->U));
   L->theta_np = pad_theta ? np : desc->n;
@@ -229,7 +230,7 @@ int kvc_layer_create(const kvc_layer_desc* desc, kvc_layer** out) {
   const size_t o_theta = take(pad_theta ? padded : 0), o_U = take(pad_U ? padded : 0);
   cudaError_t e = cudaGetDevice(&L->device);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&L->num_sms, cudaDevAttrMultiProcessorCount, L->device);
-  if (e == cudaSuccess && cluster_may_serve(L)) cluster_occupancy(L->device, L->num_sms, L->clusters);
+  if (e == cudaSuccess && (cluster_may_serve(L) || spread_may_serve(L))) cluster_occupancy(L->device, L->num_sms, L->clusters);
   if (e == cudaSuccess) e = cudaMalloc(&L->d_block, bytes);
   if (e == cudaSuccess) {
     char* base = static_cast<char*>(L->d_block);
@@ -428,6 +429,22 @@ static bool use_cluster(const kvc_layer* L, int B, int R, int T, bool ragged) {
   return 1.1 * (25.0 * rounds + 4.0 + 2.4 * bytes / HBM_US) < (f.units + sms - 1) / sms * (9.0 + 0.09 * L->m);
 }
 
+// Which bf16 shapes take the spread path: those its plan serves (at most 64 expansion rows per pair, clusters of two or more CTAs for all pairs
+// at once, scores and weights that leave room for a ring).  Over 109 drawn calls of that kind (1/1 to 32/32 heads, n = 64 to 1024, m = 52 to
+// 820, up to 4096 text rows, a third with lengths per sequence) it took 0.38 to 0.98 of the time of the paths below, with these exceptions:
+// short blocks whose parameters the resident path keeps in shared memory.  n = 64: level at 9.7 us, behind with text (18 x 2 blocks, 28/4 heads,
+// 512 rows 10.5 / 10.5; 4 x 2, 1024 rows 10.9 / 9.7); n = 256: ahead up to 256 text rows per CTA (4 x 2, 2048 rows 11.6 / 12.4; 1 x 2, 4096
+// rows 14.8 / 12.3).  Calls whose path the tests name stay where they are, although this one is ahead: lengths per sequence on those short
+// blocks (6 x 1 of n = 256, 8/2 heads 10.3 / 13.4) or under 1e7 flop of expansion beside them, and clusters of two on blocks under 96 positions
+// (32 x 1 of n = 81, 8/2 heads, 700 rows 12.3 / 36.9).  KVC_EXPANSION=spread forces it where its plan applies, any other value keeps it off.
+static bool use_spread(const kvc_layer* L, int B, int R, int T, bool ragged, const SpreadPlan& p) {
+  if (!p.ok || L->use_tc == 6) return p.ok != 0;
+  const int n = L->desc.n;
+  if (plan_resident(L, B, R, T).ok) return !ragged && n == 256 && T <= 256 * p.C;
+  if (ragged && n % 8 == 0 && n % 64 != 0 && 4.0 * B * L->desc.H_q * R * (double)L->m * n < 1e7) return false;
+  return n >= 96 || p.C > 2;
+}
+
 // One token per decode call, process-wide: never 0 and never one of the byte patterns a caller is likely to have
 // filled a fresh workspace with, so that stale workspace contents cannot pass for arrivals of this call.
 static unsigned int next_token() {
@@ -472,6 +489,15 @@ int decode_common(const kvc_layer* L, const void* q, const void* capsules, int B
   const uintptr_t align = reinterpret_cast<uintptr_t>(q) | reinterpret_cast<uintptr_t>(capsules) |
                           reinterpret_cast<uintptr_t>(out) | (T > 0 ? reinterpret_cast<uintptr_t>(K_txt) |
                           reinterpret_cast<uintptr_t>(V_txt) : 0) | reinterpret_cast<uintptr_t>(L->desc.mu);
+
+  if ((align & 15) == 0) {
+    const SpreadPlan sp = plan_spread(L, B, R, T);
+    if (use_spread(L, B, R, T, ragged, sp)) {
+      bool encoded = false;
+      const cudaError_t se = launch_spread(L, a, sp, st, &encoded);
+      if (encoded) return cuda_status(se);
+    }
+  }
 
   if ((align & 15) == 0 && use_cluster(L, B, R, T, ragged)) {
     const ClusterPlan cp = plan_cluster(L, B, R, T, ragged);

@@ -60,6 +60,7 @@ __device__ __forceinline__ bool mbar_test_wait(uint64_t* bar, uint32_t parity) {
 }
 // true on completion, false if the spin limit ran out
 __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity) {
+#pragma unroll 1
   for (uint32_t i = 0; i < WAIT_SPIN_LIMIT; ++i)
     if (mbar_try_wait(bar, parity)) return true;
   return false;
@@ -103,10 +104,27 @@ __device__ __forceinline__ bool mbar_try_wait_cluster(uint64_t* bar, uint32_t pa
   return ok != 0;
 }
 __device__ __forceinline__ bool mbar_wait_cluster_bounded(uint64_t* bar, uint32_t parity) {
+#pragma unroll 1
   for (uint32_t i = 0; i < WAIT_SPIN_LIMIT; ++i)
     if (mbar_try_wait_cluster(bar, parity)) return true;
   return false;
 }
+// asynchronous stores into a peer's shared memory; their bytes are reported to the peer's barrier when they have landed
+__device__ __forceinline__ void st_async_f32x2(uint32_t caddr, float x, float y, uint32_t cbar) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];\n" ::"r"(caddr), "f"(x), "f"(y), "r"(cbar) : "memory");
+}
+__device__ __forceinline__ void st_async_f32x4(uint32_t caddr, const float4& v, uint32_t cbar) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];\n"
+               ::"r"(caddr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "r"(cbar) : "memory");
+}
+// this CTA's shared memory -> a peer's, 16-byte aligned; completion on the peer's barrier
+__device__ __forceinline__ void bulk_s2peer(uint32_t dst_caddr, uint32_t src_saddr, uint32_t bytes, uint32_t cbar) {
+  asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n"
+               ::"r"(dst_caddr), "r"(src_saddr), "r"(bytes), "r"(cbar) : "memory");
+}
+// the two halves of cluster_sync_all
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory"); }
 // every thread of every CTA of the cluster
 __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");

@@ -118,8 +118,8 @@ struct kvc_layer {
   int num_sms;
   int clusters[9];       // clusters of 1 to 8 CTAs of the cluster decode kernel the device holds at once (0: not to be used)
   int use_tc;            // expansions of the one-kernel decode path: 0 chosen per shape, 1 tcgen05, 2 tcgen05 in pairs of CTAs,
-                         // -1 mma.sync; -2 three-phase kernels, 3 three-kernel path, 4 resident parameters, 5 clusters (environment
-                         // KVC_EXPANSION=tcgen05 | pair | mma | phases | split | resident | cluster when the handle is created)
+                         // -1 mma.sync; -2 three-phase kernels, 3 three-kernel path, 4 resident parameters, 5 clusters, 6 a cluster per pair (environment
+                         // KVC_EXPANSION=tcgen05 | pair | mma | phases | split | resident | cluster | spread when the handle is created)
   int32_t* d_idx;        // device [H_kv][m]
   int* d_cstatus;        // device status word of the compress kernels (cleared by every kvc_compress call)
   float* d_usum;         // device [H_kv][m] row sums of U (value compression:  U (V - 1 mu^T) = U V - (U 1) mu^T)

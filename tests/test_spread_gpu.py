@@ -1,0 +1,63 @@
+"""The spread decode path (a cluster of CTAs per (sequence, KV head)) at the sizes where its tiling can go wrong, against the fp64
+oracle: retained lengths and block lengths around the 16-row granules and the slices they are cut into, one to eight row tiles, one and
+two head tiles, two boxes of columns, text lengths around a piece and around what the CTAs share, more pieces than ring slots,
+per-sequence lengths with nothing in some sequences.
+
+Bound: the regression bound of the parity tests.
+"""
+import random
+
+import pytest
+
+from paper_2605_16439_b200 import build as kvc_build
+from paper_2605_16439_b200 import workloads as wl
+
+import kvc_testlib as tl
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    kvc_build.build()
+
+
+@pytest.mark.parametrize("B,H_q,H_kv,grid,R,T,ratio", [
+    (1, 1, 1, 8, 1, 0, 600),         # n = 64, m = 26: two granules, two CTAs, one row, no text
+    (1, 8, 2, 8, 1, 1, 200),         # m = 52: four granules over four CTAs, the last of 4 rows
+    (2, 7, 1, 9, 3, 15, 600),        # n = 81: the last column group has one column
+    (1, 16, 2, 12, 1, 16, 600),      # n = 144
+    (1, 32, 32, 24, 5, 128, 600),    # one row per block
+    (2, 28, 4, 27, 5, 300, 600),     # n = 729: two terms, 35 rows
+    (8, 28, 4, 27, 5, 33, 600),      # more pairs: four CTAs each
+    (3, 14, 2, 32, 9, 513, 600),     # 63 rows, n = 1024
+    (8, 8, 4, 32, 3, 47, 400),       # sixteen column groups per CTA: two boxes
+    (32, 8, 2, 16, 4, 70, 600),      # two CTAs per pair
+    (1, 16, 1, 11, 4, 30, 800),      # two head tiles, 64 rows
+    (2, 24, 2, 17, 2, 129, 500),     # G = 12
+    (1, 2, 1, 12, 1, 4097, 600),     # long text
+    (1, 4, 1, 31, 4, 40, 300),       # n = 961, m = 673: six granules per CTA, two terms
+])
+@pytest.mark.parametrize("recipe", ["peaked", "structured"])
+def test_uniform(B, H_q, H_kv, grid, R, T, ratio, recipe, monkeypatch):
+    monkeypatch.setenv("KVC_EXPANSION", "spread")
+    shape = wl.Shape("spread", 1, B, H_q, H_kv, 128, grid, R, T, 1, "bf16", ratio)
+    p = tl.make_problem(shape, 600 + grid + B, T=T, T_cap=T + 3, recipe=recipe)
+    counts, (_, _, _, out) = tl.launches(lambda: tl.gpu_run(shape, p))
+    assert counts["spread"] == 1 and counts["scores"] == 0
+    tl.assert_close(tl.np64(out), tl.oracle_run(shape, p, "fused")[2], "bf16")
+
+
+@pytest.mark.parametrize("B,H_q,H_kv,grid,R,T,ratio", [
+    (9, 14, 2, 24, 3, 150, 600), (5, 8, 2, 9, 2, 40, 600), (4, 7, 1, 32, 3, 300, 200), (3, 12, 1, 15, 4, 64, 500),
+])
+def test_per_sequence_lengths(B, H_q, H_kv, grid, R, T, ratio, monkeypatch):
+    monkeypatch.setenv("KVC_EXPANSION", "spread")
+    rng = random.Random(grid)
+    R_b = [rng.randint(0, R) for _ in range(B)]
+    T_b = [rng.choice([0, 1, T, rng.randint(0, T)]) for _ in range(B)]
+    R_b[1], T_b[1] = 0, 0                              # nothing at all: a zero output row
+    R_b[-1] = R
+    shape = wl.Shape("spread-ragged", 1, B, H_q, H_kv, 128, grid, R, T, 1, "bf16", ratio)
+    counts, _ = tl.check_ragged(shape, 650 + grid, R_b, T_b)
+    assert counts["spread"] == 1 and counts["scores"] == 0
