@@ -103,9 +103,17 @@ def _ptr(t) -> int | None:
     return t.data_ptr()
 
 
+_RAW_STREAM = getattr(torch._C, "_cuda_getCurrentRawStream", None)      # absent from builds of torch without CUDA
+
+
 def _stream(stream=None) -> int:
-    s = torch.cuda.current_stream() if stream is None else stream
-    return s.cuda_stream
+    """The stream's handle; None: the current stream of the current device (asked for as a number: the Stream object that
+    torch.cuda.current_stream() builds takes 3.3 us, as long as the launch)."""
+    if stream is not None:
+        return stream.cuda_stream
+    if _RAW_STREAM is None:
+        return torch.cuda.current_stream().cuda_stream
+    return _RAW_STREAM(torch._C._cuda_getDevice())
 
 
 def kvc_retained_len(n: int, ratio_permille: int) -> int:
@@ -297,10 +305,22 @@ def kvc_export_maps(layer: Layer, R: int):
 
 def capsule_views(layer: Layer, capsules, B: int, R: int):
     """(K_tilde [B,H_kv,R,m_k,d], V_tilde [B,H_kv,R,m_v,d]) typed views of a capsule store (no copy)."""
+    m_k, m_v, d, H = layer.m_k, layer.m_v, layer.d, layer.H_kv
+    if B > 0 and R > 0 and capsules.dim() == 1 and capsules.dtype is torch.uint8:
+        # three tensor operations instead of six (4 us instead of 7, where the smallest calls take 9)
+        try:
+            t = capsules.view(layer.dtype)
+        except RuntimeError:                        # bytes that are not whole elements: the parts below may be
+            t = None
+        kn = B * H * R * m_k * d
+        if t is not None and t.numel() >= kn + B * H * R * m_v * d:
+            at = t.storage_offset()
+            return (t.as_strided((B, H, R, m_k, d), (H * R * m_k * d, R * m_k * d, m_k * d, d, 1), at),
+                    t.as_strided((B, H, R, m_v, d), (H * R * m_v * d, R * m_v * d, m_v * d, d, 1), at + kn))
     total = kvc_capsule_bytes(layer, B, R)
-    kb = total // (layer.m_k + layer.m_v) * layer.m_k
-    return (capsules[:kb].view(layer.dtype).view(B, layer.H_kv, R, layer.m_k, layer.d),
-            capsules[kb:total].view(layer.dtype).view(B, layer.H_kv, R, layer.m_v, layer.d))
+    kb = total // (m_k + m_v) * m_k
+    return (capsules[:kb].view(layer.dtype).view(B, layer.H_kv, R, m_k, d),
+            capsules[kb:total].view(layer.dtype).view(B, layer.H_kv, R, m_v, d))
 
 
 KVC_KERNEL_COUNT = 14
