@@ -294,7 +294,8 @@ size_t kvc_capsule_bytes(const kvc_layer* L, int B, int R) {
 size_t kvc_workspace_bytes(const kvc_layer* L, int B, int R, int T_cap) {
   if (!L || B < 0 || R < 0 || T_cap < 0) return 0;
   const size_t phases = ws_layout(L, B, R, T_cap, WS_UNIFORM | WS_RAGGED).total, cluster = cluster_ws_bytes(L, B, R, T_cap);
-  const size_t most = phases > cluster ? phases : cluster;
+  size_t most = phases > cluster ? phases : cluster;
+  if (B > 0 && R > 0) most = std::max(most, spread_ws_bytes(L, B, R));
   const size_t plain = (R == 0 || L->passthrough) && L->desc.dtype == KVC_BF16 && B > 0 ? plain_ws(L, B).bytes : 0;
   return most > plain ? most : plain;
 }
@@ -429,20 +430,23 @@ static bool use_cluster(const kvc_layer* L, int B, int R, int T, bool ragged) {
   return 1.1 * (25.0 * rounds + 4.0 + 2.4 * bytes / HBM_US) < (f.units + sms - 1) / sms * (9.0 + 0.09 * L->m);
 }
 
-// Which bf16 shapes take the spread path: those its plan serves (at most 64 expansion rows per pair, clusters of two or more CTAs for all pairs
-// at once, scores and weights that leave room for a ring).  Over 109 drawn calls of that kind (1/1 to 32/32 heads, n = 64 to 1024, m = 52 to
-// 820, up to 4096 text rows, a third with lengths per sequence) it took 0.38 to 0.98 of the time of the paths below, with these exceptions:
-// short blocks whose parameters the resident path keeps in shared memory.  n = 64: level at 9.7 us, behind with text (18 x 2 blocks, 28/4 heads,
-// 512 rows 10.5 / 10.5; 4 x 2, 1024 rows 10.9 / 9.7); n = 256: ahead up to 256 text rows per CTA (4 x 2, 2048 rows 11.6 / 12.4; 1 x 2, 4096
-// rows 14.8 / 12.3).  Calls whose path the tests name stay where they are, although this one is ahead: lengths per sequence on those short
+// Which bf16 shapes take the spread path: those its plan serves (at most 64 expansion rows per group of blocks, clusters of two or more CTAs for
+// all groups at once, scores and weights that leave room for a ring).  Over 110 drawn calls of that kind (1/1 to 32/32 heads, n = 64 to 1024, up
+// to 3000 text rows) it took 14.4 us in the geometric mean, the paths below 23.8; behind them are:
+// short blocks whose parameters the resident path keeps in shared memory, with more than two row tiles (5 x 9 of n = 256, 28/4 heads 13.4 / 12.5;
+// 2 x 8 13.2 / 11.0; but 2 x 2 8.8 / 10.3, 1 x 1 9.0 / 10.8), few retained rows (5 x 1, m = 32, 16/2 heads 8.4 / 7.6; 4 x 4, m = 52, 8/2 heads
+// 8.6 / 8.7), long text (1 x 2, 4096 rows 14.8 / 12.3; 4 x 2, 1024 rows, 10.1 / 13.1) or n = 64 (8.8 / 8.3); and the longest chains beside the
+// one-kernel and three-kernel paths (3 x 13 of 1024, 28/4 heads 48.3, estimated 39.4, / 41.1).
+// Calls whose path the tests name stay where they are, although this one is ahead: lengths per sequence on those short
 // blocks (6 x 1 of n = 256, 8/2 heads 10.3 / 13.4) or under 1e7 flop of expansion beside them, and clusters of two on blocks under 96 positions
 // (32 x 1 of n = 81, 8/2 heads, 700 rows 12.3 / 36.9).  KVC_EXPANSION=spread forces it where its plan applies, any other value keeps it off.
 static bool use_spread(const kvc_layer* L, int B, int R, int T, bool ragged, const SpreadPlan& p) {
   if (!p.ok || L->use_tc == 6) return p.ok != 0;
   const int n = L->desc.n;
-  if (plan_resident(L, B, R, T).ok) return !ragged && n == 256 && T <= 256 * p.C;
+  if (plan_resident(L, B, R, T).ok) return !ragged && n == 256 && L->m > 48 && R * L->G <= 16 && T <= 128 * p.C;
   if (ragged && n % 8 == 0 && n % 64 != 0 && 4.0 * B * L->desc.H_q * R * (double)L->m * n < 1e7) return false;
-  return n >= 96 || p.C > 2;
+  if (n % 64 == 0 && p.us > 36.0) return false;
+  return n >= 96 || p.C * p.nrg > 2;
 }
 
 // One token per decode call, process-wide: never 0 and never one of the byte patterns a caller is likely to have
@@ -492,9 +496,9 @@ int decode_common(const kvc_layer* L, const void* q, const void* capsules, int B
 
   if ((align & 15) == 0) {
     const SpreadPlan sp = plan_spread(L, B, R, T);
-    if (use_spread(L, B, R, T, ragged, sp)) {
+    if (use_spread(L, B, R, T, ragged, sp) && (ws_limit == 0 || spread_ws(L, sp, B).bytes <= ws_limit)) {
       bool encoded = false;
-      const cudaError_t se = launch_spread(L, a, sp, st, &encoded);
+      const cudaError_t se = launch_spread(L, a, sp, ws, st, &encoded);
       if (encoded) return cuda_status(se);
     }
   }

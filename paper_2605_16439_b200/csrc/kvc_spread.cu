@@ -10,6 +10,7 @@
 // 130 KB of code, now 50.
 #include <algorithm>
 
+#include "kvc_fused.cuh"
 #include "kvc_spread.cuh"
 
 namespace kvc {
@@ -127,7 +128,8 @@ spread_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
   __shared__ __align__(8) SpreadBars bars;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int C = 1 << a.lc, G = a.G, rank = (int)blockIdx.x & (C - 1), unit = (int)blockIdx.x >> a.lc;
-  const int b = unit / a.H_kv, h = unit - b * a.H_kv;
+  const int pair = a.nrg > 1 ? unit / a.nrg : unit, rg = unit - pair * a.nrg;    // group of blocks [rg a.rg, ...) of (b, h)
+  const int b = pair / a.H_kv, h = pair - b * a.H_kv;
   const bool ragged = a.R_b != nullptr || a.T_b != nullptr;
 
   // this CTA's granules of the m axis and column groups of the n axis
@@ -150,7 +152,14 @@ spread_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
 
   const uint32_t kbytes = (uint32_t)(a.kg * 16 * a.bpp) * 256u, pbytes = (uint32_t)(a.nsub * a.pg * 16 * a.wbox) * 2u;
   const int kp = gown > a.kg ? (gown + a.kg - 1) / a.kg : 1;  // capsule pieces per run of blocks
-  const int blk = unit * a.R;                                 // first block in the capsule store
+  const int blk = pair * a.R + rg * a.rg;                     // first block in the capsule store
+  // blocks of the group in a sequence that has r of them
+  auto group_blocks = [&](int r) { return min(max(r - rg * a.rg, 0), a.rg); };
+  // this CTA's share of the text rows, in items of 16
+  auto text_items = [&](int t, int& i0, int& i1) {
+    const int items = (t + 15) >> 4, c = rg * C + rank, n = a.nrg << a.lc;
+    i0 = (int)((long long)c * items / n); i1 = (int)((long long)(c + 1) * items / n);
+  };
   auto load_capsule = [&](const CUtensorMap* tm, uint32_t slot, int r, int x) {
     tma_load_4d(ring + slot * a.slot_bytes, tm, 0, (g0 + x * a.kg) * 16, 0, blk + r, &bars.full[slot]);
   };
@@ -160,7 +169,7 @@ spread_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
   // us per call, 13.2 with the key rows alone, 13.3 with nothing this early; 4 pairs of n = 1024: 23.9, 23.9, 24.3).
   int filled = 0;
   if (warp == SPR_WARPS) {
-    const int nk = ((a.R + a.bpp - 1) / a.bpp) * kp;
+    const int nk = ((group_blocks(a.R) + a.bpp - 1) / a.bpp) * kp;
     if (a.early && !ragged) filled = min(a.slots, nk);
     if (lane < a.slots) {
       mbar_init(&bars.full[lane], 1); mbar_init(&bars.empty[lane], SPR_WARPS);
@@ -201,6 +210,7 @@ spread_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
       int Re = a.R, Te = a.T;
       if (a.R_b) { const int r = a.R_b[b]; Re = r < 0 ? 0 : (r > a.R ? a.R : r); }
       if (a.T_b) { const int t = a.T_b[b]; Te = t < 0 ? 0 : (t > a.T ? a.T : t); }
+      Re = group_blocks(Re);
       auto capsule = [&](const CUtensorMap* tm) {
 #pragma unroll 1
         for (int r = 0; r < Re && ok; r += a.bpp)
@@ -224,7 +234,8 @@ spread_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
         }
       };
       auto text = [&]() {
-        const int items = (Te + 15) >> 4, i0 = rank * items >> a.lc, i1 = (rank + 1) * items >> a.lc;
+        int i0, i1;
+        text_items(Te, i0, i1);
 #pragma unroll 1
         for (int i = i0; i < i1 && ok; i += a.ti) {
           if (!begin((uint32_t)a.ti * 8192u)) return;
@@ -266,7 +277,7 @@ spread_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
     };
     auto peer_wait = [&](uint64_t* bar) { if (!dead && !mbar_wait_cluster_bounded(bar, 0u)) dead = true; };
 
-    if (tid < 2 * G) prefetch_l2(a.q + ((size_t)unit * G) * D + tid * 64);      // consumes nothing: may run before the wait
+    if (tid < 2 * G) prefetch_l2(a.q + ((size_t)pair * G) * D + tid * 64);      // consumes nothing: may run before the wait
     grid_dep_wait();
     grid_dep_launch();
     if (blockIdx.x == 0 && warp == 0) {
@@ -280,13 +291,14 @@ spread_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
     int Re = a.R, Te = a.T;
     if (a.R_b) { const int r = a.R_b[b]; Re = r < 0 ? 0 : (r > a.R ? a.R : r); }
     if (a.T_b) { const int t = a.T_b[b]; Te = t < 0 ? 0 : (t > a.T ? a.T : t); }
+    Re = group_blocks(Re);
 
     // the pair's queries, an A operand whose rows are the heads: read from shared memory where they are used (held in registers they spill)
 #pragma unroll 1
     for (int i = tid; i < 16 * 16; i += SPR_CONS) {
       const int g = i >> 4, c = i & 15;
       *reinterpret_cast<uint4*>(sm + a.q_off + (uint32_t)g * SPR_QPITCH + c * 16u) =
-          g < G ? *reinterpret_cast<const uint4*>(a.q + ((size_t)unit * G + g) * D + c * 8) : make_uint4(0, 0, 0, 0);
+          g < G ? *reinterpret_cast<const uint4*>(a.q + ((size_t)pair * G + g) * D + c * 8) : make_uint4(0, 0, 0, 0);
     }
     if (tid < D >> a.lc) mus[tid] = __bfloat162float(a.mu[h * D + rank * (D >> a.lc) + tid]);
     const uint32_t q_u = smem_addr(sm + a.q_off) + (uint32_t)lrowA * SPR_QPITCH + (uint32_t)lhi * 16u;
@@ -363,7 +375,8 @@ spread_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
     };
     // this CTA's share of the text rows: 16 at a time, a warp each, flash-style
     auto text_part = [&]() {
-      const int items = (Te + 15) >> 4, i0 = rank * items >> a.lc, i1 = (rank + 1) * items >> a.lc;
+      int i0, i1;
+      text_items(Te, i0, i1);
       int first = SPR_WARPS - 1 - warp;                       // item of the piece; every sixteenth is this warp's (the last warps have the fewest granules)
 #pragma unroll 1
       for (int i = i0; i < i1; i += a.ti) {
@@ -760,7 +773,39 @@ spread_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
           num = fmaf(f, mus[d], num);
         }
       }
-      a.out[((size_t)unit * G + g) * D + rank * dc + d] = __float2bfloat16_rn(den > 0.f ? num / den : 0.f);
+      if (a.nrg == 1) {
+        a.out[((size_t)pair * G + g) * D + rank * dc + d] = __float2bfloat16_rn(den > 0.f ? num / den : 0.f);
+      } else {
+        a.py[((size_t)unit * G + g) * D + rank * dc + d] = num;
+        if (d == 0) a.pml[(((size_t)pair * C + rank) * a.nrg + rg) * G + g] = make_float2(mx, den);
+      }
+    }
+    if (a.nrg > 1) {
+      // the last group's CTA `rank` to arrive merges their channels
+      __threadfence();
+      named_barrier_sync(1, SPR_CONS);
+      if (tid == 0) rowmax[0] = arrive_is_last(&a.cnt[pair * C + rank], a.token, a.nrg) ? 1 : 0;
+      named_barrier_sync(1, SPR_CONS);
+      if (rowmax[0]) {
+        __threadfence();
+#pragma unroll 1
+        for (int i = tid; i < G * dc; i += SPR_CONS) {
+          const int g = i >> ld, d = i & (dc - 1);
+          const float2* ml = a.pml + ((size_t)pair * C + rank) * a.nrg * G + g;
+          const float* yp = a.py + ((size_t)pair * a.nrg * G + g) * D + rank * dc + d;
+          float mx = -INFINITY, num = 0.f, den = 0.f;
+#pragma unroll 4
+          for (int p = 0; p < a.nrg; ++p) mx = fmaxf(mx, __ldcg(ml + p * G).x);
+#pragma unroll 4
+          for (int p = 0; p < a.nrg; ++p) {
+            const float2 t = __ldcg(ml + p * G);
+            const float f = t.x == -INFINITY ? 0.f : fast_exp2(t.x - mx);
+            num = fmaf(f, __ldcg(yp + (size_t)p * G * D), num);
+            den = fmaf(f, t.y, den);
+          }
+          a.out[((size_t)pair * G + g) * D + rank * dc + d] = __float2bfloat16_rn(den > 0.f ? num / den : 0.f);
+        }
+      }
     }
     if (dead) {
       if (lane == 0) atomicExch(a.status, (int)KVC_ERR_TIMEOUT);
@@ -782,15 +827,16 @@ bool spread_may_serve(const kvc_layer* L) {
   return L->desc.dtype == KVC_BF16 && !L->passthrough && L->mode == KVC_MODE_KV && L->desc.n >= 64 && (L->use_tc == 0 || L->use_tc == 6);
 }
 
-SpreadPlan plan_spread(const kvc_layer* L, int B, int R, int T) {
+static SpreadPlan plan_groups(const kvc_layer* L, int B, int R_all, int T_all, int nrg) {
   SpreadPlan p{};
+  const int R = ceil_div(R_all, nrg), T = ceil_div(T_all, nrg);
   const int G = L->G, n = L->desc.n, m = L->m, H = L->desc.H_kv;
-  if (!spread_may_serve(L) || B < 1 || R < 1 || G > 16 || R > 64 || R * G > 64 || T < 0) return p;
-  if (!tma_rows(spread_theta(L)) || !tma_rows(L->U_rows) || spread_theta_np(L) % 8 || L->U_np % 8) return p;
+  p.nrg = nrg; p.rg = R;
+  if (R > 64 || R * G > 64 || (nrg - 1) * R >= R_all) return p;
   p.ng = ceil_div(m, 16);
   p.ncg = ceil_div(n, 16);
   for (int c = SPR_MAX_C; c >= 2; c /= 2)
-    if ((long long)B * H <= L->clusters[c] && p.ng >= c && p.ncg >= c) { p.C = c; break; }
+    if ((long long)B * H * nrg <= L->clusters[c] && p.ng >= c && p.ncg >= c) { p.C = c; break; }
   if (p.C == 0) return p;
   p.gs = ceil_div(p.ng, p.C);
   p.gw = ceil_div(p.ncg, p.C);
@@ -832,8 +878,57 @@ SpreadPlan plan_spread(const kvc_layer* L, int B, int R, int T) {
   p.slots = std::min((int)(room / p.slot_bytes), SPR_MAX_SLOTS);
   if (p.slots < 2 || p.ring_off - p.s_off + (uint32_t)p.slots * p.slot_bytes < SPR_WARPS * 8u * SPR_YLD * 4u) return p;
   p.smem = 1024u + (size_t)p.ring_off + (size_t)p.slots * p.slot_bytes;
+  {
+    // us of a call: the looks at pieces, the steps of the two expansions of a warp, its text items, the exchanged weights, the bytes.  Fitted
+    // (non-negative least squares of the relative error, 6 %) to 260 calls on B200: 110 drawn shapes, every number of groups they allow
+    const int items = ceil_div(ceil_div(T_all, 16), p.C * nrg), MG = p.nt > 2 ? 2 : 1, TN = p.nt > 2 ? p.nt / 2 : p.nt;
+    int tasks = 0;
+    for (int x = 0; x < p.npp; ++x) { const int c = std::min(p.pg, p.ng - x * p.pg); tasks += MG == 2 ? (c + 1) & ~1 : c; }
+    const double step = TN * p.terms * MG, pieces = 2.0 * ceil_div(R, p.bpp) * kp + 2.0 * p.npp + ceil_div(items, p.ti);
+    const double mb = ((double)B * H * nrg * p.C * (2.0 * R * p.gs * 4096.0 + items * 8192.0) + 4.0 * H * n * (double)m) * 1e-6;
+    p.us = 5.9 + (nrg > 1 ? 3.6 : 0.0) + 0.336 * pieces + 0.0292 * p.ng * step + 0.0086 * ceil_div(tasks, SPR_WARPS) * p.gw * step +
+           0.45 * ceil_div(items, SPR_WARPS) + 0.0525 * W / 1024.0 + 0.0485 * mb;
+  }
   p.ok = 1;
   return p;
+}
+
+// Groups of blocks per pair: as many as 64 expansion rows each demand, more where the estimate finds the shorter chain of a group worth the
+// merge (us per call: 1 x 31 blocks of n = 576, m = 432, 16/2 heads, 4 groups 40.5, 6 30.1, 8 25.6, the one-kernel path 43.7; 4 x 5 of 1024,
+// 28/4 heads, one 33.1, two 26.5; 1 x 5 of 576, 28/4 heads, one 15.6, two 16.8, three 15.0).  Of the 110 shapes above each takes 14.31 us (geometric
+// mean) with its best number, 14.36 with the chosen one, 15.5 with the smallest, 23.8 on the paths below.
+SpreadPlan plan_spread(const kvc_layer* L, int B, int R, int T) {
+  if (!spread_may_serve(L) || B < 1 || R < 1 || L->G > 16 || T < 0) return SpreadPlan{};
+  if (!tma_rows(spread_theta(L)) || !tma_rows(L->U_rows) || spread_theta_np(L) % 8 || L->U_np % 8) return SpreadPlan{};
+  SpreadPlan best{};
+  for (int nrg = 1; nrg <= SPR_MAX_NRG && nrg <= R; ++nrg) {
+    const SpreadPlan p = plan_groups(L, B, R, T, nrg);
+    if (p.ok && (!best.ok || p.us < best.us)) best = p;
+  }
+  return best;
+}
+
+SpreadWs spread_ws(const kvc_layer* L, const SpreadPlan& p, int B) {
+  SpreadWs w{};
+  const size_t pairs = (size_t)B * L->desc.H_kv, parts = p.ok && p.nrg > 1 ? pairs * p.nrg : 0;
+  size_t off = align_up(sizeof(int) * (pairs + 1), 256);                // behind the status word of the layout all paths share
+  auto take = [&](size_t bytes) { const size_t o = off; off = align_up(off + bytes, 256); return o; };
+  w.off_cnt = take(parts ? sizeof(unsigned long long) * pairs * p.C : 0);
+  w.off_py = take(sizeof(float) * parts * L->G * D);
+  w.off_pml = take(sizeof(float2) * parts * p.C * L->G);
+  w.bytes = off;
+  return w;
+}
+
+// enough for every T: the number of groups depends on the text, whether a number can be had does not
+size_t spread_ws_bytes(const kvc_layer* L, int B, int R) {
+  size_t most = 0;
+  if (!plan_spread(L, B, R, 0).ok) return 0;
+  for (int nrg = 1; nrg <= SPR_MAX_NRG && nrg <= R; ++nrg) {
+    const SpreadPlan p = plan_groups(L, B, R, 0, nrg);
+    if (p.ok) most = std::max(most, spread_ws(L, p, B).bytes);
+  }
+  return most;
 }
 
 template <int NT, int NH, int PL>
@@ -841,7 +936,7 @@ static cudaError_t launch_spread_inst(const CUtensorMap* tm, const SpreadArgs& a
   const cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(spread_decode_kernel<NT, NH, PL>), SPR_DYN_LIMIT);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(a.B * a.H_kv * p.C));
+  cfg.gridDim = dim3((unsigned)(a.B * a.H_kv * p.nrg * p.C));
   cfg.blockDim = dim3(SPR_THREADS);
   cfg.dynamicSmemBytes = p.smem;
   cfg.stream = st;
@@ -867,7 +962,7 @@ static cudaError_t launch_spread_nt(const CUtensorMap* tm, const SpreadArgs& a, 
   }
 }
 
-cudaError_t launch_spread(const kvc_layer* L, const DecodeArgs& d, const SpreadPlan& p, cudaStream_t st, bool* encoded) {
+cudaError_t launch_spread(const kvc_layer* L, const DecodeArgs& d, const SpreadPlan& p, char* ws, cudaStream_t st, bool* encoded) {
   *encoded = false;
   const int B = d.B, H = d.H_kv, R = d.R, m = L->m, n = L->desc.n;
   CUtensorMap tm[6];
@@ -900,6 +995,11 @@ cudaError_t launch_spread(const kvc_layer* L, const DecodeArgs& d, const SpreadP
   a.q = static_cast<const __nv_bfloat16*>(d.q);
   a.mu = static_cast<const __nv_bfloat16*>(d.mu);
   a.out = static_cast<__nv_bfloat16*>(d.out);
+  const SpreadWs w = spread_ws(L, p, B);
+  a.cnt = reinterpret_cast<unsigned long long*>(ws + w.off_cnt);
+  a.py = reinterpret_cast<float*>(ws + w.off_py);
+  a.pml = reinterpret_cast<float2*>(ws + w.off_pml);
+  a.token = d.token; a.nrg = p.nrg; a.rg = p.rg;
   a.status = d.status; a.R_b = d.R_b; a.T_b = d.T_b; a.early = d.early_capsules;
   a.B = B; a.H_kv = H; a.G = d.G; a.R = R; a.m = m; a.n = n; a.T = d.T;
   a.lc = p.C == 8 ? 3 : (p.C == 4 ? 2 : 1); a.ng = p.ng; a.gs = p.gs; a.ncg = p.ncg; a.gw = p.gw; a.nsub = p.nsub; a.gsub = p.gsub; a.wbox = p.wbox;

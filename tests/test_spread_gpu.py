@@ -1,14 +1,16 @@
 """The spread decode path (a cluster of CTAs per (sequence, KV head)) at the sizes where its tiling can go wrong, against the fp64
 oracle: retained lengths and block lengths around the 16-row granules and the slices they are cut into, one to eight row tiles, one and
 two head tiles, two boxes of columns, text lengths around a piece and around what the CTAs share, more pieces than ring slots,
-per-sequence lengths with nothing in some sequences.
+several groups of blocks, per-sequence lengths with nothing in some sequences or groups.
 
 Bound: the regression bound of the parity tests.
 """
 import random
 
 import pytest
+import torch
 
+from paper_2605_16439_b200 import binding as kvc
 from paper_2605_16439_b200 import build as kvc_build
 from paper_2605_16439_b200 import workloads as wl
 
@@ -36,6 +38,9 @@ def _built():
     (1, 16, 1, 11, 4, 30, 800),      # two head tiles, 64 rows
     (2, 24, 2, 17, 2, 129, 500),     # G = 12
     (1, 2, 1, 12, 1, 4097, 600),     # long text
+    (7, 28, 4, 10, 10, 168, 250),    # 70 rows: two groups of blocks
+    (2, 8, 2, 24, 23, 60, 375),      # 92 rows: groups of twelve and eleven blocks
+    (1, 16, 2, 9, 31, 33, 600),      # several groups, fewer text items than CTAs
     (1, 4, 1, 31, 4, 40, 300),       # n = 961, m = 673: six granules per CTA, two terms
 ])
 @pytest.mark.parametrize("recipe", ["peaked", "structured"])
@@ -50,6 +55,7 @@ def test_uniform(B, H_q, H_kv, grid, R, T, ratio, recipe, monkeypatch):
 
 @pytest.mark.parametrize("B,H_q,H_kv,grid,R,T,ratio", [
     (9, 14, 2, 24, 3, 150, 600), (5, 8, 2, 9, 2, 40, 600), (4, 7, 1, 32, 3, 300, 200), (3, 12, 1, 15, 4, 64, 500),
+    (5, 8, 2, 12, 23, 70, 600), (3, 28, 4, 13, 20, 40, 600),
 ])
 def test_per_sequence_lengths(B, H_q, H_kv, grid, R, T, ratio, monkeypatch):
     monkeypatch.setenv("KVC_EXPANSION", "spread")
@@ -61,3 +67,25 @@ def test_per_sequence_lengths(B, H_q, H_kv, grid, R, T, ratio, monkeypatch):
     shape = wl.Shape("spread-ragged", 1, B, H_q, H_kv, 128, grid, R, T, 1, "bf16", ratio)
     counts, _ = tl.check_ragged(shape, 650 + grid, R_b, T_b)
     assert counts["spread"] == 1 and counts["scores"] == 0
+
+
+@pytest.mark.parametrize("B,H_q,H_kv,grid,R,ratio", [(2, 8, 2, 24, 23, 375), (3, 28, 4, 27, 8, 750), (1, 16, 2, 9, 31, 600)])
+def test_workspace_holds_every_shorter_text(B, H_q, H_kv, grid, R, ratio, monkeypatch):
+    """The number of groups a pair's blocks are split into depends on the text: a workspace for T_cap rows serves every T below, and
+    nothing behind it is written."""
+    monkeypatch.setenv("KVC_EXPANSION", "spread")
+    T_cap = 6000
+    shape = wl.Shape("spread-ws", 1, B, H_q, H_kv, 128, grid, R, T_cap, 1, "bf16", ratio)
+    p = tl.make_problem(shape, 690 + grid, T=T_cap, T_cap=T_cap)
+    layer = tl.gpu_layer(shape, p)
+    caps = kvc.alloc_capsules(layer, B, R)
+    kvc.kvc_compress(layer, p["K_vis"].cuda(), p["V_vis"].cuda(), B, R, caps)
+    need = kvc.kvc_workspace_bytes(layer, B, R, T_cap)
+    ws = torch.full((need + (4 << 20),), 0xA5, dtype=torch.uint8, device="cuda")
+    q, K_txt, V_txt = p["q"].cuda(), p["K_txt"].cuda(), p["V_txt"].cuda()
+    out = torch.empty((B, H_q, 128), dtype=torch.bfloat16, device="cuda")
+    for T in (0, 1, 100, 700, 3000, T_cap):
+        counts, _ = tl.launches(lambda: kvc.kvc_decode_attend(layer, q, caps, B, R, K_txt, V_txt, T, T_cap, out, ws))
+        assert counts["spread"] == 1
+        assert kvc.kvc_read_device_status(layer, B, R, T, ws) == 0
+        assert bool((ws[need:] == 0xA5).all()), T
