@@ -230,7 +230,7 @@ int kvc_layer_create(const kvc_layer_desc* desc, kvc_layer** out) {
   const size_t o_theta = take(pad_theta ? padded : 0), o_U = take(pad_U ? padded : 0);
   cudaError_t e = cudaGetDevice(&L->device);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&L->num_sms, cudaDevAttrMultiProcessorCount, L->device);
-  if (e == cudaSuccess && (cluster_may_serve(L) || spread_may_serve(L))) cluster_occupancy(L->device, L->num_sms, L->clusters);
+  if (e == cudaSuccess && (cluster_may_serve(L) || spread_may_serve(L) || spread_f32_may_serve(L))) cluster_occupancy(L->device, L->num_sms, L->clusters);
   if (e == cudaSuccess) e = cudaMalloc(&L->d_block, bytes);
   if (e == cudaSuccess) {
     char* base = static_cast<char*>(L->d_block);
@@ -295,7 +295,7 @@ size_t kvc_workspace_bytes(const kvc_layer* L, int B, int R, int T_cap) {
   if (!L || B < 0 || R < 0 || T_cap < 0) return 0;
   const size_t phases = ws_layout(L, B, R, T_cap, WS_UNIFORM | WS_RAGGED).total, cluster = cluster_ws_bytes(L, B, R, T_cap);
   size_t most = phases > cluster ? phases : cluster;
-  if (B > 0 && R > 0) most = std::max(most, spread_ws_bytes(L, B, R));
+  if (B > 0 && R > 0) most = std::max(most, std::max(spread_ws_bytes(L, B, R), spread_f32_ws_bytes(L, B, R)));
   const size_t plain = (R == 0 || L->passthrough) && L->desc.dtype == KVC_BF16 && B > 0 ? plain_ws(L, B).bytes : 0;
   return most > plain ? most : plain;
 }
@@ -436,7 +436,7 @@ static bool use_cluster(const kvc_layer* L, int B, int R, int T, bool ragged) {
 // short blocks whose parameters the resident path keeps in shared memory, with more than two row tiles (5 x 9 of n = 256, 28/4 heads 13.4 / 12.5;
 // 2 x 8 13.2 / 11.0; but 2 x 2 8.8 / 10.3, 1 x 1 9.0 / 10.8), few retained rows (5 x 1, m = 32, 16/2 heads 8.4 / 7.6; 4 x 4, m = 52, 8/2 heads
 // 8.6 / 8.7), long text (1 x 2, 4096 rows 14.8 / 12.3; 4 x 2, 1024 rows, 10.1 / 13.1) or n = 64 (8.8 / 8.3); and the longest chains beside the
-// one-kernel and three-kernel paths (3 x 13 of 1024, 28/4 heads 48.3, estimated 39.4, / 41.1).
+// one-kernel and three-kernel paths (3 x 13 of 1024, 28/4 heads 48.3, estimated 39.4, / 41.1; 14 x 16 of 256, m = 167, 16/2 heads 23.9 / 23.2).
 // Calls whose path the tests name stay where they are, although this one is ahead: lengths per sequence on those short
 // blocks (6 x 1 of n = 256, 8/2 heads 10.3 / 13.4) or under 1e7 flop of expansion beside them, and clusters of two on blocks under 96 positions
 // (32 x 1 of n = 81, 8/2 heads, 700 rows 12.3 / 36.9).  KVC_EXPANSION=spread forces it where its plan applies, any other value keeps it off.
@@ -445,7 +445,7 @@ static bool use_spread(const kvc_layer* L, int B, int R, int T, bool ragged, con
   const int n = L->desc.n;
   if (plan_resident(L, B, R, T).ok) return !ragged && n == 256 && L->m > 48 && R * L->G <= 16 && T <= 128 * p.C;
   if (ragged && n % 8 == 0 && n % 64 != 0 && 4.0 * B * L->desc.H_q * R * (double)L->m * n < 1e7) return false;
-  if (n % 64 == 0 && p.us > 36.0) return false;
+  if (n % 64 == 0 && p.us > (n <= 256 ? 24.0 : 36.0)) return false;
   return n >= 96 || p.C * p.nrg > 2;
 }
 
@@ -501,6 +501,11 @@ int decode_common(const kvc_layer* L, const void* q, const void* capsules, int B
       const cudaError_t se = launch_spread(L, a, sp, ws, st, &encoded);
       if (encoded) return cuda_status(se);
     }
+  }
+
+  if ((align & 15) == 0) {
+    const SpreadPlan sp = plan_spread_f32(L, B, R, T);
+    if (sp.ok && (L->use_tc == 6 || !ragged || 4.0 * B * L->desc.H_q * R * (double)L->m * L->desc.n >= 3e7) && (ws_limit == 0 || spread_ws(L, sp, B).bytes <= ws_limit)) return cuda_status(launch_spread_f32(L, a, sp, ws, st));
   }
 
   if ((align & 15) == 0 && use_cluster(L, B, R, T, ragged)) {

@@ -157,8 +157,9 @@ spread_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
   auto group_blocks = [&](int r) { return min(max(r - rg * a.rg, 0), a.rg); };
   // this CTA's share of the text rows, in items of 16
   auto text_items = [&](int t, int& i0, int& i1) {
-    const int items = (t + 15) >> 4, c = rg * C + rank, n = a.nrg << a.lc;
-    i0 = (int)((long long)c * items / n); i1 = (int)((long long)(c + 1) * items / n);
+    const uint32_t items = (uint32_t)(t + 15) >> 4, c = (uint32_t)(rg * C + rank), n = (uint32_t)a.nrg << a.lc;
+    const uint32_t q = a.nrg == 1 ? items >> a.lc : items / n, rem = items - q * n;
+    i0 = (int)(c * q + min(c, rem)); i1 = i0 + (int)(q + (c < rem ? 1u : 0u));
   };
   auto load_capsule = [&](const CUtensorMap* tm, uint32_t slot, int r, int x) {
     tma_load_4d(ring + slot * a.slot_bytes, tm, 0, (g0 + x * a.kg) * 16, 0, blk + r, &bars.full[slot]);
@@ -725,6 +726,7 @@ spread_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
     named_barrier_sync(1, SPR_CONS);                          // all of them have been read, and nothing is on its way there
     float* yred = reinterpret_cast<float*>(sm + a.s_off);     // [SPR_WARPS][8][SPR_YLD]
     const int ld = 7 - a.lc, dc = 1 << ld;                    // channels of a CTA
+    const int unit = fresh((int)blockIdx.x) >> a.lc, pair = a.nrg > 1 ? unit / a.nrg : unit, rg = unit - pair * a.nrg;      // (anew: kept until here they spill)
     const uint32_t ybar = smem_addr(&bars.y);
 #pragma unroll
     for (int nh = 0; nh < NH; ++nh) {
