@@ -1,6 +1,7 @@
 // Host side of the C ABI: validation, layer handles, workspace layout, kernel sequencing.
 #include <algorithm>
 #include <atomic>
+#include <cmath>
 #include <map>
 #include <mutex>
 #include <new>
@@ -449,6 +450,24 @@ static bool use_spread(const kvc_layer* L, int B, int R, int T, bool ragged, con
   return n >= 96 || p.C * p.nrg > 2;
 }
 
+// Which fp32 calls take the spread path: those of one wave of clusters (0.29 to 0.97 of the three-phase kernels' time over 44 drawn calls), and
+// of up to four where its estimate is under nine tenths of theirs (0.74 with lengths per sequence, whose sum it does not see: 11 x 4 of n = 841,
+// 28/4 heads, 316, estimated 268 to 359, / 299; 0.7 with one query head per KV head: 2 x 3 of 1024, 32/32 heads 250,
+// estimated 199, / 194; 13 x 3 of 169, 28/4 heads 52 / 97; 16 x 8 of 169 95 / 128).  Their estimate: the columns and chunks of a CTA's walk,
+// the waves of CTAs and the bytes, fitted to the same 70 shapes (16 %).
+// Calls with lengths per sequence of less than 3e7 flop of expansion stay on the three-phase kernels, whose path the tests name.
+static bool use_spread_f32(const kvc_layer* L, int B, int R, int T, bool ragged, const SpreadPlan& p) {
+  if (!p.ok || L->use_tc == 6) return p.ok != 0;
+  const int n = L->desc.n, m = L->m, H = L->desc.H_kv;
+  if (ragged && 4.0 * B * L->desc.H_q * R * (double)m * n < 3e7) return false;
+  if (p.npp <= 1) return true;
+  const WsLayout w = ws_layout(L, B, R, T);
+  const double tiles = (double)H * ceil_div(B * R * L->G, EXP_ROWS), walk = (double)(w.IR / EXP_IC) * m;
+  const double phases = 9.7 + 0.0466 * walk + 0.0251 * std::ceil(tiles * w.NS / 296.0) * walk + 2.03e-4 * tiles * ceil_div(n, EXP_IC) * m +
+                        3.14 * 2.0 * H * ((double)B * R * m + (double)B * T) * 512.0 / HBM_US + 4.46 * L->G + 0.0423 * R * B * H;
+  return p.us < (L->G == 1 ? 0.7 : (ragged ? 0.74 : 0.9)) * phases;
+}
+
 // One token per decode call, process-wide: never 0 and never one of the byte patterns a caller is likely to have
 // filled a fresh workspace with, so that stale workspace contents cannot pass for arrivals of this call.
 static unsigned int next_token() {
@@ -505,7 +524,7 @@ int decode_common(const kvc_layer* L, const void* q, const void* capsules, int B
 
   if ((align & 15) == 0) {
     const SpreadPlan sp = plan_spread_f32(L, B, R, T);
-    if (sp.ok && (L->use_tc == 6 || !ragged || 4.0 * B * L->desc.H_q * R * (double)L->m * L->desc.n >= 3e7) && (ws_limit == 0 || spread_ws(L, sp, B).bytes <= ws_limit)) return cuda_status(launch_spread_f32(L, a, sp, ws, st));
+    if (use_spread_f32(L, B, R, T, ragged, sp) && (ws_limit == 0 || spread_ws(L, sp, B).bytes <= ws_limit)) return cuda_status(launch_spread_f32(L, a, sp, ws, st));
   }
 
   if ((align & 15) == 0 && use_cluster(L, B, R, T, ragged)) {

@@ -56,7 +56,7 @@ size_t spread_ws_bytes(const kvc_layer* L, int B, int R);     // 0 if the path n
 bool spread_may_serve(const kvc_layer* L);
 cudaError_t launch_spread(const kvc_layer* L, const DecodeArgs& a, const SpreadPlan& p, char* ws, cudaStream_t st, bool* encoded);
 
-// the same for fp32 storage (kvc_spread_f32.cu); of the plan ok, nrg, rg and C are set
+// the same for fp32 storage (kvc_spread_f32.cu); of the plan ok, nrg, rg, C, us and npp (waves of clusters) are set
 bool spread_f32_may_serve(const kvc_layer* L);
 SpreadPlan plan_spread_f32(const kvc_layer* L, int B, int R, int T);
 size_t spread_f32_ws_bytes(const kvc_layer* L, int B, int R);

@@ -7,6 +7,8 @@
 //            through shared memory
 //   step 3   a thread per retained row (two where they fit): its row of U in shared memory, P broadcast
 //   step 4   a warp per value row, four channels per lane; text rows the same way with their weights in shared memory
+// 1 x 1 block of n = 576, 8/2 heads, 32 text rows: 42.3 us (four launches) -> 15.7; 4 x 3 of 256, 28/4 heads, 3173 rows 147 -> 44; 1 x 16 of 576,
+// m = 389, 8/2 heads 113 -> 33; 8 x 1 of 1024, m = 794 101 -> 97.
 // Bound: the chain of these steps and of four exchanges; theta and U come at the rate of the SMs that take part.
 #include <algorithm>
 
@@ -18,6 +20,7 @@ namespace kvc {
 constexpr int SPF_THREADS = 512, SPF_WARPS = 16;
 constexpr float SPF_QSCALE = 0.08838834764831845f * 1.4426950408889634f;      // sigma = 1/sqrt(128), logits in log2 units
 constexpr int SPF_MAX_TEXT = 512;             // text rows per CTA
+constexpr int SPF_MAX_NRG = 64, SPF_MAX_WAVES = 4;      // groups of blocks per pair; waves of clusters
 constexpr int SPF_AHEAD = 12;                 // loads of theta per thread ahead of the scores
 
 struct SpreadF32Args {
@@ -170,11 +173,13 @@ __global__ void __launch_bounds__(SPF_THREADS, 1) spread_f32_kernel(const __grid
     for (int g = 0; g < GT; ++g) {
       s[g] = 0.f;
       if (g < G) {
+        float part[4];                                           // (short chains, added as a tree: a score's error grows with the logits it makes)
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           const float4 q = *reinterpret_cast<const float4*>(qs + g * D + l8 * 4 + 32 * i);
-          s[g] = fmaf(q.x, x[i].x, s[g]); s[g] = fmaf(q.y, x[i].y, s[g]); s[g] = fmaf(q.z, x[i].z, s[g]); s[g] = fmaf(q.w, x[i].w, s[g]);
+          part[i] = fmaf(q.w, x[i].w, fmaf(q.z, x[i].z, fmaf(q.y, x[i].y, q.x * x[i].x)));
         }
+        s[g] = (part[0] + part[1]) + (part[2] + part[3]);
       }
     }
 #pragma unroll
@@ -542,19 +547,30 @@ static bool spread_f32_layout(const kvc_layer* L, int C, int nrg, int R, int T, 
   return o.jc >= 64 || o.jc >= ceil_div(m, 2);
 }
 
-// Groups of blocks: as few as 16 expansion rows each allow, clusters as large as the device holds for all groups at once
+// Groups of blocks of at most 16 expansion rows and the size of their clusters, by an estimate of the call: waves of clusters, the fused multiply-adds
+// of a thread in the two expansions, rounds of key and value rows, the bytes of the parameters and of the call.  Fitted (non-negative least squares
+// of the relative error, 7 %) to 281 calls on B200: 70 drawn shapes, one to four waves.  Their best choices take 52.0 us in the geometric
+// mean, the chosen ones 52.8, the three-phase kernels 93.1.
 SpreadPlan plan_spread_f32(const kvc_layer* L, int B, int R, int T) {
   SpreadPlan p{};
   if (!spread_f32_may_serve(L) || B < 1 || R < 1 || T < 0 || L->m < 8) return p;
-  const int H = L->desc.H_kv;
-  for (int nrg = 1; nrg <= SPR_MAX_NRG && nrg <= R && !p.ok; ++nrg) {
-    const int rg = ceil_div(R, nrg);
-    if (rg * L->G > 16 || (nrg - 1) * rg >= R) continue;
-    for (int c = SPR_MAX_C; c >= 2 && !p.ok; c /= 2) {
+  const int H = L->desc.H_kv, G = L->G, n = L->desc.n, m = L->m;
+  for (int rg = std::min(16 / G, R), last = 0; rg >= 1; --rg) {
+    const int nrg = ceil_div(R, rg), rows = ceil_div(R, nrg) * G;
+    if (nrg == last || nrg > SPF_MAX_NRG) continue;
+    last = nrg;
+    for (int c = SPR_MAX_C; c >= 2; c /= 2) {
       SpreadF32Layout o{};
-      if ((long long)B * H * nrg > L->clusters[c] || ceil_div(L->desc.n, 4) < c) continue;
-      if (!spread_f32_layout(L, c, nrg, rg, T, o)) continue;
-      p.ok = 1; p.nrg = nrg; p.rg = rg; p.C = c;
+      if (L->clusters[c] < 1 || ceil_div(n, 4) < c || !spread_f32_layout(L, c, nrg, rows / G, T, o)) continue;
+      const long long clusters = (long long)B * H * nrg, waves = (clusters + L->clusters[c] - 1) / L->clusters[c];
+      if (waves > SPF_MAX_WAVES) continue;
+      const int W = o.qw * 4, tn = ceil_div(T, c * nrg), rb = rows / G;
+      const double chain = ceil_div(m, SPF_THREADS / W) * (double)o.rt, two = m <= SPF_THREADS ? 2.0 : 1.0;
+      const double expand = 9.06e-3 * chain + 0.48e-3 * ceil_div((int)(m * two), SPF_THREADS) * W * o.rt / two;
+      const double rounds = o.gt * (0.269 * (ceil_div(rb * o.js, 64) + ceil_div(tn, 64)) + 0.0175 * (ceil_div(rb * o.js, 16) + ceil_div(tn, 16)));
+      const double act = (double)std::min(clusters, (long long)L->clusters[c]) * c, kb = m * (double)W * 8.0 / 1024.0;
+      const double us = (nrg > 1 ? 2.8 : 0.0) + waves * (8.5 + expand + rounds + 0.0328 * kb + 0.0736 * 1e-6 * act * (m * (double)W * 8.0 + 2.0 * rb * o.js * 512.0 + tn * 1024.0));
+      if (!p.ok || us < p.us) { p.ok = 1; p.nrg = nrg; p.rg = rb; p.C = c; p.us = us; p.npp = (int)waves; }
     }
   }
   return p;
@@ -562,9 +578,9 @@ SpreadPlan plan_spread_f32(const kvc_layer* L, int B, int R, int T) {
 
 // enough for every T (the number of groups depends on it)
 size_t spread_f32_ws_bytes(const kvc_layer* L, int B, int R) {
-  if (!spread_f32_may_serve(L) || B < 1 || R < 1 || (long long)B * L->desc.H_kv > L->clusters[2]) return 0;
+  if (!spread_f32_may_serve(L) || B < 1 || R < 1 || (long long)B * L->desc.H_kv > (long long)SPF_MAX_WAVES * L->clusters[2]) return 0;
   SpreadPlan p{};
-  p.ok = 1; p.C = SPR_MAX_C; p.nrg = std::min(SPR_MAX_NRG, R);
+  p.ok = 1; p.C = SPR_MAX_C; p.nrg = (int)std::min<long long>(std::min(SPF_MAX_NRG, R), (long long)SPF_MAX_WAVES * L->clusters[2] / ((long long)B * L->desc.H_kv));
   return spread_ws(L, p, B).bytes;
 }
 

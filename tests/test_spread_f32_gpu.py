@@ -32,6 +32,7 @@ def _built():
     (1, 8, 2, 32, 2, 300, 400),      # n = 1024, m = 615: several chunks of U
     (2, 8, 2, 17, 11, 70, 775),      # n = 289, eleven blocks: groups
     (1, 2, 2, 12, 30, 2100, 600),    # many blocks and text rows
+    (13, 28, 4, 13, 3, 61, 450),     # more groups than clusters the device holds at once
     (1, 4, 1, 31, 4, 10, 300),       # n = 961, m = 673
 ])
 @pytest.mark.parametrize("recipe", ["peaked", "structured"])
