@@ -2,7 +2,7 @@
 //
 // Bound: a chain of dependent steps, four of them exchanges within a cluster of 0.5-1 us; the bytes take a tenth to a half of the time.
 // Measured on B200, us per call, before / now: 1 x 5 blocks of n = 576, 32/32 heads, 128 text rows (the one-kernel path on 32 SMs) 25.5 /
-// 13.1, its time line: scores until 2.5 us after the previous kernel's end, logits 4.2, probabilities 4.9, text 5.3, weights 6.4 (at their
+// 12.8, its time line: scores until 2.5 us after the previous kernel's end, logits 4.2, probabilities 4.9, text 5.3, weights 6.4 (at their
 // owners 7.4), values 9.1, out 10.4; 8 x 5 of n = 729, 28/4 heads (the cluster path) 36.2 / 27.0; 1 x 5 of 576, 28/4 heads 25.5 / 15.3; 7 x 2
 // of 576, m = 404, 38.0 / 14.8; 4 x 5 of 1024, m = 103 (three kernels) 21.1 / 12.6; 1 x 1 of 576, 8/2 heads, 16384 text rows 170 / 21.
 // Why pieces are few and large: a look at a piece by all warps, with its loops, takes some 200 cycles, issuing one some 300 (pieces of 16 KB,
@@ -278,6 +278,10 @@ spread_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
     };
     auto peer_wait = [&](uint64_t* bar) { if (!dead && !mbar_wait_cluster_bounded(bar, 0u)) dead = true; };
 
+    if (tid < D >> a.lc) mus[tid] = __bfloat162float(a.mu[h * D + rank * (D >> a.lc) + tid]);      // (a parameter)
+    // reciprocals for the divisions of small numbers below, made while the previous kernel runs
+    const uint32_t inv_full = (65536u + (uint32_t)a.kg - 1u) / (uint32_t)a.kg, cnt_last = (uint32_t)(gown - (kp - 1) * a.kg), inv_last = (65536u + cnt_last - 1u) / cnt_last;
+    const float inv_ng = 1.f / (float)a.ng;
     if (tid < 2 * G) prefetch_l2(a.q + ((size_t)pair * G) * D + tid * 64);      // consumes nothing: may run before the wait
     grid_dep_wait();
     grid_dep_launch();
@@ -301,7 +305,6 @@ spread_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
       *reinterpret_cast<uint4*>(sm + a.q_off + (uint32_t)g * SPR_QPITCH + c * 16u) =
           g < G ? *reinterpret_cast<const uint4*>(a.q + ((size_t)pair * G + g) * D + c * 8) : make_uint4(0, 0, 0, 0);
     }
-    if (tid < D >> a.lc) mus[tid] = __bfloat162float(a.mu[h * D + rank * (D >> a.lc) + tid]);
     const uint32_t q_u = smem_addr(sm + a.q_off) + (uint32_t)lrowA * SPR_QPITCH + (uint32_t)lhi * 16u;
     // 16 key rows (halves of 64 channels `half` bytes apart): c[8-key tile] = logits of (head gid (+8), keys 2 t4, + 1), in log2 units
     auto score16 = [&](uint32_t base, uint32_t half, float (&c)[2][4]) {
@@ -455,7 +458,7 @@ spread_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
           for (int x = 0; x < kp; ++x) {
             const uint32_t pc = smem_addr(acquire());
             const int cnt = min(a.kg, gown - x * a.kg), tasks = min(a.bpp, Re - r0) * cnt;
-            const uint32_t inv = (65536u + (uint32_t)cnt - 1u) / (uint32_t)cnt;      // first / cnt for the few tasks of a piece
+            const uint32_t inv = x + 1 < kp ? inv_full : inv_last;      // first / cnt for the few tasks of a piece
 #pragma unroll 1
             for (; first < tasks; first += SPR_WARPS) {
               const int bl = (int)((uint32_t)first * inv >> 16), gi = first - bl * cnt, r = r0 + bl;
@@ -625,7 +628,7 @@ spread_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
           for (int g = 0; g < MG; ++g) {
             const int k = p * a.pg + kp0 + g;
             if (g > 0 && kp0 + g >= cnt) break;
-            const int own = ((k + 1) * C - 1) / a.ng, kl = k - (own * a.ng >> a.lc);
+            const int own = (int)(((float)((k + 1) * C - 1) + 0.5f) * inv_ng), kl = k - (own * a.ng >> a.lc);
             const uint32_t bar = map_to_cta(smem_addr(&bars.w), (uint32_t)own);
             const uint32_t dst = map_to_cta(s_u + (uint32_t)(((rank * a.gs + kl) * 16 + gid) * RW + part * TN * 8 + 2 * t4) * 4u, (uint32_t)own);
 #pragma unroll
@@ -694,7 +697,7 @@ spread_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
         for (int x = 0; x < kp; ++x) {
           const uint32_t pc = smem_addr(acquire());
           const int cnt = min(a.kg, gown - x * a.kg), tasks = min(a.bpp, Re - r0) * cnt;
-          const uint32_t inv = (65536u + (uint32_t)cnt - 1u) / (uint32_t)cnt;
+          const uint32_t inv = x + 1 < kp ? inv_full : inv_last;
 #pragma unroll 1
           for (; first < tasks; first += SPR_WARPS) {
             const int bl = (int)((uint32_t)first * inv >> 16), gi = first - bl * cnt, r = r0 + bl;
@@ -863,8 +866,9 @@ static SpreadPlan plan_groups(const kvc_layer* L, int B, int R_all, int T_all, i
   p.p_off = take((uint32_t)(p.terms * RP * (p.gw * 16 + 8) * 2));
   p.ring_off = (off + 1023u) & ~1023u;
   if (p.ring_off + 1024u + 4u * 8192u >= SPR_DYN_LIMIT) return p;
-  // A piece is looked at by every warp (about 200 cycles a look): few large ones, five of which fill the ring
-  const uint32_t room = (uint32_t)SPR_DYN_LIMIT - 1024u - p.ring_off, want = room / 5 & ~1023u;
+  // A piece is looked at by every warp (about 200 cycles a look): few large ones, five of which fill the ring, four with a single row tile (1 x 5
+  // blocks of n = 576, 32/32 heads: 12.8 us, five 13.2, seven 14.2; 2 x 4 of 1024, 32/8 heads, two tiles: 18.5, 17.5, 19.5)
+  const uint32_t room = (uint32_t)SPR_DYN_LIMIT - 1024u - p.ring_off, want = room / (p.nt == 1 ? 4u : 5u) & ~1023u;
   const int kp = ceil_div(p.gs, 16);
   p.kg = ceil_div(p.gs, kp);
   p.bpp = std::max(1, std::min(kp > 1 ? 1 : R, (int)(want / ((uint32_t)p.kg * 4096u))));
