@@ -22,7 +22,9 @@ constexpr int FIT_TILE = 64;            // covariance tile per CTA
 constexpr int FIT_KC = 32;              // channels per staged chunk
 constexpr int FIT_SPLITS = 4;            // parts of the samples, one per matrix of the workspace
 constexpr int FIT_MAX_SWEEPS = 40;
-constexpr float FIT_COS_TOL2 = 1e-20f;  // one-sided: stop after a sweep whose largest squared cosine between two columns was below this
+// one-sided: stop after a sweep whose largest squared cosine between two columns was below this.  Convergence is quadratic: from 1e-11 that sweep
+// leaves at most 2e-19 (fields of 34 to 256 positions in numpy; 3e-12 -> 2e-23, 6e-10 -> 2e-21), cosines far below the outputs' rounding
+constexpr float FIT_COS_TOL2 = 1e-11f;
 constexpr double FIT_OFF_TOL2 = 1e-22;  // stop when (off-diagonal norm / diagonal norm)^2 falls below this
 
 static inline int even_up(int x) { return (x + 1) & ~1; }
@@ -414,11 +416,19 @@ __global__ void __launch_bounds__(256) fit_emit_theta_kernel(const double* __res
 // double precision a rotation took 1.05 us instead of 0.89 (both with their share of the rounds).
 // tau = 1e-5 of the largest diagonal entry keeps the columns of a rank-deficient matrix away from zero, so that its null space gets
 // orthonormal vectors too.
-template <int EPL>
+__device__ __forceinline__ double ld_cluster_f64(uint32_t caddr) {
+  double v;
+  asm volatile("ld.shared::cluster.f64 %0, [%1];\n" : "=d"(v) : "r"(caddr) : "memory");
+  return v;
+}
+
+// DS: the columns stay in shared memory, in two buffers (a round reads the peers' last one and writes the other); otherwise through L2
+template <int EPL, bool DS>
 __global__ void __launch_bounds__(640, 1) jacobi_cluster_kernel(double* __restrict__ ws, size_t head_stride, size_t off_A, size_t off_Q,
                                                                 size_t off_flag, int size, int C, int bs) {
   constexpr int LD = 32 * EPL;
-  extern __shared__ __align__(16) double cols[];                 // [2 bs][LD]
+  extern __shared__ __align__(16) double cols_all[];             // [DS ? 2 : 1][2 bs][LD]
+  double* cols = cols_all;
   __shared__ double s_red[32], s_norm[40];                       // s_norm: squared lengths of the block columns
   __shared__ float s_max[32];
   const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31, nw = bs;
@@ -510,8 +520,20 @@ __global__ void __launch_bounds__(640, 1) jacobi_cluster_kernel(double* __restri
       const int p = at(c) * bs + w, q = at(NB - 1 - c) * bs + w;
       double a[EPL], b[EPL];
       const bool shift = sweep == 0 && br == 0;
-      fetch(a, p, shift);
-      fetch(b, q, shift);
+      if (!DS || shift) {
+        fetch(a, p, shift);
+        fetch(b, q, shift);
+      } else {
+        // the block now in place x was in place x - 1 (the last for the first, block 0 stays), of CTA x or NB - 1 - x
+        auto from = [&](int pos) {
+          const int was = pos == 0 ? 0 : (pos == 1 ? NB - 1 : pos - 1);
+          return map_to_cta(smem_addr(cols + (size_t)((was < C ? 0 : bs) + w) * LD + lane), (uint32_t)(was < C ? was : NB - 1 - was));
+        };
+        const uint32_t fa = from(c), fb = from(NB - 1 - c);
+#pragma unroll
+        for (int e = 0; e < EPL; ++e) { a[e] = ld_cluster_f64(fa + e * 256u); b[e] = ld_cluster_f64(fb + e * 256u); }
+        cols = cols == cols_all ? cols_all + (size_t)2 * bs * LD : cols_all;
+      }
       double na = length2(a), nb = length2(b);
       put(b, bs + w);
       if (lane == 0) s_norm[bs + w] = nb;
@@ -548,9 +570,13 @@ __global__ void __launch_bounds__(640, 1) jacobi_cluster_kernel(double* __restri
           __syncthreads();
         }
       }
-      save(a, p);
-      get(b, bs + w);
-      save(b, q);
+      if (DS) {
+        put(a, w);
+      } else {
+        save(a, p);
+        get(b, bs + w);
+        save(b, q);
+      }
       if (br == NB - 2) {
         if (lane == 0) s_max[w] = mx;
         __syncthreads();
@@ -567,13 +593,19 @@ __global__ void __launch_bounds__(640, 1) jacobi_cluster_kernel(double* __restri
     if (worst < FIT_COS_TOL2) break;
   }
 
+  // the columns a warp finishes: the two it holds after the last round, or any two
+  auto place_of = [&](int x) {
+    if (!DS) return (2 * c + x) * bs + w;
+    const int pos = x ? NB - 1 - c : c, br = NB - 2;
+    return (pos == 0 ? 0 : (pos - 1 - br + 2 * (NB - 1)) % (NB - 1) + 1) * bs + w;
+  };
   // eigenvalues and eigenvectors: Q[i][col] = column / its length, A[col][col] = length - tau
   double len[2];
 #pragma unroll
   for (int x = 0; x < 2; ++x) {
-    const int col = (2 * c + x) * bs + w;
+    const int col = place_of(x);
     double a[EPL];
-    fetch(a, col, false);
+    if (DS) get(a, x * bs + w); else fetch(a, col, false);
     const double al = length2(a);
     len[x] = sqrt(al);
     const double inv = al > 0.0 ? 1.0 / len[x] : 0.0;
@@ -586,7 +618,7 @@ __global__ void __launch_bounds__(640, 1) jacobi_cluster_kernel(double* __restri
   cluster_sync_all();                                            // every column has been read
 #pragma unroll
   for (int x = 0; x < 2; ++x) {
-    const int col = (2 * c + x) * bs + w;
+    const int col = place_of(x);
     if (lane == 0 && col < size) A[(size_t)col * size + col] = (len[x] - tau) * (tau < 1.0 ? big : 0.0);
   }
   if (c == 0 && tid == 0) reinterpret_cast<int*>(flag)[60] = sweep;
@@ -596,13 +628,14 @@ __global__ void __launch_bounds__(640, 1) jacobi_cluster_kernel(double* __restri
 template <int EPL>
 static cudaError_t launch_jacobi_cluster(double* ws, size_t head_stride, size_t off_A, size_t off_Q, size_t off_flag, int H, int size,
                                          cudaStream_t st, bool* used) {
-  const void* fn = reinterpret_cast<const void*>(jacobi_cluster_kernel<EPL>);
+  constexpr bool DS = EPL <= 12;               // two buffers of columns fit shared memory up to 384 indices
+  const void* fn = reinterpret_cast<const void*>(jacobi_cluster_kernel<EPL, DS>);
   *used = false;
   int C = ceil_div(size, 16);
   C = C > 16 ? 16 : C;
   const int bs = ceil_div(size, 2 * C);
   if (bs > 20) return cudaSuccess;
-  const size_t smem = sizeof(double) * 2 * (size_t)bs * 32 * EPL;
+  const size_t smem = sizeof(double) * (DS ? 4 : 2) * (size_t)bs * 32 * EPL;
   cudaError_t e = ensure_dynamic_smem(fn, smem);
   if (e != cudaSuccess) return e;
   if (C > 8) e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
@@ -620,7 +653,7 @@ static cudaError_t launch_jacobi_cluster(double* ws, size_t head_stride, size_t 
   int fit = 0;
   if (C > 8 && (cudaOccupancyMaxActiveClusters(&fit, fn, &cfg) != cudaSuccess || fit < 1)) { cudaGetLastError(); return cudaSuccess; }
   *used = true;
-  return cudaLaunchKernelEx(&cfg, jacobi_cluster_kernel<EPL>, ws, head_stride, off_A, off_Q, off_flag, size, C, bs);
+  return cudaLaunchKernelEx(&cfg, jacobi_cluster_kernel<EPL, DS>, ws, head_stride, off_A, off_Q, off_flag, size, C, bs);
 }
 
 // ---- host side -------------------------------------------------------------------------------------------------
