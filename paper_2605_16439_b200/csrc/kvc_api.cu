@@ -447,6 +447,16 @@ static bool use_spread(const kvc_layer* L, int B, int R, int T, bool ragged, con
   if (plan_resident(L, B, R, T).ok) return !ragged && n == 256 && L->m > 48 && R * L->G <= 16 && T <= 128 * p.C;
   if (ragged && n % 8 == 0 && n % 64 != 0 && 4.0 * B * L->desc.H_q * R * (double)L->m * n < 1e7) return false;
   if (n % 64 == 0 && p.us > (n <= 256 ? 24.0 : 36.0)) return false;
+  if (p.waves > 1) {
+    // several waves: where it is ahead of an estimate of the cluster path (rounds of units and their tiles, the bytes; fitted to 97 uniform calls,
+    // 10 %).  Routed by it those take 0.89 of their time before in the geometric mean, none more than 3 % longer (16 x 8 of n = 144, 28/4
+    // heads, 715 rows 16.5 / 32.3; 25 x 5 of 400, 1610 rows 46 / 89; 8 x 7 of 324, 32/32 heads 74 / 88; not: 26 x 10 of 121 45 / 34)
+    const int H = L->desc.H_kv, units = H * ceil_div(B * R, CL_ROWS / L->G), NS = ceil_div(ceil_div(n, 64), n % 8 ? 2 : 4);
+    const int held = (L->num_sms > 0 ? L->num_sms : 148) * 88 / 100 / NS, rounds = ceil_div(units, held > 0 ? held : 1);
+    const double rows = 512.0 * B * R * H * (double)L->m + 4.0 * H * (double)L->m * n, text = 512.0 * B * H * (double)T;
+    const double cluster = rounds * (24.4 + 1.93 * ceil_div(L->m, 64)) - 4.2 + (1.71 * rows + 1.86 * text) / HBM_US + 0.0137 * B * H;
+    return !ragged && n >= 96 && p.us < 0.85 * cluster;
+  }
   return n >= 96 || p.C * p.nrg > 2;
 }
 
@@ -460,7 +470,7 @@ static bool use_spread_f32(const kvc_layer* L, int B, int R, int T, bool ragged,
   if (!p.ok || L->use_tc == 6) return p.ok != 0;
   const int n = L->desc.n, m = L->m, H = L->desc.H_kv;
   if (ragged && 4.0 * B * L->desc.H_q * R * (double)m * n < 3e7) return false;
-  if (p.npp <= 1) return true;
+  if (p.waves <= 1) return true;
   const WsLayout w = ws_layout(L, B, R, T);
   const double tiles = (double)H * ceil_div(B * R * L->G, EXP_ROWS), walk = (double)(w.IR / EXP_IC) * m;
   const double phases = 9.7 + 0.0466 * walk + 0.0251 * std::ceil(tiles * w.NS / 296.0) * walk + 2.03e-4 * tiles * ceil_div(n, EXP_IC) * m +

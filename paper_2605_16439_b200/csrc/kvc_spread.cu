@@ -832,7 +832,8 @@ bool spread_may_serve(const kvc_layer* L) {
   return L->desc.dtype == KVC_BF16 && !L->passthrough && L->mode == KVC_MODE_KV && L->desc.n >= 64 && (L->use_tc == 0 || L->use_tc == 6);
 }
 
-static SpreadPlan plan_groups(const kvc_layer* L, int B, int R_all, int T_all, int nrg) {
+// most_waves: 1: clusters for all groups at once; more: clusters of two, in that many waves at most
+static SpreadPlan plan_groups(const kvc_layer* L, int B, int R_all, int T_all, int nrg, int most_waves) {
   SpreadPlan p{};
   const int R = ceil_div(R_all, nrg), T = ceil_div(T_all, nrg);
   const int G = L->G, n = L->desc.n, m = L->m, H = L->desc.H_kv;
@@ -842,6 +843,11 @@ static SpreadPlan plan_groups(const kvc_layer* L, int B, int R_all, int T_all, i
   p.ncg = ceil_div(n, 16);
   for (int c = SPR_MAX_C; c >= 2; c /= 2)
     if ((long long)B * H * nrg <= L->clusters[c] && p.ng >= c && p.ncg >= c) { p.C = c; break; }
+  p.waves = 1;
+  if (p.C == 0 && most_waves > 1 && L->clusters[2] > 0 && p.ng >= 2 && p.ncg >= 2) {
+    const long long w = ((long long)B * H * nrg + L->clusters[2] - 1) / L->clusters[2];
+    if (w <= most_waves) { p.C = 2; p.waves = (int)w; }
+  }
   if (p.C == 0) return p;
   p.gs = ceil_div(p.ng, p.C);
   p.gw = ceil_div(p.ncg, p.C);
@@ -891,9 +897,12 @@ static SpreadPlan plan_groups(const kvc_layer* L, int B, int R_all, int T_all, i
     int tasks = 0;
     for (int x = 0; x < p.npp; ++x) { const int c = std::min(p.pg, p.ng - x * p.pg); tasks += MG == 2 ? (c + 1) & ~1 : c; }
     const double step = TN * p.terms * MG, pieces = 2.0 * ceil_div(R, p.bpp) * kp + 2.0 * p.npp + ceil_div(items, p.ti);
-    const double mb = ((double)B * H * nrg * p.C * (2.0 * R * p.gs * 4096.0 + items * 8192.0) + 4.0 * H * n * (double)m) * 1e-6;
+    const double at_once = p.waves > 1 ? L->clusters[2] : (double)B * H * nrg;
+    const double mb = (at_once * p.C * (2.0 * R * p.gs * 4096.0 + items * 8192.0) + 4.0 * H * n * (double)m) * 1e-6;
     p.us = 5.9 + (nrg > 1 ? 3.6 : 0.0) + 0.336 * pieces + 0.0292 * p.ng * step + 0.0086 * ceil_div(tasks, SPR_WARPS) * p.gw * step +
            0.45 * ceil_div(items, SPR_WARPS) + 0.0525 * W / 1024.0 + 0.0485 * mb;
+    // (394 calls of 220 shapes, one to four waves: 6 %)
+    if (p.waves > 1) p.us = 0.9 + p.waves * (0.63 + 0.86 * p.us);
   }
   p.ok = 1;
   return p;
@@ -908,8 +917,14 @@ SpreadPlan plan_spread(const kvc_layer* L, int B, int R, int T) {
   if (!tma_rows(spread_theta(L)) || !tma_rows(L->U_rows) || spread_theta_np(L) % 8 || L->U_np % 8) return SpreadPlan{};
   SpreadPlan best{};
   for (int nrg = 1; nrg <= SPR_MAX_NRG && nrg <= R; ++nrg) {
-    const SpreadPlan p = plan_groups(L, B, R, T, nrg);
+    const SpreadPlan p = plan_groups(L, B, R, T, nrg, 1);
     if (p.ok && (!best.ok || p.us < best.us)) best = p;
+  }
+  // more groups than clusters the device holds: beside the paths for block lengths off 64 only (the others are ahead of a second wave: 30 x 2
+  // blocks of n = 576, 28/4 heads 43 / 21.5; 21 x 2 of 1024 79 / 70)
+  for (int nrg = 1; !best.ok && L->desc.n % 64 != 0 && nrg <= SPR_MAX_NRG && nrg <= R; ++nrg) {
+    const SpreadPlan p = plan_groups(L, B, R, T, nrg, SPR_MAX_WAVES);
+    if (p.ok) best = p;
   }
   return best;
 }
@@ -931,7 +946,7 @@ size_t spread_ws_bytes(const kvc_layer* L, int B, int R) {
   size_t most = 0;
   if (!plan_spread(L, B, R, 0).ok) return 0;
   for (int nrg = 1; nrg <= SPR_MAX_NRG && nrg <= R; ++nrg) {
-    const SpreadPlan p = plan_groups(L, B, R, 0, nrg);
+    const SpreadPlan p = plan_groups(L, B, R, 0, nrg, SPR_MAX_WAVES);
     if (p.ok) most = std::max(most, spread_ws(L, p, B).bytes);
   }
   return most;

@@ -22,6 +22,7 @@ constexpr int SPR_THREADS = SPR_CONS + 32;            // + TMA producer
 constexpr int SPR_MAX_C = 8;
 constexpr int SPR_MAX_SLOTS = 24;
 constexpr int SPR_MAX_NRG = 8;
+constexpr int SPR_MAX_WAVES = 4;
 constexpr uint32_t SPR_QPITCH = 272;                  // bytes per staged query row (conflict-free ldmatrix)
 constexpr int SPR_YLD = 132;                          // pitch of a head's row in the reduction over the warps
 
@@ -29,6 +30,7 @@ struct SpreadPlan {
   int ok;
   int nrg, rg;           // groups of blocks per (sequence, KV head), blocks of a group
   int C;                 // CTAs per group
+  int waves;             // of clusters
   int nt;                // 8-row tiles of expansion rows (1, 2, 4, 6, 8)
   int terms;             // bf16 terms of S and P
   int ng, gs;            // 16-row granules of the m axis, and the most of them a CTA has
@@ -56,7 +58,7 @@ size_t spread_ws_bytes(const kvc_layer* L, int B, int R);     // 0 if the path n
 bool spread_may_serve(const kvc_layer* L);
 cudaError_t launch_spread(const kvc_layer* L, const DecodeArgs& a, const SpreadPlan& p, char* ws, cudaStream_t st, bool* encoded);
 
-// the same for fp32 storage (kvc_spread_f32.cu); of the plan ok, nrg, rg, C, us and npp (waves of clusters) are set
+// the same for fp32 storage (kvc_spread_f32.cu); of the plan ok, nrg, rg, C, waves and us are set
 bool spread_f32_may_serve(const kvc_layer* L);
 SpreadPlan plan_spread_f32(const kvc_layer* L, int B, int R, int T);
 size_t spread_f32_ws_bytes(const kvc_layer* L, int B, int R);

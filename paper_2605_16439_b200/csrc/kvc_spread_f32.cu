@@ -570,7 +570,7 @@ SpreadPlan plan_spread_f32(const kvc_layer* L, int B, int R, int T) {
       const double rounds = o.gt * (0.269 * (ceil_div(rb * o.js, 64) + ceil_div(tn, 64)) + 0.0175 * (ceil_div(rb * o.js, 16) + ceil_div(tn, 16)));
       const double act = (double)std::min(clusters, (long long)L->clusters[c]) * c, kb = m * (double)W * 8.0 / 1024.0;
       const double us = (nrg > 1 ? 2.8 : 0.0) + waves * (8.5 + expand + rounds + 0.0328 * kb + 0.0736 * 1e-6 * act * (m * (double)W * 8.0 + 2.0 * rb * o.js * 512.0 + tn * 1024.0));
-      if (!p.ok || us < p.us) { p.ok = 1; p.nrg = nrg; p.rg = rb; p.C = c; p.us = us; p.npp = (int)waves; }
+      if (!p.ok || us < p.us) { p.ok = 1; p.nrg = nrg; p.rg = rb; p.C = c; p.us = us; p.waves = (int)waves; }
     }
   }
   return p;

@@ -41,6 +41,8 @@ def _built():
     (7, 28, 4, 10, 10, 168, 250),    # 70 rows: two groups of blocks
     (2, 8, 2, 24, 23, 60, 375),      # 92 rows: groups of twelve and eleven blocks
     (1, 16, 2, 9, 31, 33, 600),      # several groups, fewer text items than CTAs
+    (24, 28, 4, 12, 2, 40, 600),     # more pairs than clusters the device holds at once
+    (11, 32, 8, 11, 18, 30, 600),    # the same with groups
     (1, 4, 1, 31, 4, 40, 300),       # n = 961, m = 673: six granules per CTA, two terms
 ])
 @pytest.mark.parametrize("recipe", ["peaked", "structured"])
