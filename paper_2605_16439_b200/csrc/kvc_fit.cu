@@ -407,15 +407,22 @@ __global__ void __launch_bounds__(256) fit_emit_theta_kernel(const double* __res
 // them one after the other per sweep whatever the machine's width, 11 to 14 sweeps.  So everything else is taken out of that chain: a
 // cluster of C CTAs owns a matrix, its columns form 2 C blocks of bs, in each of the 2 C - 1 rounds of a sweep a CTA holds two blocks
 // in shared memory (a warp per pair, the first block's column kept in registers) and rotates all pairs between them (in the first
-// round also those inside), and between rounds the columns go through L2 behind one cluster barrier (about 3 us); no launch, no host
-// round trip.  n = 256, 4 heads on B200: 3.2 ms (n = 103: 0.85 ms); the two-sided form took two launches of 4 us per round, 24 and 8 ms.
-// Half as many CTAs with twice the warps: 3.8 ms (the rotations of 16 warps are bound by shared memory).
-// The angle is taken in single precision: it only steers the convergence (off-diagonal cosines fall by 1e-7 at worst per sweep once
-// they are small); cosine and sine are made from its tangent in double precision, so that the rotation is orthogonal.  The squared
-// lengths that the angle needs are carried along and taken anew in every round; with them as two more dot products and the angle in
+// round also those inside), and between rounds the columns go to their next CTA behind one cluster barrier: through distributed shared
+// memory up to 384 indices, beyond that (two buffers don't fit) through L2 (about 3 us per round); no launch, no host round trip.  Both
+// fits of n = 256, m = 154, 4 heads on B200: 3.9 ms (4.3 with the divisions and the square root of the angle
+// rounded exactly and everything behind the dot product, 4.6 through L2; the two-sided form, two launches of 4 us per round, above 24).
+// Half as many CTAs with twice the warps took a fifth longer (the rotations of 16 warps are bound by shared memory).
+// The angle is taken in single precision, with approximate divisions: it only steers the convergence (off-diagonal cosines fall by 1e-7
+// at worst per sweep once they are small); cosine and sine are made from its tangent in double precision, so that the rotation is
+// orthogonal.  The squared lengths that the angle needs are carried along and taken anew in every round; with them as two more dot products and the angle in
 // double precision a rotation took 1.05 us instead of 0.89 (both with their share of the rounds).
 // tau = 1e-5 of the largest diagonal entry keeps the columns of a rank-deficient matrix away from zero, so that its null space gets
 // orthonormal vectors too.
+__device__ __forceinline__ float sqrt_approx(float x) {
+  float y;
+  asm("sqrt.approx.f32 %0, %1;\n" : "=f"(y) : "f"(x));
+  return y;
+}
 __device__ __forceinline__ double ld_cluster_f64(uint32_t caddr) {
   double v;
   asm volatile("ld.shared::cluster.f64 %0, [%1];\n" : "=d"(v) : "r"(caddr) : "memory");
@@ -460,22 +467,26 @@ __global__ void __launch_bounds__(640, 1) jacobi_cluster_kernel(double* __restri
   };
   // rotates columns a, b towards orthogonality; na, nb: their squared lengths, carried along
   auto rotate = [&](double (&a)[EPL], double (&b)[EPL], double& na, double& nb) {
+    // what the angle needs of the lengths, made while the dot product is on its way (approximate: it only steers)
+    // the lengths are numbers between 1e-10 and the size; 0 for an index beyond the matrix, whose cosine then is NaN
+    const float diff = (float)(nb - na), inv_len = rsqrtf((float)na) * rsqrtf((float)nb);
     double g0 = 0.0, g1 = 0.0;
 #pragma unroll
     for (int e = 0; e < EPL; e += 2) { g0 = fma(a[e], b[e], g0); g1 = fma(a[e + 1], b[e + 1], g1); }
     double ga = g0 + g1;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) ga += __shfl_xor_sync(0xffffffffu, ga, o);
-    const float gf = (float)ga, cosine = gf * rsqrtf((float)na) * rsqrtf((float)nb);      // NaN for a zero column (an index beyond the matrix)
+    const float gf = (float)ga, cosine = gf * inv_len;
     const float cos2 = cosine * cosine;
     if (!(cos2 > 1e-30f)) return;
     mx = fmaxf(mx, cos2);
-    const float z = (float)(nb - na) / (2.f * gf);
-    const float tf = (z >= 0.f ? 1.f : -1.f) / (fabsf(z) + sqrtf(fmaf(z, z, 1.f)));
+    const float z = __fdividef(diff, 2.f * gf);
+    const float tf = __fdividef(z >= 0.f ? 1.f : -1.f, fabsf(z) + sqrt_approx(fmaf(z, z, 1.f)));
     const double t = (double)tf, d = fma(t, t, 1.0);
-    double cs = (double)rsqrtf(fmaf(tf, tf, 1.f));                // two Newton steps: 1e-7 -> 1e-14 -> rounding
-    cs = cs * fma(-0.5 * d, cs * cs, 1.5);
-    cs = cs * fma(-0.5 * d, cs * cs, 1.5);
+    // 1 / sqrt(d): the approximation's relative error 1e-7 becomes its cube in one Halley step, and the rounding's
+    double cs = (double)rsqrtf(fmaf(tf, tf, 1.f));
+    const double err = fma(-d, cs * cs, 1.0);
+    cs = fma(cs * err, fma(0.375, err, 0.5), cs);
     const double sn = cs * t;
     na = fma(-t, ga, na);
     nb = fma(t, ga, nb);
@@ -586,7 +597,7 @@ __global__ void __launch_bounds__(640, 1) jacobi_cluster_kernel(double* __restri
           atomicMax(reinterpret_cast<int*>(flag) + sweep, __float_as_int(m));
         }
       }
-      cluster_sync_all();                                        // the columns (and the sweep's maximum) are in L2 for their next owners
+      cluster_sync_all();                                        // the columns (and the sweep's maximum) can be read by their next owners
     }
     const float worst = __ldcg(flag + sweep);
     ++sweep;
