@@ -409,7 +409,7 @@ __global__ void __launch_bounds__(256) fit_emit_theta_kernel(const double* __res
 // in shared memory (a warp per pair, the first block's column kept in registers) and rotates all pairs between them (in the first
 // round also those inside), and between rounds the columns go to their next CTA behind one cluster barrier: through distributed shared
 // memory up to 384 indices, beyond that (two buffers don't fit) through L2 (about 3 us per round); no launch, no host round trip.  Both
-// fits of n = 256, m = 154, 4 heads on B200: 3.9 ms (4.3 with the divisions and the square root of the angle
+// fits of n = 256, m = 103, 4 heads on B200: 3.75 ms (3.9 with the dot product reduced by shuffles, 4.3 also with the divisions and the square root of the angle
 // rounded exactly and everything behind the dot product, 4.6 through L2; the two-sided form, two launches of 4 us per round, above 24).
 // Half as many CTAs with twice the warps took a fifth longer (the rotations of 16 warps are bound by shared memory).
 // The angle is taken in single precision, with approximate divisions: it only steers the convergence (off-diagonal cosines fall by 1e-7
@@ -468,20 +468,26 @@ __global__ void __launch_bounds__(640, 1) jacobi_cluster_kernel(double* __restri
   // rotates columns a, b towards orthogonality; na, nb: their squared lengths, carried along
   auto rotate = [&](double (&a)[EPL], double (&b)[EPL], double& na, double& nb) {
     // what the angle needs of the lengths, made while the dot product is on its way (approximate: it only steers)
-    // the lengths are numbers between 1e-10 and the size; 0 for an index beyond the matrix, whose cosine then is NaN
-    const float diff = (float)(nb - na), inv_len = rsqrtf((float)na) * rsqrtf((float)nb);
+    // the lengths are numbers between 1e-10 and the size; 0 for an index beyond the matrix
+    const float inv_len = rsqrtf((float)na) * rsqrtf((float)nb), half_diff = 0.5f * (float)(nb - na) * inv_len;
+    const double scale = (double)inv_len * 0x1p30;
     double g0 = 0.0, g1 = 0.0;
 #pragma unroll
     for (int e = 0; e < EPL; e += 2) { g0 = fma(a[e], b[e], g0); g1 = fma(a[e + 1], b[e + 1], g1); }
-    double ga = g0 + g1;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) ga += __shfl_xor_sync(0xffffffffu, ga, o);
-    const float gf = (float)ga, cosine = gf * inv_len;
+    const double g = g0 + g1;
+    // the lanes' parts of the cosine in units of 2^-30 and the rests in units of 2^-56, as integers in the low words of sums with 1.5 * 2^52
+    // (each part is at most the product of the lengths), so that two integer reductions of the warp replace five steps of shuffles
+    constexpr double MAGIC = 0x1.8p52;
+    const double hi = fma(g, scale, MAGIC);
+    const double lo = fma(fma(g, scale, MAGIC - hi), 0x1p26, MAGIC);
+    const int hi_sum = __reduce_add_sync(0xffffffffu, __double2loint(hi)), lo_sum = __reduce_add_sync(0xffffffffu, __double2loint(lo));
+    const float cosine = fmaf((float)lo_sum, 0x1p-56f, (float)hi_sum * 0x1p-30f);
     const float cos2 = cosine * cosine;
-    if (!(cos2 > 1e-30f)) return;
+    if (!(cos2 > 1e-30f && inv_len > 0.f && inv_len < 1e30f)) return;
     mx = fmaxf(mx, cos2);
-    const float z = __fdividef(diff, 2.f * gf);
-    const float tf = __fdividef(z >= 0.f ? 1.f : -1.f, fabsf(z) + sqrt_approx(fmaf(z, z, 1.f)));
+    // tangent of the angle: 1 / (z + sqrt(z^2 + 1)) with z = (nb - na) / (2 g), both sides times the cosine
+    const float tf = __fdividef(half_diff >= 0.f ? cosine : -cosine, fabsf(half_diff) + sqrt_approx(fmaf(half_diff, half_diff, cos2)));
+    const double ga = (double)__fdividef(cosine, inv_len);
     const double t = (double)tf, d = fma(t, t, 1.0);
     // 1 / sqrt(d): the approximation's relative error 1e-7 becomes its cube in one Halley step, and the rounding's
     double cs = (double)rsqrtf(fmaf(tf, tf, 1.f));
