@@ -403,19 +403,20 @@ __global__ void __launch_bounds__(256) fit_emit_theta_kernel(const double* __res
 }
 
 // ---- one-sided Jacobi, one launch ----------------------------------------------------------------------------------------
-// Bound: latency of a rotation (a dot product over a column reduced across a warp, the angle, the update: about 850 cycles), n - 1 of
+// Bound: latency of a rotation (a dot product over a column reduced across a warp, the angle, the update; its warps issue in a quarter of the cycles), n - 1 of
 // them one after the other per sweep whatever the machine's width, 11 to 14 sweeps.  So everything else is taken out of that chain: a
 // cluster of C CTAs owns a matrix, its columns form 2 C blocks of bs, in each of the 2 C - 1 rounds of a sweep a CTA holds two blocks
 // in shared memory (a warp per pair, the first block's column kept in registers) and rotates all pairs between them (in the first
 // round also those inside), and between rounds the columns go to their next CTA behind one cluster barrier: through distributed shared
 // memory up to 384 indices, beyond that (two buffers don't fit) through L2 (about 3 us per round); no launch, no host round trip.  Both
-// fits of n = 256, m = 103, 4 heads on B200: 3.75 ms (3.9 with the dot product reduced by shuffles, 4.3 also with the divisions and the square root of the angle
-// rounded exactly and everything behind the dot product, 4.6 through L2; the two-sided form, two launches of 4 us per round, above 24).
+// fits of n = 256, m = 103, 4 heads on B200: 3.75 ms, of it 2.6 and 0.6 here (3.9 with the dot product reduced by shuffles, 4.3 also with
+// the divisions and the square root of the angle rounded exactly and everything behind the dot product, 4.6 through L2; the two-sided form,
+// two launches of 4 us per round, above 24).
 // Half as many CTAs with twice the warps took a fifth longer (the rotations of 16 warps are bound by shared memory).
 // The angle is taken in single precision, with approximate divisions: it only steers the convergence (off-diagonal cosines fall by 1e-7
 // at worst per sweep once they are small); cosine and sine are made from its tangent in double precision, so that the rotation is
-// orthogonal.  The squared lengths that the angle needs are carried along and taken anew in every round; with them as two more dot products and the angle in
-// double precision a rotation took 1.05 us instead of 0.89 (both with their share of the rounds).
+// orthogonal.  The squared lengths that the angle needs are carried along and taken anew in every round; with them as two more dot products
+// and the angle in double precision a rotation took 1.05 us where this took 0.89 then (both with their share of the rounds).
 // tau = 1e-5 of the largest diagonal entry keeps the columns of a rank-deficient matrix away from zero, so that its null space gets
 // orthonormal vectors too.
 __device__ __forceinline__ float sqrt_approx(float x) {
