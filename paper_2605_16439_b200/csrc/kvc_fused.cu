@@ -167,7 +167,7 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
         for (int part = 0; part < 3; ++part) {
           const int count = part == 1 ? nts : stages_of(bg, r0);
           for (int c = 0; c < count; ++c) {
-            if (!mbar_wait_bounded(&bars.empty[slot], phase)) { atomicExch(a.status, (int)KVC_ERR_TIMEOUT); return; }
+            if (!mbar_wait_bounded<RG>(&bars.empty[slot], phase)) { atomicExch(a.status, (int)KVC_ERR_TIMEOUT); return; }
             unsigned char* dst = sm + slot * a.stage_bytes;
             uint64_t* bar = &bars.full[slot];
             if (part == 1) {
@@ -211,7 +211,7 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
       for (int part = 0; part < 3; ++part) {
         const int count = part == 1 ? nts : a.NJ;
         for (int c = 0; c < count; ++c) {
-          if (!mbar_wait_bounded(&bars.empty[slot], phase)) { atomicExch(a.status, (int)KVC_ERR_TIMEOUT); return; }
+          if (!mbar_wait_bounded<RG>(&bars.empty[slot], phase)) { atomicExch(a.status, (int)KVC_ERR_TIMEOUT); return; }
           unsigned char* dst = sm + slot * a.stage_bytes;
           uint64_t* bar = &bars.full[slot];
           if (part == 1) {
@@ -284,7 +284,7 @@ fused_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
   bool dead = false;
   // every lane of the calling warp waits; the lanes leave the polling loop together again before any warp-wide instruction
   auto wait_on = [&](uint64_t* bar, uint32_t parity) {
-    if (!dead && !mbar_wait_bounded(bar, parity)) dead = true;
+    if (!dead && !mbar_wait_bounded<RG>(bar, parity)) dead = true;
     __syncwarp();
   };
   // the stage in `slot` has been consumed by this warp
