@@ -98,9 +98,10 @@ KVC_API int kvc_retained_len(int n, int ratio_permille);
  * the logits in registers up to n = 640, with per-sequence lengths up to 1024; or on tcgen05 with the logits in tensor memory), for
  * uniform calls of longer blocks as three kernels (streaming scores, tcgen05 expansion per 128 rows and range of the n axis, streaming
  * output), or as one kernel of CTA clusters that share the n axis: block lengths off 64, the smallest and the many-round
- * calls with groups of query heads, and per-sequence lengths where it is ahead.  What none of them takes, and block lengths off 64 with few
+ * calls with groups of query heads, and per-sequence lengths where it is ahead.  Calls whose (sequence, KV head) pairs leave the device idle
+ * take a kernel that spreads each pair over a cluster of CTAs, in fp32 storage too.  What none of them takes, and block lengths off 64 with few
  * query heads per KV head where they are ahead, goes to the generic three-phase kernels.  The library picks per shape
- * (same results within the bf16 tolerance).  The environment variable KVC_EXPANSION = "tcgen05" | "mma" | "pair" | "split" | "resident" | "cluster", read
+ * (same results within the bf16 tolerance).  The environment variable KVC_EXPANSION = "tcgen05" | "mma" | "pair" | "split" | "resident" | "cluster" | "spread", read
  * when the handle is created, forces one of them where it applies ("pair": the tcgen05 one-kernel path run by clusters of two
  * CTAs per (sequence, KV head)); "phases" forces the generic three-phase kernels that also serve fp32 storage. */
 KVC_API int kvc_layer_create(const kvc_layer_desc* desc, kvc_layer** out);
