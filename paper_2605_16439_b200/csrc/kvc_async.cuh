@@ -110,10 +110,16 @@ __device__ __forceinline__ bool mbar_try_wait_cluster(uint64_t* bar, uint32_t pa
       : "=r"(ok) : "r"(smem_addr(bar)), "r"(parity) : "memory");
   return ok != 0;
 }
+template <bool ROLLED = true>
 __device__ __forceinline__ bool mbar_wait_cluster_bounded(uint64_t* bar, uint32_t parity) {
+  if constexpr (ROLLED) {
 #pragma unroll 1
-  for (uint32_t i = 0; i < WAIT_SPIN_LIMIT; ++i)
-    if (mbar_try_wait_cluster(bar, parity)) return true;
+    for (uint32_t i = 0; i < WAIT_SPIN_LIMIT; ++i)
+      if (mbar_try_wait_cluster(bar, parity)) return true;
+  } else {
+    for (uint32_t i = 0; i < WAIT_SPIN_LIMIT; ++i)
+      if (mbar_try_wait_cluster(bar, parity)) return true;
+  }
   return false;
 }
 // asynchronous stores into a peer's shared memory; their bytes are reported to the peer's barrier when they have landed
