@@ -10,8 +10,7 @@
 // 130 KB of code, now 50.
 #include <algorithm>
 
-#include "kvc_fused.cuh"
-#include "kvc_spread.cuh"
+#include "kvc_spread_end.cuh"
 
 namespace kvc {
 
@@ -682,7 +681,7 @@ spread_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
 #pragma unroll
       for (int o = 8; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
       mx = fmaxf(mx, hstat[warp].x);
-      l = t.x == -INFINITY ? 0.f : t.y * fast_exp2(t.x - mx);
+      l = t.y * spread_weight(t.x, mx);
 #pragma unroll
       for (int o = 8; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
       if (lane < C) st_async_f32x2(map_to_cta(smem_addr(&ystat[rank * 16 + warp]), (uint32_t)lane), mx, l, map_to_cta(smem_addr(&bars.y), (uint32_t)lane));
@@ -757,61 +756,7 @@ spread_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
     cluster_arrive();                                         // nothing is sent to a peer after this
     peer_wait(&bars.y);
     __syncwarp();
-#pragma unroll 1
-    for (int i = tid; i < G * dc; i += SPR_CONS) {
-      const int g = i >> ld, d = i & (dc - 1);
-      float mx = -INFINITY, num = 0.f, den = 0.f;
-#pragma unroll 2
-      for (int c = 0; c < C; ++c) mx = fmaxf(mx, ystat[c * 16 + g].x);
-      if (mx != -INFINITY) {
-#pragma unroll 2
-        for (int c = 0; c < C; ++c) {
-          const float2 t = ystat[c * 16 + g];
-          const float f = t.x == -INFINITY ? 0.f : fast_exp2(t.x - mx);
-          num = fmaf(f, yrecv[(c * G + g) * dc + d], num);
-          den = fmaf(f, t.y, den);
-        }
-        const float2 v = hstat[g];
-        if (v.x != -INFINITY) {
-          const float f = fast_exp2(v.x - mx) * v.y;
-          den += f;
-          num = fmaf(f, mus[d], num);
-        }
-      }
-      if (a.nrg == 1) {
-        a.out[((size_t)pair * G + g) * D + rank * dc + d] = __float2bfloat16_rn(den > 0.f ? num / den : 0.f);
-      } else {
-        a.py[((size_t)unit * G + g) * D + rank * dc + d] = num;
-        if (d == 0) a.pml[(((size_t)pair * C + rank) * a.nrg + rg) * G + g] = make_float2(mx, den);
-      }
-    }
-    if (a.nrg > 1) {
-      // the last group's CTA `rank` to arrive merges their channels
-      __threadfence();
-      named_barrier_sync(1, SPR_CONS);
-      if (tid == 0) rowmax[0] = arrive_is_last(&a.cnt[pair * C + rank], a.token, a.nrg) ? 1 : 0;
-      named_barrier_sync(1, SPR_CONS);
-      if (rowmax[0]) {
-        __threadfence();
-#pragma unroll 1
-        for (int i = tid; i < G * dc; i += SPR_CONS) {
-          const int g = i >> ld, d = i & (dc - 1);
-          const float2* ml = a.pml + ((size_t)pair * C + rank) * a.nrg * G + g;
-          const float* yp = a.py + ((size_t)pair * a.nrg * G + g) * D + rank * dc + d;
-          float mx = -INFINITY, num = 0.f, den = 0.f;
-#pragma unroll 4
-          for (int p = 0; p < a.nrg; ++p) mx = fmaxf(mx, __ldcg(ml + p * G).x);
-#pragma unroll 4
-          for (int p = 0; p < a.nrg; ++p) {
-            const float2 t = __ldcg(ml + p * G);
-            const float f = t.x == -INFINITY ? 0.f : fast_exp2(t.x - mx);
-            num = fmaf(f, __ldcg(yp + (size_t)p * G * D), num);
-            den = fmaf(f, t.y, den);
-          }
-          a.out[((size_t)pair * G + g) * D + rank * dc + d] = __float2bfloat16_rn(den > 0.f ? num / den : 0.f);
-        }
-      }
-    }
+    spread_end<SPR_CONS>(a, C, G, ld, dc, tid, pair, unit, rg, rank, ystat, yrecv, hstat, mus, &rowmax[0], [] { named_barrier_sync(1, SPR_CONS); });
     if (dead) {
       if (lane == 0) atomicExch(a.status, (int)KVC_ERR_TIMEOUT);
       __nanosleep(50000);                                     // what a peer has sent and this CTA gave up on still lands in its memory

@@ -12,8 +12,7 @@
 // Bound: the chain of these steps and of four exchanges; theta and U come at the rate of the SMs that take part.
 #include <algorithm>
 
-#include "kvc_fused.cuh"
-#include "kvc_spread.cuh"
+#include "kvc_spread_end.cuh"
 
 namespace kvc {
 
@@ -361,7 +360,7 @@ __global__ void __launch_bounds__(SPF_THREADS, 1) spread_f32_kernel(const __grid
     float s = 0.f;
 #pragma unroll 1
     for (int t = lane; t < tn; t += 32) {
-      const float p = fast_exp2(ts[t * GT + warp] - mx);
+      const float p = spread_weight(ts[t * GT + warp], mx);
       ts[t * GT + warp] = p;
       s += p;
     }
@@ -446,61 +445,7 @@ __global__ void __launch_bounds__(SPF_THREADS, 1) spread_f32_kernel(const __grid
   cluster_arrive();                                            // nothing is sent to a peer after this
   peer_wait(&bar_y);
   __syncwarp();
-#pragma unroll 1
-  for (int i = tid; i < G * dc; i += SPF_THREADS) {
-    const int g = i >> ld, d = i & (dc - 1);
-    float mx = -INFINITY, num = 0.f, den = 0.f;
-#pragma unroll 2
-    for (int c = 0; c < C; ++c) mx = fmaxf(mx, ystat[c * 16 + g].x);
-    if (mx != -INFINITY) {
-#pragma unroll 2
-      for (int c = 0; c < C; ++c) {
-        const float2 t = ystat[c * 16 + g];
-        const float f = t.x == -INFINITY ? 0.f : fast_exp2(t.x - mx);
-        num = fmaf(f, yrecv[(c * G + g) * dc + d], num);
-        den = fmaf(f, t.y, den);
-      }
-      const float2 v = hstat[g];
-      if (v.x != -INFINITY) {
-        const float f = fast_exp2(v.x - mx) * v.y;
-        den += f;
-        num = fmaf(f, mus[d], num);
-      }
-    }
-    if (a.nrg == 1) {
-      a.out[((size_t)pair * G + g) * D + rank * dc + d] = den > 0.f ? num / den : 0.f;
-    } else {
-      a.py[((size_t)unit * G + g) * D + rank * dc + d] = num;
-      if (d == 0) a.pml[(((size_t)pair * C + rank) * a.nrg + rg) * G + g] = make_float2(mx, den);
-    }
-  }
-  if (a.nrg > 1) {
-    // the last group's CTA `rank` to arrive merges their channels
-    __threadfence();
-    __syncthreads();
-    if (tid == 0) s_last = arrive_is_last(&a.cnt[pair * C + rank], a.token, a.nrg) ? 1 : 0;
-    __syncthreads();
-    if (s_last) {
-      __threadfence();
-#pragma unroll 1
-      for (int i = tid; i < G * dc; i += SPF_THREADS) {
-        const int g = i >> ld, d = i & (dc - 1);
-        const float2* ml = a.pml + ((size_t)pair * C + rank) * a.nrg * G + g;
-        const float* yp = a.py + ((size_t)pair * a.nrg * G + g) * D + rank * dc + d;
-        float mx = -INFINITY, num = 0.f, den = 0.f;
-#pragma unroll 4
-        for (int p = 0; p < a.nrg; ++p) mx = fmaxf(mx, __ldcg(ml + p * G).x);
-#pragma unroll 4
-        for (int p = 0; p < a.nrg; ++p) {
-          const float2 t = __ldcg(ml + p * G);
-          const float f = t.x == -INFINITY ? 0.f : fast_exp2(t.x - mx);
-          num = fmaf(f, __ldcg(yp + (size_t)p * G * D), num);
-          den = fmaf(f, t.y, den);
-        }
-        a.out[((size_t)pair * G + g) * D + rank * dc + d] = den > 0.f ? num / den : 0.f;
-      }
-    }
-  }
+  spread_end<SPF_THREADS>(a, C, G, ld, dc, tid, pair, unit, rg, rank, ystat, yrecv, hstat, mus, &s_last, [] { __syncthreads(); });
   if (dead) {
     if (lane == 0) atomicExch(a.status, (int)KVC_ERR_TIMEOUT);
     __nanosleep(50000);                                        // what a peer has sent and this CTA gave up on still lands in its memory
