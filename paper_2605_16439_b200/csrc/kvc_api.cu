@@ -451,7 +451,7 @@ static bool use_spread(const kvc_layer* L, int B, int R, int T, bool ragged, con
     // several waves: where it is ahead of an estimate of the cluster path (rounds of units and their tiles, the bytes; fitted to 97 uniform calls,
     // 10 %).  Routed by it those take 0.89 of their time before in the geometric mean, none more than 3 % longer (16 x 8 of n = 144, 28/4
     // heads, 715 rows 16.5 / 32.3; 25 x 5 of 400, 1610 rows 46 / 89; 8 x 7 of 324, 32/32 heads 74 / 88; not: 26 x 10 of 121 45 / 34)
-    const int H = L->desc.H_kv, units = H * ceil_div(B * R, CL_ROWS / L->G), NS = ceil_div(ceil_div(n, 64), n % 8 ? 2 : 4);
+    const int H = L->desc.H_kv, units = H * ceil_div(B * R, CL_ROWS / L->G), NS = ceil_div(ceil_div(n, 64), p.terms == 2 ? 2 : 4);
     const int held = (L->num_sms > 0 ? L->num_sms : 148) * 88 / 100 / NS, rounds = ceil_div(units, held > 0 ? held : 1);
     const double rows = 512.0 * B * R * H * (double)L->m + 4.0 * H * (double)L->m * n, text = 512.0 * B * H * (double)T;
     const double cluster = rounds * (24.4 + 1.93 * ceil_div(L->m, 64)) - 4.2 + (1.71 * rows + 1.86 * text) / HBM_US + 0.0137 * B * H;
@@ -524,7 +524,7 @@ int decode_common(const kvc_layer* L, const void* q, const void* capsules, int B
                           reinterpret_cast<uintptr_t>(V_txt) : 0) | reinterpret_cast<uintptr_t>(L->desc.mu);
 
   if ((align & 15) == 0) {
-    const SpreadPlan sp = plan_spread(L, B, R, T);
+    const SpreadPlan sp = plan_spread(L, B, R, T, ragged);
     if (use_spread(L, B, R, T, ragged, sp) && (ws_limit == 0 || spread_ws(L, sp, B).bytes <= ws_limit)) {
       bool encoded = false;
       const cudaError_t se = launch_spread(L, a, sp, ws, st, &encoded);

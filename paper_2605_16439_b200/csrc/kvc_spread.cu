@@ -10,6 +10,8 @@
 // 130 KB of code, now 50.
 #include <algorithm>
 
+#include "kvc_cluster.cuh"
+#include "kvc_split.cuh"
 #include "kvc_spread_end.cuh"
 
 namespace kvc {
@@ -777,8 +779,18 @@ bool spread_may_serve(const kvc_layer* L) {
   return L->desc.dtype == KVC_BF16 && !L->passthrough && L->mode == KVC_MODE_KV && L->desc.n >= 64 && (L->use_tc == 0 || L->use_tc == 6);
 }
 
+// bf16 terms of the scores and probabilities: two where the general paths keep them in two or in fp32 (cluster_terms: n no multiple of 8, or more
+// than some 720 retained rows), but one for the uniform calls of such long rows that the three-kernel or the one-kernel path takes, which
+// carry one.  4 x 3 blocks of n = 1024, m = 820, 28/4 heads, with lengths per sequence, relative error of the output against 64 bits on peaked
+// softmaxes: one term 3.9e-3, two 1.7e-3 (its rounding to bf16).
+static int spread_terms(const kvc_layer* L, int B, int R, int T, bool ragged) {
+  if (cluster_terms(L) == 1) return 1;
+  const bool one = !ragged && L->desc.n % 64 == 0 && ((plan_split(L, B, R).ok && T <= 64 * SP_OUT_ROWS * SP_TEXT_CHUNK) || plan_fused(L, B, R).ok);
+  return one ? 1 : 2;
+}
+
 // most_waves: 1: clusters for all groups at once; more: clusters of two, in that many waves at most
-static SpreadPlan plan_groups(const kvc_layer* L, int B, int R_all, int T_all, int nrg, int most_waves) {
+static SpreadPlan plan_groups(const kvc_layer* L, int B, int R_all, int T_all, int nrg, int most_waves, int terms) {
   SpreadPlan p{};
   const int R = ceil_div(R_all, nrg), T = ceil_div(T_all, nrg);
   const int G = L->G, n = L->desc.n, m = L->m, H = L->desc.H_kv;
@@ -800,8 +812,7 @@ static SpreadPlan plan_groups(const kvc_layer* L, int B, int R_all, int T_all, i
   p.nt = ceil_div(R * G, 8);
   if (p.nt > 1) p.nt = (p.nt + 1) & ~1;
   if (G > 8 && p.nt == 6) p.nt = 8;
-  // as the paths before it: one bf16 term, or two where the three-phase kernels kept the scores and probabilities in fp32
-  p.terms = n % 8 == 0 ? 1 : 2;
+  p.terms = terms;
   p.nsub = p.gw > 15 ? 2 : 1;
   p.gsub = ceil_div(p.gw, p.nsub);
   p.wbox = p.gsub * 16 + 8;
@@ -857,18 +868,19 @@ static SpreadPlan plan_groups(const kvc_layer* L, int B, int R_all, int T_all, i
 // merge (us per call: 1 x 31 blocks of n = 576, m = 432, 16/2 heads, 4 groups 40.5, 6 30.1, 8 25.6, the one-kernel path 43.7; 4 x 5 of 1024,
 // 28/4 heads, one 33.1, two 26.5; 1 x 5 of 576, 28/4 heads, one 15.6, two 16.8, three 15.0).  Of the 110 shapes above each takes 14.31 us (geometric
 // mean) with its best number, 14.36 with the chosen one, 15.5 with the smallest, 23.8 on the paths below.
-SpreadPlan plan_spread(const kvc_layer* L, int B, int R, int T) {
+SpreadPlan plan_spread(const kvc_layer* L, int B, int R, int T, bool ragged) {
   if (!spread_may_serve(L) || B < 1 || R < 1 || L->G > 16 || T < 0) return SpreadPlan{};
   if (!tma_rows(spread_theta(L)) || !tma_rows(L->U_rows) || spread_theta_np(L) % 8 || L->U_np % 8) return SpreadPlan{};
   SpreadPlan best{};
+  const int terms = spread_terms(L, B, R, T, ragged);
   for (int nrg = 1; nrg <= SPR_MAX_NRG && nrg <= R; ++nrg) {
-    const SpreadPlan p = plan_groups(L, B, R, T, nrg, 1);
+    const SpreadPlan p = plan_groups(L, B, R, T, nrg, 1, terms);
     if (p.ok && (!best.ok || p.us < best.us)) best = p;
   }
   // more groups than clusters the device holds: beside the paths for block lengths off 64 only (the others are ahead of a second wave: 30 x 2
   // blocks of n = 576, 28/4 heads 43 / 21.5; 21 x 2 of 1024 79 / 70)
   for (int nrg = 1; !best.ok && L->desc.n % 64 != 0 && nrg <= SPR_MAX_NRG && nrg <= R; ++nrg) {
-    const SpreadPlan p = plan_groups(L, B, R, T, nrg, SPR_MAX_WAVES);
+    const SpreadPlan p = plan_groups(L, B, R, T, nrg, SPR_MAX_WAVES, terms);
     if (p.ok) best = p;
   }
   return best;
@@ -886,14 +898,15 @@ SpreadWs spread_ws(const kvc_layer* L, const SpreadPlan& p, int B) {
   return w;
 }
 
-// enough for every T: the number of groups depends on the text, whether a number can be had does not
+// enough for every T and for lengths per sequence: the number of groups and of terms depends on them, whether a number of groups can be had only on the terms
 size_t spread_ws_bytes(const kvc_layer* L, int B, int R) {
   size_t most = 0;
-  if (!plan_spread(L, B, R, 0).ok) return 0;
-  for (int nrg = 1; nrg <= SPR_MAX_NRG && nrg <= R; ++nrg) {
-    const SpreadPlan p = plan_groups(L, B, R, 0, nrg, SPR_MAX_WAVES);
-    if (p.ok) most = std::max(most, spread_ws(L, p, B).bytes);
-  }
+  if (!plan_spread(L, B, R, 0, false).ok && !plan_spread(L, B, R, 0, true).ok) return 0;
+  for (int terms = 1; terms <= cluster_terms(L); ++terms)
+    for (int nrg = 1; nrg <= SPR_MAX_NRG && nrg <= R; ++nrg) {
+      const SpreadPlan p = plan_groups(L, B, R, 0, nrg, SPR_MAX_WAVES, terms);
+      if (p.ok) most = std::max(most, spread_ws(L, p, B).bytes);
+    }
   return most;
 }
 

@@ -52,7 +52,7 @@ struct SpreadWs {
   size_t bytes;
 };
 
-SpreadPlan plan_spread(const kvc_layer* L, int B, int R, int T);
+SpreadPlan plan_spread(const kvc_layer* L, int B, int R, int T, bool ragged);
 SpreadWs spread_ws(const kvc_layer* L, const SpreadPlan& p, int B);
 size_t spread_ws_bytes(const kvc_layer* L, int B, int R);     // 0 if the path never applies
 bool spread_may_serve(const kvc_layer* L);

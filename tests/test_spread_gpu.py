@@ -7,9 +7,11 @@ Bound: the regression bound of the parity tests.
 """
 import random
 
+import numpy as np
 import pytest
 import torch
 
+from oracle import kvcapsule_oracle as orc
 from paper_2605_16439_b200 import binding as kvc
 from paper_2605_16439_b200 import build as kvc_build
 from paper_2605_16439_b200 import workloads as wl
@@ -91,3 +93,37 @@ def test_workspace_holds_every_shorter_text(B, H_q, H_kv, grid, R, ratio, monkey
         assert counts["spread"] == 1
         assert kvc.kvc_read_device_status(layer, B, R, T, ws) == 0
         assert bool((ws[need:] == 0xA5).all()), T
+
+
+@pytest.mark.parametrize("B,H_q,H_kv,grid,R,T,ratio,lengths", [
+    (4, 28, 4, 32, 3, 300, 200, True),       # n = 1024, m = 820
+    (2, 8, 8, 32, 2, 60, 250, True),         # m = 768, one query head per KV head
+    (1, 4, 1, 32, 1, 40, 280, True),         # m = 738
+    (2, 8, 2, 36, 1, 100, 200, False),       # n = 1296, m = 1037: no whole multiple of 64
+])
+def test_long_score_rows_keep_both_terms(B, H_q, H_kv, grid, R, T, ratio, lengths):
+    """Rows of scores too long for the tensor-core expansion of the three-phase kernels keep scores and probabilities in two bf16 terms or in
+    fp32 on every path that serves them, by default routing.
+
+    Bound, relative 2-norm against 64 bits on the stored capsules: the rounding of the output, at most 2^-9 of every entry, and 1e-4 for
+    two terms (16 bits: 5e-6 on this recipe at m = 820; one term 3.8e-3)."""
+    shape = wl.Shape("spread-terms", 1, B, H_q, H_kv, 128, grid, R, T, 1, "bf16", ratio)
+    p = tl.make_problem(shape, 640 + grid + B, T=T, T_cap=T, recipe="peaked")
+    layer = tl.gpu_layer(shape, p)
+    caps = kvc.alloc_capsules(layer, B, R)
+    kvc.kvc_compress(layer, p["K_vis"].cuda(), p["V_vis"].cuda(), B, R, caps)
+    K_t, V_t = (tl.np64(x) for x in kvc.capsule_views(layer, caps, B, R))
+    q, K_txt, V_txt = p["q"].cuda(), p["K_txt"].cuda(), p["V_txt"].cuda()
+    out = torch.empty((B, H_q, 128), dtype=torch.bfloat16, device="cuda")
+    ws = kvc.alloc_workspace(layer, B, R, T)
+    R_b, T_b = [R - b % R for b in range(B)], [T - b for b in range(B)]
+    if lengths:
+        i32 = lambda x: torch.tensor(x, dtype=torch.int32, device="cuda")
+        kvc.kvc_decode_attend_ragged(layer, q, caps, B, R, i32(R_b), K_txt, V_txt, T, i32(T_b), T, out, ws)
+    else:
+        R_b, T_b = [R] * B, [T] * B
+        kvc.kvc_decode_attend(layer, q, caps, B, R, K_txt, V_txt, T, T, out, ws)
+    want = orc.decode_attend_ragged(tl.np64(p["q"]), K_t, V_t, tl.np64(p["theta"]), tl.np64(p["U"]), tl.np64(p["mu"]), tl.np64(p["K_txt"]),
+                                    tl.np64(p["V_txt"]), R_b, T_b, "kv")
+    err = float(np.linalg.norm(tl.np64(out) - want) / np.linalg.norm(want))
+    assert err <= 2.0 ** -9 + 1e-4, err
