@@ -22,9 +22,12 @@ constexpr int FIT_TILE = 64;            // covariance tile per CTA
 constexpr int FIT_KC = 32;              // channels per staged chunk
 constexpr int FIT_SPLITS = 4;            // parts of the samples, one per matrix of the workspace
 constexpr int FIT_MAX_SWEEPS = 40;
-// one-sided: stop after a sweep whose largest squared cosine between two columns was below this.  Convergence is quadratic: from 1e-11 that sweep
-// leaves at most 2e-19 (fields of 34 to 256 positions in numpy; 3e-12 -> 2e-23, 6e-10 -> 2e-21), cosines far below the outputs' rounding
-constexpr float FIT_COS_TOL2 = 1e-11f;
+// one-sided: stop after a sweep whose largest squared cosine between two columns was below this.  Convergence is quadratic only between
+// eigenvalues that stand apart: 32 blocks of n = 256 go 4e-7, 1e-12, 2e-26, but in a cluster, and fewer samples than positions always make one of
+// the null space, the squares fall by a factor of ten a sweep (one block of 256: 8e-12, 8e-13, 7e-13, 3e-14, 3e-15, 2e-18, 8e-26), and a sweep
+// may show a drop from elsewhere while the cluster's are still coming.  Stopped at 1e-11, rows of U were 1.2e-6 from orthonormal there, and
+// eigenvalues equal to 1e-5 off by 1e-6 of the largest; 32 blocks of 256 took one sweep less, both fits 3.76 ms instead of 3.93
+constexpr float FIT_COS_TOL2 = 1e-20f;
 constexpr double FIT_OFF_TOL2 = 1e-22;  // stop when (off-diagonal norm / diagonal norm)^2 falls below this
 
 static inline int even_up(int x) { return (x + 1) & ~1; }
@@ -404,14 +407,14 @@ __global__ void __launch_bounds__(256) fit_emit_theta_kernel(const double* __res
 
 // ---- one-sided Jacobi, one launch ----------------------------------------------------------------------------------------
 // Bound: latency of a rotation (a dot product over a column reduced across a warp, the angle, the update; its warps issue in a quarter of the cycles), n - 1 of
-// them one after the other per sweep whatever the machine's width, 11 to 14 sweeps.  So everything else is taken out of that chain: a
+// them one after the other per sweep whatever the machine's width, 12 to 15 sweeps, some 25 where there are fewer samples than positions.  So everything else is taken out of that chain: a
 // cluster of C CTAs owns a matrix, its columns form 2 C blocks of bs, in each of the 2 C - 1 rounds of a sweep a CTA holds two blocks
 // in shared memory (a warp per pair, the first block's column kept in registers) and rotates all pairs between them (in the first
 // round also those inside), and between rounds the columns go to their next CTA behind one cluster barrier: through distributed shared
 // memory up to 384 indices, beyond that (two buffers don't fit) through L2 (about 3 us per round); no launch, no host round trip.  Both
-// fits of n = 256, m = 103, 4 heads on B200: 3.75 ms, of it 2.6 and 0.6 here (3.9 with the dot product reduced by shuffles, 4.3 also with
-// the divisions and the square root of the angle rounded exactly and everything behind the dot product, 4.6 through L2; the two-sided form,
-// two launches of 4 us per round, above 24).
+// fits of n = 256, m = 103, 4 heads on B200: 3.93 ms in 14 sweeps (at 13 sweeps 3.75, and 3.9 with the dot product reduced by shuffles, 4.3 also
+// with the divisions and the square root of the angle rounded exactly and everything behind the dot product, 4.6 through L2; the two-sided
+// form, two launches of 4 us per round, above 24).
 // Half as many CTAs with twice the warps took a fifth longer (the rotations of 16 warps are bound by shared memory).
 // The angle is taken in single precision, with approximate divisions: it only steers the convergence (off-diagonal cosines fall by 1e-7
 // at worst per sweep once they are small); cosine and sine are made from its tangent in double precision, so that the rotation is
