@@ -418,7 +418,7 @@ __global__ void __launch_bounds__(256) fit_emit_theta_kernel(const double* __res
 // Half as many CTAs with twice the warps took a fifth longer (the rotations of 16 warps are bound by shared memory).
 // The angle is taken in single precision, with approximate divisions: it only steers the convergence (off-diagonal cosines fall by 1e-7
 // at worst per sweep once they are small); cosine and sine are made from its tangent in double precision, so that the rotation is
-// orthogonal.  The squared lengths that the angle needs are carried along and taken anew in every round; with them as two more dot products
+// orthogonal.  The squared lengths that the angle needs are carried along and taken anew in every round, and where one falls below a quarter; with them as two more dot products
 // and the angle in double precision a rotation took 1.05 us where this took 0.89 then (both with their share of the rounds).
 // tau = 1e-5 of the largest diagonal entry keeps the columns of a rank-deficient matrix away from zero, so that its null space gets
 // orthonormal vectors too.
@@ -480,7 +480,8 @@ __global__ void __launch_bounds__(640, 1) jacobi_cluster_kernel(double* __restri
     for (int e = 0; e < EPL; e += 2) { g0 = fma(a[e], b[e], g0); g1 = fma(a[e + 1], b[e + 1], g1); }
     const double g = g0 + g1;
     // the lanes' parts of the cosine in units of 2^-30 and the rests in units of 2^-56, as integers in the low words of sums with 1.5 * 2^52
-    // (each part is at most the product of the lengths), so that two integer reductions of the warp replace five steps of shuffles
+    // (the parts together are at most the product of the lengths, 2^30, and 2^31 with lengths carried as below), so that two integer reductions
+    // of the warp replace five steps of shuffles
     constexpr double MAGIC = 0x1.8p52;
     const double hi = fma(g, scale, MAGIC);
     const double lo = fma(fma(g, scale, MAGIC - hi), 0x1p26, MAGIC);
@@ -498,6 +499,7 @@ __global__ void __launch_bounds__(640, 1) jacobi_cluster_kernel(double* __restri
     const double err = fma(-d, cs * cs, 1.0);
     cs = fma(cs * err, fma(0.375, err, 0.5), cs);
     const double sn = cs * t;
+    const double na0 = na, nb0 = nb;
     na = fma(-t, ga, na);
     nb = fma(t, ga, nb);
 #pragma unroll
@@ -506,6 +508,9 @@ __global__ void __launch_bounds__(640, 1) jacobi_cluster_kernel(double* __restri
       a[e] = cs * x - sn * y;
       b[e] = sn * x + cs * y;
     }
+    // a column that was nearly parallel to the other loses most of its length, and what is left is no larger than the rounding of t ga: taken anew
+    if (na < 0.25 * na0) na = length2(a);
+    if (nb < 0.25 * nb0) nb = length2(b);
   };
   auto get = [&](double (&x)[EPL], int slot) {
 #pragma unroll
