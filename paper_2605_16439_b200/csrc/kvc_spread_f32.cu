@@ -226,23 +226,30 @@ __global__ void __launch_bounds__(SPF_THREADS, 1) spread_f32_kernel(const __grid
     float acc[RT];
 #pragma unroll
     for (int k = 0; k < RT; ++k) acc[k] = 0.f;
-    auto fma_rows = [&](const float* v, float x) {
+    auto fma_rows = [&](float (&sum)[RT], const float* v, float x) {
 #pragma unroll
       for (int k = 0; k < RT; k += 4) {
         const float4 s = *reinterpret_cast<const float4*>(v + k);
-        acc[k] = fmaf(s.x, x, acc[k]); acc[k + 1] = fmaf(s.y, x, acc[k + 1]); acc[k + 2] = fmaf(s.z, x, acc[k + 2]); acc[k + 3] = fmaf(s.w, x, acc[k + 3]);
+        sum[k] = fmaf(s.x, x, sum[k]); sum[k + 1] = fmaf(s.y, x, sum[k + 1]); sum[k + 2] = fmaf(s.z, x, sum[k + 2]); sum[k + 3] = fmaf(s.w, x, sum[k + 3]);
       }
     };
     if (mine) {
 #pragma unroll
-      for (int e = 0; e < SPF_AHEAD; ++e) if (kl + e * KL < m) fma_rows(S + (kl + e * KL) * RT, th[e]);
+      for (int e = 0; e < SPF_AHEAD; ++e) if (kl + e * KL < m) fma_rows(acc, S + (kl + e * KL) * RT, th[e]);
 #pragma unroll 1
       for (int j = kl + SPF_AHEAD * KL; j < m; j += 8 * KL) {
         float t[8];
 #pragma unroll
         for (int e = 0; e < 8; ++e) t[e] = j + e * KL < m ? __ldg(theta + (size_t)(j + e * KL) * n + col) : 0.f;
+        // eight products at a time: in one chain over all of a thread's rows, where few threads share a column (n = 1024 on two CTAs: one), the
+        // error was 1.7 times that of the three-phase kernels' four chains, now 0.7 (16 x 2 blocks of n = 900, 8/2 heads)
+        float part[RT];
 #pragma unroll
-        for (int e = 0; e < 8; ++e) if (j + e * KL < m) fma_rows(S + (j + e * KL) * RT, t[e]);
+        for (int k = 0; k < RT; ++k) part[k] = 0.f;
+#pragma unroll
+        for (int e = 0; e < 8; ++e) if (j + e * KL < m) fma_rows(part, S + (j + e * KL) * RT, t[e]);
+#pragma unroll
+        for (int k = 0; k < RT; ++k) acc[k] += part[k];
       }
 #pragma unroll
       for (int k = 0; k < RT; k += 4) *reinterpret_cast<float4*>(red + (size_t)tid * RL + k) = make_float4(acc[k], acc[k + 1], acc[k + 2], acc[k + 3]);
@@ -253,9 +260,12 @@ __global__ void __launch_bounds__(SPF_THREADS, 1) spread_f32_kernel(const __grid
       const int c = i / (RT / 4), k = (i - c * (RT / 4)) * 4;
       float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
       if (c < W)
-        for (int p = 0; p < KL; ++p) {
-          const float4 x = *reinterpret_cast<const float4*>(red + (size_t)(p * W + c) * RL + k);
-          s.x += x.x; s.y += x.y; s.z += x.z; s.w += x.w;
+        for (int p = 0; p < KL; p += 4) {
+          float4 x[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) x[e] = p + e < KL ? *reinterpret_cast<const float4*>(red + (size_t)((p + e) * W + c) * RL + k) : make_float4(0.f, 0.f, 0.f, 0.f);
+          s.x += (x[0].x + x[1].x) + (x[2].x + x[3].x); s.y += (x[0].y + x[1].y) + (x[2].y + x[3].y);
+          s.z += (x[0].z + x[1].z) + (x[2].z + x[3].z); s.w += (x[0].w + x[1].w) + (x[2].w + x[3].w);
         }
       *reinterpret_cast<float4*>(P + c * RL + k) = s;
     }
@@ -266,6 +276,7 @@ __global__ void __launch_bounds__(SPF_THREADS, 1) spread_f32_kernel(const __grid
       for (int c = lane; c < W; c += 32) mx = fmaxf(mx, P[c * RL + warp]);
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+      mx = ceilf(mx);                                          // a whole number: the factors between CTAs, blocks and text are powers of two, exact
 #pragma unroll 1
       for (int c = lane; c < W4; c += 32) {
         const float p = c < W ? fast_exp2(P[c * RL + warp] - mx) : 0.f;
@@ -285,7 +296,7 @@ __global__ void __launch_bounds__(SPF_THREADS, 1) spread_f32_kernel(const __grid
     for (int t = lane; t < tn; t += 32) mx = fmaxf(mx, ts[t * GT + warp]);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    if (lane == 0) tmax[warp] = mx;
+    if (lane == 0) tmax[warp] = ceilf(mx);
   }
   if (Re > 0) {
     // ---------------- step 3 ----------------
