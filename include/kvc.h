@@ -307,7 +307,7 @@ typedef enum {
   KVC_KERNEL_CLUSTER = 14,        /* of FUSED: the kernel of CTA clusters that share the n axis */
   KVC_KERNEL_PLAIN = 15,          /* of FUSED: attention over rows stored verbatim */
   KVC_KERNEL_COMPRESS = 16,       /* of PROJECT_VALUES (GATHER_KEYS where no side is projected): the one-kernel bf16 compression */
-  KVC_KERNEL_SPREAD = 17,         /* of CLUSTER: the kernel of clusters that serve one (sequence, KV head) each */
+  KVC_KERNEL_SPREAD = 17,         /* of FUSED: the kernels of clusters that serve one (sequence, KV head) each, bf16 and fp32 */
   KVC_KERNEL_ID_END = 18
 } kvc_kernel_id;
 KVC_API int kvc_profile_start(int max_launches);

@@ -350,5 +350,5 @@ def kvc_profile_read() -> dict:
 
 
 def kvc_profile_parts() -> dict:
-    """The same for the kernels that kvc_profile_read counts among others (cluster and plain under fused, compress under project_values)."""
+    """The same for the kernels that kvc_profile_read counts among others (cluster, plain and spread under fused, compress under project_values)."""
     return _profile(range(KVC_KERNEL_COUNT, KVC_KERNEL_ID_END))

@@ -62,7 +62,7 @@ int kvc_profile_read(int kernel_id, double* total_ms, long long* launches) {
   double t = 0;
   long long n = 0;
   for (size_t i = 0; i < p.kid.size(); ++i) {
-    if (p.kid[i] != kernel_id && p.part[i] != kernel_id && !(kernel_id == KVC_KERNEL_CLUSTER && p.part[i] == KVC_KERNEL_SPREAD)) continue;
+    if (p.kid[i] != kernel_id && p.part[i] != kernel_id) continue;
     float ms = 0.f;
     if (cudaEventElapsedTime(&ms, p.ev[2 * i], p.ev[2 * i + 1]) != cudaSuccess) return KVC_ERR_CUDA;
     t += ms;

@@ -98,7 +98,7 @@ def gpu_run(shape: wl.Shape, p, dev="cuda", mode: str = "kv"):
 
 
 def launches(fn):
-    """({kernel name: launches}, result) of fn run with the library's event brackets on; cluster, plain and compress beside what they count under."""
+    """({kernel name: launches}, result) of fn run with the library's event brackets on; cluster, plain, spread and compress beside what they count under."""
     kvc.kvc_profile_start(64)
     try:
         out = fn()

@@ -83,16 +83,17 @@ def test_long_runs_of_sequences_without_blocks(B, H_q, H_kv, grid, R, T, ratio, 
     assert counts["cluster"] == 1 and counts["scores"] == 0
 
 
-@pytest.mark.parametrize("H_q,H_kv,B,R,grid,T,ratio,cluster", [
-    (16, 16, 64, 2, 9, 60, 875, False), (4, 4, 64, 2, 9, 700, 600, False), (8, 2, 32, 1, 9, 700, 600, False), (16, 16, 7, 2, 31, 60, 875, False),
-    (8, 2, 16, 5, 19, 60, 600, True), (4, 4, 7, 2, 27, 60, 600, True), (28, 4, 1, 1, 9, 60, 875, True),
+@pytest.mark.parametrize("H_q,H_kv,B,R,grid,T,ratio,path", [
+    (16, 16, 64, 2, 9, 60, 875, "phases"), (4, 4, 64, 2, 9, 700, 600, "phases"), (8, 2, 32, 1, 9, 700, 600, "phases"),
+    (16, 16, 7, 2, 31, 60, 875, "phases"), (28, 4, 1, 1, 9, 60, 875, "cluster"), (28, 4, 40, 3, 9, 60, 600, "cluster"),
+    (8, 2, 16, 5, 19, 60, 600, "spread"), (4, 4, 7, 2, 27, 60, 600, "spread"),
 ])
-def test_odd_block_lengths_take_the_faster_path(H_q, H_kv, B, R, grid, T, ratio, cluster):
-    """Block lengths off the tensor-core expansion of the three-phase kernels: both sides of the rule, by default routing."""
+def test_routing_of_odd_block_lengths(H_q, H_kv, B, R, grid, T, ratio, path):
+    """Block lengths off the tensor-core expansion of the three-phase kernels: every side of the rules, by default routing."""
     shape = wl.Shape("odd-route", 1, B, H_q, H_kv, 128, grid, R, T, 1, "bf16", ratio)
     p = tl.make_problem(shape, 850 + grid, T=T, T_cap=T, recipe="peaked")
     counts, (_, _, _, out) = tl.launches(lambda: tl.gpu_run(shape, p))
-    assert counts["cluster"] == int(cluster) and counts["scores"] == 1 - int(cluster)
+    assert [counts[k] for k in ("cluster", "spread", "scores")] == [int(path == k) for k in ("cluster", "spread", "phases")]
     tl.assert_close(tl.np64(out), tl.oracle_run(shape, p, "fused")[2], "bf16")
 
 
@@ -121,8 +122,11 @@ def test_workspace_holds_every_shorter_text(B, H_q, H_kv, grid, R, ratio, monkey
         assert bool((ws[need:] == 0xA5).all()), T
 
 
-def test_static_entry_point_takes_the_cluster_path():
-    """8 x 5 blocks of n = 729: the workspace of the call itself fits the fixed scratch."""
+@pytest.mark.parametrize("path,forced", [("spread", None), ("cluster", "cluster")])
+def test_static_entry_point_takes_the_path(path, forced, monkeypatch):
+    """8 x 5 blocks of n = 729: the workspace of the call itself fits the fixed scratch, on the path it takes by default and on the cluster path."""
+    if forced:
+        monkeypatch.setenv("KVC_EXPANSION", forced)
     shape = wl.Shape("cluster-static", 1, 8, 28, 4, 128, 27, 5, 300, 1, "bf16", 600)
     p = tl.make_problem(shape, 890, T=300, T_cap=300, recipe="peaked")
     layer = tl.gpu_layer(shape, p)
@@ -132,6 +136,6 @@ def test_static_entry_point_takes_the_cluster_path():
     run = lambda: kvc.kvc_decode_attend_static(layer, p["q"].to(DEV), caps, 8, 5, p["K_txt"].to(DEV), p["V_txt"].to(DEV), 300, 300, out)
     run()
     counts, _ = tl.launches(run)
-    assert counts["cluster"] == 1 and counts["scores"] == 0
+    assert [counts[k] for k in ("cluster", "spread", "scores")] == [int(path == "cluster"), int(path == "spread"), 0]
     assert kvc.kvc_workspace_bytes(layer, 8, 5, 300) <= kvc.kvc_static_scratch_bytes()
     tl.assert_close(tl.np64(out), tl.oracle_run(shape, p, "fused")[2], "bf16")

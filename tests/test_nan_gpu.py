@@ -78,4 +78,4 @@ def _check(B, H_q, H_kv, grid, R, T, ratio, dtype, where, lengths):
 def test_spread_path(B, H_q, H_kv, grid, R, T, ratio, dtype, where, lengths, monkeypatch):
     monkeypatch.setenv("KVC_EXPANSION", "spread")
     counts = _check(B, H_q, H_kv, grid, R, T, ratio, dtype, where, lengths)
-    assert counts["spread"] == 1 and counts["scores"] == 0
+    assert counts["spread"] == 1 and counts["cluster"] == counts["scores"] == 0

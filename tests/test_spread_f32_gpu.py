@@ -40,7 +40,7 @@ def test_uniform(B, H_q, H_kv, grid, R, T, ratio, recipe):
     shape = wl.Shape("spread-f32", 1, B, H_q, H_kv, 128, grid, R, T, 1, "f32", ratio)
     p = tl.make_problem(shape, 640 + grid + B, T=T, T_cap=T + 3, recipe=recipe)
     counts, (_, _, _, out) = tl.launches(lambda: tl.gpu_run(shape, p))
-    assert counts["spread"] == 1 and counts["scores"] == 0
+    assert counts["spread"] == 1 and counts["cluster"] == counts["scores"] == 0
     tl.assert_close(tl.np64(out), tl.oracle_run(shape, p, "fused")[2], "f32")
 
 
@@ -54,7 +54,7 @@ def test_per_sequence_lengths(B, H_q, H_kv, grid, R, T, ratio, monkeypatch):
     R_b[-1] = R
     shape = wl.Shape("spread-f32-ragged", 1, B, H_q, H_kv, 128, grid, R, T, 1, "f32", ratio)
     counts, _ = tl.check_ragged(shape, 660 + grid, R_b, T_b)
-    assert counts["spread"] == 1 and counts["scores"] == 0
+    assert counts["spread"] == 1 and counts["cluster"] == counts["scores"] == 0
 
 
 @pytest.mark.parametrize("B,H_q,H_kv,grid,R,T,ratio", [

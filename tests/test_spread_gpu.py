@@ -53,7 +53,7 @@ def test_uniform(B, H_q, H_kv, grid, R, T, ratio, recipe, monkeypatch):
     shape = wl.Shape("spread", 1, B, H_q, H_kv, 128, grid, R, T, 1, "bf16", ratio)
     p = tl.make_problem(shape, 600 + grid + B, T=T, T_cap=T + 3, recipe=recipe)
     counts, (_, _, _, out) = tl.launches(lambda: tl.gpu_run(shape, p))
-    assert counts["spread"] == 1 and counts["scores"] == 0
+    assert counts["spread"] == 1 and counts["cluster"] == counts["scores"] == 0
     tl.assert_close(tl.np64(out), tl.oracle_run(shape, p, "fused")[2], "bf16")
 
 
@@ -70,7 +70,7 @@ def test_per_sequence_lengths(B, H_q, H_kv, grid, R, T, ratio, monkeypatch):
     R_b[-1] = R
     shape = wl.Shape("spread-ragged", 1, B, H_q, H_kv, 128, grid, R, T, 1, "bf16", ratio)
     counts, _ = tl.check_ragged(shape, 650 + grid, R_b, T_b)
-    assert counts["spread"] == 1 and counts["scores"] == 0
+    assert counts["spread"] == 1 and counts["cluster"] == counts["scores"] == 0
 
 
 @pytest.mark.parametrize("B,H_q,H_kv,grid,R,ratio", [(2, 8, 2, 24, 23, 375), (3, 28, 4, 27, 8, 750), (1, 16, 2, 9, 31, 600)])
