@@ -293,7 +293,7 @@ __global__ void __launch_bounds__(256) merge_kernel(DecodeArgs a) {
   float4 num = make_float4(0.f, 0.f, 0.f, 0.f);
   for (int p = 0; p < np; ++p) {
     const float2 v = st[p];
-    if (v.x == -INFINITY) continue;              // a piece without rows (text chunks beyond T)
+    if (v.x == -INFINITY && v.y == 0.f) continue;      // a piece without rows (text chunks beyond T); a NaN leaves the maximum alone and shows in the sum
     const float sc = __expf(v.x - mx);
     den = fmaf(sc, v.y, den);
     const float4 y = *reinterpret_cast<const float4*>(yp + (size_t)p * D + lane * 4);
