@@ -391,8 +391,8 @@ resident_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_con
       for (int w = 0; w < RS_WARPS; ++w) {
         const float* sy = reinterpret_cast<const float*>(sm + a.off_ring + region(w));
         const float* ss = sy + 8 * D;
-        if (has_items(w) && ss[head] != -INFINITY) {
-          const float f = fast_exp2(ss[head] - Mx);
+        if (has_items(w)) {
+          const float f = ss[head] == -INFINITY ? 0.f : fast_exp2(ss[head] - Mx);      // (a NaN leaves the maximum alone and shows in sum and outputs: kept)
           Ls = fmaf(f, ss[8 + head], Ls);
           Vs = fmaf(f, ss[16 + head], Vs);
           const float4 v = *reinterpret_cast<const float4*>(sy + head * D + lane * 4);

@@ -83,7 +83,7 @@ def test_spread_path(B, H_q, H_kv, grid, R, T, ratio, dtype, where, lengths, mon
 
 @pytest.mark.parametrize("lengths", [False, True])
 @pytest.mark.parametrize("where", ["query", "key", "text key", "value", "text value"])
-@pytest.mark.parametrize("path,grid,dtype", [("phases", 24, "bf16"), ("phases", 24, "f32"), ("phases", 27, "bf16"),
+@pytest.mark.parametrize("path,grid,dtype", [("phases", 24, "bf16"), ("phases", 24, "f32"), ("phases", 27, "bf16"), ("resident", 16, "bf16"),
                                              ("mma", 24, "bf16"), ("tcgen05", 24, "bf16"), ("split", 32, "bf16"), ("cluster", 24, "bf16")])
 def test_other_paths(path, grid, dtype, where, lengths, monkeypatch):
     monkeypatch.setenv("KVC_EXPANSION", path)
@@ -91,7 +91,7 @@ def test_other_paths(path, grid, dtype, where, lengths, monkeypatch):
     assert counts["spread"] == 0
 
 
-@pytest.mark.parametrize("path,grid,R", [("phases", 16, 12)])
+@pytest.mark.parametrize("path,grid,R", [("resident", 16, 12), ("phases", 16, 12)])
 def test_whole_parts_of_nan(path, grid, R, monkeypatch):
     """No text row, one query of NaN: every part that is joined has a NaN for a sum and nothing for a maximum."""
     monkeypatch.setenv("KVC_EXPANSION", path)
