@@ -91,8 +91,32 @@ def test_other_paths(path, grid, dtype, where, lengths, monkeypatch):
     assert counts["spread"] == 0
 
 
-@pytest.mark.parametrize("path,grid,R", [("resident", 16, 12), ("phases", 16, 12)])
-def test_whole_parts_of_nan(path, grid, R, monkeypatch):
+@pytest.mark.parametrize("lengths", [False, True])
+@pytest.mark.parametrize("path,grid,R,dtype", [
+    ("resident", 16, 12, "bf16"), ("phases", 16, 12, "bf16"), ("phases", 16, 12, "f32"), ("mma", 24, 12, "bf16"), ("tcgen05", 24, 12, "bf16"),
+    ("split", 32, 6, "bf16"), ("cluster", 24, 24, "bf16"), ("spread", 24, 24, "bf16"), ("spread", 17, 11, "f32"),
+])
+def test_whole_parts_of_nan(path, grid, R, dtype, lengths, monkeypatch):
     """No text row, one query of NaN: every part that is joined has a NaN for a sum and nothing for a maximum."""
     monkeypatch.setenv("KVC_EXPANSION", path)
-    _check(2, 8, 2, grid, R, 0, 600, "bf16", "query", False)
+    _check(2, 8, 2, grid, R, 0, 600, dtype, "query", lengths)
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("S", [1, 70, 3000])
+def test_uncompressed_attention(S, dtype):
+    gen = torch.Generator().manual_seed(S)
+    B, H_q, H_kv = 2, 8, 2
+    q, K, V = (torch.randn(x, generator=gen).to(wl.torch_dtype(dtype)) for x in ((B, H_q, 128), (B, H_kv, S, 128), (B, H_kv, S, 128)))
+    q[1, -1, 5] = float("nan")
+    K[0, 0, S // 2, 3] = float("nan")
+    V[0, 1, S - 1, 9] = float("nan")
+    layer = kvc.Layer(H_q, H_kv, 128, 64, 0, wl.torch_dtype(dtype))
+    ws = kvc.alloc_workspace(layer, B, 0, S)
+    out = torch.empty((B, H_q, 128), dtype=wl.torch_dtype(dtype), device=DEV)
+    kvc.kvc_attend_full(layer, q.to(DEV), K.to(DEV), V.to(DEV), B, S, S, out, ws)
+    x = torch.einsum("bhgd,bhsd->bhgs", q.double().view(B, H_kv, -1, 128) * 128 ** -0.5, K.double())
+    want = torch.einsum("bhgs,bhsd->bhgd", torch.softmax(x, -1), V.double()).reshape(B, H_q, 128).numpy()
+    got = tl.np64(out)
+    np.testing.assert_array_equal(np.isnan(got), np.isnan(want))
+    tl.assert_close(np.nan_to_num(got), np.nan_to_num(want), dtype)
