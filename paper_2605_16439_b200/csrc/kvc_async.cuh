@@ -58,8 +58,9 @@ __device__ __forceinline__ bool mbar_test_wait(uint64_t* bar, uint32_t parity) {
       : "=r"(ok) : "r"(smem_addr(bar)), "r"(parity) : "memory");
   return ok != 0;
 }
-// true on completion, false if the spin limit ran out.  ROLLED: the loop is left rolled, which keeps the code around the wait small (16 x 8 blocks
-// of n = 1024: 47.2 us a call unrolled, 46.0 rolled); the uniform one-kernel path takes 1 % less with the compiler's choice
+// true on completion, false if the spin limit ran out.  ROLLED: the loop is left rolled, which keeps the code around the wait small (three-kernel
+// path, 16 x 8 blocks of n = 1024: 47.2 us a call unrolled, 46.0 rolled; cluster path, 26 calls it takes by default: 69.2 and 67.4 in the geometric
+// mean, none longer by more than 0.1).  The uniform one-kernel path takes 1 % less with the compiler's choice
 template <bool ROLLED = true>
 __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity) {
   if constexpr (ROLLED) {
@@ -110,16 +111,10 @@ __device__ __forceinline__ bool mbar_try_wait_cluster(uint64_t* bar, uint32_t pa
       : "=r"(ok) : "r"(smem_addr(bar)), "r"(parity) : "memory");
   return ok != 0;
 }
-template <bool ROLLED = true>
 __device__ __forceinline__ bool mbar_wait_cluster_bounded(uint64_t* bar, uint32_t parity) {
-  if constexpr (ROLLED) {
 #pragma unroll 1
-    for (uint32_t i = 0; i < WAIT_SPIN_LIMIT; ++i)
-      if (mbar_try_wait_cluster(bar, parity)) return true;
-  } else {
-    for (uint32_t i = 0; i < WAIT_SPIN_LIMIT; ++i)
-      if (mbar_try_wait_cluster(bar, parity)) return true;
-  }
+  for (uint32_t i = 0; i < WAIT_SPIN_LIMIT; ++i)
+    if (mbar_try_wait_cluster(bar, parity)) return true;
   return false;
 }
 // asynchronous stores into a peer's shared memory; their bytes are reported to the peer's barrier when they have landed

@@ -260,7 +260,7 @@ __device__ __forceinline__ bool cl_text_part(const CUtensorMap& tmKt, const CUte
       const int nv = min(16, n_rows - r0);
       // ---- keys
       uint32_t s = us_cnt % CL_TEXT_SLOTS;
-      if (!dead && !mbar_wait_bounded<false>(&bars.text[warp][s], (us_cnt / CL_TEXT_SLOTS) & 1u)) dead = true;
+      if (!dead && !mbar_wait_bounded(&bars.text[warp][s], (us_cnt / CL_TEXT_SLOTS) & 1u)) dead = true;
       __syncwarp();
       float cc[2][4];
       {
@@ -325,7 +325,7 @@ __device__ __forceinline__ bool cl_text_part(const CUtensorMap& tmKt, const CUte
       }
       // ---- values
       s = us_cnt % CL_TEXT_SLOTS;
-      if (!dead && !mbar_wait_bounded<false>(&bars.text[warp][s], (us_cnt / CL_TEXT_SLOTS) & 1u)) dead = true;
+      if (!dead && !mbar_wait_bounded(&bars.text[warp][s], (us_cnt / CL_TEXT_SLOTS) & 1u)) dead = true;
       __syncwarp();
       const bool ragged_rows = a.T_b != nullptr && nv < 16;
       if (ragged_rows) {
@@ -489,7 +489,7 @@ cluster_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
       // last one has been consumed when the slot's empty barrier has left that parity's phase (a slot never filled passes at once).
       uint32_t kb = 0, vb = 0, xb = 0;
       bool ok = true;
-      auto drained = [&](uint64_t* empty, uint32_t bits, int s) { if (ok && !mbar_wait_bounded<false>(&empty[s], ((bits >> s) & 1u) ^ 1u)) ok = false; };
+      auto drained = [&](uint64_t* empty, uint32_t bits, int s) { if (ok && !mbar_wait_bounded(&empty[s], ((bits >> s) & 1u) ^ 1u)) ok = false; };
       bool waited = ragged;
       if (!a.early && !waited) { grid_dep_wait(); waited = true; }
       const int spg = a.nV / CL_GROUPS;                                       // value slots per group
@@ -628,7 +628,7 @@ cluster_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
     uint32_t xs = 0, xb = 0, round = 0, wpass = 0;              // bit s of xb: parity of the fills of slot s taken so far
     bool dead = false;
     auto wait_on = [&](uint64_t* bar, uint32_t parity) {
-      if (!dead && !mbar_wait_bounded<false>(bar, parity)) dead = true;
+      if (!dead && !mbar_wait_bounded(bar, parity)) dead = true;
       __syncwarp();
       tc_fence_after();
     };
@@ -775,7 +775,7 @@ cluster_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
 #pragma unroll
             for (int ks = 0; ks < 8; ++ks) ldsm_x4(qa[ks], qrow + (uint32_t)ks * 32u);
           }
-          if (!dead && !mbar_wait_bounded<false>(&bars.kfull[s], (kb >> s) & 1u)) dead = true;
+          if (!dead && !mbar_wait_bounded(&bars.kfull[s], (kb >> s) & 1u)) dead = true;
           kb ^= 1u << s;
           __syncwarp();
           const uint32_t k_u = ring_u + s * CL_TILE_BYTES;
@@ -844,7 +844,7 @@ cluster_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
         const uint32_t trow = tb + ((uint32_t)(rg * 32) << 16);
         const bool work = rg * 32 < rows;
         unsigned char* sm_p = sm;
-        if (!dead && !mbar_wait_bounded<false>(&bars.l_done, round & 1u)) dead = true;
+        if (!dead && !mbar_wait_bounded(&bars.l_done, round & 1u)) dead = true;
         __syncwarp();
         tc_fence_after();
         const int cb = (hf * (NWc >> 5) / CL_GROUPS) * 32, ce = ((hf + 1) * (NWc >> 5) / CL_GROUPS) * 32;
@@ -936,7 +936,7 @@ cluster_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
         const int row = rg * 32 + lane, hf = grp;
         const uint32_t trow = tb + ((uint32_t)(rg * 32) << 16);
         const bool work = rg * 32 < rows;
-        if (!dead && !mbar_wait_bounded<false>(&bars.w_done, wpass & 1u)) dead = true;
+        if (!dead && !mbar_wait_bounded(&bars.w_done, wpass & 1u)) dead = true;
         ++wpass;
         __syncwarp();
         tc_fence_after();
@@ -1054,7 +1054,7 @@ cluster_decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
               }
             }
           }
-          if (!dead && !mbar_wait_bounded<false>(&bars.vfull[s], (vb >> s) & 1u)) dead = true;
+          if (!dead && !mbar_wait_bounded(&bars.vfull[s], (vb >> s) & 1u)) dead = true;
           vb ^= 1u << s;
           __syncwarp();
           if (jt * CL_TILE + rg * 16 < a.m) {
