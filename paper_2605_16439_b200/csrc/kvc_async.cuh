@@ -59,8 +59,9 @@ __device__ __forceinline__ bool mbar_test_wait(uint64_t* bar, uint32_t parity) {
   return ok != 0;
 }
 // true on completion, false if the spin limit ran out.  ROLLED: the loop is left rolled, which keeps the code around the wait small (three-kernel
-// path, 16 x 8 blocks of n = 1024: 47.2 us a call unrolled, 46.0 rolled; cluster path, 26 calls it takes by default: 69.2 and 67.4 in the geometric
-// mean, none longer by more than 0.1).  The uniform one-kernel path takes 1 % less with the compiler's choice
+// path, 16 x 8 blocks of n = 1024: 47.2 us a call unrolled, 46.0 rolled; cluster path, 26 calls it takes by default: 68.9 and 67.3 in the geometric
+// mean).  The uniform one-kernel path takes 1 % less with the compiler's choice, the cluster path's text warps about 1 % (35 calls of 1000 to 3800 text
+// rows 126.8 and 125.5, where with all waits unrolled they take 128.9; 30 x 10 blocks of n = 81, 3800 rows 71.1 and 67.8)
 template <bool ROLLED = true>
 __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity) {
   if constexpr (ROLLED) {

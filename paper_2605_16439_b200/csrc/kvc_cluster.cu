@@ -260,7 +260,7 @@ __device__ __forceinline__ bool cl_text_part(const CUtensorMap& tmKt, const CUte
       const int nv = min(16, n_rows - r0);
       // ---- keys
       uint32_t s = us_cnt % CL_TEXT_SLOTS;
-      if (!dead && !mbar_wait_bounded(&bars.text[warp][s], (us_cnt / CL_TEXT_SLOTS) & 1u)) dead = true;
+      if (!dead && !mbar_wait_bounded<false>(&bars.text[warp][s], (us_cnt / CL_TEXT_SLOTS) & 1u)) dead = true;
       __syncwarp();
       float cc[2][4];
       {
@@ -325,7 +325,7 @@ __device__ __forceinline__ bool cl_text_part(const CUtensorMap& tmKt, const CUte
       }
       // ---- values
       s = us_cnt % CL_TEXT_SLOTS;
-      if (!dead && !mbar_wait_bounded(&bars.text[warp][s], (us_cnt / CL_TEXT_SLOTS) & 1u)) dead = true;
+      if (!dead && !mbar_wait_bounded<false>(&bars.text[warp][s], (us_cnt / CL_TEXT_SLOTS) & 1u)) dead = true;
       __syncwarp();
       const bool ragged_rows = a.T_b != nullptr && nv < 16;
       if (ragged_rows) {
