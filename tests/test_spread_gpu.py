@@ -127,3 +127,17 @@ def test_long_score_rows_keep_both_terms(B, H_q, H_kv, grid, R, T, ratio, length
                                     tl.np64(p["V_txt"]), R_b, T_b, "kv")
     err = float(np.linalg.norm(tl.np64(out) - want) / np.linalg.norm(want))
     assert err <= 2.0 ** -9 + 1e-4, err
+
+
+@pytest.mark.parametrize("B,H_q,H_kv,grid,R,T,ratio,path", [
+    (8, 16, 1, 16, 1, 26, 875, "one"), (5, 12, 1, 16, 2, 267, 850, "one"), (1, 12, 1, 8, 12, 197, 875, "one"),
+    (3, 12, 1, 16, 2, 576, 275, "spread"), (3, 12, 1, 24, 5, 260, 750, "spread"), (11, 16, 1, 32, 1, 1, 550, "spread"),
+    (9, 16, 1, 23, 4, 3, 550, "spread"), (13, 10, 1, 32, 12, 325, 725, "split"),
+])
+def test_routing_with_more_than_eight_query_heads_per_kv_head(B, H_q, H_kv, grid, R, T, ratio, path):
+    """Both sides of the rule that compares the path's estimate with one of the path it stands before, by default routing."""
+    shape = wl.Shape("spread-route", 1, B, H_q, H_kv, 128, grid, R, T, 1, "bf16", ratio)
+    p = tl.make_problem(shape, 670 + grid + B, T=T, T_cap=T, recipe="peaked")
+    counts, (_, _, _, out) = tl.launches(lambda: tl.gpu_run(shape, p))
+    assert [counts["spread"], counts["fused"] - counts["spread"], counts["split_output"]] == [int(path == x) for x in ("spread", "one", "split")]
+    tl.assert_close(tl.np64(out), tl.oracle_run(shape, p, "fused")[2], "bf16")
