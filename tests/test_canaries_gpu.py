@@ -1,6 +1,6 @@
 """Guard regions around every buffer the library writes: compress, decode (every default path, the ragged and one-sided
 calls) and the fits must leave the bytes in front of and behind their outputs, the capsule store and the workspace
-untouched.  (A stand-in for a memory checker: it catches stray writes next to the caller's buffers, not reads.)"""
+untouched, on every path of the library.  (A stand-in for a memory checker: it catches stray writes next to the caller's buffers, not reads.)"""
 import numpy as np
 import pytest
 import torch
@@ -38,21 +38,31 @@ class Guarded:
         return bool((self.raw[:self.off] == PATTERN).all()) and bool((self.raw[self.off + self.n:] == PATTERN).all())
 
 
-CASES = [  # B, H_q, H_kv, grid, R, T, dtype, mode
-    (2, 4, 4, 24, 3, 70, "bf16", "kv"),      # mma.sync one-kernel path (n = 576)
-    (2, 14, 2, 32, 3, 130, "bf16", "kv"),    # three-kernel path (n = 1024)
-    (3, 14, 2, 16, 5, 77, "bf16", "kv"),     # resident path (n = 256), partials in the workspace
-    (2, 8, 2, 12, 2, 33, "f32", "kv"),       # three-phase kernels
-    (2, 6, 2, 8, 3, 9, "bf16", "k"),
-    (2, 6, 2, 8, 3, 9, "f32", "v"),
-    (2, 4, 2, 8, 2, 0, "bf16", "kv"),        # no text
-    (38, 2, 2, 32, 1, 0, "bf16", "kv"),      # three-kernel path, one CTA of the output kernel per pair, no text
-    (40, 8, 8, 16, 2, 20, "bf16", "kv"),     # resident path, more pairs than SMs
+CASES = [  # B, H_q, H_kv, grid, R, T, dtype, mode, path forced (None: as the library picks), kernels of a uniform call
+    (2, 4, 4, 24, 3, 70, "bf16", "kv", None, {"fused", "spread"}),
+    (2, 8, 2, 24, 23, 60, "bf16", "kv", None, {"fused", "spread"}),        # several groups of blocks, partials in the workspace
+    (2, 8, 2, 12, 2, 33, "f32", "kv", None, {"fused", "spread"}),
+    (2, 8, 2, 17, 11, 70, "f32", "kv", None, {"fused", "spread"}),         # several groups
+    (2, 4, 4, 24, 3, 70, "bf16", "kv", "mma", {"fused"}),
+    (2, 14, 2, 32, 3, 130, "bf16", "kv", "tcgen05", {"fused_tc"}),
+    (2, 14, 2, 32, 3, 130, "bf16", "kv", "pair", {"fused_pair"}),
+    (2, 14, 2, 32, 3, 130, "bf16", "kv", "split", {"split_scores", "split_expand", "split_output"}),
+    (2, 14, 2, 27, 3, 130, "bf16", "kv", "cluster", {"fused", "cluster"}),
+    (3, 14, 2, 16, 5, 77, "bf16", "kv", "resident", {"resident"}),         # partials in the workspace
+    (2, 8, 2, 12, 2, 33, "bf16", "kv", "phases", {"scores", "expand", "combine", "output", "merge"}),
+    (2, 8, 2, 12, 2, 33, "f32", "kv", "phases", {"scores", "expand", "combine", "output", "merge"}),
+    (2, 6, 2, 8, 3, 9, "bf16", "k", None, {"scores", "expand", "combine", "output", "merge"}),
+    (2, 6, 2, 8, 3, 9, "f32", "v", None, {"scores", "expand", "combine", "output", "merge"}),
+    (2, 4, 2, 8, 2, 0, "bf16", "kv", None, {"resident"}),                  # no text
+    (38, 2, 2, 32, 1, 0, "bf16", "kv", "split", {"split_scores", "split_expand", "split_output"}),     # one CTA of the output kernel per pair, no text
+    (40, 8, 8, 16, 2, 20, "bf16", "kv", None, {"resident"}),               # more pairs than SMs
 ]
 
 
-@pytest.mark.parametrize("B,H_q,H_kv,grid,R,T,dtype,mode", CASES)
-def test_compress_and_decode_write_only_inside_their_buffers(B, H_q, H_kv, grid, R, T, dtype, mode):
+@pytest.mark.parametrize("B,H_q,H_kv,grid,R,T,dtype,mode,path,kernels", CASES)
+def test_compress_and_decode_write_only_inside_their_buffers(B, H_q, H_kv, grid, R, T, dtype, mode, path, kernels, monkeypatch):
+    if path:
+        monkeypatch.setenv("KVC_EXPANSION", path)
     shape = wl.Shape("canary", 1, B, H_q, H_kv, 128, grid, R, T, 1, dtype, 600)
     T_cap = T + 5
     p = tl.make_problem(shape, 77 + grid + R, T=T, T_cap=T_cap, recipe="peaked")
@@ -65,9 +75,11 @@ def test_compress_and_decode_write_only_inside_their_buffers(B, H_q, H_kv, grid,
     kvc.kvc_compress(layer, p["K_vis"].to(DEV), p["V_vis"].to(DEV), B, R, caps.payload)
     K_txt = p["K_txt"].to(DEV) if T_cap > 0 else None
     V_txt = p["V_txt"].to(DEV) if T_cap > 0 else None
-    for _ in range(2):                                   # the second call reads the settled store early
-        kvc.kvc_decode_attend(layer, p["q"].to(DEV), caps.payload, B, R, K_txt, V_txt, T, T_cap, out_t, ws.payload)
+    run = lambda: kvc.kvc_decode_attend(layer, p["q"].to(DEV), caps.payload, B, R, K_txt, V_txt, T, T_cap, out_t, ws.payload)
+    counts, _ = tl.launches(run)
+    run()                                                # the second call reads the settled store early
     torch.cuda.synchronize()
+    assert {k for k, v in counts.items() if v} == kernels
     assert caps.intact() and ws.intact() and out.intact()
     assert kvc.kvc_read_device_status(layer, B, R, T, ws.payload) == 0
     _, _, want = tl.oracle_run(shape, p, "fused", mode)

@@ -391,17 +391,21 @@ def _fused_launches(fn):
         torch.cuda.synchronize()
     finally:
         kvc.kvc_profile_stop()
-    out = {k: v[1] for k, v in kvc.kvc_profile_read().items()}
+    out = {k: v[1] for k, v in {**kvc.kvc_profile_read(), **kvc.kvc_profile_parts()}.items()}
     kvc.kvc_profile_start(0)
     kvc.kvc_profile_stop()
     return out
 
 
 def test_bf16_block_lengths_of_the_configurations_take_the_one_kernel_path():
-    shape = tl.small(wl.CONFIGS[1], B=2, H_q=4, H_kv=4)
+    shape = tl.small(wl.CONFIGS[1], B=40, H_q=4, H_kv=4, R=2)
     p = tl.make_problem(shape, 131, T=40, T_cap=48)
     counts = _fused_launches(lambda: tl.gpu_run(shape, p))
-    assert counts["fused"] == 1 and counts["scores"] == 0 and counts["output"] == 0
+    assert counts["fused"] == 1 and counts["spread"] == counts["cluster"] == 0 and counts["scores"] == 0 and counts["output"] == 0
+    # few pairs: a cluster of CTAs for each
+    shape1 = tl.small(wl.CONFIGS[1], B=2, H_q=4, H_kv=4)
+    p1 = tl.make_problem(shape1, 133, T=40, T_cap=48)
+    assert _fused_launches(lambda: tl.gpu_run(shape1, p1))["spread"] == 1
     # a block length that is not a multiple of 64 goes through the three-phase kernels
     shape2 = wl.Shape("odd-n", 1, 2, 4, 2, 128, 7, 2, 9, 1, "bf16")
     p2 = tl.make_problem(shape2, 132)
@@ -420,22 +424,33 @@ def test_bf16_block_lengths_of_the_configurations_take_the_one_kernel_path():
     (1, 16, 1, 8, 3, 20),      # G = 16: two head tiles, one block per unit
     (1, 12, 2, 32, 2, 64),     # n = 1024
 ])
-def test_one_kernel_path_edges(B, H_q, H_kv, grid, R, T):
+@pytest.mark.parametrize("path", [None, "mma"])
+def test_one_kernel_path_edges(B, H_q, H_kv, grid, R, T, path, monkeypatch):
+    """As the library routes them (the smallest calls to the spread path) and through the one-kernel paths."""
+    if path:
+        monkeypatch.setenv("KVC_EXPANSION", path)
     shape = wl.Shape("fused-edge", 1, B, H_q, H_kv, 128, grid, R, T, 1, "bf16")
     p = tl.make_problem(shape, 140 + B + 7 * R + T, T=T, T_cap=T + 5)
-    _check(shape, p)
+    counts = _fused_launches(lambda: _check(shape, p))
+    if path:
+        assert counts["fused"] + counts["fused_tc"] + counts["fused_pair"] == 1 and counts["spread"] == counts["cluster"] == counts["scores"] == 0
 
 
 # per-layer ratios of a pyramid schedule (Sec. 2.4, Sec. 3.2: shallow layers compress less, deep layers more): every retained
-# length between 0.3 and 0.9 on the 7B block lengths goes through the same one-kernel path as the uniform 0.6
+# length between 0.3 and 0.9 on the 7B block lengths goes through the same path as the uniform 0.6
 @pytest.mark.parametrize("ratio", [300, 375, 450, 525, 600, 675, 750, 825, 900])
 @pytest.mark.parametrize("ci,kw", [(1, dict(B=2, H_q=4, H_kv=4, R=3)), (2, dict(B=1, H_q=14, H_kv=2, R=3))])
-def test_pyramid_schedule_ratios_on_the_7b_block_lengths(ci, kw, ratio):
+@pytest.mark.parametrize("forced", [False, True])
+def test_pyramid_schedule_ratios_on_the_7b_block_lengths(ci, kw, ratio, forced, monkeypatch):
+    """These few pairs take the spread path; forced, the path that larger batches of the block length take."""
+    if forced:
+        monkeypatch.setenv("KVC_EXPANSION", {1: "mma", 2: "split"}[ci])
     shape = tl.small(wl.CONFIGS[ci], ratio_permille=ratio, **kw)
     p = tl.make_problem(shape, 900 + ci + ratio, T=70, T_cap=80)
     counts = _fused_launches(lambda: _check(shape, p))
-    # one kernel per call for the LLaVA-NeXT block length, the three-kernel bf16 path for the Qwen2-VL one
-    assert counts["fused"] + counts["fused_tc"] + counts["fused_pair"] + counts["split_output"] == 1 and counts["scores"] == 0
+    # forced: one kernel per call for the LLaVA-NeXT block length, the three-kernel bf16 path for the Qwen2-VL one
+    assert counts["spread"] == int(not forced) and counts["split_output"] == int(forced and ci == 2) and counts["scores"] == 0
+    assert counts["fused"] + counts["fused_tc"] + counts["fused_pair"] == int(not forced or ci == 1)
 
 
 @pytest.mark.parametrize("B,H_q,H_kv,grid,R,T,ratio", [
