@@ -307,16 +307,16 @@ def capsule_views(layer: Layer, capsules, B: int, R: int):
     """(K_tilde [B,H_kv,R,m_k,d], V_tilde [B,H_kv,R,m_v,d]) typed views of a capsule store (no copy)."""
     m_k, m_v, d, H = layer.m_k, layer.m_v, layer.d, layer.H_kv
     if B > 0 and R > 0 and capsules.dim() == 1 and capsules.dtype is torch.uint8:
-        # three tensor operations instead of six (4 us instead of 7, where the smallest calls take 9)
+        # four tensor operations instead of six (5.5 us instead of 8, where the smallest calls take 9); no storage offset is read: it would be
+        # a constant of a traced graph, and what does not return a tensor cannot be compiled
         try:
             t = capsules.view(layer.dtype)
         except RuntimeError:                        # bytes that are not whole elements: the parts below may be
             t = None
         kn = B * H * R * m_k * d
         if t is not None and t.numel() >= kn + B * H * R * m_v * d:
-            at = t.storage_offset()
-            return (t.as_strided((B, H, R, m_k, d), (H * R * m_k * d, R * m_k * d, m_k * d, d, 1), at),
-                    t.as_strided((B, H, R, m_v, d), (H * R * m_v * d, R * m_v * d, m_v * d, d, 1), at + kn))
+            return (t.as_strided((B, H, R, m_k, d), (H * R * m_k * d, R * m_k * d, m_k * d, d, 1)),
+                    t[kn:].as_strided((B, H, R, m_v, d), (H * R * m_v * d, R * m_v * d, m_v * d, d, 1)))
     total = kvc_capsule_bytes(layer, B, R)
     kb = total // (m_k + m_v) * m_k
     return (capsules[:kb].view(layer.dtype).view(B, layer.H_kv, R, m_k, d),
