@@ -478,7 +478,9 @@ static bool use_spread(const kvc_layer* L, int B, int R, int T, bool ragged, con
   return n >= 96 || p.C * p.nrg > 2;
 }
 
-// Which fp32 calls take the spread path: those of one wave of clusters (0.29 to 0.97 of the three-phase kernels' time over 44 drawn calls), and
+// Which fp32 calls take the spread path (410 of 492 drawn ones, half the three-phase kernels' time in the geometric mean; three of them are longer than
+// there, with one query head per KV head and many retained rows, at worst 2 x 2 of n = 729, m = 438, 32/32 heads, 158 / 138, which neither
+// estimate tells apart): those of one wave of clusters (0.29 to 0.97 of the three-phase kernels' time over 44 drawn calls), and
 // of up to four where its estimate is under nine tenths of theirs (0.74 with lengths per sequence, whose sum it does not see: 11 x 4 of n = 841,
 // 28/4 heads, 316, estimated 268 to 359, / 299; 0.7 with one query head per KV head: 2 x 3 of 1024, 32/32 heads 250,
 // estimated 199, / 194; 13 x 3 of 169, 28/4 heads 52 / 97; 16 x 8 of 169 95 / 128).  Their estimate: the columns and chunks of a CTA's walk,

@@ -1,10 +1,11 @@
 // Spread decode kernel (see kvc_spread.cuh) and its host side.
 //
 // Bound: a chain of dependent steps, four of them exchanges within a cluster of 0.5-1 us; the bytes take a tenth to a half of the time.
-// Measured on B200, us per call, before / now: 1 x 5 blocks of n = 576, 32/32 heads, 128 text rows (the one-kernel path on 32 SMs) 25.5 /
-// 12.8, its time line: scores until 2.5 us after the previous kernel's end, logits 4.2, probabilities 4.9, text 5.3, weights 6.4 (at their
-// owners 7.4), values 9.1, out 10.4; 8 x 5 of n = 729, 28/4 heads (the cluster path) 36.2 / 27.0; 1 x 5 of 576, 28/4 heads 25.5 / 15.3; 7 x 2
-// of 576, m = 404, 38.0 / 14.8; 4 x 5 of 1024, m = 103 (three kernels) 21.1 / 12.6; 1 x 1 of 576, 8/2 heads, 16384 text rows 170 / 21.
+// Measured on B200, us per call of a captured graph back to back, the path before / this one: 1 x 5 blocks of n = 576, 32/32 heads, 128 text
+// rows (the one-kernel path on 32 SMs) 25.0 / 12.3 (32 layers in turn 12.7; its time line: scores until 2.5 us after the previous kernel's end,
+// logits 4.2, probabilities 4.9, text 5.3, weights 6.4, at their owners 7.4, values 9.1, out 10.4); 8 x 5 of n = 729, 28/4 heads (the cluster
+// path) 36.6 / 26.9; 1 x 5 of 576, 28/4 heads 24.2 / 13.0; 7 x 2 of 576, m = 404, 37.6 / 14.4; 4 x 5 of 1024, m = 103 (three kernels) 20.6 /
+// 11.9; 1 x 1 of 576, 8/2 heads, 16384 text rows 168 / 19.4.
 // Why pieces are few and large: a look at a piece by all warps, with its loops, takes some 200 cycles, issuing one some 300 (pieces of 16 KB,
 // 21 of them in the first shape: 19.7 us, of 39 KB: 16.9).  Why every loop that need not be is kept rolled: unrolled, the kernel was 100 to
 // 130 KB of code, now 50.

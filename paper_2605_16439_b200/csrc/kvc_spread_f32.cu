@@ -7,8 +7,9 @@
 //            through shared memory
 //   step 3   a thread per retained row (two where they fit): its row of U in shared memory, P broadcast
 //   step 4   a warp per value row, four channels per lane; text rows the same way with their weights in shared memory
-// 1 x 1 block of n = 576, 8/2 heads, 32 text rows: 42.3 us (four launches) -> 15.7; 4 x 3 of 256, 28/4 heads, 3173 rows 147 -> 44; 1 x 16 of 576,
-// m = 389, 8/2 heads 113 -> 33; 8 x 1 of 1024, m = 794 101 -> 97.
+// 1 x 1 block of n = 576, 8/2 heads, 32 text rows: 35.1 us (four launches) -> 13.6; 4 x 3 of 256, 28/4 heads, 3173 rows 123 -> 35; 1 x 16 of 576,
+// m = 389, 8/2 heads 108 -> 31; 8 x 1 of 1024, m = 794 87 -> 81 (calls of a captured graph back to back).
+// Error against 64 bits, 59 shapes, relative to the three-phase kernels': 0.81 with peaked softmaxes, 0.94 with flat ones (geometric means).
 // Bound: the chain of these steps and of four exchanges; theta and U come at the rate of the SMs that take part.
 #include <algorithm>
 
