@@ -73,10 +73,10 @@ def test_per_sequence_lengths(B, H_q, H_kv, grid, R, T, ratio, monkeypatch):
     assert counts["spread"] == 1 and counts["cluster"] == counts["scores"] == 0
 
 
-@pytest.mark.parametrize("B,H_q,H_kv,grid,R,ratio", [(2, 8, 2, 24, 23, 375), (3, 28, 4, 27, 8, 750), (1, 16, 2, 9, 31, 600)])
+@pytest.mark.parametrize("B,H_q,H_kv,grid,R,ratio", [(2, 8, 2, 24, 23, 375), (3, 28, 4, 27, 8, 750), (1, 16, 2, 9, 31, 600), (2, 14, 2, 32, 9, 200)])
 def test_workspace_holds_every_shorter_text(B, H_q, H_kv, grid, R, ratio, monkeypatch):
-    """The number of groups a pair's blocks are split into depends on the text: a workspace for T_cap rows serves every T below, and
-    nothing behind it is written."""
+    """The number of groups a pair's blocks are split into depends on the text, and at n = 1024, m = 820 the terms on whether the lengths are
+    given per sequence: a workspace for T_cap rows serves every T below and both calls, and nothing behind it is written."""
     monkeypatch.setenv("KVC_EXPANSION", "spread")
     T_cap = 6000
     shape = wl.Shape("spread-ws", 1, B, H_q, H_kv, 128, grid, R, T_cap, 1, "bf16", ratio)
@@ -88,8 +88,13 @@ def test_workspace_holds_every_shorter_text(B, H_q, H_kv, grid, R, ratio, monkey
     ws = torch.full((need + (4 << 20),), 0xA5, dtype=torch.uint8, device="cuda")
     q, K_txt, V_txt = p["q"].cuda(), p["K_txt"].cuda(), p["V_txt"].cuda()
     out = torch.empty((B, H_q, 128), dtype=torch.bfloat16, device="cuda")
+    full = torch.full((B,), R, dtype=torch.int32, device="cuda")
     for T in (0, 1, 100, 700, 3000, T_cap):
         counts, _ = tl.launches(lambda: kvc.kvc_decode_attend(layer, q, caps, B, R, K_txt, V_txt, T, T_cap, out, ws))
+        assert counts["spread"] == 1
+        assert kvc.kvc_read_device_status(layer, B, R, T, ws) == 0
+        ragged = lambda: kvc.kvc_decode_attend_ragged(layer, q, caps, B, R, full, K_txt, V_txt, T, None, T_cap, out, ws)
+        counts, _ = tl.launches(ragged)
         assert counts["spread"] == 1
         assert kvc.kvc_read_device_status(layer, B, R, T, ws) == 0
         assert bool((ws[need:] == 0xA5).all()), T
