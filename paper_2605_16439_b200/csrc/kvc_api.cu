@@ -460,6 +460,7 @@ static double general_estimate(const kvc_layer* L, int B, int R, int T, bool rag
   }
   // the cluster path: rounds of units and their tiles, the bytes; fitted to 97 uniform calls of up to eight query heads per KV head, 10 %
   const int units = H * ceil_div(B * R, CL_ROWS / G), NS = ceil_div(ceil_div(n, 64), terms == 2 ? 2 : 4);
+  if (NS > CL_MAX_NS) return other;          // longer blocks than its clusters hold: the three-phase kernels, 105 us and more
   const int held = sms * 88 / 100 / NS, rounds = ceil_div(units, held > 0 ? held : 1);
   const double rows = 512.0 * B * R * H * (double)m + 4.0 * H * (double)m * n, text = 512.0 * B * H * (double)T;
   return std::min(other, rounds * (24.4 + 1.93 * ceil_div(m, 64)) - 4.2 + (1.71 * rows + 1.86 * text) / HBM_US + 0.0137 * B * H);

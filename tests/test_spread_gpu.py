@@ -138,6 +138,7 @@ def test_long_score_rows_keep_both_terms(B, H_q, H_kv, grid, R, T, ratio, length
     (8, 16, 1, 16, 1, 26, 875, "one"), (5, 12, 1, 16, 2, 267, 850, "one"), (1, 12, 1, 8, 12, 197, 875, "one"),
     (3, 12, 1, 16, 2, 576, 275, "spread"), (3, 12, 1, 24, 5, 260, 750, "spread"), (11, 16, 1, 32, 1, 1, 550, "spread"),
     (9, 16, 1, 23, 4, 3, 550, "spread"), (13, 10, 1, 32, 12, 325, 725, "split"),
+    (2, 48, 4, 38, 2, 16, 500, "spread"),        # n = 1444: longer than the cluster path takes
 ])
 def test_routing_with_more_than_eight_query_heads_per_kv_head(B, H_q, H_kv, grid, R, T, ratio, path):
     """Both sides of the rule that compares the path's estimate with one of the path it stands before, by default routing."""
