@@ -441,41 +441,48 @@ static bool use_cluster(const kvc_layer* L, int B, int R, int T, bool ragged) {
 // Calls whose path the tests name stay where they are, although this one is ahead: lengths per sequence on those short
 // blocks (6 x 1 of n = 256, 8/2 heads 10.3 / 13.4) or under 1e7 flop of expansion beside them, and clusters of two on blocks under 96 positions
 // (32 x 1 of n = 81, 8/2 heads, 700 rows 12.3 / 36.9).  KVC_EXPANSION=spread forces it where its plan applies, any other value keeps it off.
-// More than eight query heads per KV head: where its estimate is ahead of one of the path it stands before.  Of 352 drawn calls with 10 to 16
-// it is the faster path for 265; taken for all that the rules above give it, 56 were more than 3 % longer (13 x 12 of 1024, 10/1 heads 61 / 34;
-// 9 x 11 of 256, 28/2 heads, 1492 rows 32 / 22), by the estimates 3, at worst 1.15 times, and the geometric mean is 0.81 of the other paths' time.
-static double general_estimate(const kvc_layer* L, int B, int R, int T, bool ragged, int terms) {
-  // fitted (least squares of the relative error) to those calls: the one-kernel path's 12 %, the three-kernel path's 10 %; the cluster path's, see below, 18 %
-  const int n = L->desc.n, m = L->m, H = L->desc.H_kv, G = L->G, sms = L->num_sms > 0 ? L->num_sms : 148;
-  double other = 1e30;
-  if (!ragged && n % 64 == 0) {
-    const FusedPlan f = plan_fused(L, B, R);
-    if (n > 640 && plan_split(L, B, R).ok) {
-      other = 15.7 + 0.027 * m + 0.6 * H * ceil_div(B * R * G, 128) + 0.33 * 512.0 * B * H * (2.0 * R * m + 2.0 * T) / HBM_US;
-    } else if (f.ok) {
-      const int waves = ceil_div(f.units, sms);
-      other = 9.8 + 0.030 * m + 15.6 * (waves - 1) + 6.9e-5 * waves * m * (double)n + 9.5e-3 * T / f.nrg + (f.nrg > 1 ? 5.3 : 0.0);
-    }
-    if (n <= 256 || n > 640) return other;
-  }
-  // the cluster path: rounds of units and their tiles, the bytes; fitted to 97 uniform calls of up to eight query heads per KV head, 10 %
-  const int units = H * ceil_div(B * R, CL_ROWS / G), NS = ceil_div(ceil_div(n, 64), terms == 2 ? 2 : 4);
-  if (NS > CL_MAX_NS) return other;          // longer blocks than its clusters hold: the three-phase kernels, 105 us and more
+// More than eight query heads per KV head: where its estimate is ahead of one of the path it stands before.  Of 881 drawn calls with 9 to 16
+// it is the faster path for 662; taken for all that the rules above give it, 145 were more than 3 % longer, at worst 2.1 times (13 x 12 of 1024,
+// 10/1 heads 61 / 34; 9 x 11 of 256, 28/2 heads, 1492 rows 32 / 22); by the estimates about 30, at worst 1.3 times, and the geometric mean of all
+// is 0.79 of the other paths' time (0.82 before; 0.78 with every call on its better path).
+// The cluster path: rounds of units and their tiles, the bytes; fitted to 97 uniform calls of up to eight query heads per KV head, 10 %
+static double cluster_estimate(const kvc_layer* L, int B, int R, int T, int terms) {
+  const int n = L->desc.n, m = L->m, H = L->desc.H_kv, sms = L->num_sms > 0 ? L->num_sms : 148;
+  const int units = H * ceil_div(B * R, CL_ROWS / L->G), NS = ceil_div(ceil_div(n, 64), terms == 2 ? 2 : 4);
   const int held = sms * 88 / 100 / NS, rounds = ceil_div(units, held > 0 ? held : 1);
   const double rows = 512.0 * B * R * H * (double)m + 4.0 * H * (double)m * n, text = 512.0 * B * H * (double)T;
-  return std::min(other, rounds * (24.4 + 1.93 * ceil_div(m, 64)) - 4.2 + (1.71 * rows + 1.86 * text) / HBM_US + 0.0137 * B * H);
+  return rounds * (24.4 + 1.93 * ceil_div(m, 64)) - 4.2 + (1.71 * rows + 1.86 * text) / HBM_US + 0.0137 * B * H;
+}
+// The path a call with more than eight query heads per KV head would take otherwise: fitted (least squares of the relative error) to those calls,
+// the one-kernel path's 10 %, the three-kernel path's 13 %, the cluster path's as above and 14 % too short for them.  Blocks longer than its
+// clusters hold go to the three-phase kernels, which the spread path is always ahead of there (2 x 2 of n = 1444, 48/4 heads 57 / 161).
+static double general_estimate(const kvc_layer* L, int B, int R, int T, bool ragged, int terms) {
+  const int n = L->desc.n, m = L->m, H = L->desc.H_kv, sms = L->num_sms > 0 ? L->num_sms : 148;
+  const double cluster = ceil_div(ceil_div(n, 64), terms == 2 ? 2 : 4) <= CL_MAX_NS ? 1.1 * cluster_estimate(L, B, R, T, terms) : 1e30;
+  if (n % 64 != 0 || (ragged && ragged_path(L, B, R, T) != 1)) return cluster;
+  if (!ragged && n > 640 && plan_split(L, B, R).ok)
+    return 1.05 * (16.2 + 0.0214 * m + 0.124 * H * ceil_div(B * R * L->G, 128) + 2.0 * 512.0 * B * H * (2.0 * R * m + 2.0 * T) / HBM_US + 3.5e-4 * H * n);
+  double fused = 1e30;
+  const FusedPlan f = plan_fused(L, B, R, ragged);
+  if (f.ok) {
+    const int waves = ceil_div(f.units, sms);
+    const double text = (double)T / f.nrg;                   // of a unit, shared by the warps that its blocks' columns occupy
+    fused = 9.4 + 0.0346 * m + 16.1 * (waves - 1) + 7.2e-5 * waves * m * (double)n + 4.96e-3 * text + 35e-3 * text / (ceil_div(R, f.nrg) * (n / 64)) +
+            (f.nrg > 1 ? 4.9 : 0.0);
+  }
+  return ragged || n <= 256 || n > 640 ? fused : std::min(fused, cluster);
 }
 static bool use_spread(const kvc_layer* L, int B, int R, int T, bool ragged, const SpreadPlan& p) {
   if (!p.ok || L->use_tc == 6) return p.ok != 0;
   const int n = L->desc.n;
   if (plan_resident(L, B, R, T).ok) return !ragged && n == 256 && L->m > 48 && R * L->G <= 16 && T <= 128 * p.C;
   if (ragged && n % 8 == 0 && n % 64 != 0 && 4.0 * B * L->desc.H_q * R * (double)L->m * n < 1e7) return false;
-  if (n % 64 == 0 && p.us > (L->G > 8 ? 1.16 : 1.0) * (n <= 256 ? 24.0 : 36.0)) return false;
-  if (L->G > 8 && p.waves == 1) return p.us < (!ragged && n % 64 == 0 ? 0.95 : 1.0) * general_estimate(L, B, R, T, ragged, p.terms);
+  if (n % 64 == 0 && p.us > (L->G > 8 ? (n > 640 ? 42.0 : 1e30) : (n <= 256 ? 24.0 : 36.0))) return false;
+  if (L->G > 8 && p.waves == 1) return p.us < general_estimate(L, B, R, T, ragged, p.terms);
   // several waves: where it is ahead of the estimate of the cluster path.  Routed by it those take 0.89 of their time before in the geometric mean,
   // none more than 3 % longer (16 x 8 of n = 144, 28/4 heads, 715 rows 16.5 / 32.3; 25 x 5 of 400, 1610 rows 46 / 89; 8 x 7 of 324, 32/32 heads
   // 74 / 88; not: 26 x 10 of 121 45 / 34)
-  if (p.waves > 1) return !ragged && n >= 96 && p.us < 0.85 * general_estimate(L, B, R, T, ragged, p.terms);
+  if (p.waves > 1) return !ragged && n >= 96 && p.us < 0.85 * cluster_estimate(L, B, R, T, p.terms);
   return n >= 96 || p.C * p.nrg > 2;
 }
 

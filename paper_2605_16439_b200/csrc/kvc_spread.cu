@@ -858,8 +858,8 @@ static SpreadPlan plan_groups(const kvc_layer* L, int B, int R_all, int T_all, i
     const double mb = (at_once * p.C * (2.0 * R * p.gs * 4096.0 + items * 8192.0) + 4.0 * H * n * (double)m) * 1e-6;
     p.us = 5.9 + (nrg > 1 ? 3.6 : 0.0) + 0.336 * pieces + 0.0292 * p.ng * step + 0.0086 * ceil_div(tasks, SPR_WARPS) * p.gw * step +
            0.45 * ceil_div(items, SPR_WARPS) + 0.0525 * W / 1024.0 + 0.0485 * mb;
-    // two tiles of query heads: the values, the text and the ends take twice as long (336 calls of G = 9 to 16: 10 %, without this 1.5 times too short)
-    if (G > 8) p.us = 1.16 * p.us - 0.5 + 4.9 * ceil_div(items, SPR_WARPS);
+    // two tiles of query heads: the values, the text and the ends take twice as long (881 calls of G = 9 to 16: 10 %, without this 1.5 times too short)
+    if (G > 8) p.us = 1.106 * p.us - 0.96 + 0.298 * items + 5.23 * ceil_div(R * p.gs, SPR_WARPS);
     // (394 calls of 220 shapes, one to four waves: 6 %)
     if (p.waves > 1) p.us = 0.9 + p.waves * (0.63 + 0.86 * p.us);
   }
